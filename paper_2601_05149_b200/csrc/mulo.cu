@@ -13,6 +13,7 @@
 #include "mulo_islands.cuh"
 #include "mulo_lane.cuh"
 #include "mulo_full.cuh"
+#include "mulo_rows.cuh"
 #include "mulo_stream.cuh"
 
 using namespace mulo;
@@ -967,6 +968,83 @@ static size_t plan_lane(const mulo_ctx* ctx, const DevParams& d, LaneArgs* s) {
   return dyn;
 }
 
+// ---- rows with a top-k cut, NW warps per row (mulo_rows.cuh) ----------------------------
+
+#ifndef MULO_RNW
+#define MULO_RNW 2
+#endif
+constexpr int kRowsWarps = MULO_RNW;
+
+// Fills `s` and returns the dynamic shared memory of a CTA, or 0 if these parameters are not eligible.
+static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, int nw, RowsArgs* s) {
+  if (d.top_k <= 0 || (d.pool_k > 1 && !sample)) return 0;
+  const int V = d.V, k = d.top_k;
+  if (V < 1024 || d.r > 4) return 0;
+  const int esz = d.bf16 ? 2 : 4, ids = 16 / esz;
+  // Candidates aimed for beyond k: 3.5 standard deviations of the count of entries above a fixed value near the
+  // k-th largest (a row that misses, about one in two thousand, is streamed again); more for rows without a
+  // prediction.
+  const double p = (double)k / V;
+  const int margin = (int)fmax(48.0, 3.5 * sqrt(k * (1.0 - p)));
+  const int margin_boot = margin + 3 * margin / 4;
+  if ((double)(k + margin_boot) > 0.5 * V) return 0;
+  s->row_bytes = (uint32_t)(V * esz);
+  const int pieces = (int)((s->row_bytes + kRPieceBytes - 1) / kRPieceBytes);
+  s->ppw = (pieces + nw - 1) / nw;
+  s->n_words = (s->ppw + 3) / 4;
+  // A list column holds the candidates of two threads: their share plus 3.6 standard deviations of that
+  // binomial count (3 for a row without prediction); a thread's own at most 64.
+  auto rows_for = [&](int count, double threads, double dev) {
+    const double pc = (double)count / V, mu = threads * s->ppw * ids * pc;
+    return mu + dev * sqrt(mu * (1.0 - pc));
+  };
+  if (rows_for(k + margin, 1.0, 4.5) > 64.0) return 0;
+  s->R = (int)ceil(fmax(rows_for(k + margin, 2.0, 3.6), rows_for(k + margin_boot, 2.0, 3.0))) + 1 + kRSlack;
+  if (s->R < 32) s->R = 32;
+  s->margin = margin;
+  s->a_theta = (float)inv_norm_cdf(1.0 - p);
+  s->a_boot = (float)inv_norm_cdf(1.0 - (double)(k + margin_boot) / V);
+  s->a_max = (float)inv_norm_cdf(1.0 - 0.5 / V);
+  const size_t dyn = rows_layout(*s, nw, d.bf16, sample);
+  if (2 * (dyn + sizeof(RowsSmem<8>) + 1024) > (size_t)ctx->smem_optin) return 0;   // too few rows in flight per SM
+  return dyn;
+}
+
+template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
+static bool launch_rows_p(const mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
+  auto kern = k_round_rows<BF16, HAS_U, SAMPLE, PLAIN, NW>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, dyn) != cudaSuccess || per_sm < 1) {
+    cudaGetLastError();
+    return false;
+  }
+  int grid = ctx->sm_count * per_sm;
+  if (grid > s.n_units) grid = s.n_units;
+  kern<<<grid, NW * 32, dyn, st>>>(s);
+  return true;
+}
+
+template <bool BF16, bool HAS_U, bool SAMPLE, int NW>
+static bool launch_rows_t(const mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
+  const bool plain = s.P.invT == 1.0f && s.row_bytes % (4u * kRPieceBytes * NW) == 0;
+  return plain ? launch_rows_p<BF16, HAS_U, SAMPLE, true, NW>(ctx, s, dyn, st)
+               : launch_rows_p<BF16, HAS_U, SAMPLE, false, NW>(ctx, s, dyn, st);
+}
+
+template <int NW>
+static bool launch_rows(const mulo_ctx* ctx, const RowsArgs& s, bool sample, size_t dyn, cudaStream_t st) {
+  const bool hu = s.uncond != nullptr;
+  if (sample)
+    return s.P.bf16 ? launch_rows_t<true, false, true, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, true, NW>(ctx, s, dyn, st);
+  if (s.P.bf16)
+    return hu ? launch_rows_t<true, true, false, NW>(ctx, s, dyn, st) : launch_rows_t<true, false, false, NW>(ctx, s, dyn, st);
+  return hu ? launch_rows_t<false, true, false, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, false, NW>(ctx, s, dyn, st);
+}
+
 // ---- rows without a top-k cut: the resident-row kernel ------------------------------------
 // Eligible: top-k off, V = 256 * W with W a multiple of the ids in 16 bytes, and the rows of one
 // position (draft row if q is needed, conditional, unconditional) within a CTA's shared memory.
@@ -1172,6 +1250,22 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
   // fast path: the streaming kernel in its sampling mode (top-k on, and a workspace large
   // enough for the list of cells it may leave to the general routines)
   Workspace w;
+  RowsArgs ra;
+  memset(&ra, 0, sizeof ra);
+  const size_t rdyn = (ctx->force_dense || check_ws(ctx, p, &w) != MULO_OK) ? 0 : plan_rows(ctx, a.P, true, kRowsWarps, &ra);
+  if (rdyn) {
+    ra.P = a.P;
+    ra.cond = a.draft;
+    ra.sample_out = draft_tok_lo;
+    ra.dev_status = w.status;
+    ra.fail_list = w.fail_list;
+    ra.n_units = p->B * a.P.h * a.P.w;
+    if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
+    if (launch_rows<kRowsWarps>(ctx, ra, true, rdyn, st)) {
+      k_sample_failed<<<2 * ctx->sm_count, kThreads, 0, st>>>(a, w.fail_list, w.status + kFailCount);
+      return launched(ctx, 2);
+    }
+  }
   StreamArgs sa;
   memset(&sa, 0, sizeof sa);
   const size_t sdyn = (ctx->force_dense || check_ws(ctx, p, &w) != MULO_OK) ? 0 : plan_stream(ctx, a.P, &sa);
@@ -1378,6 +1472,21 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     fa.n_parents = p->B * a.P.h * a.P.w;
     fast = launch_full(ctx, fa, fdyn, st);
     if (fast) fast_launches = 1;
+  }
+  RowsArgs ra;
+  memset(&ra, 0, sizeof ra);
+  const size_t rdyn = (ctx->force_dense || ctx->no_lane || fast) ? 0 : plan_rows(ctx, a.P, false, kRowsWarps, &ra);
+  if (rdyn) {
+    ra.P = a.P;
+    ra.cond = a.cond; ra.uncond = a.uncond; ra.draft = a.draft; ra.draft_tok_lo = draft_tok_lo;
+    ra.p_tok = p_tok; ra.q_tok = q_tok; ra.accept_prob = accept_prob;
+    ra.flags = w.flags; ra.cand_res = w.cand_res; ra.cand_tgt = w.cand_tgt;
+    ra.dev_status = w.status;
+    ra.fail_list = w.fail_list;
+    ra.n_units = p->B * p->H * p->W;
+    if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
+    fast = launch_rows<kRowsWarps>(ctx, ra, false, rdyn, st);
+    if (fast) k_verify_failed<<<2 * ctx->sm_count, kThreads, dyn, st>>>(a, w.fail_list, w.status + kFailCount);
   }
   LaneArgs la;
   memset(&la, 0, sizeof la);

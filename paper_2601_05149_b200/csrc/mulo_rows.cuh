@@ -1,0 +1,1041 @@
+// The fast path for rows with a top-k cut: NW warps per row.
+//
+// A CTA owns a contiguous range of target rows (in parent order).  Per parent it streams the draft row and then
+// the target rows under it, each ONCE.  Warp w owns the w-th contiguous NW-th of the ids.
+//
+//   stream     512-byte pieces of the warp's part (16 bytes per lane) through registers, kRDepth pieces in
+//              flight per warp, the next row asked into L2 by a bulk prefetch.  Per id: unpack, CFG mix (packed
+//              fp32, one IEEE rounding per step), compare with a predicted pivot and a predicated append to the
+//              thread's PRIVATE list plus a bit in its survivor mask (one word per four pieces).  The loads run
+//              on into the next row, so a row's first pieces are in registers when its turn comes.
+//   lists      threads t and t + 32 (of an even and the next odd warp) share a column of R rows, growing towards
+//              each other.
+//   first pass over the list: exp against a predicted maximum.  Entries above the selection window are done
+//              with here (their exp replaces the logit in the list); those in the window go into a 256-bin
+//              histogram and a bit mask.
+//   selection  the bin that holds the k-th largest; the window's entries once more: above the bin -> exp, below
+//              -> 0, in the bin -> set aside, ranked exactly, written back.  From here on the list holds the
+//              row's weights, zeros below the threshold included.
+//   draws      warp sums of p (target) or of max(0, p - q) (residual; the sum of p minus that of min(p, q) over
+//              the ids that both rows kept, found by intersecting the masks).  The warp that owns u * total walks
+//              its part -- mask word, piece, lane, id -- while the others go on with the next row.
+//
+// Three block barriers per row.  Pivot, histogram scale and exp reference are predicted from the CTA's previous
+// rows of the same kind; a row without prediction takes them from the mean and spread of its first pieces.  A
+// row whose prediction misses (too few candidates, a full column, rank beyond the histogram, maximum far from the
+// reference) is streamed again with corrected values; one that still fails, or has too many ties at the
+// threshold, goes to a list that a second launch works off with the general routines, so results never depend
+// on the prediction.
+#pragma once
+
+#include "mulo_lane.cuh"
+
+namespace mulo {
+
+#ifndef MULO_RDEPTH
+#define MULO_RDEPTH 4
+#endif
+#ifndef MULO_RWARPS
+#define MULO_RWARPS 16
+#endif
+constexpr int kRDepth = MULO_RDEPTH;     // pieces in flight per warp
+constexpr int kRPieceBytes = 512;        // 16 bytes per lane
+constexpr int kRBins = 256;
+constexpr int kRSetAside = 128;          // entries of the crossing bin that are ranked exactly
+constexpr int kRTries = 6;               // times a row is streamed before it is given up
+constexpr int kRSlack = 8;               // list rows kept free between the two lists of a column: one piece's entries
+constexpr float kRMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
+
+struct RowsArgs {
+  DevParams P;
+  const char* cond;
+  const char* uncond;
+  const char* draft;
+  const int32_t* draft_tok_lo;
+  float* p_tok;
+  float* q_tok;
+  float* accept_prob;
+  uint8_t* flags;
+  int32_t* cand_res;
+  int32_t* cand_tgt;
+  int32_t* sample_out;      // SAMPLE: the drafter's token per cell
+  uint32_t* dev_status;
+  int32_t* fail_list;
+  int n_units;              // target rows, parent by parent (SAMPLE: low-res cells)
+  uint32_t row_bytes;
+  int ppw;                  // pieces of a warp's part of a row
+  int n_words;              // mask words per thread: ceil(ppw / 4)
+  int R;                    // rows of a list column (shared by two threads)
+  uint32_t o_dlist, o_tmask, o_dmask;   // dynamic shared memory: the lists first, then these
+  int margin;
+  float a_theta, a_boot, a_max;
+};
+
+template <int NW>
+struct RowsSmem {
+  alignas(16) unsigned hist[kRBins + 4];   // (+ one bin that rounding may reach)
+  alignas(16) float closer[4][32];         // -inf: what a thread past its list's end reads
+  alignas(16) float sa_z[kRSetAside];      // (before the set-aside: where such a thread writes)
+  unsigned short sa_at[kRSetAside];        // the entry's place (index in its owner's list << 8 | thread)
+  LanePredictor pred[2];                   // draft rows / target rows
+  double w_all[NW];                        // exp sums of each warp without the crossing bin
+  double w_t[NW], w_r[NW];                 // weights of a draw, per warp
+  double e_tok;
+  float z_tok;
+  uint32_t rnd[2][16][3];                  // uniforms of the parent's children, by parity of the parent
+  unsigned n_sa;
+  int wn[NW];
+  unsigned wmax[NW];
+  float red[NW][3];
+  unsigned char cnt[NW * 32];
+  unsigned char over[NW];
+};
+
+// Dynamic shared memory of a CTA (bytes); the parts' offsets go into `s`.
+inline uint32_t rows_layout(RowsArgs& s, int nw, bool bf16, bool sample) {
+  const uint32_t cols = (uint32_t)s.R * (uint32_t)(nw / 2);
+  uint32_t off = cols * 128u;   // the target row's lists
+  auto take = [&](uint32_t bytes) {
+    const uint32_t o = off;
+    off += bytes;
+    return o;
+  };
+  s.o_dlist = take(sample ? 0u : cols * (bf16 ? 64u : 128u));
+  s.o_tmask = take((uint32_t)s.n_words * nw * 128u);
+  s.o_dmask = sample ? s.o_tmask : take((uint32_t)s.n_words * nw * 128u);
+  return off;
+}
+
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// a logit of the draft list (bf16 or fp32)
+template <bool BF16>
+__device__ __forceinline__ void dlist_put(uint32_t addr, float z) {
+  if (BF16) asm volatile("{\n\t.reg .b16 h;\n\tcvt.rn.bf16.f32 h, %1;\n\tst.shared.b16 [%0], h;\n\t}" ::"r"(addr), "f"(z) : "memory");
+  else sts_f32(addr, z);
+}
+template <bool BF16>
+__device__ __forceinline__ float dlist_get(uint32_t addr) {
+  if (!BF16) return lds_f32(addr);
+  uint16_t v;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+  return __uint_as_float((uint32_t)v << 16);
+}
+__device__ __forceinline__ uint4 ldg_stream(const char* p) {   // 16 bytes, read once: not kept in L1
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+__device__ __forceinline__ void prefetch_l2(const char* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// Appends z to the thread's list if z >= pivot (cursor step: one list row of 128 bytes, up or down) and
+// marks its bit.
+template <int BIT>
+__device__ __forceinline__ void row_put(float z, float pivot, uint32_t& cur, uint32_t step, uint32_t& m) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ge.f32 p, %2, %3;\n\t"
+      "@p st.shared.f32 [%0], %2;\n\t"
+      "@p add.u32 %0, %0, %4;\n\t"
+      "@p or.b32 %1, %1, %5;\n\t}"
+      : "+r"(cur), "+r"(m)
+      : "f"(z), "f"(pivot), "r"(step), "n"(1u << BIT)
+      : "memory");
+}
+
+// The pre-processed logits of a piece (8 bf16 / 4 fp32 ids), two per packed instruction: d = c - u;
+// v = fma(s, d, u); z = v * invT, each half one IEEE rounding.
+template <bool BF16, bool ROW_U, bool SCALE, int J>
+__device__ __forceinline__ float2 row_pair(const uint4& c, const uint4& u, float2 s2, float2 t2) {
+  float2 v, un;
+  if (BF16) {
+    const uint32_t cw = word_of<J>(c);
+    v = make_float2(bf16_lo(cw), bf16_hi(cw));
+    if (ROW_U) {
+      const uint32_t uw = word_of<J>(u);
+      un = make_float2(bf16_lo(uw), bf16_hi(uw));
+    }
+  } else {
+    v = make_float2(__uint_as_float(word_of<(2 * J) & 3>(c)), __uint_as_float(word_of<(2 * J + 1) & 3>(c)));
+    if (ROW_U)
+      un = make_float2(__uint_as_float(word_of<(2 * J) & 3>(u)), __uint_as_float(word_of<(2 * J + 1) & 3>(u)));
+  }
+  if (ROW_U) v = __ffma2_rn(s2, __ffma2_rn(un, make_float2(-1.f, -1.f), v), un);   // fma(u, -1, c) rounds as c - u
+  if (SCALE) v = __fmul2_rn(v, t2);
+  return v;
+}
+template <bool BF16, bool ROW_U, bool SCALE, int BIT0>
+__device__ __forceinline__ void row_piece(const uint4& c, const uint4& u, float2 s2, float2 t2, float pivot,
+                                          uint32_t& cur, uint32_t step, uint32_t& m) {
+  float2 z = row_pair<BF16, ROW_U, SCALE, 0>(c, u, s2, t2);
+  row_put<BIT0>(z.x, pivot, cur, step, m);
+  row_put<BIT0 + 1>(z.y, pivot, cur, step, m);
+  z = row_pair<BF16, ROW_U, SCALE, 1>(c, u, s2, t2);
+  row_put<BIT0 + 2>(z.x, pivot, cur, step, m);
+  row_put<BIT0 + 3>(z.y, pivot, cur, step, m);
+  if (BF16) {
+    z = row_pair<BF16, ROW_U, SCALE, 2>(c, u, s2, t2);
+    row_put<(BIT0 + 4) & 31>(z.x, pivot, cur, step, m);
+    row_put<(BIT0 + 5) & 31>(z.y, pivot, cur, step, m);
+    z = row_pair<BF16, ROW_U, SCALE, 3>(c, u, s2, t2);
+    row_put<(BIT0 + 6) & 31>(z.x, pivot, cur, step, m);
+    row_put<(BIT0 + 7) & 31>(z.y, pivot, cur, step, m);
+  }
+}
+
+// Double division, out of line.
+__device__ __noinline__ double rows_div(double a, double b) { return a / b; }
+
+// PLAIN: T = 1 and every piece a thread's whole 16 bytes (V splits evenly), so no scaling and no bounds checks.
+template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
+__global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
+  constexpr int NT = NW * 32;
+  constexpr int IDS = BF16 ? 8 : 4;              // ids per lane per piece
+  constexpr int PIECE_BITS = (1 << IDS) - 1;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  __shared__ RowsSmem<NW> sm;
+  const DevParams& P = a.P;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int unit = (int)(((long long)a.n_units * blockIdx.x) / gridDim.x);
+  const int u_end = (int)(((long long)a.n_units * (blockIdx.x + 1)) / gridDim.x);
+  if (unit >= u_end) return;
+  const int rr = SAMPLE ? 1 : P.r * P.r;
+  const uint32_t row_bytes = a.row_bytes;
+  const int n_words = a.n_words, R = a.R;
+
+  // ---- this thread's places in shared memory.  Lists grow upwards (even warps) or downwards (odd warps).
+  const bool up = (warp & 1) == 0;
+  const uint32_t my = smem_u32(dyn);
+  const uint32_t first_row = (uint32_t)(warp >> 1) * (uint32_t)R + (up ? 0u : (uint32_t)(R - 1));
+  const uint32_t step = up ? 128u : 0u - 128u;
+  const uint32_t tl = my + (uint32_t)lane * 4u + first_row * 128u;
+  const uint32_t low4 = up ? 0u : 0u - 384u;       // from an entry to the lowest address of the four from it on
+  // the draft row's kept logits (bf16 if they came as such: exact, half the memory)
+  constexpr uint32_t DROW = BF16 ? 64u : 128u;
+  const uint32_t dstep = up ? DROW : 0u - DROW;
+  const uint32_t dl = my + a.o_dlist + (uint32_t)lane * (DROW / 32u) + first_row * DROW;
+  const uint32_t tm = my + a.o_tmask + (uint32_t)tid * 4u, dm = my + a.o_dmask + (uint32_t)tid * 4u;
+  const uint32_t hbase = smem_u32(sm.hist) - (__float_as_uint(kRMagic) << 2);
+  const uint32_t closer = smem_u32(sm.closer) + (uint32_t)lane * 4u, dump = smem_u32(sm.sa_z) + (uint32_t)lane * 4u;
+
+#pragma unroll 1
+  for (int i = tid; i < kRBins + 4; i += NT) sm.hist[i] = 0;
+#pragma unroll 1
+  for (int i = tid; i < 128; i += NT) (&sm.closer[0][0])[i] = -INFINITY;
+  if (tid < 2) {
+    LanePredictor& pr = sm.pred[tid];
+    pr.have = 0;
+    pr.age = 0;
+    pr.theta = 0.f; pr.rho = 1.f; pr.mx = 0.f;
+    pr.pivot = 0.f; pr.inv_w = 0.f; pr.ref = 0.f;
+    pr.shift = 0.f; pr.step = 0.f; pr.dir = 0;
+    sm.n_sa = 0;
+  }
+  __syncthreads();
+
+  // ---- where the current row is.  parent = low-res cell (b, ca, cc); child (di, dj) of a target row.
+  int parent, b, ca, cc, di = 0, dj = 0;
+  {
+    parent = unit / rr;
+    const int child = unit - parent * rr, hw = P.h * P.w;
+    b = parent / hw;
+    const int rem = parent - b * hw;
+    ca = rem / P.w;
+    cc = rem - ca * P.w;
+    if (!SAMPLE) {
+      di = child / P.r;
+      dj = child - di * P.r;
+    }
+  }
+  auto target_index = [&]() -> uint32_t {
+    return ((uint32_t)b * P.H + (uint32_t)(ca * P.r + di)) * P.W + (uint32_t)(cc * P.r + dj);
+  };
+  auto next_parent = [&]() {
+    ++parent;
+    di = dj = 0;
+    if (++cc == P.w) {
+      cc = 0;
+      if (++ca == P.h) {
+        ca = 0;
+        ++b;
+      }
+    }
+  };
+
+  // ---- this thread's part of a row: np pieces from part_off on
+  const uint32_t part_off = (uint32_t)(warp * a.ppw) * kRPieceBytes + (uint32_t)lane * 16u;
+  const int np = part_off < row_bytes ? min(a.ppw, (int)((row_bytes - part_off + kRPieceBytes - 1) / kRPieceBytes)) : 0;
+  uint4 c[kRDepth], u[kRDepth];   // the pieces in flight
+  const uint4 none = make_uint4(~0u, ~0u, ~0u, ~0u);   // NaN in either type: never appended
+#pragma unroll
+  for (int j = 0; j < kRDepth; ++j) c[j] = u[j] = none;
+  auto prologue = [&](const char* rc, const char* ru) {
+#pragma unroll
+    for (int j = 0; j < kRDepth; ++j) {
+      c[j] = j < np ? ldg_stream(rc + j * kRPieceBytes) : none;
+      if (HAS_U) u[j] = j < np && ru ? ldg_stream(ru + j * kRPieceBytes) : none;
+    }
+  };
+  const float2 s2 = make_float2(P.cfg_scale, P.cfg_scale), t2 = make_float2(P.invT, P.invT);
+
+  // ---- one row through the registers into the list; the loads run on into the row (nc, nu).  Returns
+  //      the list's end.  (All row pointers are this thread's: part_off is in them.)
+  auto stream_t = [&](auto row_u_tag, const char* rc, const char* ru, const char* nc, const char* nu, float pivot,
+                      uint32_t cur, uint32_t lim, uint32_t mask_at) -> uint32_t {
+    constexpr bool ROW_U = decltype(row_u_tag)::value;
+#pragma unroll 1
+    for (int w = 0; w < n_words; ++w) {
+      const bool last = w + 1 == n_words;
+      // the pieces to ask for: kRDepth ahead; those of the next word may be the next row's first
+      const char* const fc = last ? nc : rc + 4 * kRPieceBytes;
+      const char* const fu = !HAS_U ? nullptr : last ? nu : ROW_U ? ru + 4 * kRPieceBytes : nullptr;
+      const bool do_u = HAS_U && fu != nullptr;
+      const int f0 = last ? 0 : 4 * w + 4;
+      uint32_t m = 0;
+#define MULO_PIECE(J)                                                                                      \
+  {                                                                                                        \
+    constexpr int S = J % kRDepth, A = (J + kRDepth) & 3;                                                  \
+    constexpr bool SAME = J + kRDepth < 4;                                                                 \
+    cur = up ? min(cur, lim) : max(cur, lim);                                                              \
+    row_piece<BF16, ROW_U, !PLAIN, J * IDS>(c[S], u[S], s2, t2, pivot, cur, step, m);                      \
+    const char* const pc = SAME ? rc : fc;                                                                 \
+    const char* const pu = SAME ? ru : fu;                                                                 \
+    const bool want_u = SAME ? ROW_U : do_u;                                                               \
+    if (PLAIN) {                                                                                           \
+      c[S] = ldg_stream(pc + A * kRPieceBytes);                                                            \
+      if (HAS_U && want_u) u[S] = ldg_stream(pu + A * kRPieceBytes);                                       \
+    } else {                                                                                               \
+      const bool in = (SAME ? 4 * w : f0) + A < np;                                                        \
+      c[S] = in ? ldg_stream(pc + A * kRPieceBytes) : none;                                                \
+      if (HAS_U) u[S] = in && want_u ? ldg_stream(pu + A * kRPieceBytes) : none;                           \
+    }                                                                                                      \
+  }
+      MULO_PIECE(0) MULO_PIECE(1) MULO_PIECE(2) MULO_PIECE(3)
+#undef MULO_PIECE
+      sts_u32(mask_at + (uint32_t)(w * NT) * 4u, m);
+      rc += 4 * kRPieceBytes;
+      if (HAS_U && ROW_U) ru += 4 * kRPieceBytes;
+    }
+    return cur;
+  };
+
+  // ---- pivot, histogram scale and exp reference of a row whose first pieces are in registers
+  auto boot_pivot = [&](bool row_u, float shift, float& pivot, float& inv_w, float& ref, float& per) {
+    float s1 = 0.f, sq = 0.f, cnt = 0.f;
+    auto add = [&](float z) {
+      if (z == z) {
+        s1 += z;
+        sq += z * z;
+        cnt += 1.f;
+      }
+    };
+#pragma unroll
+    for (int j = 0; j < kRDepth; ++j) {
+      const uint32_t cw[4] = {c[j].x, c[j].y, c[j].z, c[j].w}, uw[4] = {u[j].x, u[j].y, u[j].z, u[j].w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (BF16) {
+          add(mix_logit(bf16_lo(cw[k]), bf16_lo(uw[k]), row_u, P.cfg_scale, P.invT));
+          add(mix_logit(bf16_hi(cw[k]), bf16_hi(uw[k]), row_u, P.cfg_scale, P.invT));
+        } else {
+          add(mix_logit(__uint_as_float(cw[k]), __uint_as_float(uw[k]), row_u, P.cfg_scale, P.invT));
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s1 += __shfl_xor_sync(kFull, s1, o);
+      sq += __shfl_xor_sync(kFull, sq, o);
+      cnt += __shfl_xor_sync(kFull, cnt, o);
+    }
+    if (lane == 0) {
+      sm.red[warp][0] = s1;
+      sm.red[warp][1] = sq;
+      sm.red[warp][2] = cnt;
+    }
+    __syncthreads();
+    s1 = sq = cnt = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      s1 += sm.red[w][0];
+      sq += sm.red[w][1];
+      cnt += sm.red[w][2];
+    }
+    __syncthreads();
+    const float mean = s1 / cnt;
+    const float sd = sqrtf(fmaxf(sq / cnt - mean * mean, 1e-20f));
+    const float d = fmaxf((a.a_theta - a.a_boot) * sd, 1e-20f);
+    pivot = mean + (a.a_boot + shift) * sd;
+    inv_w = (float)kRBins / (3.0f * d);   // (a predicted row's histogram spans 2 d)
+    ref = mean + a.a_max * sd;
+    per = d / (1.75f * (float)a.margin);  // distance per candidate near the pivot
+  };
+
+  bool is_q = !SAMPLE;                    // the row in work is a draft row
+  uint32_t g = (uint32_t)parent;          // ... and its index in its tensor
+
+  // ---- first pass over the list (see the top of the file); returns the exp sum of the entries above the window.
+  //      A draft row (Q) puts its logits into the draft list instead of their exps into its own.  Written with
+  //      predicated PTX: left to the compiler, every entry becomes two branches.
+  auto pass_one = [&](auto q_tag, int n, float inv_w, float hoff, float c0, uint32_t& low_a, uint32_t& low_b) -> float {
+    constexpr bool Q = decltype(q_tag)::value;
+    const int n_max = __reduce_max_sync(kFull, n);
+    float mx = -INFINITY, s0 = 0.f, s1 = 0.f;
+    low_a = low_b = 0;
+    const uint32_t end = tl + (uint32_t)n * step;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) sts_f32(end + (uint32_t)k * step, -INFINITY);
+    const float hm = hoff + kRMagic;
+    const float T = 1.0f / P.invT;   // (fl(v * invT) * T rounds back to the bf16 value v)
+    uint32_t ad = tl + low4, dd = dl + (up ? 0u : 0u - 3u * DROW);
+#pragma unroll 1
+    for (int i = 0; i < n_max; i += 4, ad += 4 * step, dd += 4 * dstep) {
+      const bool in = i < n;
+      const uint32_t from = in ? ad : closer, to = in ? ad : dump;
+      float z[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) z[k] = lds_f32(from + k * 128);
+      uint32_t l4 = 0;
+#define MULO_ENTRY(K, S)                                                                       \
+  {                                                                                            \
+    const float e = ex2f(fmaf(z[K], kLog2e, c0));                                              \
+    const uint32_t bin = __float_as_uint(fmaf(z[K], inv_w, hm));                               \
+    if (Q)                                                                                     \
+      asm volatile(                                                                            \
+          "{\n\t.reg .pred p;\n\t.reg .u32 t;\n\t"                                             \
+          "sub.u32 t, %2, %3;\n\t"                                                             \
+          "setp.le.u32 p, t, %4;\n\t"                                                          \
+          "@p red.shared.add.u32 [%5], 1;\n\t"                                                 \
+          "@p or.b32 %0, %0, %6;\n\t"                                                          \
+          "@!p add.f32 %1, %1, %7;\n\t}"                                                       \
+          : "+r"(l4), "+f"(S)                                                                  \
+          : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(hbase + (bin << 2)), "n"(1 << K), "f"(e) \
+          : "memory");                                                                         \
+    else                                                                                       \
+      asm volatile(                                                                            \
+          "{\n\t.reg .pred p;\n\t.reg .u32 t;\n\t"                                             \
+          "sub.u32 t, %2, %3;\n\t"                                                             \
+          "setp.le.u32 p, t, %4;\n\t"                                                          \
+          "@p red.shared.add.u32 [%5], 1;\n\t"                                                 \
+          "@p or.b32 %0, %0, %6;\n\t"                                                          \
+          "@!p add.f32 %1, %1, %7;\n\t"                                                        \
+          "@!p st.shared.f32 [%8 + %9], %7;\n\t}"                                              \
+          : "+r"(l4), "+f"(S)                                                                  \
+          : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(hbase + (bin << 2)), "n"(1 << K), "f"(e), "r"(to), "n"(K * 128) \
+          : "memory");                                                                         \
+    if (Q && in) dlist_put<BF16>(dd + K * DROW, BF16 && !PLAIN ? __fmul_rn(z[K], T) : z[K]);   \
+  }
+      MULO_ENTRY(0, s0) MULO_ENTRY(1, s1) MULO_ENTRY(2, s0) MULO_ENTRY(3, s1)
+#undef MULO_ENTRY
+      mx = fmaxf(mx, fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])));
+      if (i < 32) low_a |= l4 << i;   // (uniform)
+      else low_b |= l4 << (i & 31);
+    }
+    const unsigned mk = __reduce_max_sync(kFull, float_key(mx));
+    const int nw = __reduce_add_sync(kFull, n);
+    sm.cnt[tid] = (unsigned char)n;
+    if (lane == 0) {
+      sm.wn[warp] = nw;
+      sm.wmax[warp] = mk;
+    }
+    return s0 + s1;
+  };
+
+  // ---- the window's entries once more (after the crossing bin is known): the exp of those above it and 0 for those
+  //      below replace the logit (draft row: those below leave the draft list); returns the exp sum of those above
+  auto window = [&](uint32_t low_a, uint32_t low_b, float inv_w, float hoff, float c0, int bstar) -> float {
+    const float hm = hoff + kRMagic;
+    const uint32_t bm = __float_as_uint(kRMagic) + (uint32_t)bstar;
+    const uint32_t flip = up ? 0u : 3u;
+    float s = 0.f;
+    uint32_t first = 0;
+    auto one = [&](uint32_t bit) {
+      const uint32_t i = first + ((uint32_t)__popc(bit - 1u) ^ flip), at = tl + i * step;
+      const float z = lds_f32(bit ? at : closer);
+      const uint32_t bin = __float_as_uint(fmaf(z, inv_w, hm));   // (-inf: as unsigned above every bin; its exp is 0)
+      float e = ex2f(fmaf(z, kLog2e, c0));
+      e = bin > bm ? e : 0.f;
+      s += e;
+      if (is_q) {
+        if (bin < bm) dlist_put<BF16>(dl + i * dstep, -INFINITY);
+      } else if (bit) {
+        sts_f32(at, e);
+      }
+      if (bin == bm) {
+        const unsigned k = atomicAdd(&sm.n_sa, 1u) & (unsigned)(kRSetAside - 1);
+        sm.sa_z[k] = z;
+        sm.sa_at[k] = (unsigned short)(i << 8 | (uint32_t)tid);
+      }
+    };
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const int trips = __reduce_max_sync(kFull, __popc(low_a));
+#pragma unroll 1
+      for (int t = 0; t < trips; t += 2) {
+        const uint32_t b0 = low_a & (0u - low_a);
+        low_a ^= b0;
+        const uint32_t b1 = low_a & (0u - low_a);
+        low_a ^= b1;
+        one(b0);
+        one(b1);
+      }
+      low_a = low_b;
+      first = 32;
+    }
+    return s;
+  };
+
+  auto count_failure = [&](int reason) {   // one thread
+    if (reason < 1 || reason > 4) return;
+    const int slot = reason == 1 ? kCntListFull : reason == 2 ? kCntTooFew : reason == 3 ? kCntAboveRange : kCntCrowdedBin;
+    atomicAdd(a.dev_status + slot, 1u);
+  };
+  auto defer = [&](uint32_t g) {           // one thread: position (cell) g goes to the general routines
+    const unsigned at = atomicAdd(a.dev_status + kFailCount, 1u);
+    a.fail_list[at] = (int32_t)g;
+    atomicAdd(a.dev_status + kCntRows, 1u);
+    atomicOr(a.dev_status, MULO_DEV_DENSE_FALLBACK);
+  };
+
+  auto row_c = [&](bool q, uint32_t g) -> const char* { return (q ? a.draft : a.cond) + (size_t)g * row_bytes; };
+  auto row_u = [&](bool q, uint32_t g) -> const char* { return HAS_U && !q ? a.uncond + (size_t)g * row_bytes : nullptr; };
+  auto part = [&](const char* row) -> const char* { return row ? row + part_off : nullptr; };
+  auto prefetch = [&](const char* rc, const char* ru) {   // one thread
+    prefetch_l2(rc, row_bytes);
+    if (HAS_U && ru) prefetch_l2(ru, row_bytes);
+  };
+
+  int tries = 0, tok = 0, child = 0;      // child: which row under the parent
+  int partner_n = 0;                      // entries of the previous target row in the list this thread's list grows towards
+  float c0_q = 0.f, Zq = 1.f;             // of the parent's draft row
+  double q_tok = 0.0;
+  int tok_next = SAMPLE ? 0 : __ldg(a.draft_tok_lo + parent);
+  float pivot = 0.f, inv_w = 0.f, ref = 0.f, per = 0.f, lo = 0.f, hi = 0.f;   // of the row in work
+  prologue(part(row_c(is_q, g)), nullptr);
+  if (tid == 0) prefetch(row_c(is_q, g), nullptr);
+
+#pragma unroll 1
+  for (;;) {
+    const char* const rc = row_c(is_q, g);
+    const char* const ru = row_u(is_q, g);
+    // ---- the row after this one
+    bool nq = false, more = true;
+    uint32_t ng = 0;
+    if (SAMPLE) {
+      more = unit + 1 < u_end;
+      ng = more ? g + 1 : g;
+    } else if (is_q) {
+      ng = target_index();
+    } else if (unit + 1 >= u_end) {
+      more = false;
+      ng = g;
+    } else {
+      if (dj + 1 < P.r || di + 1 < P.r) {
+        if (++dj == P.r) {
+          dj = 0;
+          ++di;
+        }
+        ng = target_index();
+      } else {
+        nq = true;
+        ng = (uint32_t)parent + 1u;
+        tok_next = __ldg(a.draft_tok_lo + ng);
+      }
+    }
+    const char* const nc = row_c(nq, ng);            // (no row left: this one's first pieces again)
+    const char* const nu = more ? row_u(nq, ng) : nullptr;
+    // the logit of x~ in this row: asked for now, used after the first pass
+    float raw_c = 0.f, raw_u = 0.f;
+    if (!SAMPLE) {
+      if (is_q) {
+        tok = tok_next;
+        if (tok < 0 || tok >= P.V) {
+          if (tid == 0) atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
+          tok = min(max(tok, 0), P.V - 1);
+        }
+      }
+      if (warp == NW - 1) {
+        RowSrc src;
+        src.cond = rc; src.uncond = nullptr; src.s = 0.f; src.invT = 1.f; src.V = P.V; src.bf16 = BF16;
+        raw_c = load1(src, tok);
+        if (HAS_U && !is_q) {
+          src.cond = ru;
+          raw_u = load1(src, tok);
+        }
+      }
+    }
+
+    LanePredictor& pr = sm.pred[is_q ? 0 : 1];
+    if (tries == 0) {   // (a row streamed again keeps its corrected values)
+      lo = -INFINITY;
+      hi = INFINITY;
+      if (pr.have) {
+        pivot = pr.pivot;
+        inv_w = pr.inv_w;
+        ref = pr.ref;
+        per = 1.0f / pr.rho;
+      } else {
+        boot_pivot(HAS_U && !is_q, pr.shift, pivot, inv_w, ref, per);
+      }
+    }
+
+    const uint32_t mask_at = is_q ? dm : tm;
+    const uint32_t lim = tl + (uint32_t)(R - kRSlack - partner_n) * step;   // a piece appends at most 8 entries
+    const uint32_t end = HAS_U && !is_q
+                             ? stream_t(std::integral_constant<bool, HAS_U>{}, part(rc), part(ru), part(nc), part(nu), pivot, tl, lim, mask_at)
+                             : stream_t(std::false_type{}, part(rc), part(ru), part(nc), part(nu), pivot, tl, lim, mask_at);
+    if (more && tid == 0) prefetch(nc, nu);
+    const int n_raw = (int)(up ? end - tl : tl - end) >> 7;
+    const int n = min(n_raw, 64);
+    // (a list that passed its limit, or would leave its neighbour's next row no room)
+    const bool over = (up ? end > lim : end < lim) || n_raw > 64 || n_raw > R - 2 * kRSlack;
+    const float c0 = -ref * kLog2e, hoff = -pivot * inv_w;
+    uint32_t low_a, low_b;
+    float s_t = is_q ? pass_one(std::integral_constant<bool, !SAMPLE>{}, n, inv_w, hoff, c0, low_a, low_b)
+                     : pass_one(std::false_type{}, n, inv_w, hoff, c0, low_a, low_b);
+    {
+      const bool any_over = __any_sync(kFull, over);
+      if (lane == 0) sm.over[warp] = any_over;
+    }
+    if (!SAMPLE && warp == NW - 1) {
+      // the token's own weight, in double from the same exponent as the list entries (its z against theta later)
+      raw_c = mix_logit(raw_c, raw_u, HAS_U && !is_q, P.cfg_scale, P.invT);
+      const double e = lane_exp2((double)raw_c * (double)kLog2e + (double)c0);
+      if (lane == 0) {
+        sm.e_tok = e;
+        sm.z_tok = raw_c;
+      }
+    }
+    if (!SAMPLE && is_q && warp == 0 && lane < rr) {   // the uniforms of the parent's rows
+      const int ddi = lane / P.r, ddj = lane - ddi * P.r;
+      const uint32_t t = (uint32_t)(ca * P.r + ddi) * P.W + (uint32_t)(cc * P.r + ddj);
+      const uint4 v = lane_philox(make_uint4(t, (uint32_t)b + P.image_offset, P.round, 0u), make_uint2(P.seed_lo, P.seed_hi));
+      sm.rnd[parent & 1][lane][0] = v.x;
+      sm.rnd[parent & 1][lane][1] = v.y;
+      sm.rnd[parent & 1][lane][2] = v.z;
+    }
+    __syncthreads();   // ---- barrier 1
+    int n_all = 0, reason = 0;
+    unsigned mk = 0;
+    bool any_over = false;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      n_all += sm.wn[w];
+      mk = max(mk, sm.wmax[w]);
+      any_over |= sm.over[w] != 0;
+    }
+    const float mx = key_float(mk);
+    const int pair_n = sm.cnt[tid ^ 32];
+#pragma unroll
+    for (int w = 0; w < NW; w += 2)   // (three rows close each of the two lists)
+      any_over |= (int)sm.cnt[w * 32 + lane] + (int)sm.cnt[w * 32 + 32 + lane] + 6 > R;
+    if (__any_sync(kFull, any_over)) reason = 1;
+    else if (n_all < P.top_k) reason = 2;
+    else if (!(fabsf(mx - ref) <= kNearRefGap)) reason = 5;
+    unsigned cum = 0, in_bin = 0;
+    int bstar = 0;
+    const int rank = n_all - P.top_k + 1;   // 1-based rank from the bottom of the k-th largest
+    if (reason == 0) {
+      // ---- the bin that holds the k-th largest: which eight bins, then which of them
+      const uint4 h0 = *reinterpret_cast<const uint4*>(sm.hist + lane * 8);
+      const uint4 h1 = *reinterpret_cast<const uint4*>(sm.hist + lane * 8 + 4);
+      const unsigned own = ((h0.x + h0.y) + (h0.z + h0.w)) + ((h1.x + h1.y) + (h1.z + h1.w));
+      unsigned inc = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += t;
+      }
+      const unsigned owners = __ballot_sync(kFull, inc >= (unsigned)rank);
+      if (owners == 0) {
+        reason = 3;
+      } else {
+        const int src = __ffs(owners) - 1;
+        cum = __shfl_sync(kFull, inc - own, src);
+        const unsigned h = sm.hist[src * 8 + (lane & 7)];
+        inc = h;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+          const unsigned t = __shfl_up_sync(kFull, inc, o, 8);
+          if ((lane & 7) >= o) inc += t;
+        }
+        const int k = __ffs(__ballot_sync(kFull, cum + inc >= (unsigned)rank)) - 1;
+        bstar = src * 8 + k;
+        in_bin = __shfl_sync(kFull, h, k);
+        cum += __shfl_sync(kFull, inc - h, k);
+        if (in_bin > (unsigned)kRSetAside) reason = 4;
+      }
+    }
+    float theta = 0.f;
+    int n_ge = 0;
+    double Z = 0.0, w_own = 0.0;
+    if (reason == 0) {
+      s_t += window(low_a, low_b, inv_w, hoff, c0, bstar);
+      w_own = warp_sum((double)s_t);
+      if (lane == 0) sm.w_all[warp] = w_own;
+    }
+    __syncthreads();   // ---- barrier 2
+#pragma unroll 1
+    for (int i = tid; i < kRBins + 4; i += NT) sm.hist[i] = 0;
+    if (reason == 0) {
+      // ---- the crossing bin's entries: exact rank, and back into the lists
+      const int want = rank - (int)cum, mcount = (int)in_bin;
+      float vmin = INFINITY, vmax = -INFINITY;
+#pragma unroll 1
+      for (int i = lane; i < mcount; i += 32) {
+        const float v = sm.sa_z[i];
+        vmin = fminf(vmin, v);
+        vmax = fmaxf(vmax, v);
+      }
+      const unsigned kmin = __reduce_min_sync(kFull, float_key(vmin)), kmax = __reduce_max_sync(kFull, float_key(vmax));
+      int less_at = 0;
+      theta = key_float(kmin);
+      if (kmin != kmax) {   // several values in the bin: rank them
+        float th = 0.f;
+        bool found = false;
+#pragma unroll 1
+        for (int i = lane; i < mcount; i += 32) {
+          const float vi = sm.sa_z[i];
+          int less = 0, leq = 0;
+#pragma unroll 1
+          for (int k = 0; k < mcount; ++k) {
+            const float vk = sm.sa_z[k];
+            less += vk < vi;
+            leq += vk <= vi;
+          }
+          if (less < want && want <= leq) {
+            th = vi;
+            less_at = less;
+            found = true;
+          }
+        }
+        const unsigned fm = __ballot_sync(kFull, found);
+        const int fs = fm ? __ffs(fm) - 1 : 0;   // (always found: the bin holds the rank)
+        theta = __shfl_sync(kFull, th, fs);
+        less_at = __shfl_sync(kFull, less_at, fs);
+      }
+      n_ge = n_all - (int)cum - less_at;
+      double all = 0.0, own = 0.0;   // (values of one bin share their exponent: their sums in double are exact)
+#pragma unroll 1
+      for (int i = lane; i < mcount; i += 32) {
+        const float v = sm.sa_z[i];
+        const uint32_t at = sm.sa_at[i];
+        const float e = v >= theta ? ex2f(fmaf(v, kLog2e, c0)) : 0.f;
+        all += (double)e;
+        if ((int)((at & 0xffu) >> 5) == warp) {
+          own += (double)e;
+          const uint32_t col = (at & 31u) - (uint32_t)lane, idx = at >> 8;   // to the owner's column
+          if (!is_q) sts_f32(tl + col * 4u + idx * step, e);
+          else if (!(v >= theta)) dlist_put<BF16>(dl + col * (DROW / 32u) + idx * dstep, -INFINITY);
+        }
+      }
+      all = warp_sum(all);
+      own = warp_sum(own);
+      w_own += own;
+      Z = all;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) Z += sm.w_all[w];
+    }
+    const bool ok = reason == 0 && Z > 0.0 && Z < 1e300;
+    const bool again = !ok && reason != 0 && reason != 4 && tries + 1 < kRTries;
+    if (tid == 32 && !again)
+      lane_learn(&pr, ok, reason, theta, pivot, n_all, n_ge, mx, a.margin, a.a_theta, a.a_boot);
+
+    if (!ok) {   // CTA-uniform
+      __syncthreads();   // ---- barrier 3
+      if (tid == 0) sm.n_sa = 0;
+      partner_n = 0;     // (nothing of this row is read any more)
+      if (again) {
+        // once more, with the pivot moved by the candidates it was off by (a column was full: aim low in the
+        // margin; the values tried so far bracket it), or with the maximum just found
+        ++tries;
+        if (reason == 5) {
+          ref = mx;
+        } else {
+          const float aim = (float)P.top_k + (reason == 2 ? 0.75f : 0.3f) * (float)a.margin;
+          float next = pivot + ((float)n_all - aim) * per;
+          if (reason == 2) hi = pivot;
+          else lo = pivot;
+          if (!(next > lo && next < hi))
+            next = lo > -INFINITY && hi < INFINITY ? 0.5f * (lo + hi) : pivot + (reason == 2 ? -1.f : 1.f) * (float)a.margin * per;
+          per *= 2.0f;   // (should the density be off, the next correction is larger)
+          pivot = next;
+        }
+        prologue(part(rc), part(ru));
+        if (!SAMPLE && !is_q && more && !nq) {   // (the position was advanced to the next row above)
+          if (--dj < 0) {
+            dj = P.r - 1;
+            --di;
+          }
+        }
+        continue;
+      }
+      tries = 0;
+      if (tid == 0) count_failure(reason);
+      if (!is_q) {
+        if (tid == 0) defer(g);
+      } else {
+        // the draft row is lost: its parent's rows go with it (those of this CTA)
+#pragma unroll 1
+        while (true) {
+          if (tid == 0) defer(target_index());
+          ++unit;
+          if (dj + 1 < P.r || di + 1 < P.r) {
+            if (++dj == P.r) {
+              dj = 0;
+              ++di;
+            }
+            if (unit >= u_end) break;
+          } else {
+            break;
+          }
+        }
+        if (unit >= u_end) break;
+        next_parent();
+        g = (uint32_t)parent;
+        tok_next = __ldg(a.draft_tok_lo + parent);
+        prologue(part(row_c(true, g)), nullptr);
+        continue;
+      }
+    } else if (!SAMPLE && is_q) {
+      tries = 0;
+      // ---- a draft row ends here
+      c0_q = c0;
+      Zq = (float)Z;
+      q_tok = sm.z_tok >= theta ? rows_div(sm.e_tok, Z) : 0.0;
+      if (q_tok <= 0.0 && tid == 0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
+      __syncthreads();   // ---- barrier 3
+      if (tid == 0) sm.n_sa = 0;
+      partner_n = 0;
+    } else {
+      tries = 0;
+      // ---- the decision (Eq. 1 / Eq. 5) and what has to be drawn, the same in every warp
+      int pending = kDrawTarget;
+      double u_res = 0.0, u_tgt;
+      if (SAMPLE) {
+        const uint32_t cell = g - (uint32_t)b * (uint32_t)(P.h * P.w);
+        const uint4 v = lane_philox(make_uint4(cell, (uint32_t)b + P.image_offset, P.round, 1u), make_uint2(P.seed_lo, P.seed_hi));
+        u_tgt = uniform24(v.x);
+      } else {
+        const uint32_t* const rnd = sm.rnd[parent & 1][child];
+        const double e_tok = sm.z_tok >= theta ? sm.e_tok : 0.0;
+        int accepted;
+        if (P.accept_mode == MULO_ACCEPT_THRESHOLD) accepted = e_tok >= P.tau * Z;
+        else if (q_tok <= 0.0) accepted = e_tok > 0.0;
+        else accepted = uniform24(rnd[0]) * q_tok * Z < e_tok;
+        u_res = uniform24(rnd[1]);
+        u_tgt = uniform24(rnd[2]);
+        if (tid == 0) {
+          a.flags[g] = accepted ? 0 : 1;
+          if (a.p_tok || a.q_tok || a.accept_prob)
+            lane_write_probs(a.p_tok, a.q_tok, a.accept_prob, g, e_tok, q_tok, Z,
+                             P.accept_mode == MULO_ACCEPT_THRESHOLD);
+        }
+        pending = draws_for(P.resample_mode, accepted);
+      }
+      // weights in units of e = exp(z - ref): p -> e, q -> ratio * e_q
+      const float ratio = __fdividef((float)Z, Zq);
+      auto q_weight = [&](uint32_t at) -> float {
+        float zq = dlist_get<BF16>(at);
+        if (BF16 && !PLAIN) zq = __fmul_rn(zq, P.invT);
+        return __fmul_rn(ex2f(fmaf(zq, kLog2e, c0_q)), ratio);
+      };
+      if (lane == 0) sm.w_t[warp] = w_own;
+      if (!SAMPLE && (pending & kDrawResidual)) {
+        // sum of max(0, p - q) = p - min(p, q); min is not zero only where both rows kept the id
+        __syncwarp();   // (the crossing bin's entries, written back by other lanes)
+        uint32_t tp = tl, dp = dl;
+        float mins = 0.f;
+#pragma unroll 1
+        for (int w = 0; w < n_words; ++w) {
+          const uint32_t m = lds_u32(tm + (uint32_t)(w * NT) * 4u), d = lds_u32(dm + (uint32_t)(w * NT) * 4u);
+          uint32_t im = m & d;
+          const int trips = __reduce_max_sync(kFull, __popc(im));
+          auto both = [&](uint32_t bit) -> float {
+            const uint32_t below = bit - 1u;
+            const float e = lds_f32(tp + (uint32_t)__popc(m & below) * step);
+            const float q = q_weight(dp + (uint32_t)__popc(d & below) * dstep);
+            return bit ? fminf(e, q) : 0.f;
+          };
+#pragma unroll 1
+          for (int i = 0; i < trips; i += 2) {
+            const uint32_t b0 = im & (0u - im);
+            im ^= b0;
+            const uint32_t b1 = im & (0u - im);
+            im ^= b1;
+            mins += both(b0);
+            mins += both(b1);
+          }
+          tp += (uint32_t)__popc(m) * step;
+          dp += (uint32_t)__popc(d) * dstep;
+        }
+        const double wr = fmax(w_own - warp_sum((double)mins), 0.0);
+        if (lane == 0) sm.w_r[warp] = wr;
+      }
+      __syncthreads();   // ---- barrier 3
+      if (tid == 0) sm.n_sa = 0;
+      partner_n = pair_n;   // (this row's entries may still be walked when the next row is streamed)
+      bool no_mass = false;
+#pragma unroll 1
+      while (pending) {
+        const bool is_res = (pending & kDrawResidual) != 0;
+        const bool resid = !SAMPLE && is_res && !no_mass;
+        const double* const ws = resid ? sm.w_r : sm.w_t;
+        double total = 0.0, below = 0.0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+          if (w == warp) below = total;
+          total += ws[w];
+        }
+        if (!(total > 0.0)) {
+          if (resid) {
+            no_mass = true;   // the same draw again, from the target weights
+            continue;
+          }
+          pending &= ~(is_res ? kDrawResidual : kDrawTarget);
+          no_mass = false;
+          continue;
+        }
+        const double yt = (is_res ? u_res : u_tgt) * total;
+        const double w_mine = ws[warp];
+        if (below <= yt && yt < below + w_mine) {   // warp-uniform: this warp owns u * total
+          // ---- mask word, piece, lane, id
+          __syncwarp();
+          double y = yt - below;
+          auto weight = [&](uint32_t ta, bool both, uint32_t da) -> float {
+            float e = lds_f32(ta);
+            if (resid && both) e = fmaxf(__fsub_rn(e, q_weight(da)), 0.f);
+            return e;
+          };
+          // sum of this lane's entries under the mask bits `m` of a word whose entries start at (ta, da)
+          auto lane_sum = [&](uint32_t m, uint32_t d, uint32_t ta, uint32_t da) -> float {
+            const int trips = __reduce_max_sync(kFull, __popc(m));
+            float s = 0.f;
+#pragma unroll 1
+            for (int i = 0; i < trips; ++i) {
+              const uint32_t bit = m & (0u - m);
+              m ^= bit;
+              if (bit) {
+                s += weight(ta, (d & bit) != 0, da + (uint32_t)__popc(d & (bit - 1u)) * dstep);
+                ta += step;
+              }
+            }
+            return s;
+          };
+          uint32_t ta = tl, da = dl, m = 0, d = 0;
+          int wd = 0, last_wd = -1;
+          bool seek = false;   // rounding left the sums short: take the last word with weight
+#pragma unroll 1
+          for (;;) {
+            m = lds_u32(tm + (uint32_t)(wd * NT) * 4u);
+            d = resid ? lds_u32(dm + (uint32_t)(wd * NT) * 4u) : 0u;
+            const double t = warp_sum((double)lane_sum(m, d, ta, da));
+            if (t > 0.0) last_wd = wd;
+            if (seek ? wd == last_wd : y < t) break;
+            if (!seek) y -= t;
+            ta += (uint32_t)__popc(m) * step;
+            da += (uint32_t)__popc(d) * dstep;
+            if (++wd == n_words) {
+              if (last_wd < 0) break;
+              seek = true;
+              y = 1e300;
+              wd = 0;
+              ta = tl;
+              da = dl;
+#pragma unroll 1
+              while (wd < last_wd) {   // (where the last word starts)
+                ta += (uint32_t)__popc(lds_u32(tm + (uint32_t)(wd * NT) * 4u)) * step;
+                if (resid) da += (uint32_t)__popc(lds_u32(dm + (uint32_t)(wd * NT) * 4u)) * dstep;
+                ++wd;
+              }
+            }
+          }
+          int32_t* const out = SAMPLE ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
+          if (last_wd < 0) {   // a sum that was rounding noise of a difference
+            if (lane == 0) defer(g);
+          } else {
+            float v = 0.f, v_last = 0.f;
+            int pj = -1, pj_last = 0;
+#pragma unroll 1
+            for (int p = 0; p < 4; ++p) {
+              const uint32_t bits = (uint32_t)PIECE_BITS << (p * IDS), under = (1u << (p * IDS)) - 1u;
+              v = lane_sum(m & bits, d, ta + (uint32_t)__popc(m & under) * step, da);
+              const double t = warp_sum((double)v);
+              if (t > 0.0) {
+                pj_last = p;
+                v_last = v;
+              }
+              if (y < t) {
+                pj = p;
+                break;
+              }
+              y -= t;
+            }
+            if (pj < 0) {
+              pj = pj_last;
+              v = v_last;
+              y = 1e300;
+            }
+            double inc = (double)v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const double t = __shfl_up_sync(kFull, inc, o);
+              if (lane >= o) inc += t;
+            }
+            double exc = __shfl_up_sync(kFull, inc, 1);
+            if (lane == 0) exc = 0.0;
+            unsigned hit = __ballot_sync(kFull, v > 0.f && inc > y), has = __ballot_sync(kFull, v > 0.f);
+            const int src = hit ? __ffs(hit) - 1 : 31 - __clz(has);
+            y -= __shfl_sync(kFull, exc, src);
+            if (!hit) y = 1e300;
+            const uint32_t om = __shfl_sync(kFull, m, src), od = __shfl_sync(kFull, d, src);
+            const uint32_t ota = __shfl_sync(kFull, ta, src), oda = __shfl_sync(kFull, da, src);
+            const uint32_t bit = lane < IDS ? 1u << (pj * IDS + lane) : 0u;
+            float w = 0.f;
+            if (om & bit)
+              w = weight(ota + (uint32_t)__popc(om & (bit - 1u)) * step, (od & bit) != 0,
+                         oda + (uint32_t)__popc(od & (bit - 1u)) * dstep);
+            double run = (double)w;
+#pragma unroll
+            for (int o = 1; o < IDS; o <<= 1) {
+              const double t = __shfl_up_sync(kFull, run, o);
+              if (lane >= o) run += t;
+            }
+            hit = __ballot_sync(kFull, w > 0.f && run > y);
+            has = __ballot_sync(kFull, w > 0.f);
+            const int chosen = hit ? __ffs(hit) - 1 : 31 - __clz(has);
+            if (lane == chosen) *out = ((warp * a.ppw + wd * 4 + pj) * 32 + src) * IDS + chosen;
+          }
+        } else if (warp == NW - 1 && yt >= below + w_mine) {
+          // (u * total rounded up to the total itself cannot be: u <= 1 - 2^-24; kept for the last bits of the sum)
+          if (lane == 0) defer(g);
+        }
+        pending &= ~(is_res ? kDrawResidual : kDrawTarget);
+        no_mass = false;
+      }
+    }
+
+    // ---- on to the next row (its first pieces are in registers)
+    if (!is_q) ++unit;
+    if (!more) break;
+    if (!SAMPLE) {
+      if (is_q) child = di * P.r + dj;
+      else ++child;
+    }
+    if (SAMPLE || nq) next_parent();
+    is_q = nq;
+    g = ng;
+  }
+}
+
+}  // namespace mulo
