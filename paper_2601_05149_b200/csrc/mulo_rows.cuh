@@ -1,10 +1,11 @@
 // The fast path for rows with a top-k cut: NW warps per row.
 //
 // A CTA owns a contiguous range of target rows (in parent order).  Per parent it streams the draft row and then
-// the target rows under it, each ONCE.  Warp w owns the w-th contiguous NW-th of the ids.
+// the target rows under it, each ONCE.  The ids are split into 4 NW contiguous parts, one for every group of eight
+// lanes.
 //
-//   stream     512-byte pieces of the warp's part (16 bytes per lane) through registers, kRDepth pieces in
-//              flight per warp, the next row asked into L2 by a bulk prefetch.  Per id: unpack, CFG mix (packed
+//   stream     128-byte pieces of each group's part (16 bytes per lane) through registers, kRDepth pieces in
+//              flight per lane, the next row asked into L2 by a bulk prefetch.  Per id: unpack, CFG mix (packed
 //              fp32, one IEEE rounding per step), compare with a predicted pivot and a predicated append to the
 //              thread's PRIVATE list plus a bit in its survivor mask (one word per four pieces).  The loads run
 //              on into the next row, so a row's first pieces are in registers when its turn comes.
@@ -16,11 +17,12 @@
 //   selection  the bin that holds the k-th largest; the window's entries once more: above the bin -> exp, below
 //              -> 0, in the bin -> set aside, ranked exactly, written back.  From here on the list holds the
 //              row's weights, zeros below the threshold included.
-//   draws      warp sums of p (target) or of max(0, p - q) (residual; the sum of p minus that of min(p, q) over
-//              the ids that both rows kept, found by intersecting the masks).  The warp that owns u * total walks
-//              its part -- mask word, piece, lane, id -- while the others go on with the next row.
+//   draws      sums of p (target) or of max(0, p - q) (residual; the sum of p minus that of min(p, q) over the ids
+//              that both rows kept, found by intersecting the masks) per thread, group and warp.  The warp that
+//              owns u * total searches the owning group's part -- a quarter of it per eight lanes, then a quarter of
+//              that, down to a piece, a lane, an id -- while the others go on with the next row.
 //
-// Three block barriers per row.  Pivot, histogram scale and exp reference are predicted from the CTA's previous
+// Three block barriers per row (a further draw takes one more).  Pivot, histogram scale and exp reference are predicted from the CTA's previous
 // rows of the same kind; a row without prediction takes them from the mean and spread of its first pieces.  A
 // row whose prediction misses (too few candidates, a full column, rank beyond the histogram, maximum far from the
 // reference) is streamed again with corrected values; one that still fails, or has too many ties at the
@@ -39,11 +41,11 @@ namespace mulo {
 #define MULO_RWARPS 16
 #endif
 constexpr int kRDepth = MULO_RDEPTH;     // pieces in flight per warp
-constexpr int kRPieceBytes = 512;        // 16 bytes per lane
+constexpr int kRPieceBytes = 128;        // of a group: 16 bytes per lane
 constexpr int kRBins = 256;
 constexpr int kRSetAside = 128;          // entries of the crossing bin that are ranked exactly
 constexpr int kRTries = 6;               // times a row is streamed before it is given up
-constexpr int kRSlack = 8;               // list rows kept free between the two lists of a column: one piece's entries
+constexpr int kRSlack = 12;              // list rows kept free between the two lists of a column: a piece's entries and the closing ones
 constexpr float kRMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
 
 struct RowsArgs {
@@ -63,8 +65,8 @@ struct RowsArgs {
   int32_t* fail_list;
   int n_units;              // target rows, parent by parent (SAMPLE: low-res cells)
   uint32_t row_bytes;
-  int ppw;                  // pieces of a warp's part of a row
-  int n_words;              // mask words per thread: ceil(ppw / 4)
+  int ppg;                  // pieces of a group's part of a row
+  int n_words;              // mask words per thread: ceil(ppg / 4)
   int R;                    // rows of a list column (shared by two threads)
   uint32_t o_dlist, o_tmask, o_dmask;   // dynamic shared memory: the lists first, then these
   int margin;
@@ -79,7 +81,7 @@ struct RowsSmem {
   unsigned short sa_at[kRSetAside];        // the entry's place (index in its owner's list << 8 | thread)
   LanePredictor pred[2];                   // draft rows / target rows
   double w_all[NW];                        // exp sums of each warp without the crossing bin
-  double w_t[NW], w_r[NW];                 // weights of a draw, per warp
+  double w_draw[2][NW];                    // weights of a draw, per warp; consecutive draws alternate
   double e_tok;
   float z_tok;
   uint32_t rnd[2][16][3];                  // uniforms of the parent's children, by parity of the parent
@@ -201,7 +203,6 @@ template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
 __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
   constexpr int NT = NW * 32;
   constexpr int IDS = BF16 ? 8 : 4;              // ids per lane per piece
-  constexpr int PIECE_BITS = (1 << IDS) - 1;
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ RowsSmem<NW> sm;
   const DevParams& P = a.P;
@@ -218,12 +219,13 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
   const uint32_t my = smem_u32(dyn);
   const uint32_t first_row = (uint32_t)(warp >> 1) * (uint32_t)R + (up ? 0u : (uint32_t)(R - 1));
   const uint32_t step = up ? 128u : 0u - 128u;
-  const uint32_t tl = my + (uint32_t)lane * 4u + first_row * 128u;
+  uint32_t col = (uint32_t)lane;                   // this thread's column (see `rot` below)
+  uint32_t tl = my + first_row * 128u + col * 4u;
   const uint32_t low4 = up ? 0u : 0u - 384u;       // from an entry to the lowest address of the four from it on
   // the draft row's kept logits (bf16 if they came as such: exact, half the memory)
   constexpr uint32_t DROW = BF16 ? 64u : 128u;
   const uint32_t dstep = up ? DROW : 0u - DROW;
-  const uint32_t dl = my + a.o_dlist + (uint32_t)lane * (DROW / 32u) + first_row * DROW;
+  uint32_t dl = my + a.o_dlist + first_row * DROW + col * (DROW / 32u);
   const uint32_t tm = my + a.o_tmask + (uint32_t)tid * 4u, dm = my + a.o_dmask + (uint32_t)tid * 4u;
   const uint32_t hbase = smem_u32(sm.hist) - (__float_as_uint(kRMagic) << 2);
   const uint32_t closer = smem_u32(sm.closer) + (uint32_t)lane * 4u, dump = smem_u32(sm.sa_z) + (uint32_t)lane * 4u;
@@ -273,8 +275,8 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
   };
 
   // ---- this thread's part of a row: np pieces from part_off on
-  const uint32_t part_off = (uint32_t)(warp * a.ppw) * kRPieceBytes + (uint32_t)lane * 16u;
-  const int np = part_off < row_bytes ? min(a.ppw, (int)((row_bytes - part_off + kRPieceBytes - 1) / kRPieceBytes)) : 0;
+  const uint32_t part_off = (uint32_t)((tid >> 3) * a.ppg) * kRPieceBytes + (uint32_t)(lane & 7) * 16u;
+  const int np = part_off < row_bytes ? min(a.ppg, (int)((row_bytes - part_off + kRPieceBytes - 1) / kRPieceBytes)) : 0;
   uint4 c[kRDepth], u[kRDepth];   // the pieces in flight
   const uint4 none = make_uint4(~0u, ~0u, ~0u, ~0u);   // NaN in either type: never appended
 #pragma unroll
@@ -515,6 +517,9 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
     if (HAS_U && ru) prefetch_l2(ru, row_bytes);
   };
 
+  // A column can be too full for its two threads although both have few enough entries: when a row is streamed
+  // again for that, the odd warps' threads move to other columns (lane ^ rot).
+  uint32_t rot = 0;
   int tries = 0, tok = 0, child = 0;      // child: which row under the parent
   int partner_n = 0;                      // entries of the previous target row in the list this thread's list grows towards
   float c0_q = 0.f, Zq = 1.f;             // of the parent's draft row
@@ -589,6 +594,9 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
       }
     }
 
+    col = (uint32_t)lane ^ (up ? 0u : rot);
+    tl = my + first_row * 128u + col * 4u;
+    if (is_q) dl = my + a.o_dlist + first_row * DROW + col * (DROW / 32u);
     const uint32_t mask_at = is_q ? dm : tm;
     const uint32_t lim = tl + (uint32_t)(R - kRSlack - partner_n) * step;   // a piece appends at most 8 entries
     const uint32_t end = HAS_U && !is_q
@@ -635,10 +643,10 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
       any_over |= sm.over[w] != 0;
     }
     const float mx = key_float(mk);
-    const int pair_n = sm.cnt[tid ^ 32];
+    const int pair_n = sm.cnt[(uint32_t)tid ^ 32u ^ rot];
 #pragma unroll
     for (int w = 0; w < NW; w += 2)   // (three rows close each of the two lists)
-      any_over |= (int)sm.cnt[w * 32 + lane] + (int)sm.cnt[w * 32 + 32 + lane] + 6 > R;
+      any_over |= (int)sm.cnt[w * 32 + lane] + (int)sm.cnt[w * 32 + 32 + (lane ^ (int)rot)] + 6 > R;
     if (__any_sync(kFull, any_over)) reason = 1;
     else if (n_all < P.top_k) reason = 2;
     else if (!(fabsf(mx - ref) <= kNearRefGap)) reason = 5;
@@ -678,11 +686,11 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
     }
     float theta = 0.f;
     int n_ge = 0;
-    double Z = 0.0, w_own = 0.0;
+    double Z = 0.0;
     if (reason == 0) {
       s_t += window(low_a, low_b, inv_w, hoff, c0, bstar);
-      w_own = warp_sum((double)s_t);
-      if (lane == 0) sm.w_all[warp] = w_own;
+      const double w = warp_sum((double)s_t);
+      if (lane == 0) sm.w_all[warp] = w;
     }
     __syncthreads();   // ---- barrier 2
 #pragma unroll 1
@@ -725,23 +733,32 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
         less_at = __shfl_sync(kFull, less_at, fs);
       }
       n_ge = n_all - (int)cum - less_at;
-      double all = 0.0, own = 0.0;   // (values of one bin share their exponent: their sums in double are exact)
+      // (values of one bin share their exponent: sums of them in double are exact, whatever the order)
+      double all = (double)mcount * (double)ex2f(fmaf(theta, kLog2e, c0));
+      if (kmin != kmax) {
+        all = 0.0;
 #pragma unroll 1
-      for (int i = lane; i < mcount; i += 32) {
-        const float v = sm.sa_z[i];
-        const uint32_t at = sm.sa_at[i];
-        const float e = v >= theta ? ex2f(fmaf(v, kLog2e, c0)) : 0.f;
-        all += (double)e;
-        if ((int)((at & 0xffu) >> 5) == warp) {
-          own += (double)e;
-          const uint32_t col = (at & 31u) - (uint32_t)lane, idx = at >> 8;   // to the owner's column
-          if (!is_q) sts_f32(tl + col * 4u + idx * step, e);
-          else if (!(v >= theta)) dlist_put<BF16>(dl + col * (DROW / 32u) + idx * dstep, -INFINITY);
+        for (int i = lane; i < mcount; i += 32) {
+          const float v = sm.sa_z[i];
+          if (v >= theta) all += (double)ex2f(fmaf(v, kLog2e, c0));
         }
+        all = warp_sum(all);
       }
-      all = warp_sum(all);
-      own = warp_sum(own);
-      w_own += own;
+      if (kmin != kmax || !is_q) {   // (a draft row keeps its logits: nothing changes unless some fall below)
+        double own = 0.0;
+#pragma unroll 1
+        for (int i = 0; i < mcount; ++i) {
+          const uint32_t at = sm.sa_at[i];
+          if ((int)(at & 0xffu) == tid) {
+            const float v = sm.sa_z[i];
+            const float e = v >= theta ? ex2f(fmaf(v, kLog2e, c0)) : 0.f;
+            own += (double)e;
+            if (!is_q) sts_f32(tl + (at >> 8) * step, e);
+            else if (!(v >= theta)) dlist_put<BF16>(dl + (at >> 8) * dstep, -INFINITY);
+          }
+        }
+        s_t = (float)((double)s_t + own);
+      }
       Z = all;
 #pragma unroll
       for (int w = 0; w < NW; ++w) Z += sm.w_all[w];
@@ -759,6 +776,7 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
         // once more, with the pivot moved by the candidates it was off by (a column was full: aim low in the
         // margin; the values tried so far bracket it), or with the maximum just found
         ++tries;
+        if (reason == 1) rot = (uint32_t)(11 * tries) & 31u;
         if (reason == 5) {
           ref = mx;
         } else {
@@ -781,6 +799,7 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
         continue;
       }
       tries = 0;
+      rot = 0;
       if (tid == 0) count_failure(reason);
       if (!is_q) {
         if (tid == 0) defer(g);
@@ -850,181 +869,213 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
         if (BF16 && !PLAIN) zq = __fmul_rn(zq, P.invT);
         return __fmul_rn(ex2f(fmaf(zq, kLog2e, c0_q)), ratio);
       };
-      if (lane == 0) sm.w_t[warp] = w_own;
-      if (!SAMPLE && (pending & kDrawResidual)) {
-        // sum of max(0, p - q) = p - min(p, q); min is not zero only where both rows kept the id
-        __syncwarp();   // (the crossing bin's entries, written back by other lanes)
-        uint32_t tp = tl, dp = dl;
-        float mins = 0.f;
-#pragma unroll 1
-        for (int w = 0; w < n_words; ++w) {
-          const uint32_t m = lds_u32(tm + (uint32_t)(w * NT) * 4u), d = lds_u32(dm + (uint32_t)(w * NT) * 4u);
-          uint32_t im = m & d;
-          const int trips = __reduce_max_sync(kFull, __popc(im));
-          auto both = [&](uint32_t bit) -> float {
-            const uint32_t below = bit - 1u;
-            const float e = lds_f32(tp + (uint32_t)__popc(m & below) * step);
-            const float q = q_weight(dp + (uint32_t)__popc(d & below) * dstep);
-            return bit ? fminf(e, q) : 0.f;
-          };
-#pragma unroll 1
-          for (int i = 0; i < trips; i += 2) {
-            const uint32_t b0 = im & (0u - im);
-            im ^= b0;
-            const uint32_t b1 = im & (0u - im);
-            im ^= b1;
-            mins += both(b0);
-            mins += both(b1);
-          }
-          tp += (uint32_t)__popc(m) * step;
-          dp += (uint32_t)__popc(d) * dstep;
-        }
-        const double wr = fmax(w_own - warp_sum((double)mins), 0.0);
-        if (lane == 0) sm.w_r[warp] = wr;
-      }
-      __syncthreads();   // ---- barrier 3
-      if (tid == 0) sm.n_sa = 0;
-      partner_n = pair_n;   // (this row's entries may still be walked when the next row is streamed)
+      partner_n = pair_n;   // (this row's entries may still be searched when the next row is streamed)
       bool no_mass = false;
+      int dcall = 0;
 #pragma unroll 1
-      while (pending) {
+      do {
         const bool is_res = (pending & kDrawResidual) != 0;
         const bool resid = !SAMPLE && is_res && !no_mass;
-        const double* const ws = resid ? sm.w_r : sm.w_t;
+        float v_t = s_t;
+        if (resid) {
+          // sum of max(0, p - q) = p - min(p, q); min is not zero only where both rows kept the id
+          uint32_t tp = tl, dp = dl;
+          float mins = 0.f;
+#pragma unroll 1
+          for (int w = 0; w < n_words; ++w) {
+            const uint32_t m = lds_u32(tm + (uint32_t)(w * NT) * 4u), d = lds_u32(dm + (uint32_t)(w * NT) * 4u);
+            uint32_t im = m & d;
+            const int trips = __reduce_max_sync(kFull, __popc(im));
+            auto both = [&]() -> float {   // the next entry of the intersection
+              const uint32_t bit = im & (0u - im), below = bit - 1u;
+              im ^= bit;
+              const float e = lds_f32(tp + (uint32_t)__popc(m & below) * step);
+              const float q = q_weight(dp + (uint32_t)__popc(d & below) * dstep);
+              return bit ? fminf(e, q) : 0.f;
+            };
+#pragma unroll 1
+            for (int i = 0; i < trips; i += 4) {   // four at a time: their chains overlap
+              const float v0 = both(), v1 = both(), v2 = both(), v3 = both();
+              mins += (v0 + v1) + (v2 + v3);
+            }
+            tp += (uint32_t)__popc(m) * step;
+            dp += (uint32_t)__popc(d) * dstep;
+          }
+          v_t = fmaxf(s_t - mins, 0.f);
+        }
+        double w_grp = (double)v_t;   // of this lane's group
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) w_grp += __shfl_xor_sync(kFull, w_grp, o);
+        double w_mine = w_grp + __shfl_xor_sync(kFull, w_grp, 8);
+        w_mine += __shfl_xor_sync(kFull, w_mine, 16);
+        double* const ws = sm.w_draw[dcall & 1];
+        ++dcall;
+        if (lane == 0) ws[warp] = w_mine;
+        __syncthreads();   // ---- barrier 3
+        if (tid == 0) sm.n_sa = 0;
         double total = 0.0, below = 0.0;
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
           if (w == warp) below = total;
           total += ws[w];
         }
-        if (!(total > 0.0)) {
-          if (resid) {
-            no_mass = true;   // the same draw again, from the target weights
-            continue;
-          }
-          pending &= ~(is_res ? kDrawResidual : kDrawTarget);
-          no_mass = false;
+        if (!(total > 0.0) && resid) {
+          no_mass = true;   // the same draw again, from the target weights
           continue;
         }
         const double yt = (is_res ? u_res : u_tgt) * total;
-        const double w_mine = ws[warp];
-        if (below <= yt && yt < below + w_mine) {   // warp-uniform: this warp owns u * total
-          // ---- mask word, piece, lane, id
+        if (total > 0.0 && below <= yt && yt < below + w_mine) {   // warp-uniform: this warp owns u * total
           __syncwarp();
-          double y = yt - below;
-          auto weight = [&](uint32_t ta, bool both, uint32_t da) -> float {
-            float e = lds_f32(ta);
-            if (resid && both) e = fmaxf(__fsub_rn(e, q_weight(da)), 0.f);
+          // which group
+          int q = 0, q_last = 0;
+          double y_d = yt - below, w_q = 0.0;
+          bool found = false;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const double w = __shfl_sync(kFull, w_grp, 8 * k);
+            if (!found && w > 0.0) {
+              q_last = k;
+              w_q = w;
+              found = y_d < w;
+              if (!found) y_d -= w;
+            }
+          }
+          q = q_last;   // (rounding left the sums short: the last group with weight)
+          // Sums of the group's part in fixed point: 2^31 = its weight.  Every eight lanes take a quarter of the
+          // pieces in question, lane j of them the entries of the group's lane j.
+          const float to_fx = __fdividef(2147483648.0f, (float)w_q);
+          uint32_t y = found ? __double2uint_rz(y_d * (double)to_fx) : ~0u;
+          const uint32_t odd = up ? 0u : rot;
+          const int k8 = lane >> 3;
+          int L = q * 8 + (lane & 7);   // the lane whose entries this lane looks at
+          uint32_t d = 0, da = 0;       // draft mask of the word in work and where its entries start
+          auto weight = [&](uint32_t bit, uint32_t at) -> float {
+            float e = fmaxf(lds_f32(bit ? at : closer), 0.f);   // (the closer's -inf)
+            if (resid) {
+              const float qv = q_weight(da + (uint32_t)__popc(d & (bit - 1u)) * dstep);
+              e = (d & bit) ? fmaxf(__fsub_rn(e, qv), 0.f) : e;
+            }
             return e;
           };
-          // sum of this lane's entries under the mask bits `m` of a word whose entries start at (ta, da)
-          auto lane_sum = [&](uint32_t m, uint32_t d, uint32_t ta, uint32_t da) -> float {
-            const int trips = __reduce_max_sync(kFull, __popc(m));
-            float s = 0.f;
+          // fixed-point sum of lane L's entries in pieces [pa, pb)
+          auto part_sum = [&](int pa, int pb) -> uint32_t {
+            const uint32_t l4 = (uint32_t)(L - lane) * 4u, to = ((uint32_t)L ^ odd) - col;
+            uint32_t ta = tl + to * 4u, mw = tm + l4, dw = dm + l4;
+            da = dl + to * (DROW / 32u);
+            float sum = 0.f;
+            int w = 0;
 #pragma unroll 1
-            for (int i = 0; i < trips; ++i) {
-              const uint32_t bit = m & (0u - m);
-              m ^= bit;
-              if (bit) {
-                s += weight(ta, (d & bit) != 0, da + (uint32_t)__popc(d & (bit - 1u)) * dstep);
-                ta += step;
-              }
+            for (; w < (pa >> 2); ++w) {
+              ta += (uint32_t)__popc(lds_u32(mw)) * step;
+              if (resid) da += (uint32_t)__popc(lds_u32(dw)) * dstep;
+              mw += NT * 4u;
+              dw += NT * 4u;
             }
-            return s;
+#pragma unroll 1
+            for (; 4 * w < pb; ++w) {
+              const uint32_t m = lds_u32(mw);
+              d = resid ? lds_u32(dw) : 0u;
+              mw += NT * 4u;
+              dw += NT * 4u;
+              const int from = max(pa - 4 * w, 0) * IDS, to_bit = min(pb - 4 * w, 4) * IDS;
+              const uint32_t skip = (1u << from) - 1u;
+              uint32_t mm = m & ~skip & (to_bit < 32 ? (1u << to_bit) - 1u : ~0u);
+              uint32_t at = ta + (uint32_t)__popc(m & skip) * step;
+              while (mm) {
+                const uint32_t b0 = mm & (0u - mm);
+                mm ^= b0;
+                const uint32_t b1 = mm & (0u - mm);
+                mm ^= b1;
+                const uint32_t b2 = mm & (0u - mm);
+                mm ^= b2;
+                const float v0 = weight(b0, at), v1 = weight(b1, at + step), v2 = weight(b2, at + 2 * step);
+                sum += (v0 + v1) + v2;
+                at += 3 * step;
+              }
+              ta += (uint32_t)__popc(m) * step;
+              da += (uint32_t)__popc(d) * dstep;
+            }
+            return __float2uint_rn(__fmul_rn(sum, to_fx));
           };
-          uint32_t ta = tl, da = dl, m = 0, d = 0;
-          int wd = 0, last_wd = -1;
-          bool seek = false;   // rounding left the sums short: take the last word with weight
-#pragma unroll 1
+          int s0 = 0, len = a.ppg;
+          uint32_t v;
           for (;;) {
-            m = lds_u32(tm + (uint32_t)(wd * NT) * 4u);
-            d = resid ? lds_u32(dm + (uint32_t)(wd * NT) * 4u) : 0u;
-            const double t = warp_sum((double)lane_sum(m, d, ta, da));
-            if (t > 0.0) last_wd = wd;
-            if (seek ? wd == last_wd : y < t) break;
-            if (!seek) y -= t;
-            ta += (uint32_t)__popc(m) * step;
-            da += (uint32_t)__popc(d) * dstep;
-            if (++wd == n_words) {
-              if (last_wd < 0) break;
-              seek = true;
-              y = 1e300;
-              wd = 0;
-              ta = tl;
-              da = dl;
-#pragma unroll 1
-              while (wd < last_wd) {   // (where the last word starts)
-                ta += (uint32_t)__popc(lds_u32(tm + (uint32_t)(wd * NT) * 4u)) * step;
-                if (resid) da += (uint32_t)__popc(lds_u32(dm + (uint32_t)(wd * NT) * 4u)) * dstep;
-                ++wd;
+            const int sub = (len + 3) >> 2, pa = s0 + min(k8 * sub, len), pb = s0 + min(k8 * sub + sub, len);
+            v = pa < pb ? part_sum(pa, pb) : 0u;
+            __syncwarp();
+            if (sub == 1) break;
+            uint32_t t = v;
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) t += __shfl_xor_sync(kFull, t, o);
+            int pick = 0;
+            bool hit = false;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t w = __shfl_sync(kFull, t, 8 * k);
+              if (!hit && w > 0) {
+                pick = k;
+                hit = y < w;
+                if (!hit && y != ~0u) y -= w;
               }
             }
+            if (!hit) y = ~0u;
+            s0 += pick * sub;
+            len = min(sub, len - pick * sub);
           }
+          // the four pieces, lane by lane
+          uint32_t inc = v;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += t;
+          }
+          unsigned hit = __ballot_sync(kFull, v > 0 && inc > y), has = __ballot_sync(kFull, v > 0);
+          const int src = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : 0;
+          y = hit ? y - __shfl_sync(kFull, inc - v, src) : ~0u;
+          // ... and the ids of the one found: lane i takes id i
+          const int piece = s0 + (src >> 3);
+          L = q * 8 + (src & 7);
+          float w = 0.f;
+          {
+            const uint32_t l4 = (uint32_t)(L - lane) * 4u, to = ((uint32_t)L ^ odd) - col;
+            uint32_t ta = tl + to * 4u, mw = tm + l4, dw = dm + l4;
+            da = dl + to * (DROW / 32u);
+#pragma unroll 1
+            for (int k = 0; k < (piece >> 2); ++k) {
+              ta += (uint32_t)__popc(lds_u32(mw)) * step;
+              if (resid) da += (uint32_t)__popc(lds_u32(dw)) * dstep;
+              mw += NT * 4u;
+              dw += NT * 4u;
+            }
+            const uint32_t m = lds_u32(mw);
+            d = resid ? lds_u32(dw) : 0u;
+            const uint32_t bit = lane < IDS ? m & (1u << ((piece & 3) * IDS + lane)) : 0u;
+            w = weight(bit, ta + (uint32_t)__popc(m & (bit - 1u)) * step);
+          }
+          inc = __float2uint_rn(__fmul_rn(w, to_fx));
+#pragma unroll
+          for (int o = 1; o < IDS; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += t;
+          }
+          hit = __ballot_sync(kFull, w > 0.f && inc > y);
+          has = __ballot_sync(kFull, w > 0.f);
+          // (no id with weight: a sum that was rounding noise of a difference -- to the general routines)
+          const int chosen = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : -1;
           int32_t* const out = SAMPLE ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
-          if (last_wd < 0) {   // a sum that was rounding noise of a difference
-            if (lane == 0) defer(g);
-          } else {
-            float v = 0.f, v_last = 0.f;
-            int pj = -1, pj_last = 0;
-#pragma unroll 1
-            for (int p = 0; p < 4; ++p) {
-              const uint32_t bits = (uint32_t)PIECE_BITS << (p * IDS), under = (1u << (p * IDS)) - 1u;
-              v = lane_sum(m & bits, d, ta + (uint32_t)__popc(m & under) * step, da);
-              const double t = warp_sum((double)v);
-              if (t > 0.0) {
-                pj_last = p;
-                v_last = v;
-              }
-              if (y < t) {
-                pj = p;
-                break;
-              }
-              y -= t;
-            }
-            if (pj < 0) {
-              pj = pj_last;
-              v = v_last;
-              y = 1e300;
-            }
-            double inc = (double)v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const double t = __shfl_up_sync(kFull, inc, o);
-              if (lane >= o) inc += t;
-            }
-            double exc = __shfl_up_sync(kFull, inc, 1);
-            if (lane == 0) exc = 0.0;
-            unsigned hit = __ballot_sync(kFull, v > 0.f && inc > y), has = __ballot_sync(kFull, v > 0.f);
-            const int src = hit ? __ffs(hit) - 1 : 31 - __clz(has);
-            y -= __shfl_sync(kFull, exc, src);
-            if (!hit) y = 1e300;
-            const uint32_t om = __shfl_sync(kFull, m, src), od = __shfl_sync(kFull, d, src);
-            const uint32_t ota = __shfl_sync(kFull, ta, src), oda = __shfl_sync(kFull, da, src);
-            const uint32_t bit = lane < IDS ? 1u << (pj * IDS + lane) : 0u;
-            float w = 0.f;
-            if (om & bit)
-              w = weight(ota + (uint32_t)__popc(om & (bit - 1u)) * step, (od & bit) != 0,
-                         oda + (uint32_t)__popc(od & (bit - 1u)) * dstep);
-            double run = (double)w;
-#pragma unroll
-            for (int o = 1; o < IDS; o <<= 1) {
-              const double t = __shfl_up_sync(kFull, run, o);
-              if (lane >= o) run += t;
-            }
-            hit = __ballot_sync(kFull, w > 0.f && run > y);
-            has = __ballot_sync(kFull, w > 0.f);
-            const int chosen = hit ? __ffs(hit) - 1 : 31 - __clz(has);
-            if (lane == chosen) *out = ((warp * a.ppw + wd * 4 + pj) * 32 + src) * IDS + chosen;
-          }
-        } else if (warp == NW - 1 && yt >= below + w_mine) {
-          // (u * total rounded up to the total itself cannot be: u <= 1 - 2^-24; kept for the last bits of the sum)
-          if (lane == 0) defer(g);
+          if (lane == chosen) *out = ((((warp * 4 + q) * a.ppg + piece) << 3) + (src & 7)) * IDS + chosen;
+          if (chosen < 0 && lane == 0) defer(g);
         }
         pending &= ~(is_res ? kDrawResidual : kDrawTarget);
         no_mass = false;
-      }
+      } while (pending);
     }
 
+    if (rot != 0) {   // (the next row's columns pair up differently: nobody may still be walking this one's)
+      __syncthreads();
+      rot = 0;
+      partner_n = 0;
+    }
     // ---- on to the next row (its first pieces are in registers)
     if (!is_q) ++unit;
     if (!more) break;
