@@ -992,14 +992,14 @@ static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, in
   const int pieces = (int)((s->row_bytes + kRPieceBytes - 1) / kRPieceBytes);
   s->ppg = (pieces + 4 * nw - 1) / (4 * nw);
   s->n_words = (s->ppg + 3) / 4;
-  // A list column holds the candidates of two threads: their share plus 4.2 standard deviations of that
+  // A list column holds the candidates of two threads: their share plus 3.6 standard deviations of that
   // binomial count (3 for a row without prediction); a thread's own at most 64.
   auto rows_for = [&](int count, double threads, double dev) {
     const double pc = (double)count / V, mu = threads * s->ppg * ids * pc;
     return mu + dev * sqrt(mu * (1.0 - pc));
   };
   if (rows_for(k + margin, 1.0, 4.5) > 64.0) return 0;
-  s->R = (int)ceil(fmax(rows_for(k + margin, 2.0, 4.2), rows_for(k + margin_boot, 2.0, 3.0))) + 1 + kRSlack;
+  s->R = (int)ceil(fmax(rows_for(k + margin, 2.0, 3.6), rows_for(k + margin_boot, 2.0, 3.0))) + 1 + kRSlack;
   if (s->R < 32) s->R = 32;
   s->margin = margin;
   s->a_theta = (float)inv_norm_cdf(1.0 - p);

@@ -18,11 +18,11 @@
 //              -> 0, in the bin -> set aside, ranked exactly, written back.  From here on the list holds the
 //              row's weights, zeros below the threshold included.
 //   draws      sums of p (target) or of max(0, p - q) (residual; the sum of p minus that of min(p, q) over the ids
-//              that both rows kept, found by intersecting the masks) per thread, group and warp.  The warp that
-//              owns u * total searches the owning group's part -- a quarter of it per eight lanes, then a quarter of
-//              that, down to a piece, a lane, an id -- while the others go on with the next row.
+//              that both rows kept, found by intersecting the masks) per thread and group.  The group that owns
+//              u * total is searched by the whole CTA, a mask word or so per eight threads; the owner's warp takes
+//              it from there (piece, lane, id) while the others go on with the next row.
 //
-// Three block barriers per row (a further draw takes one more).  Pivot, histogram scale and exp reference are predicted from the CTA's previous
+// Three block barriers per draft row, four per target row.  Pivot, histogram scale and exp reference are predicted from the CTA's previous
 // rows of the same kind; a row without prediction takes them from the mean and spread of its first pieces.  A
 // row whose prediction misses (too few candidates, a full column, rank beyond the histogram, maximum far from the
 // reference) is streamed again with corrected values; one that still fails, or has too many ties at the
@@ -81,7 +81,8 @@ struct RowsSmem {
   unsigned short sa_at[kRSetAside];        // the entry's place (index in its owner's list << 8 | thread)
   LanePredictor pred[2];                   // draft rows / target rows
   double w_all[NW];                        // exp sums of each warp without the crossing bin
-  double w_draw[2][NW];                    // weights of a draw, per warp; consecutive draws alternate
+  double w_draw[2][NW * 4];                // weights of a draw, per group; consecutive draws alternate
+  uint32_t fx[2][NW * 4];                  // ... and of the parts of the owning group
   double e_tok;
   float z_tok;
   uint32_t rnd[2][16][3];                  // uniforms of the parent's children, by parity of the parent
@@ -519,9 +520,10 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
 
   // A column can be too full for its two threads although both have few enough entries: when a row is streamed
   // again for that, the odd warps' threads move to other columns (lane ^ rot).
-  uint32_t rot = 0;
+  uint32_t rot = 0, rot_q = 0;            // of the row in work / of the parent's draft row
   int tries = 0, tok = 0, child = 0;      // child: which row under the parent
   int partner_n = 0;                      // entries of the previous target row in the list this thread's list grows towards
+  int partner_q = 0;                      // ... and of the draft row's list
   float c0_q = 0.f, Zq = 1.f;             // of the parent's draft row
   double q_tok = 0.0;
   int tok_next = SAMPLE ? 0 : __ldg(a.draft_tok_lo + parent);
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
     tl = my + first_row * 128u + col * 4u;
     if (is_q) dl = my + a.o_dlist + first_row * DROW + col * (DROW / 32u);
     const uint32_t mask_at = is_q ? dm : tm;
-    const uint32_t lim = tl + (uint32_t)(R - kRSlack - partner_n) * step;   // a piece appends at most 8 entries
+    const uint32_t lim = tl + (uint32_t)(R - kRSlack - (is_q ? max(partner_n, partner_q) : partner_n)) * step;   // a piece appends at most 8 entries
     const uint32_t end = HAS_U && !is_q
                              ? stream_t(std::integral_constant<bool, HAS_U>{}, part(rc), part(ru), part(nc), part(nu), pivot, tl, lim, mask_at)
                              : stream_t(std::false_type{}, part(rc), part(ru), part(nc), part(nu), pivot, tl, lim, mask_at);
@@ -771,7 +773,8 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
     if (!ok) {   // CTA-uniform
       __syncthreads();   // ---- barrier 3
       if (tid == 0) sm.n_sa = 0;
-      partner_n = 0;     // (nothing of this row is read any more)
+      partner_n = 0;     // (nothing of the target rows before is read any more)
+      if (is_q) partner_q = 0;
       if (again) {
         // once more, with the pivot moved by the candidates it was off by (a column was full: aim low in the
         // margin; the values tried so far bracket it), or with the maximum just found
@@ -836,6 +839,8 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
       __syncthreads();   // ---- barrier 3
       if (tid == 0) sm.n_sa = 0;
       partner_n = 0;
+      partner_q = pair_n;
+      rot_q = rot;
     } else {
       tries = 0;
       // ---- the decision (Eq. 1 / Eq. 5) and what has to be drawn, the same in every warp
@@ -903,178 +908,181 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
           }
           v_t = fmaxf(s_t - mins, 0.f);
         }
-        double w_grp = (double)v_t;   // of this lane's group
+        constexpr int NG = NW * 4;   // groups, and sets of eight threads in the search
+        double w_grp = (double)v_t;
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) w_grp += __shfl_xor_sync(kFull, w_grp, o);
-        double w_mine = w_grp + __shfl_xor_sync(kFull, w_grp, 8);
-        w_mine += __shfl_xor_sync(kFull, w_mine, 16);
         double* const ws = sm.w_draw[dcall & 1];
+        uint32_t* const fxs = sm.fx[dcall & 1];
         ++dcall;
-        if (lane == 0) ws[warp] = w_mine;
+        if ((lane & 7) == 0) ws[tid >> 3] = w_grp;
         __syncthreads();   // ---- barrier 3
         if (tid == 0) sm.n_sa = 0;
-        double total = 0.0, below = 0.0;
+        // the group that owns u * total (the same in every warp)
+        w_grp = ws[lane & (NG - 1)];
+        double inc_d = w_grp;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) {
-          if (w == warp) below = total;
-          total += ws[w];
+        for (int o = 1; o < NG; o <<= 1) {
+          const double t = __shfl_up_sync(kFull, inc_d, o, NG);
+          if ((lane & (NG - 1)) >= o) inc_d += t;
         }
-        if (!(total > 0.0) && resid) {
-          no_mass = true;   // the same draw again, from the target weights
-          continue;
-        }
-        const double yt = (is_res ? u_res : u_tgt) * total;
-        if (total > 0.0 && below <= yt && yt < below + w_mine) {   // warp-uniform: this warp owns u * total
-          __syncwarp();
-          // which group
-          int q = 0, q_last = 0;
-          double y_d = yt - below, w_q = 0.0;
-          bool found = false;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const double w = __shfl_sync(kFull, w_grp, 8 * k);
-            if (!found && w > 0.0) {
-              q_last = k;
-              w_q = w;
-              found = y_d < w;
-              if (!found) y_d -= w;
-            }
+        const double total = __shfl_sync(kFull, inc_d, NG - 1);
+        if (!(total > 0.0)) {
+          if (resid) {
+            no_mass = true;   // the same draw again, from the target weights
+            continue;
           }
-          q = q_last;   // (rounding left the sums short: the last group with weight)
-          // Sums of the group's part in fixed point: 2^31 = its weight.  Every eight lanes take a quarter of the
-          // pieces in question, lane j of them the entries of the group's lane j.
-          const float to_fx = __fdividef(2147483648.0f, (float)w_q);
-          uint32_t y = found ? __double2uint_rz(y_d * (double)to_fx) : ~0u;
-          const uint32_t odd = up ? 0u : rot;
-          const int k8 = lane >> 3;
-          int L = q * 8 + (lane & 7);   // the lane whose entries this lane looks at
-          uint32_t d = 0, da = 0;       // draft mask of the word in work and where its entries start
+        } else {
+          const double yt = (is_res ? u_res : u_tgt) * total;
+          double exc_d = __shfl_up_sync(kFull, inc_d, 1, NG);
+          if ((lane & (NG - 1)) == 0) exc_d = 0.0;
+          const unsigned hit_g = __ballot_sync(kFull, lane < NG && inc_d > yt), has_g = __ballot_sync(kFull, lane < NG && w_grp > 0.0);
+          const int og = hit_g ? __ffs(hit_g) - 1 : 31 - __clz(has_g);
+          // sums over the group's part in fixed point: 2^31 = its weight
+          const float to_fx = __fdividef(2147483648.0f, (float)__shfl_sync(kFull, w_grp, og));
+          uint32_t y = hit_g ? __double2uint_rz((yt - __shfl_sync(kFull, exc_d, og)) * (double)to_fx) : ~0u;
+          // the thread of the group whose entries this thread looks at, and where they are
+          const int own = og * 8 + (lane & 7);
+          const bool o_up = ((own >> 5) & 1) == 0;
+          const uint32_t o_row = (uint32_t)(own >> 6) * (uint32_t)R + (o_up ? 0u : (uint32_t)(R - 1));
+          const uint32_t o_step = o_up ? 128u : 0u - 128u, o_dstep = o_up ? DROW : 0u - DROW;
+          const uint32_t o_tm = my + a.o_tmask + (uint32_t)own * 4u, o_dm = my + a.o_dmask + (uint32_t)own * 4u;
+          const uint32_t o_tl = my + o_row * 128u + (((uint32_t)own & 31u) ^ (o_up ? 0u : rot)) * 4u;
+          const uint32_t o_dl = my + a.o_dlist + o_row * DROW + (((uint32_t)own & 31u) ^ (o_up ? 0u : rot_q)) * (DROW / 32u);
+          uint32_t m = 0, d = 0, ta = 0, da = 0;   // masks of the word in work and where its entries start
           auto weight = [&](uint32_t bit, uint32_t at) -> float {
             float e = fmaxf(lds_f32(bit ? at : closer), 0.f);   // (the closer's -inf)
             if (resid) {
-              const float qv = q_weight(da + (uint32_t)__popc(d & (bit - 1u)) * dstep);
+              const float qv = q_weight(da + (uint32_t)__popc(d & (bit - 1u)) * o_dstep);
               e = (d & bit) ? fmaxf(__fsub_rn(e, qv), 0.f) : e;
             }
             return e;
           };
-          // fixed-point sum of lane L's entries in pieces [pa, pb)
-          auto part_sum = [&](int pa, int pb) -> uint32_t {
-            const uint32_t l4 = (uint32_t)(L - lane) * 4u, to = ((uint32_t)L ^ odd) - col;
-            uint32_t ta = tl + to * 4u, mw = tm + l4, dw = dm + l4;
-            da = dl + to * (DROW / 32u);
+          auto entries = [&](uint32_t mm, uint32_t at) -> uint32_t {   // fixed-point sum of the entries at the bits mm
             float sum = 0.f;
-            int w = 0;
 #pragma unroll 1
-            for (; w < (pa >> 2); ++w) {
-              ta += (uint32_t)__popc(lds_u32(mw)) * step;
-              if (resid) da += (uint32_t)__popc(lds_u32(dw)) * dstep;
-              mw += NT * 4u;
-              dw += NT * 4u;
-            }
-#pragma unroll 1
-            for (; 4 * w < pb; ++w) {
-              const uint32_t m = lds_u32(mw);
-              d = resid ? lds_u32(dw) : 0u;
-              mw += NT * 4u;
-              dw += NT * 4u;
-              const int from = max(pa - 4 * w, 0) * IDS, to_bit = min(pb - 4 * w, 4) * IDS;
-              const uint32_t skip = (1u << from) - 1u;
-              uint32_t mm = m & ~skip & (to_bit < 32 ? (1u << to_bit) - 1u : ~0u);
-              uint32_t at = ta + (uint32_t)__popc(m & skip) * step;
-              while (mm) {
-                const uint32_t b0 = mm & (0u - mm);
-                mm ^= b0;
-                const uint32_t b1 = mm & (0u - mm);
-                mm ^= b1;
-                const uint32_t b2 = mm & (0u - mm);
-                mm ^= b2;
-                const float v0 = weight(b0, at), v1 = weight(b1, at + step), v2 = weight(b2, at + 2 * step);
-                sum += (v0 + v1) + v2;
-                at += 3 * step;
-              }
-              ta += (uint32_t)__popc(m) * step;
-              da += (uint32_t)__popc(d) * dstep;
+            while (mm) {
+              const uint32_t b0 = mm & (0u - mm);
+              mm ^= b0;
+              const uint32_t b1 = mm & (0u - mm);
+              mm ^= b1;
+              const uint32_t b2 = mm & (0u - mm);
+              mm ^= b2;
+              const float v0 = weight(b0, at), v1 = weight(b1, at + o_step), v2 = weight(b2, at + 2 * o_step);
+              sum += (v0 + v1) + v2;
+              at += 3 * o_step;
             }
             return __float2uint_rn(__fmul_rn(sum, to_fx));
           };
-          int s0 = 0, len = a.ppg;
-          uint32_t v;
-          for (;;) {
-            const int sub = (len + 3) >> 2, pa = s0 + min(k8 * sub, len), pb = s0 + min(k8 * sub + sub, len);
-            v = pa < pb ? part_sum(pa, pb) : 0u;
+          auto go_to = [&](int w) {   // the state of word w
+            ta = o_tl;
+            da = o_dl;
+#pragma unroll 1
+            for (int k = 0; k < w; ++k) {
+              ta += (uint32_t)__popc(lds_u32(o_tm + (uint32_t)(k * NT) * 4u)) * o_step;
+              if (resid) da += (uint32_t)__popc(lds_u32(o_dm + (uint32_t)(k * NT) * 4u)) * o_dstep;
+            }
+          };
+          auto load_word = [&](int w) {
+            m = lds_u32(o_tm + (uint32_t)(w * NT) * 4u);
+            d = resid ? lds_u32(o_dm + (uint32_t)(w * NT) * 4u) : 0u;
+          };
+          auto next_word = [&]() {
+            ta += (uint32_t)__popc(m) * o_step;
+            da += (uint32_t)__popc(d) * o_dstep;
+          };
+          const int wps = (n_words + NG - 1) / NG;   // words per set of eight threads
+          {
+            const int w0 = min((tid >> 3) * wps, n_words), w1 = min(w0 + wps, n_words);
+            uint32_t v = 0;
+            go_to(w0);
+#pragma unroll 1
+            for (int w = w0; w < w1; ++w) {
+              load_word(w);
+              v += entries(m, ta);
+              next_word();
+            }
             __syncwarp();
-            if (sub == 1) break;
-            uint32_t t = v;
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) t += __shfl_xor_sync(kFull, t, o);
-            int pick = 0;
-            bool hit = false;
+            for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+            if ((lane & 7) == 0) fxs[tid >> 3] = v;
+          }
+          __syncthreads();   // ---- barrier 4
+          if (warp == (og >> 2)) {
+            uint32_t v = fxs[lane & (NG - 1)], inc = v;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const uint32_t w = __shfl_sync(kFull, t, 8 * k);
-              if (!hit && w > 0) {
-                pick = k;
-                hit = y < w;
-                if (!hit && y != ~0u) y -= w;
+            for (int o = 1; o < NG; o <<= 1) {
+              const uint32_t t = __shfl_up_sync(kFull, inc, o, NG);
+              if ((lane & (NG - 1)) >= o) inc += t;
+            }
+            unsigned hit = __ballot_sync(kFull, lane < NG && v > 0 && inc > y), has = __ballot_sync(kFull, lane < NG && v > 0);
+            int src = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : 0;
+            y = hit ? y - __shfl_sync(kFull, inc - v, src) : ~0u;
+            // the set's words one by one: eight lanes to a piece
+            const uint32_t piece_bits = ((1u << IDS) - 1u) << ((lane >> 3) * IDS), under = (1u << ((lane >> 3) * IDS)) - 1u;
+            const int w0 = src * wps, w1 = min(w0 + wps, n_words);
+            int w = w0, last_w = w0;
+            bool seek = false;   // rounding left the sums short: the last word with weight
+            go_to(w0);
+#pragma unroll 1
+            for (;;) {
+              load_word(w);
+              v = entries(m & piece_bits, ta + (uint32_t)__popc(m & under) * o_step);
+              __syncwarp();
+              const uint32_t t = __reduce_add_sync(kFull, v);
+              if (t > 0) last_w = w;
+              if (seek ? w == last_w : y < t) break;
+              if (y != ~0u) y -= t;
+              next_word();
+              if (++w == w1) {
+                seek = true;
+                y = ~0u;
+                w = last_w;
+                go_to(w);
               }
             }
-            if (!hit) y = ~0u;
-            s0 += pick * sub;
-            len = min(sub, len - pick * sub);
-          }
-          // the four pieces, lane by lane
-          uint32_t inc = v;
+            inc = v;
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += t;
-          }
-          unsigned hit = __ballot_sync(kFull, v > 0 && inc > y), has = __ballot_sync(kFull, v > 0);
-          const int src = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : 0;
-          y = hit ? y - __shfl_sync(kFull, inc - v, src) : ~0u;
-          // ... and the ids of the one found: lane i takes id i
-          const int piece = s0 + (src >> 3);
-          L = q * 8 + (src & 7);
-          float w = 0.f;
-          {
-            const uint32_t l4 = (uint32_t)(L - lane) * 4u, to = ((uint32_t)L ^ odd) - col;
-            uint32_t ta = tl + to * 4u, mw = tm + l4, dw = dm + l4;
-            da = dl + to * (DROW / 32u);
-#pragma unroll 1
-            for (int k = 0; k < (piece >> 2); ++k) {
-              ta += (uint32_t)__popc(lds_u32(mw)) * step;
-              if (resid) da += (uint32_t)__popc(lds_u32(dw)) * dstep;
-              mw += NT * 4u;
-              dw += NT * 4u;
+            for (int o = 1; o < 32; o <<= 1) {
+              const uint32_t t = __shfl_up_sync(kFull, inc, o);
+              if (lane >= o) inc += t;
             }
-            const uint32_t m = lds_u32(mw);
-            d = resid ? lds_u32(dw) : 0u;
-            const uint32_t bit = lane < IDS ? m & (1u << ((piece & 3) * IDS + lane)) : 0u;
-            w = weight(bit, ta + (uint32_t)__popc(m & (bit - 1u)) * step);
-          }
-          inc = __float2uint_rn(__fmul_rn(w, to_fx));
+            hit = __ballot_sync(kFull, v > 0 && inc > y);
+            has = __ballot_sync(kFull, v > 0);
+            src = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : 0;
+            y = hit ? y - __shfl_sync(kFull, inc - v, src) : ~0u;
+            // ... and the ids of the lane found: lane i takes id i
+            m = __shfl_sync(kFull, m, src);
+            d = __shfl_sync(kFull, d, src);
+            ta = __shfl_sync(kFull, ta, src);
+            da = __shfl_sync(kFull, da, src);
+            const uint32_t bit = lane < IDS ? m & (1u << ((src >> 3) * IDS + lane)) : 0u;
+            const float wt = weight(bit, ta + (uint32_t)__popc(m & (bit - 1u)) * o_step);
+            inc = __float2uint_rn(__fmul_rn(wt, to_fx));
 #pragma unroll
-          for (int o = 1; o < IDS; o <<= 1) {
-            const uint32_t t = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += t;
+            for (int o = 1; o < IDS; o <<= 1) {
+              const uint32_t t = __shfl_up_sync(kFull, inc, o);
+              if (lane >= o) inc += t;
+            }
+            hit = __ballot_sync(kFull, wt > 0.f && inc > y);
+            has = __ballot_sync(kFull, wt > 0.f);
+            // (no id with weight: a sum that was rounding noise of a difference -- to the general routines)
+            const int chosen = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : -1;
+            int32_t* const out = SAMPLE ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
+            if (lane == chosen) *out = (((og * a.ppg + w * 4 + (src >> 3)) << 3) + (src & 7)) * IDS + chosen;
+            if (chosen < 0 && lane == 0) defer(g);
           }
-          hit = __ballot_sync(kFull, w > 0.f && inc > y);
-          has = __ballot_sync(kFull, w > 0.f);
-          // (no id with weight: a sum that was rounding noise of a difference -- to the general routines)
-          const int chosen = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : -1;
-          int32_t* const out = SAMPLE ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
-          if (lane == chosen) *out = ((((warp * 4 + q) * a.ppg + piece) << 3) + (src & 7)) * IDS + chosen;
-          if (chosen < 0 && lane == 0) defer(g);
         }
         pending &= ~(is_res ? kDrawResidual : kDrawTarget);
         no_mass = false;
       } while (pending);
     }
 
-    if (rot != 0) {   // (the next row's columns pair up differently: nobody may still be walking this one's)
+    if (rot != 0 || (nq && rot_q != 0)) {   // (the next row's columns pair up differently: nobody may still be at this one's)
       __syncthreads();
       rot = 0;
       partner_n = 0;
+      if (nq) partner_q = 0;
     }
     // ---- on to the next row (its first pieces are in registers)
     if (!is_q) ++unit;
