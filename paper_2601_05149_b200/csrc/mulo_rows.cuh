@@ -607,8 +607,9 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
     if (more && tid == 0) prefetch(nc, nu);
     const int n_raw = (int)(up ? end - tl : tl - end) >> 7;
     const int n = min(n_raw, 64);
-    // (a list that passed its limit, or would leave its neighbour's next row no room)
-    const bool over = (up ? end > lim : end < lim) || n_raw > 64 || n_raw > R - 2 * kRSlack;
+    // (a list that reached its limit was held there: its entries are incomplete; one of more than R - kRSlack
+    // entries would leave its neighbour's next row no room at all)
+    const bool over = (up ? end >= lim : end <= lim) || n_raw > 64 || n_raw > R - kRSlack;
     const float c0 = -ref * kLog2e, hoff = -pivot * inv_w;
     uint32_t low_a, low_b;
     float s_t = is_q ? pass_one(std::integral_constant<bool, !SAMPLE>{}, n, inv_w, hoff, c0, low_a, low_b)
