@@ -777,20 +777,21 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
       partner_n = 0;     // (nothing of the target rows before is read any more)
       if (is_q) partner_q = 0;
       if (again) {
-        // once more, with the pivot moved by the candidates it was off by (a column was full: aim low in the
-        // margin; the values tried so far bracket it), or with the maximum just found
+        // once more: with the maximum just found, with other columns, or with the pivot moved by the candidates it
+        // was off by (the values that were too high and too low bracket it)
         ++tries;
+        const bool first_full = reason == 1 && rot == 0 && n_all <= P.top_k + 2 * a.margin;
         if (reason == 1) rot = (uint32_t)(11 * tries) & 31u;
         if (reason == 5) {
           ref = mx;
-        } else {
-          const float aim = (float)P.top_k + (reason == 2 ? 0.75f : 0.3f) * (float)a.margin;
+        } else if (!first_full) {
+          const float aim = (float)P.top_k + (reason == 1 ? 0.4f : 0.7f) * (float)a.margin;
           float next = pivot + ((float)n_all - aim) * per;
           if (reason == 2) hi = pivot;
-          else lo = pivot;
+          if (reason == 3) lo = pivot;
           if (!(next > lo && next < hi))
             next = lo > -INFINITY && hi < INFINITY ? 0.5f * (lo + hi) : pivot + (reason == 2 ? -1.f : 1.f) * (float)a.margin * per;
-          per *= 2.0f;   // (should the density be off, the next correction is larger)
+          if (reason != 1) per *= 1.5f;   // (should the density be off, the next correction is larger)
           pivot = next;
         }
         prologue(part(rc), part(ru));
