@@ -11,7 +11,6 @@
 #include "../../include/mulo.h"
 #include "mulo_dense.cuh"
 #include "mulo_islands.cuh"
-#include "mulo_lane.cuh"
 #include "mulo_full.cuh"
 #include "mulo_rows.cuh"
 #include "mulo_stream.cuh"
@@ -554,7 +553,6 @@ struct mulo_ctx {
   std::vector<cudaEvent_t> ev;   // start/stop pairs around the fused row kernel
   size_t ev_used;
   int force_dense;               // diagnostics: never take the fast top-k path
-  int no_lane;                   // diagnostics: never take the lane-private kernel
 };
 
 static const size_t kStatusBytes = 256;
@@ -674,7 +672,6 @@ mulo_status mulo_create(mulo_ctx** out, int device) {
   c->launches = 0;
   c->ev_used = 0;
   c->force_dense = 0;
-  c->no_lane = 0;
   *out = c;
   return MULO_OK;
 }
@@ -876,107 +873,10 @@ static bool launch_stream(const mulo_ctx* ctx, const StreamArgs& s, size_t dyn, 
   return hu ? launch_stream_t<false, true>(ctx, s, dyn, st) : launch_stream_t<false, false>(ctx, s, dyn, st);
 }
 
-// ---- the lane-private fast path (V = 256 * W, W <= 64) ---------------------------------
-
-typedef CUresult (*TensorMapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                      const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                      CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's tensor-map encoder, looked up once (host code only; no device work, no allocation).
-static TensorMapEncodeFn tensor_map_encoder() {
-  static std::once_flag once;
-  static TensorMapEncodeFn fn = nullptr;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = (TensorMapEncodeFn)p;
-    else
-      cudaGetLastError();
-  });
-  return fn;
-}
-
-// A logit tensor [rows, V] seen as [rows][256 threads][W ids]; one box = one phase of one warp's
-// part of a row: the next 32 bytes of the id range of each of its 32 lanes, laid down with the
-// 32-byte swizzle.
-static bool encode_row_map(CUtensorMap* tm, const void* base, size_t rows, int V, bool bf16) {
-  TensorMapEncodeFn enc = tensor_map_encoder();
-  if (!enc || rows == 0 || rows > 0xffffffffull) return false;
-  const int esz = bf16 ? 2 : 4, W = V / kLThreads;
-  const cuuint64_t gdim[3] = {(cuuint64_t)W, (cuuint64_t)kLThreads, (cuuint64_t)rows};
-  const cuuint64_t gstr[2] = {(cuuint64_t)W * esz, (cuuint64_t)V * esz};
-  const cuuint32_t box[3] = {(cuuint32_t)(32 / esz), 32u, 1u};   // one warp's lanes
-  const cuuint32_t es[3] = {1u, 1u, 1u};
-  return enc(tm, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base),
-             gdim, gstr, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// Fills `s` and returns the dynamic shared memory the lane kernel needs, or 0 if these
-// parameters are not eligible.
-static size_t plan_lane(const mulo_ctx* ctx, const DevParams& d, LaneArgs* s) {
-  if (d.top_k <= 0 || d.pool_k > 1) return 0;
-  const int V = d.V, k = d.top_k;
-  const int ids = d.bf16 ? 16 : 8;
-  if (V % (kLThreads * ids) != 0 || V / kLThreads > 64) return 0;
-  if (!tensor_map_encoder()) return 0;
-  // candidates aimed for beyond k: six standard deviations of the count of entries above a fixed
-  // value near the k-th largest (a row that comes up short is redone by the general routines, and
-  // even one such row costs more than the margin does)
-  const double p = (double)k / V;
-  const int margin = (int)fmax(64.0, 6.0 * sqrt(k * (1.0 - p)));
-  const int margin_boot = margin + 3 * margin / 4;   // rows without a prediction
-  if ((double)(k + margin_boot) > 0.5 * V) return 0;
-  // A list column serves two threads and holds four stacks (each thread's entries of the draft row
-  // and of the current target row): the bootstrap density's mean for 4 W ids plus six and a half
-  // standard deviations of that binomial count.  Three CTAs per SM are worth a somewhat shorter
-  // column (five and a half deviations).
-  const double pb = (double)(k + margin_boot) / V;
-  const double mu = (double)(V / kLThreads) * pb, var = mu * (1.0 - pb);   // entries of one thread in one row
-  const double quad_mean = 4.0 * mu, quad_sd = sqrt(4.0 * var);
-  // ... and a thread stops appending when fewer rows than one phase's ids are left before the other
-  // thread's stack, so the column must also hold both draft stacks, what the thread has gathered
-  // by its last phase, and one more phase
-  const int n_ph = (V / kLThreads) / ids;
-  const double part = (double)(n_ph - 1) / n_ph;
-  auto rows_needed = [&](double dev) {
-    const double a1 = quad_mean + dev * quad_sd + 2.0;
-    const double a2 = (2.0 + part) * mu + dev * sqrt(var * (2.0 + part * part)) + ids + 2.0;
-    return (int)ceil(fmax(a1, a2));
-  };
-  int R = rows_needed(6.5);
-  if (R < 16) R = 16;
-  const size_t fixed = sizeof(LaneSmem) + 128 + 1024 + 256 + (size_t)kLRing;
-  const size_t per_cta3 = (size_t)228 * 1024 / 3;
-  if (per_cta3 > fixed) {
-    const int R3 = (int)((per_cta3 - fixed) / 512);
-    if (R3 < R && R3 >= rows_needed(5.5)) R = R3;
-  }
-  // one thread's own entries must fit the 32-bit mask of its low entries
-  if (0.25 * quad_mean + 6.5 * sqrt(0.25 * quad_mean * (1.0 - pb)) > 32.0) return 0;
-  const size_t dyn = 256 + (size_t)kLRing + (size_t)R * 512;
-  if (dyn + sizeof(LaneSmem) + 128 + 1024 > (size_t)ctx->smem_optin) return 0;
-  s->W = V / kLThreads;
-  s->n_ph = s->W / ids;
-  s->R = R;
-  s->margin = margin;
-  s->a_theta = (float)inv_norm_cdf(1.0 - p);
-  s->a_boot = (float)inv_norm_cdf(1.0 - (double)(k + margin_boot) / V);
-  s->a_max = (float)inv_norm_cdf(1.0 - 0.5 / V);
-  return dyn;
-}
-
 // ---- rows with a top-k cut, NW warps per row (mulo_rows.cuh) ----------------------------
 
-#ifndef MULO_RNW
-#define MULO_RNW 2
-#endif
-constexpr int kRowsWarps = MULO_RNW;
-
-// Fills `s` and returns the dynamic shared memory of a CTA, or 0 if these parameters are not eligible.
-static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, int nw, RowsArgs* s) {
+// Fills `s` and returns the dynamic shared memory of a CTA of nw warps, or 0 if these parameters are not eligible.
+static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample, int nw, RowsArgs* s) {
   if (d.top_k <= 0 || (d.pool_k > 1 && !sample)) return 0;
   const int V = d.V, k = d.top_k;
   if (V < 1024 || d.r > 4) return 0;
@@ -1010,6 +910,14 @@ static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, in
   return dyn;
 }
 
+// Two warps per row where their lists hold the candidates, else four.  Two is the faster one wherever both do: what
+// every warp of a row repeats (bin search, ranking, decision) is a third of the instructions.
+static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, RowsArgs* s, int* nw) {
+  for (*nw = 2; *nw <= 4; *nw += 2)
+    if (const size_t dyn = plan_rows_nw(ctx, d, sample, *nw, s)) return dyn;
+  return 0;
+}
+
 template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
 static bool launch_rows_p(const mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
   auto kern = k_round_rows<BF16, HAS_U, SAMPLE, PLAIN, NW>;
@@ -1036,13 +944,17 @@ static bool launch_rows_t(const mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cu
 }
 
 template <int NW>
-static bool launch_rows(const mulo_ctx* ctx, const RowsArgs& s, bool sample, size_t dyn, cudaStream_t st) {
+static bool launch_rows_nw(const mulo_ctx* ctx, const RowsArgs& s, bool sample, size_t dyn, cudaStream_t st) {
   const bool hu = s.uncond != nullptr;
   if (sample)
     return s.P.bf16 ? launch_rows_t<true, false, true, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, true, NW>(ctx, s, dyn, st);
   if (s.P.bf16)
     return hu ? launch_rows_t<true, true, false, NW>(ctx, s, dyn, st) : launch_rows_t<true, false, false, NW>(ctx, s, dyn, st);
   return hu ? launch_rows_t<false, true, false, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, false, NW>(ctx, s, dyn, st);
+}
+
+static bool launch_rows(const mulo_ctx* ctx, const RowsArgs& s, bool sample, int nw, size_t dyn, cudaStream_t st) {
+  return nw == 2 ? launch_rows_nw<2>(ctx, s, sample, dyn, st) : launch_rows_nw<4>(ctx, s, sample, dyn, st);
 }
 
 // ---- rows without a top-k cut: the resident-row kernel ------------------------------------
@@ -1087,37 +999,6 @@ static bool launch_full(const mulo_ctx* ctx, const FullArgs& s, size_t dyn, cuda
   const bool hu = s.uncond != nullptr;
   if (s.P.bf16) return hu ? launch_full_t<true, true>(ctx, s, dyn, st) : launch_full_t<true, false>(ctx, s, dyn, st);
   return hu ? launch_full_t<false, true>(ctx, s, dyn, st) : launch_full_t<false, false>(ctx, s, dyn, st);
-}
-
-template <bool BF16, bool HAS_U>
-static bool launch_lane_t(const mulo_ctx* ctx, const LaneArgs& s, const CUtensorMap& tc, const CUtensorMap& tu,
-                          const CUtensorMap& tq, size_t dyn, cudaStream_t st) {
-  auto kern = k_round_lane<BF16, HAS_U>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kLThreads, dyn) != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    return false;
-  }
-  int grid = ctx->sm_count * per_sm;
-  if (grid > s.n_parents) grid = s.n_parents;
-  kern<<<grid, kLThreads, dyn, st>>>(s, tc, tu, tq);
-  return true;
-}
-
-static bool launch_lane(const mulo_ctx* ctx, const LaneArgs& s, size_t dyn, cudaStream_t st) {
-  const DevParams& d = s.P;
-  CUtensorMap tc, tu, tq;
-  const size_t rows = (size_t)d.B * d.H * d.W, cells = (size_t)d.B * d.h * d.w;
-  if (!encode_row_map(&tc, s.cond, rows, d.V, d.bf16)) return false;
-  if (!encode_row_map(&tu, s.uncond ? s.uncond : s.cond, rows, d.V, d.bf16)) return false;
-  if (!encode_row_map(&tq, s.draft, cells, d.V, d.bf16)) return false;
-  const bool hu = s.uncond != nullptr;
-  if (d.bf16) return hu ? launch_lane_t<true, true>(ctx, s, tc, tu, tq, dyn, st) : launch_lane_t<true, false>(ctx, s, tc, tu, tq, dyn, st);
-  return hu ? launch_lane_t<false, true>(ctx, s, tc, tu, tq, dyn, st) : launch_lane_t<false, false>(ctx, s, tc, tu, tq, dyn, st);
 }
 
 static size_t mask_smem(const mulo_params* p) { return (size_t)3 * p->H * ((p->W + 31) / 32) * 4; }
@@ -1252,7 +1133,8 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
   Workspace w;
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
-  const size_t rdyn = (ctx->force_dense || check_ws(ctx, p, &w) != MULO_OK) ? 0 : plan_rows(ctx, a.P, true, kRowsWarps, &ra);
+  int rnw = 0;
+  const size_t rdyn = (ctx->force_dense || check_ws(ctx, p, &w) != MULO_OK) ? 0 : plan_rows(ctx, a.P, true, &ra, &rnw);
   if (rdyn) {
     ra.P = a.P;
     ra.cond = a.draft;
@@ -1261,7 +1143,7 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
     ra.fail_list = w.fail_list;
     ra.n_units = p->B * a.P.h * a.P.w;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
-    if (launch_rows<kRowsWarps>(ctx, ra, true, rdyn, st)) {
+    if (launch_rows(ctx, ra, true, rnw, rdyn, st)) {
       k_sample_failed<<<2 * ctx->sm_count, kThreads, 0, st>>>(a, w.fail_list, w.status + kFailCount);
       return launched(ctx, 2);
     }
@@ -1475,7 +1357,8 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
   }
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
-  const size_t rdyn = (ctx->force_dense || ctx->no_lane || fast) ? 0 : plan_rows(ctx, a.P, false, kRowsWarps, &ra);
+  int rnw = 0;
+  const size_t rdyn = (ctx->force_dense || fast) ? 0 : plan_rows(ctx, a.P, false, &ra, &rnw);
   if (rdyn) {
     ra.P = a.P;
     ra.cond = a.cond; ra.uncond = a.uncond; ra.draft = a.draft; ra.draft_tok_lo = draft_tok_lo;
@@ -1485,22 +1368,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     ra.fail_list = w.fail_list;
     ra.n_units = p->B * p->H * p->W;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
-    fast = launch_rows<kRowsWarps>(ctx, ra, false, rdyn, st);
-    if (fast) k_verify_failed<<<2 * ctx->sm_count, kThreads, dyn, st>>>(a, w.fail_list, w.status + kFailCount);
-  }
-  LaneArgs la;
-  memset(&la, 0, sizeof la);
-  const size_t ldyn = (ctx->force_dense || ctx->no_lane || fast) ? 0 : plan_lane(ctx, a.P, &la);
-  if (ldyn) {
-    la.P = a.P;
-    la.cond = a.cond; la.uncond = a.uncond; la.draft = a.draft; la.draft_tok_lo = draft_tok_lo;
-    la.p_tok = p_tok; la.q_tok = q_tok; la.accept_prob = accept_prob;
-    la.flags = w.flags; la.cand_res = w.cand_res; la.cand_tgt = w.cand_tgt;
-    la.dev_status = w.status;
-    la.fail_list = w.fail_list;
-    la.n_parents = p->B * a.P.h * a.P.w;
-    if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
-    fast = launch_lane(ctx, la, ldyn, st);
+    fast = launch_rows(ctx, ra, false, rnw, rdyn, st);
     if (fast) k_verify_failed<<<2 * ctx->sm_count, kThreads, dyn, st>>>(a, w.fail_list, w.status + kFailCount);
   }
   StreamArgs sa;
@@ -1542,16 +1410,17 @@ mulo_status mulo_round_kernel(const mulo_ctx* ctx, const mulo_params* p, int has
   const mulo_status s = validate(p);
   if (s != MULO_OK) return s;
   const DevParams d = to_dev(p);
-  LaneArgs la;
+  RowsArgs ra;
   StreamArgs sa;
-  memset(&la, 0, sizeof la);
+  int nw;
+  memset(&ra, 0, sizeof ra);
   memset(&sa, 0, sizeof sa);
   *kernel = MULO_KERNEL_GENERAL;
   if (ctx->force_dense) return MULO_OK;
   FullArgs fa;
   memset(&fa, 0, sizeof fa);
   if (plan_full(ctx, d, has_uncond != 0, &fa)) *kernel = MULO_KERNEL_FULL;
-  else if (!ctx->no_lane && plan_lane(ctx, d, &la)) *kernel = MULO_KERNEL_LANE;
+  else if (plan_rows(ctx, d, false, &ra, &nw)) *kernel = MULO_KERNEL_LANE;
   else if (plan_stream(ctx, d, &sa)) *kernel = MULO_KERNEL_STREAM;
   return MULO_OK;
 }

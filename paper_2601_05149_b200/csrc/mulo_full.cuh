@@ -26,7 +26,7 @@
 // draw's owner thread is in ascending id).
 #pragma once
 
-#include "mulo_lane.cuh"
+#include "mulo_rows.cuh"
 
 namespace mulo {
 

@@ -4,8 +4,8 @@
 // the target rows under it, each ONCE.  The ids are split into 4 NW contiguous parts, one for every group of eight
 // lanes.
 //
-//   stream     128-byte pieces of each group's part (16 bytes per lane) through registers, kRDepth pieces in
-//              flight per lane, the next row asked into L2 by a bulk prefetch.  Per id: unpack, CFG mix (packed
+//   stream     128-byte pieces of each group's part (16 bytes per lane) through registers, four in flight per lane
+//              (two when sampling), the next row asked into L2 by a bulk prefetch.  Per id: unpack, CFG mix (packed
 //              fp32, one IEEE rounding per step), compare with a predicted pivot and a predicated append to the
 //              thread's PRIVATE list plus a bit in its survivor mask (one word per four pieces).  The loads run
 //              on into the next row, so a row's first pieces are in registers when its turn comes.
@@ -30,23 +30,32 @@
 // on the prediction.
 #pragma once
 
-#include "mulo_lane.cuh"
+#include <cuda.h>
+
+#include "mulo_stream.cuh"
 
 namespace mulo {
 
-#ifndef MULO_RDEPTH
-#define MULO_RDEPTH 4
-#endif
-#ifndef MULO_RWARPS
-#define MULO_RWARPS 16
-#endif
-constexpr int kRDepth = MULO_RDEPTH;     // pieces in flight per warp
 constexpr int kRPieceBytes = 128;        // of a group: 16 bytes per lane
 constexpr int kRBins = 256;
 constexpr int kRSetAside = 128;          // entries of the crossing bin that are ranked exactly
 constexpr int kRTries = 6;               // times a row is streamed before it is given up
 constexpr int kRSlack = 12;              // list rows kept free between the two lists of a column: a piece's entries and the closing ones
 constexpr float kRMagic = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer in the low mantissa bits
+
+constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kNearRefGap = 8.0f;      // a row whose maximum lies further from the predicted exp reference is streamed again
+                                         // against its own maximum (large exponents cost relative accuracy)
+
+// running prediction for one kind of row (draft / target), per CTA
+struct LanePredictor {
+  int have;
+  int age;                    // rows learnt from since the prediction was last lost
+  float theta, rho, mx;       // running k-th largest, density below it, row maximum
+  float pivot, inv_w, ref;    // what the next row starts from (valid while have != 0)
+  float shift, step;          // bootstrap adaptation, as in the general streaming kernel
+  int dir;
+};
 
 struct RowsArgs {
   DevParams P;
@@ -76,6 +85,7 @@ struct RowsArgs {
 template <int NW>
 struct RowsSmem {
   alignas(16) unsigned hist[kRBins + 4];   // (+ one bin that rounding may reach)
+  unsigned spill[32];                      // where the entries outside the window are counted
   alignas(16) float closer[4][32];         // -inf: what a thread past its list's end reads
   alignas(16) float sa_z[kRSetAside];      // (before the set-aside: where such a thread writes)
   unsigned short sa_at[kRSetAside];        // the entry's place (index in its owner's list << 8 | thread)
@@ -107,6 +117,31 @@ inline uint32_t rows_layout(RowsArgs& s, int nw, bool bf16, bool sample) {
   s.o_tmask = take((uint32_t)s.n_words * nw * 128u);
   s.o_dmask = sample ? s.o_tmask : take((uint32_t)s.n_words * nw * 128u);
   return off;
+}
+
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float lds_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void sts_f32(uint32_t addr, float v) {
+  asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+// 2^t by the special-function unit (relative error about 2^-22)
+__device__ __forceinline__ float ex2f(float t) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(t));
+  return r;
+}
+
+template <int J>
+__device__ __forceinline__ uint32_t word_of(const uint4& v) {
+  return J == 0 ? v.x : J == 1 ? v.y : J == 2 ? v.z : v.w;
 }
 
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
@@ -196,14 +231,99 @@ __device__ __forceinline__ void row_piece(const uint4& c, const uint4& u, float2
   }
 }
 
+// 2^x in double, out of line: three call sites, a few hundred instructions each otherwise
+__device__ __noinline__ double lane_exp2(double x) { return exp2(x); }
+
+// Philox4x32-10 as a rolled loop (one thread per row runs it; the unrolled form is ten times the code)
+__device__ __noinline__ uint4 lane_philox(uint4 c, uint2 k) {
+#pragma unroll 1
+  for (int i = 0; i < 10; ++i) {
+    const uint32_t a = 0xD2511F53u, b = 0xCD9E8D57u;
+    const uint32_t h0 = __umulhi(a, c.x), l0 = a * c.x;
+    const uint32_t h1 = __umulhi(b, c.z), l1 = b * c.z;
+    c = make_uint4(h1 ^ c.y ^ k.x, l1, h0 ^ c.w ^ k.y, l0);
+    k.x += 0x9E3779B9u;
+    k.y += 0xBB67AE85u;
+  }
+  return c;
+}
+
+// The optional probability outputs of a position (one thread; out of line: double divisions).
+__device__ __noinline__ void lane_write_probs(float* p_tok, float* q_tok_out, float* accept_prob, size_t g, double e_tok,
+                                              double q_tok, double Z, bool threshold_rule) {
+  const double p = e_tok / Z;
+  if (p_tok) p_tok[g] = (float)p;
+  if (q_tok_out) q_tok_out[g] = (float)q_tok;
+  if (accept_prob) {
+    double thr;
+    if (threshold_rule) thr = p;
+    else if (q_tok <= 0.0) thr = p > 0.0 ? 1.0 : 0.0;
+    else thr = fmin(1.0, p / q_tok);
+    accept_prob[g] = (float)thr;
+  }
+}
+
+// The predictor of one kind of row after a row (ok: theta found exactly).  One thread; out of line.
+__device__ __noinline__ void lane_learn(LanePredictor* prp, bool ok, int reason, float theta, float pivot, int n,
+                                        int n_ge, float mx, int margin, float a_theta, float a_boot) {
+  LanePredictor pr = *prp;
+  if (!ok) {
+    pr.have = 0;
+    pr.age = 0;
+    const int dir = reason == 2 ? -1 : (reason == 1 || reason == 3) ? 1 : 0;
+    if (dir != 0) {
+      const float unit = 0.5f * (a_theta - a_boot);
+      if (pr.dir == 0) pr.step = unit;
+      else if (pr.dir == dir) pr.step = fminf(2.0f * pr.step, 64.0f * unit);
+      else pr.step = fmaxf(0.5f * pr.step, 0.25f * unit);
+      pr.shift += (float)dir * pr.step;
+      pr.dir = dir;
+    }
+  } else {
+    pr.dir = 0;
+    const int below = n - n_ge;   // candidates in [pivot, theta)
+    // running means: a plain average over the first four rows, weight 1/4 for the newest after that
+    const float w_new = pr.have ? fmaxf(0.25f, 1.0f / (float)(pr.age + 1)) : 1.0f;
+    float rho = pr.rho;
+    bool rho_ok = pr.have != 0;
+    if (theta > pivot && below >= 16) {
+      const float r_new = (float)below / (theta - pivot);
+      rho = pr.have ? pr.rho + w_new * (r_new - pr.rho) : r_new;
+      rho_ok = true;
+    }
+    if (!rho_ok) {
+      pr.have = 0;
+      pr.age = 0;
+    } else {
+      pr.theta = pr.have ? pr.theta + w_new * (theta - pr.theta) : theta;
+      pr.mx = pr.have ? pr.mx + w_new * (mx - pr.mx) : mx;
+      pr.rho = rho;
+      pr.have = 1;
+      if (pr.age < 8) ++pr.age;
+      // a prediction that rests on a single row carries that row's noise in the threshold and in
+      // the density: the row after it aims for a wider margin
+      const float d = (pr.age < 2 ? 1.4f : 1.0f) * (float)margin / rho;
+      pr.pivot = pr.theta - d;
+      pr.inv_w = (float)kRBins / (2.0f * d);   // the histogram spans twice the distance pivot -> threshold
+      pr.ref = pr.mx;
+    }
+  }
+  *prp = pr;
+}
+
 // Double division, out of line.
 __device__ __noinline__ double rows_div(double a, double b) { return a / b; }
 
+// Warps per SM the kernel is compiled for: 16 (128 registers, four pieces in flight; eight CTAs of two warps are also
+// what the lists of V = 16384, top-k 2000 leave room for), 24 for the sampling kernel, which keeps no draft list.
+__host__ __device__ constexpr int rows_warps(bool sample) { return sample ? 24 : 16; }
+
 // PLAIN: T = 1 and every piece a thread's whole 16 bytes (V splits evenly), so no scaling and no bounds checks.
 template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
-__global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
+__global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
   constexpr int NT = NW * 32;
   constexpr int IDS = BF16 ? 8 : 4;              // ids per lane per piece
+  constexpr int kRDepth = SAMPLE ? 2 : 4;        // pieces in flight per lane
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ RowsSmem<NW> sm;
   const DevParams& P = a.P;
@@ -230,6 +350,7 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
   const uint32_t tm = my + a.o_tmask + (uint32_t)tid * 4u, dm = my + a.o_dmask + (uint32_t)tid * 4u;
   const uint32_t hbase = smem_u32(sm.hist) - (__float_as_uint(kRMagic) << 2);
   const uint32_t closer = smem_u32(sm.closer) + (uint32_t)lane * 4u, dump = smem_u32(sm.sa_z) + (uint32_t)lane * 4u;
+  const uint32_t dl_dump = smem_u32(sm.sa_z) + (uint32_t)lane * (DROW / 32u), spill = smem_u32(sm.spill) + (uint32_t)lane * 4u;
 
 #pragma unroll 1
   for (int i = tid; i < kRBins + 4; i += NT) sm.hist[i] = 0;
@@ -404,42 +525,37 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
 #pragma unroll 1
     for (int i = 0; i < n_max; i += 4, ad += 4 * step, dd += 4 * dstep) {
       const bool in = i < n;
-      const uint32_t from = in ? ad : closer, to = in ? ad : dump;
+      const uint32_t from = in ? ad : closer, to = !Q && in ? ad : dump;
       float z[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) z[k] = lds_f32(from + k * 128);
       uint32_t l4 = 0;
+// (entries outside the window count in a word of their own lane: a predicated reduction becomes a branch)
 #define MULO_ENTRY(K, S)                                                                       \
   {                                                                                            \
     const float e = ex2f(fmaf(z[K], kLog2e, c0));                                              \
     const uint32_t bin = __float_as_uint(fmaf(z[K], inv_w, hm));                               \
-    if (Q)                                                                                     \
-      asm volatile(                                                                            \
-          "{\n\t.reg .pred p;\n\t.reg .u32 t;\n\t"                                             \
-          "sub.u32 t, %2, %3;\n\t"                                                             \
-          "setp.le.u32 p, t, %4;\n\t"                                                          \
-          "@p red.shared.add.u32 [%5], 1;\n\t"                                                 \
-          "@p or.b32 %0, %0, %6;\n\t"                                                          \
-          "@!p add.f32 %1, %1, %7;\n\t}"                                                       \
-          : "+r"(l4), "+f"(S)                                                                  \
-          : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(hbase + (bin << 2)), "n"(1 << K), "f"(e) \
-          : "memory");                                                                         \
-    else                                                                                       \
-      asm volatile(                                                                            \
-          "{\n\t.reg .pred p;\n\t.reg .u32 t;\n\t"                                             \
-          "sub.u32 t, %2, %3;\n\t"                                                             \
-          "setp.le.u32 p, t, %4;\n\t"                                                          \
-          "@p red.shared.add.u32 [%5], 1;\n\t"                                                 \
-          "@p or.b32 %0, %0, %6;\n\t"                                                          \
-          "@!p add.f32 %1, %1, %7;\n\t"                                                        \
-          "@!p st.shared.f32 [%8 + %9], %7;\n\t}"                                              \
-          : "+r"(l4), "+f"(S)                                                                  \
-          : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(hbase + (bin << 2)), "n"(1 << K), "f"(e), "r"(to), "n"(K * 128) \
-          : "memory");                                                                         \
-    if (Q && in) dlist_put<BF16>(dd + K * DROW, BF16 && !PLAIN ? __fmul_rn(z[K], T) : z[K]);   \
+    const uint32_t at = hbase + (bin << 2);                                                    \
+    asm volatile(                                                                              \
+        "{\n\t.reg .pred p;\n\t.reg .u32 t, w;\n\t"                                            \
+        "sub.u32 t, %2, %3;\n\t"                                                               \
+        "setp.le.u32 p, t, %4;\n\t"                                                            \
+        "selp.u32 w, %5, %10, p;\n\t"                                                          \
+        "red.shared.add.u32 [w], 1;\n\t"                                                       \
+        "@p or.b32 %0, %0, %6;\n\t"                                                            \
+        "@!p add.f32 %1, %1, %7;\n\t"                                                          \
+        "@!p st.shared.f32 [%8 + %9], %7;\n\t}"                                                \
+        : "+r"(l4), "+f"(S)                                                                    \
+        : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(at), "n"(1 << K), "f"(e), "r"(to), "n"(K * 128), "r"(spill) \
+        : "memory");                                                                           \
   }
       MULO_ENTRY(0, s0) MULO_ENTRY(1, s1) MULO_ENTRY(2, s0) MULO_ENTRY(3, s1)
 #undef MULO_ENTRY
+      if (Q) {   // (rows past the end of the list take -inf, or go where nobody reads)
+        const uint32_t dt = in ? dd : dl_dump;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) dlist_put<BF16>(dt + k * DROW, BF16 && !PLAIN ? __fmul_rn(z[k], T) : z[k]);
+      }
       mx = fmaxf(mx, fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])));
       if (i < 32) low_a |= l4 << i;   // (uniform)
       else low_b |= l4 << (i & 31);
@@ -462,23 +578,25 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
     const uint32_t flip = up ? 0u : 3u;
     float s = 0.f;
     uint32_t first = 0;
-    auto one = [&](uint32_t bit) {
-      const uint32_t i = first + ((uint32_t)__popc(bit - 1u) ^ flip), at = tl + i * step;
-      const float z = lds_f32(bit ? at : closer);
+    auto one = [&](uint32_t bit, uint32_t& i, float& z) -> bool {   // does the entry lie in the crossing bin?
+      i = first + ((uint32_t)__popc(bit - 1u) ^ flip);
+      const uint32_t at = tl + i * step;
+      z = lds_f32(bit ? at : closer);
       const uint32_t bin = __float_as_uint(fmaf(z, inv_w, hm));   // (-inf: as unsigned above every bin; its exp is 0)
       float e = ex2f(fmaf(z, kLog2e, c0));
       e = bin > bm ? e : 0.f;
       s += e;
       if (is_q) {
         if (bin < bm) dlist_put<BF16>(dl + i * dstep, -INFINITY);
-      } else if (bit) {
-        sts_f32(at, e);
+      } else {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(at), "f"(e), "r"(bit) : "memory");
       }
-      if (bin == bm) {
-        const unsigned k = atomicAdd(&sm.n_sa, 1u) & (unsigned)(kRSetAside - 1);
-        sm.sa_z[k] = z;
-        sm.sa_at[k] = (unsigned short)(i << 8 | (uint32_t)tid);
-      }
+      return bin == bm;
+    };
+    auto aside = [&](uint32_t i, float z) {
+      const unsigned k = atomicAdd(&sm.n_sa, 1u) & (unsigned)(kRSetAside - 1);
+      sm.sa_z[k] = z;
+      sm.sa_at[k] = (unsigned short)(i << 8 | (uint32_t)tid);
     };
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
@@ -489,8 +607,13 @@ __global__ void __launch_bounds__(NW * 32, MULO_RWARPS / NW) k_round_rows(const 
         low_a ^= b0;
         const uint32_t b1 = low_a & (0u - low_a);
         low_a ^= b1;
-        one(b0);
-        one(b1);
+        uint32_t i0, i1;
+        float z0, z1;
+        const bool h0 = one(b0, i0, z0), h1 = one(b1, i1, z1);
+        if (h0 || h1) {
+          if (h0) aside(i0, z0);
+          if (h1) aside(i1, z1);
+        }
       }
       low_a = low_b;
       first = 32;
