@@ -37,7 +37,6 @@ UNIT = "positions/s"
 # (traffic grows in proportion to the positions, every row being read once).  An entry is removed when
 # its kernel changes, and the line then reports null until the counters have been taken again.
 TRAFFIC_BYTES_PER_POSITION = {
-    ("C4", "lane"): 74268.0,   # 608.4 MB per launch of 8192 positions (algorithmic: 73,752 B per position)
     ("P4", "full"): 66598.0,   # 545.6 MB per launch of 8192 positions (algorithmic: 67,560 B; the lists come from L2)
 }
 L2_BYTES = 126 << 20
@@ -298,7 +297,7 @@ def run_ours(args, cfg):
     achieved = alg_bytes / (row_avg_ms * 1e-3) / 1e9
     which = ctx.round_kernel(p, cfg.has_uncond)
     kernel = {"full": "k_round_full",
-              "lane": "k_round_lane (+ k_verify_failed for rows that left the fast path)",
+              "lane": "k_round_rows (+ k_verify_failed for rows that left the fast path)",
               "stream": "k_round_stream (+ k_verify_failed for rows that left the fast path)",
               "general": "k_verify_rows"}[which]
     roofline = {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak,

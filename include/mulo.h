@@ -154,9 +154,9 @@ mulo_status mulo_kernel_launches(const mulo_ctx* ctx, uint64_t* count);
  *                        V <= 16384 in bf16 with classifier-free guidance): rows are made resident
  *                        in shared memory and every entry is exponentiated once; with Eq. 5 and
  *                        redraws from the target distribution the draft logits are not read;
- *   MULO_KERNEL_LANE     top-k on, pooling off, V a multiple of 4096 (bf16) or 2048 (fp32) and
- *                        at most 16384: every thread of a CTA owns a contiguous range of the
- *                        vocabulary, rows are streamed once through per-warp shared-memory rings;
+ *   MULO_KERNEL_LANE     top-k on, pooling off, V >= 1024, rows whose candidates fit the kernel's lists (k up
+ *                        to about a third of V): two or four warps per row, every thread keeps the candidates of
+ *                        the ids it reads, rows are streamed once through registers;
  *   MULO_KERNEL_STREAM   top-k on, V >= 1024 (with pooling, V <= 16384), any other shape: rows
  *                        streamed once in chunks, candidates compacted per segment;
  *   MULO_KERNEL_GENERAL  everything else (top-k off, tiny vocabularies): one CTA per row, the

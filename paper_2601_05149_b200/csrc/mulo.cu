@@ -656,8 +656,10 @@ const char* mulo_status_string(mulo_status s) {
 mulo_status mulo_create(mulo_ctx** out, int device) {
   if (!out) return MULO_ERR_INVALID_ARG;
   *out = nullptr;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) {
+  // (two attributes: the whole property struct takes the driver 2 to 40 ms)
+  int sm_count = 0, smem_optin = 0;
+  if (cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device) != cudaSuccess) {
     cudaGetLastError();
     return MULO_ERR_CUDA;
   }
@@ -665,8 +667,8 @@ mulo_status mulo_create(mulo_ctx** out, int device) {
   mulo_ctx* c = new (std::nothrow) mulo_ctx();
   if (!c) return MULO_ERR_INVALID_ARG;
   c->device = device;
-  c->sm_count = prop.multiProcessorCount;
-  c->smem_optin = (int)prop.sharedMemPerBlockOptin;
+  c->sm_count = sm_count;
+  c->smem_optin = smem_optin;
   c->ws = nullptr;
   c->ws_bytes = 0;
   c->launches = 0;
