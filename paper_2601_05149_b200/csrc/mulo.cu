@@ -6,11 +6,13 @@
 
 #include <mutex>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/mulo.h"
 #include "mulo_dense.cuh"
 #include "mulo_islands.cuh"
+#include "mulo_resident.cuh"
 #include "mulo_full.cuh"
 #include "mulo_rows.cuh"
 #include "mulo_stream.cuh"
@@ -74,23 +76,41 @@ __device__ __forceinline__ PoolSmem carve_pool(const DevParams& P, unsigned char
   return ps;
 }
 
+// The kernels of the general path come in two versions: RES for vocabularies whose rows stay in shared memory, and
+// the one that reads the row from L1/L2 again and again (V > 49152).
+template <bool RES>
+using GeneralScratch = std::conditional_t<RES, ResScratch, BlockScratch>;
+
+__device__ __forceinline__ void round_z(double& Z) {   // Z_q as the stages hand it on: an fp32 (hi, lo) pair
+  const float hi = (float)Z, lo = (float)(Z - (double)hi);
+  Z = (double)hi + (double)lo;
+}
+
 // mulo_upsample_pool: one CTA per low-res cell.
-__global__ void __launch_bounds__(kThreads) k_upsample_pool(RowKernelArgs a) {
-  __shared__ BlockScratch bs;
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_upsample_pool(RowKernelArgs a) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
   const DevParams& P = a.P;
   const int cell = blockIdx.x;   // b*h*w + ca*w + cc
   const int b = cell / (P.h * P.w), rem = cell % (P.h * P.w), ca = rem / P.w, cc = rem % P.w;
   RowSrc qr = draft_row(a, cell);
+  const int tok = checked_token(a.draft_tok_lo[cell], P.V, a.dev_status);
   RowStats sq;
-  dense_row_stats(qr, P.top_k, bs, sq.theta, sq.m, sq.Z);
+  float zq;
+  if constexpr (RES) {
+    int calls = 0;
+    res_row_stats(ResRow(reinterpret_cast<float*>(dyn), P.V), qr, P.top_k, sc, calls, tok, zq, sq);
+  } else {
+    dense_row_stats(qr, P.top_k, sc, sq.theta, sq.m, sq.Z);
+    zq = load1(qr, tok);
+  }
   if (threadIdx.x == 0) {
-    const int tok = checked_token(a.draft_tok_lo[cell], P.V, a.dev_status);
     const float Zhi = (float)sq.Z, Zlo = (float)(sq.Z - (double)Zhi);
     a.stats_out[(size_t)cell * 4 + 0] = sq.theta;
     a.stats_out[(size_t)cell * 4 + 1] = sq.m;
     a.stats_out[(size_t)cell * 4 + 2] = Zhi;
     a.stats_out[(size_t)cell * 4 + 3] = Zlo;
-    float zq = load1(qr, tok);
     double q = (zq >= sq.theta) ? exp((double)zq - (double)sq.m) / ((double)Zhi + (double)Zlo) : 0.0;
     for (int di = 0; di < P.r; ++di)
       for (int dj = 0; dj < P.r; ++dj) {
@@ -101,38 +121,56 @@ __global__ void __launch_bounds__(kThreads) k_upsample_pool(RowKernelArgs a) {
   }
 }
 
+// The inverse-CDF draw of uniform u from softmax(topk(row / T)); one thread writes the token to *out.
+template <bool RES>
+__device__ __forceinline__ void draw_row(const RowSrc& src, int top_k, double u, GeneralScratch<RES>& sc, unsigned char* dyn, int32_t* out) {
+  RowStats st;
+  if constexpr (RES) {
+    const ResRow row(reinterpret_cast<float*>(dyn), src.V);
+    int calls = 0;
+    float unused;
+    const ResSums sums = res_row_stats(row, src, top_k, sc, calls, -1, unused, st);
+    res_pick(row, sums, u, [&](int x) -> double { return (double)row.at(x); }, out);
+  } else {
+    dense_row_stats(src, top_k, sc, st.theta, st.m, st.Z);
+    __syncthreads();
+    const float invZ = (float)(1.0 / st.Z);
+    // lambda = 0 and no special token: the weights are the probabilities themselves
+    const int tok = dense_draw(src, src, st, st, invZ, invZ, 0.0f, -1, 0.0, nullptr, u, sc);
+    if (threadIdx.x == 0) *out = tok;
+  }
+}
+
 // The drafter's own draw (Sec. 3.2 Step 1) for one low-res cell by the general routines:
 // q = softmax(topk(l_q / T)), inverse CDF with word 0 of the tag-1 Philox stream.
-__device__ inline void sample_cell(const RowKernelArgs& a, int cell, BlockScratch& bs) {
+template <bool RES>
+__device__ __forceinline__ void sample_cell(const RowKernelArgs& a, int cell, GeneralScratch<RES>& sc, unsigned char* dyn) {
   const DevParams& P = a.P;
   const int b = cell / (P.h * P.w), rem = cell % (P.h * P.w);
-  RowSrc qr = draft_row(a, cell);
-  RowStats sq;
-  dense_row_stats(qr, P.top_k, bs, sq.theta, sq.m, sq.Z);
-  __syncthreads();
-  const float invZ = (float)(1.0 / sq.Z);
   const uint4 rnd = philox4x32_10(make_uint4((uint32_t)rem, (uint32_t)b + P.image_offset, P.round, 1u),
                                   make_uint2(P.seed_lo, P.seed_hi));
-  // lambda = 0 and no special token: the weights are q itself
-  const int tok = dense_draw(qr, qr, sq, sq, invZ, invZ, 0.0f, -1, 0.0, nullptr, uniform24(rnd.x), bs);
-  if (threadIdx.x == 0) a.out_tok[cell] = tok;
+  draw_row<RES>(draft_row(a, cell), P.top_k, uniform24(rnd.x), sc, dyn, a.out_tok + cell);
 }
 
 // mulo_sample_draft, general path: one CTA per low-res cell.
-__global__ void __launch_bounds__(kThreads) k_sample_draft(RowKernelArgs a) {
-  __shared__ BlockScratch bs;
-  sample_cell(a, blockIdx.x, bs);
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_sample_draft(RowKernelArgs a) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
+  sample_cell<RES>(a, blockIdx.x, sc, dyn);
 }
 
-// Second launch of mulo_sample_draft's fast path: the cells the streaming kernel put on its list.
-__global__ void __launch_bounds__(kThreads) k_sample_failed(RowKernelArgs a, const int32_t* fail_list,
+// Second launch of mulo_sample_draft's fast path: the cells the fast kernel put on its list.
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_sample_failed(RowKernelArgs a, const int32_t* fail_list,
                                                             const uint32_t* fail_count) {
-  __shared__ BlockScratch bs;
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
   const size_t total = (size_t)a.P.B * a.P.h * a.P.w;
   const size_t n = min((size_t)*fail_count, total);
   for (size_t idx = blockIdx.x; idx < n; idx += gridDim.x) {
     const size_t cell = (size_t)fail_list[idx];
-    if (cell < total) sample_cell(a, (int)cell, bs);
+    if (cell < total) sample_cell<RES>(a, (int)cell, sc, dyn);
     __syncthreads();
   }
 }
@@ -186,6 +224,13 @@ __global__ void __launch_bounds__(256) k_redraw_fill(const int32_t* __restrict__
   }
 }
 
+// a 4-byte load that is neither taken from the read-only cache nor moved
+__device__ __forceinline__ int ld_fresh(const int32_t* p) {
+  int v;
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 struct RedrawArgs {
   DevParams P;
   const char* cond;
@@ -198,14 +243,32 @@ struct RedrawArgs {
 
 // One step: every position of the step's slice of the list draws its token from the target
 // distribution of the given logits; uniform = word 0 of Philox at (t, image, round, 1 + s).
-__global__ void __launch_bounds__(kThreads) k_redraw_step(RedrawArgs a) {
-  __shared__ BlockScratch bs;
+// Steps follow one another by the thousand, a handful of positions each, so a step is bound by latency: the launch
+// may begin while the kernel before it in the stream still runs (programmatic dependent launch), asks its rows into
+// L2 -- a hint: nothing is read -- and waits for that kernel before it reads anything it uses.
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_redraw_step(RedrawArgs a) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
   const DevParams& P = a.P;
-  const int beg = a.offsets[a.s], end = a.offsets[a.s + 1];
   const size_t N = (size_t)P.H * P.W, total = (size_t)P.B * N;
   const size_t bytes = (size_t)P.V * (P.bf16 ? 2 : 4);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (threadIdx.x == 0) {
+    const int beg = ld_fresh(a.offsets + a.s), end = ld_fresh(a.offsets + a.s + 1);
+    const long long i = (long long)beg + (long long)blockIdx.x;
+    if (beg >= 0 && i < end && i < (long long)total) {
+      const size_t g = (size_t)(uint32_t)ld_fresh(a.pos_list + i);
+      if (g < total) {
+        prefetch_l2(a.cond + g * bytes, (uint32_t)bytes);
+        if (a.uncond) prefetch_l2(a.uncond + g * bytes, (uint32_t)bytes);
+      }
+    }
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int beg = ld_fresh(a.offsets + a.s), end = ld_fresh(a.offsets + a.s + 1);
   for (int i = beg + (int)blockIdx.x; i < end; i += (int)gridDim.x) {
-    const size_t g = (size_t)a.pos_list[i];
+    const size_t g = (size_t)ld_fresh(a.pos_list + i);
     if (g < total) {   // block-uniform
       const uint32_t b = (uint32_t)(g / N), t = (uint32_t)(g - (size_t)b * N);
       RowSrc tr;
@@ -215,14 +278,9 @@ __global__ void __launch_bounds__(kThreads) k_redraw_step(RedrawArgs a) {
       tr.invT = P.invT;
       tr.V = P.V;
       tr.bf16 = P.bf16;
-      RowStats sp;
-      dense_row_stats(tr, P.top_k, bs, sp.theta, sp.m, sp.Z);
-      __syncthreads();
-      const float invZ = (float)(1.0 / sp.Z);
       const uint4 rnd = philox4x32_10(make_uint4(t, b + P.image_offset, P.round, 1u + (uint32_t)a.s),
                                       make_uint2(P.seed_lo, P.seed_hi));
-      const int tok = dense_draw(tr, tr, sp, sp, invZ, invZ, 0.0f, -1, 0.0, nullptr, uniform24(rnd.x), bs);
-      if (threadIdx.x == 0) a.out_tok[g] = tok;
+      draw_row<RES>(tr, P.top_k, uniform24(rnd.x), sc, dyn, a.out_tok + g);
     }
     __syncthreads();
   }
@@ -249,60 +307,86 @@ __global__ void __launch_bounds__(256) k_downsample(const int32_t* __restrict__ 
   y[cell] = best_tok;
 }
 
+// Statistics of a draft row by the general routines, Z_q rounded as the stages hand it on.
+template <bool RES>
+__device__ __forceinline__ void general_draft_stats(const DevParams& P, const RowSrc& qr, GeneralScratch<RES>& sc, unsigned char* dyn,
+                                                    RowStats& sq) {
+  if constexpr (RES) {
+    int calls = 0;
+    float unused;
+    res_row_stats(ResRow(reinterpret_cast<float*>(dyn), P.V), qr, P.top_k, sc, calls, -1, unused, sq);
+    __syncthreads();   // the row's memory is free again
+  } else {
+    dense_row_stats(qr, P.top_k, sc, sq.theta, sq.m, sq.Z);
+  }
+  round_z(sq.Z);
+}
+// One position by the general routines (its results are valid in thread 0).
+template <bool RES, class WantDraws>
+__device__ __forceinline__ void general_position(const RowKernelArgs& a, const RowSrc& tr, const RowSrc& qr, const RowStats& sq,
+                                                 int tok, uint32_t image, uint32_t t, bool decide, int given_accept,
+                                                 WantDraws want, GeneralScratch<RES>& sc, unsigned char* dyn, PositionOut& o) {
+  const DevParams& P = a.P;
+  if constexpr (RES) {
+    int calls = 0;
+    res_position(P, ResRow(reinterpret_cast<float*>(dyn), P.V), tr, qr, sq, tok, a.nn, image, t, decide, given_accept, want, sc,
+                 calls, a.dev_status, o);
+  } else {
+    dense_position(P, tr, qr, sq, tok, a.nn, image, t, decide, given_accept, want, sc, carve_pool(P, dyn), a.dev_status, o);
+  }
+}
+__device__ __forceinline__ void store_position(const RowKernelArgs& a, size_t g, const PositionOut& o) {   // one thread
+  a.flags[g] = o.accepted ? 0 : 1;
+  a.cand_res[g] = o.tok_residual;
+  a.cand_tgt[g] = o.tok_target;
+  if (a.p_tok) a.p_tok[g] = o.p_tok;
+  if (a.q_tok) a.q_tok[g] = o.q_tok;
+  if (a.accept_prob) a.accept_prob[g] = o.accept_prob;
+}
+__device__ __forceinline__ RowStats given_stats(const RowKernelArgs& a, size_t cell) {
+  RowStats sq;
+  sq.theta = a.stats_in[cell * 4 + 0];
+  sq.m = a.stats_in[cell * 4 + 1];
+  sq.Z = (double)a.stats_in[cell * 4 + 2] + (double)a.stats_in[cell * 4 + 3];
+  return sq;
+}
+
 // mulo_verify (FUSED = false): one CTA per target position, draft statistics given.
 // mulo_round  (FUSED = true):  one CTA per low-res cell: draft statistics, then its
 // r*r children; accept flags and candidate draws go to the workspace.
-template <bool FUSED>
-__global__ void __launch_bounds__(kThreads) k_verify_rows(RowKernelArgs a) {
-  __shared__ BlockScratch bs;
+template <bool FUSED, bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_verify_rows(RowKernelArgs a) {
   extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
   const DevParams& P = a.P;
-  PoolSmem ps = carve_pool(P, dyn);
   const int N = P.H * P.W;
   if (FUSED) {
     const int cell = blockIdx.x;
     const int b = cell / (P.h * P.w), rem = cell % (P.h * P.w), ca = rem / P.w, cc = rem % P.w;
     RowSrc qr = draft_row(a, cell);
     RowStats sq;
-    dense_row_stats(qr, P.top_k, bs, sq.theta, sq.m, sq.Z);
-    {   // the unfused path stores Z_q as an fp32 (hi, lo) pair; keep both paths identical
-      const float Zhi = (float)sq.Z, Zlo = (float)(sq.Z - (double)Zhi);
-      sq.Z = (double)Zhi + (double)Zlo;
-    }
+    general_draft_stats<RES>(P, qr, sc, dyn, sq);
     const int tok = checked_token(a.draft_tok_lo[cell], P.V, a.dev_status);
     for (int di = 0; di < P.r; ++di)
       for (int dj = 0; dj < P.r; ++dj) {
         const int t = (ca * P.r + di) * P.W + cc * P.r + dj;
         const size_t g = (size_t)b * N + t;
-        RowSrc tr = target_row(a, g);
         PositionOut o;
         const int mode = P.resample_mode;
-        dense_position(P, tr, qr, sq, tok, a.nn, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
-                       [mode](int acc) { return draws_for(mode, acc); }, bs, ps, a.dev_status, o);
-        if (threadIdx.x == 0) {
-          a.flags[g] = o.accepted ? 0 : 1;
-          a.cand_res[g] = o.tok_residual;
-          a.cand_tgt[g] = o.tok_target;
-          if (a.p_tok) a.p_tok[g] = o.p_tok;
-          if (a.q_tok) a.q_tok[g] = o.q_tok;
-          if (a.accept_prob) a.accept_prob[g] = o.accept_prob;
-        }
+        general_position<RES>(a, target_row(a, g), qr, sq, tok, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
+                              [mode](int acc) { return draws_for(mode, acc); }, sc, dyn, o);
+        if (threadIdx.x == 0) store_position(a, g, o);
         __syncthreads();
       }
   } else {
     const size_t g = blockIdx.x;
     const int b = (int)(g / N), t = (int)(g % N), i = t / P.W, j = t % P.W;
     const size_t cell = ((size_t)b * P.h + i / P.r) * P.w + j / P.r;
-    RowSrc qr = draft_row(a, cell);
-    RowStats sq;
-    sq.theta = a.stats_in[cell * 4 + 0];
-    sq.m = a.stats_in[cell * 4 + 1];
-    sq.Z = (double)a.stats_in[cell * 4 + 2] + (double)a.stats_in[cell * 4 + 3];
+    const RowStats sq = given_stats(a, cell);
     const int tok = checked_token(a.draft_tok_hi[g], P.V, a.dev_status);
-    RowSrc tr = target_row(a, g);
     PositionOut o;
-    dense_position(P, tr, qr, sq, tok, a.nn, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
-                   [](int) { return (int)kDrawNone; }, bs, ps, a.dev_status, o);
+    general_position<RES>(a, target_row(a, g), draft_row(a, cell), sq, tok, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
+                          [](int) { return (int)kDrawNone; }, sc, dyn, o);
     if (threadIdx.x == 0) {
       a.flags[g] = o.accepted ? 0 : 1;
       a.p_tok[g] = o.p_tok;
@@ -312,14 +396,14 @@ __global__ void __launch_bounds__(kThreads) k_verify_rows(RowKernelArgs a) {
   }
 }
 
-// Second launch of mulo_round's fast path: the positions the streaming kernel put on its
-// list (rows whose pivot prediction failed), done by the dense routines, one CTA at a time.
-__global__ void __launch_bounds__(kThreads) k_verify_failed(RowKernelArgs a, const int32_t* fail_list,
+// Second launch of mulo_round's fast paths: the positions the fast kernel put on its
+// list (rows whose prediction failed), done by the general routines, one CTA at a time.
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_verify_failed(RowKernelArgs a, const int32_t* fail_list,
                                                             const uint32_t* fail_count) {
-  __shared__ BlockScratch bs;
   extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
   const DevParams& P = a.P;
-  PoolSmem ps = carve_pool(P, dyn);
   const int N = P.H * P.W;
   const size_t total = (size_t)P.B * N;
   const size_t n = min((size_t)*fail_count, total);
@@ -330,25 +414,13 @@ __global__ void __launch_bounds__(kThreads) k_verify_failed(RowKernelArgs a, con
     const size_t cell = ((size_t)b * P.h + i / P.r) * P.w + j / P.r;
     RowSrc qr = draft_row(a, cell);
     RowStats sq;
-    dense_row_stats(qr, P.top_k, bs, sq.theta, sq.m, sq.Z);
-    {   // Z_q rounded as everywhere else (fp32 hi + lo)
-      const float Zhi = (float)sq.Z, Zlo = (float)(sq.Z - (double)Zhi);
-      sq.Z = (double)Zhi + (double)Zlo;
-    }
+    general_draft_stats<RES>(P, qr, sc, dyn, sq);
     const int tok = checked_token(a.draft_tok_lo[cell], P.V, a.dev_status);
-    RowSrc tr = target_row(a, g);
     PositionOut o;
     const int mode = P.resample_mode;
-    dense_position(P, tr, qr, sq, tok, a.nn, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
-                   [mode](int acc) { return draws_for(mode, acc); }, bs, ps, a.dev_status, o);
-    if (threadIdx.x == 0) {
-      a.flags[g] = o.accepted ? 0 : 1;
-      a.cand_res[g] = o.tok_residual;
-      a.cand_tgt[g] = o.tok_target;
-      if (a.p_tok) a.p_tok[g] = o.p_tok;
-      if (a.q_tok) a.q_tok[g] = o.q_tok;
-      if (a.accept_prob) a.accept_prob[g] = o.accept_prob;
-    }
+    general_position<RES>(a, target_row(a, g), qr, sq, tok, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
+                          [mode](int acc) { return draws_for(mode, acc); }, sc, dyn, o);
+    if (threadIdx.x == 0) store_position(a, g, o);
     __syncthreads();
   }
 }
@@ -370,11 +442,11 @@ __device__ __forceinline__ bool covered_by_other(const uint32_t* rej, int Ww, in
 }
 
 // mulo_resample: one CTA per target position; positions outside R_X copy x~.
-__global__ void __launch_bounds__(kThreads) k_resample_rows(RowKernelArgs a) {
-  __shared__ BlockScratch bs;
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_resample_rows(RowKernelArgs a) {
   extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
   const DevParams& P = a.P;
-  PoolSmem ps = carve_pool(P, dyn);
   const int N = P.H * P.W, Ww = (P.W + 31) / 32;
   const size_t g = blockIdx.x;
   const int b = (int)(g / N), t = (int)(g % N), i = t / P.W, j = t % P.W;
@@ -400,17 +472,12 @@ __global__ void __launch_bounds__(kThreads) k_resample_rows(RowKernelArgs a) {
     }
   } else use_res = rejected;
   const size_t cell = ((size_t)b * P.h + i / P.r) * P.w + j / P.r;
-  RowSrc qr = draft_row(a, cell);
-  RowStats sq;
-  sq.theta = a.stats_in[cell * 4 + 0];
-  sq.m = a.stats_in[cell * 4 + 1];
-  sq.Z = (double)a.stats_in[cell * 4 + 2] + (double)a.stats_in[cell * 4 + 3];
+  const RowStats sq = given_stats(a, cell);
   const int tok = checked_token(tok_raw, P.V, a.dev_status);
-  RowSrc tr = target_row(a, g);
   PositionOut o;
   const int draw = use_res ? kDrawResidual : kDrawTarget;
-  dense_position(P, tr, qr, sq, tok, a.nn, (uint32_t)b + P.image_offset, (uint32_t)t, false, !rejected,
-                 [draw](int) { return draw; }, bs, ps, a.dev_status, o);
+  general_position<RES>(a, target_row(a, g), draft_row(a, cell), sq, tok, (uint32_t)b + P.image_offset, (uint32_t)t, false,
+                        !rejected, [draw](int) { return draw; }, sc, dyn, o);
   if (threadIdx.x == 0) a.out_tok[g] = use_res ? o.tok_residual : o.tok_target;
 }
 
@@ -553,6 +620,8 @@ struct mulo_ctx {
   std::vector<cudaEvent_t> ev;   // start/stop pairs around the fused row kernel
   size_t ev_used;
   int force_dense;               // diagnostics: never take the fast top-k path
+  struct Ready { const void* kernel; size_t dyn; int per_sm; };
+  std::vector<Ready> ready;      // kernels whose shared-memory cap is raised, and the CTAs of them an SM holds
 };
 
 static const size_t kStatusBytes = 256;
@@ -780,17 +849,51 @@ static mulo_status launched(mulo_ctx* ctx, int n) {
   return MULO_OK;
 }
 
-template <class K>
-static bool raise_smem(K kernel, size_t bytes, const mulo_ctx* ctx) {
-  if (bytes + sizeof(BlockScratch) + 1024 > (size_t)ctx->smem_optin) return false;
-  if (bytes > 0)
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-  return true;
+// Dynamic shared memory of the general path's kernels.
+static size_t general_smem(const DevParams& d, bool pooling) {
+  if (resident_fits(d.V)) return resident_bytes(d.V);
+  return pooling ? pool_smem_bytes(d) : 0;
 }
 
+// CTAs of `threads` with `dyn` bytes of dynamic shared memory that an SM holds; 0 if the kernel cannot run so.  The
+// kernel's shared-memory cap is raised on the way -- always to all that the device allows, so that contexts and threads
+// that set it for the same kernel agree.  Asked once per context, kernel and size.
+template <class K>
+static int ctas_per_sm(mulo_ctx* ctx, K kernel, int threads, size_t dyn) {
+  const void* const key = (const void*)kernel;
+  for (const mulo_ctx::Ready& r : ctx->ready)
+    if (r.kernel == key && r.dyn == dyn) return r.per_sm;
+  cudaFuncAttributes fa;
+  int per_sm = 0;
+  if (cudaFuncGetAttributes(&fa, key) != cudaSuccess || dyn + fa.sharedSizeBytes > (size_t)ctx->smem_optin ||
+      cudaFuncSetAttribute(key, cudaFuncAttributeMaxDynamicSharedMemorySize, ctx->smem_optin - (int)fa.sharedSizeBytes) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, dyn) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (ctx->ready.size() >= 64) ctx->ready.clear();
+  ctx->ready.push_back({key, dyn, per_sm});
+  return per_sm;
+}
+
+// Launches one of the general path's kernels in the version for this vocabulary; false if it cannot run.
+#define MULO_LAUNCH_GENERAL(KERNEL, grid, dyn, st, ...)                                     \
+  (resident_fits(a.P.V)                                                                     \
+       ? launch_general(ctx, KERNEL(true), (unsigned)(grid), dyn, st, __VA_ARGS__)          \
+       : launch_general(ctx, KERNEL(false), (unsigned)(grid), dyn, st, __VA_ARGS__))
+template <class K, class... A>
+static bool launch_general(mulo_ctx* ctx, K kernel, unsigned grid, size_t dyn, cudaStream_t st, const A&... args) {
+  if (ctas_per_sm(ctx, kernel, kThreads, dyn) < 1) return false;
+  kernel<<<grid, kThreads, dyn, st>>>(args...);
+  return true;
+}
+#define K_UPSAMPLE(RES) k_upsample_pool<RES>
+#define K_SAMPLE(RES) k_sample_draft<RES>
+#define K_SAMPLE_FAILED(RES) k_sample_failed<RES>
+#define K_VERIFY(RES) k_verify_rows<false, RES>
+#define K_ROUND(RES) k_verify_rows<true, RES>
+#define K_ROUND_FAILED(RES) k_verify_failed<RES>
+#define K_RESAMPLE(RES) k_resample_rows<RES>
 
 // ---- the fast top-k path of mulo_round -------------------------------------------------
 
@@ -845,24 +948,17 @@ static size_t plan_stream(const mulo_ctx* ctx, const DevParams& d, StreamArgs* s
 }
 
 template <bool BF16, bool HAS_U, bool SAMPLE = false, bool POOL = false>
-static bool launch_stream_t(const mulo_ctx* ctx, const StreamArgs& s, size_t dyn, cudaStream_t st) {
+static bool launch_stream_t(mulo_ctx* ctx, const StreamArgs& s, size_t dyn, cudaStream_t st) {
   auto kern = k_round_stream<BF16, HAS_U, SAMPLE, POOL>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSThreads, dyn) != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    return false;
-  }
+  const int per_sm = ctas_per_sm(ctx, kern, kSThreads, dyn);
+  if (per_sm < 1) return false;
   int grid = ctx->sm_count * per_sm;
   if (grid > s.n_parents) grid = s.n_parents;
   kern<<<grid, kSThreads, dyn, st>>>(s);
   return true;
 }
 
-static bool launch_stream(const mulo_ctx* ctx, const StreamArgs& s, size_t dyn, cudaStream_t st) {
+static bool launch_stream(mulo_ctx* ctx, const StreamArgs& s, size_t dyn, cudaStream_t st) {
   const bool hu = s.uncond != nullptr;
   if (s.P.pool_k > 1) {
     if (s.P.bf16)
@@ -921,17 +1017,10 @@ static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, Ro
 }
 
 template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
-static bool launch_rows_p(const mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
+static bool launch_rows_p(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
   auto kern = k_round_rows<BF16, HAS_U, SAMPLE, PLAIN, NW>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, dyn) != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    return false;
-  }
+  const int per_sm = ctas_per_sm(ctx, kern, NW * 32, dyn);
+  if (per_sm < 1) return false;
   int grid = ctx->sm_count * per_sm;
   if (grid > s.n_units) grid = s.n_units;
   kern<<<grid, NW * 32, dyn, st>>>(s);
@@ -939,14 +1028,14 @@ static bool launch_rows_p(const mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cu
 }
 
 template <bool BF16, bool HAS_U, bool SAMPLE, int NW>
-static bool launch_rows_t(const mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
+static bool launch_rows_t(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
   const bool plain = s.P.invT == 1.0f && s.row_bytes % (16u * kRPieceBytes * NW) == 0;
   return plain ? launch_rows_p<BF16, HAS_U, SAMPLE, true, NW>(ctx, s, dyn, st)
                : launch_rows_p<BF16, HAS_U, SAMPLE, false, NW>(ctx, s, dyn, st);
 }
 
 template <int NW>
-static bool launch_rows_nw(const mulo_ctx* ctx, const RowsArgs& s, bool sample, size_t dyn, cudaStream_t st) {
+static bool launch_rows_nw(mulo_ctx* ctx, const RowsArgs& s, bool sample, size_t dyn, cudaStream_t st) {
   const bool hu = s.uncond != nullptr;
   if (sample)
     return s.P.bf16 ? launch_rows_t<true, false, true, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, true, NW>(ctx, s, dyn, st);
@@ -955,7 +1044,7 @@ static bool launch_rows_nw(const mulo_ctx* ctx, const RowsArgs& s, bool sample, 
   return hu ? launch_rows_t<false, true, false, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, false, NW>(ctx, s, dyn, st);
 }
 
-static bool launch_rows(const mulo_ctx* ctx, const RowsArgs& s, bool sample, int nw, size_t dyn, cudaStream_t st) {
+static bool launch_rows(mulo_ctx* ctx, const RowsArgs& s, bool sample, int nw, size_t dyn, cudaStream_t st) {
   return nw == 2 ? launch_rows_nw<2>(ctx, s, sample, dyn, st) : launch_rows_nw<4>(ctx, s, sample, dyn, st);
 }
 
@@ -980,24 +1069,17 @@ static size_t plan_full(const mulo_ctx* ctx, const DevParams& d, bool has_u, Ful
 }
 
 template <bool BF16, bool HAS_U>
-static bool launch_full_t(const mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
+static bool launch_full_t(mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
   auto kern = k_round_full<BF16, HAS_U>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFThreads, dyn) != cudaSuccess || per_sm < 1) {
-    cudaGetLastError();
-    return false;
-  }
+  const int per_sm = ctas_per_sm(ctx, kern, kFThreads, dyn);
+  if (per_sm < 1) return false;
   int grid = ctx->sm_count * per_sm;
   if (grid > s.n_parents) grid = s.n_parents;
   kern<<<grid, kFThreads, dyn, st>>>(s);
   return true;
 }
 
-static bool launch_full(const mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
+static bool launch_full(mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
   const bool hu = s.uncond != nullptr;
   if (s.P.bf16) return hu ? launch_full_t<true, true>(ctx, s, dyn, st) : launch_full_t<true, false>(ctx, s, dyn, st);
   return hu ? launch_full_t<false, true>(ctx, s, dyn, st) : launch_full_t<false, false>(ctx, s, dyn, st);
@@ -1043,7 +1125,7 @@ mulo_status mulo_upsample_pool(mulo_ctx* ctx, const mulo_params* p, const void* 
   a.stats_out = draft_stats_lo;
   a.q_tok_hi_out = q_tok_hi;
   a.dev_status = (uint32_t*)ctx->ws;
-  k_upsample_pool<<<p->B * a.P.h * a.P.w, kThreads, 0, (cudaStream_t)stream>>>(a);
+  if (!MULO_LAUNCH_GENERAL(K_UPSAMPLE, p->B * a.P.h * a.P.w, general_smem(a.P, false), (cudaStream_t)stream, a)) return MULO_ERR_CUDA;
   return launched(ctx, 1);
 }
 
@@ -1110,7 +1192,23 @@ mulo_status mulo_redraw_step(mulo_ctx* ctx, const mulo_params* p, int32_t s_inde
   a.out_tok = out_tok;
   a.s = s_index;
   // the step's positions are counted on the device: a fixed grid strides over them
-  k_redraw_step<<<2 * ctx->sm_count, kThreads, 0, (cudaStream_t)stream>>>(a);
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3((unsigned)(2 * ctx->sm_count));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = general_smem(a.P, false);
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  const bool res = resident_fits(a.P.V);
+  cfg.numAttrs = res ? 1 : 0;   // (the version for larger vocabularies reads through the read-only cache)
+  if (ctas_per_sm(ctx, res ? k_redraw_step<true> : k_redraw_step<false>, kThreads, cfg.dynamicSmemBytes) < 1) return MULO_ERR_CUDA;
+  if (cudaLaunchKernelEx(&cfg, res ? k_redraw_step<true> : k_redraw_step<false>, a) != cudaSuccess) {
+    cudaGetLastError();
+    return MULO_ERR_CUDA;
+  }
   return launched(ctx, 1);
 }
 
@@ -1146,7 +1244,7 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
     ra.n_units = p->B * a.P.h * a.P.w;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
     if (launch_rows(ctx, ra, true, rnw, rdyn, st)) {
-      k_sample_failed<<<2 * ctx->sm_count, kThreads, 0, st>>>(a, w.fail_list, w.status + kFailCount);
+      if (!MULO_LAUNCH_GENERAL(K_SAMPLE_FAILED, 2 * ctx->sm_count, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
       return launched(ctx, 2);
     }
   }
@@ -1164,11 +1262,11 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
     const bool fast = a.P.bf16 ? launch_stream_t<true, false, true>(ctx, sa, sdyn, st)
                                : launch_stream_t<false, false, true>(ctx, sa, sdyn, st);
     if (fast) {
-      k_sample_failed<<<2 * ctx->sm_count, kThreads, 0, st>>>(a, w.fail_list, w.status + kFailCount);
+      if (!MULO_LAUNCH_GENERAL(K_SAMPLE_FAILED, 2 * ctx->sm_count, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
       return launched(ctx, 2);
     }
   }
-  k_sample_draft<<<p->B * a.P.h * a.P.w, kThreads, 0, st>>>(a);
+  if (!MULO_LAUNCH_GENERAL(K_SAMPLE, p->B * a.P.h * a.P.w, general_smem(a.P, false), st, a)) return MULO_ERR_CUDA;
   return launched(ctx, 1);
 }
 
@@ -1215,10 +1313,9 @@ mulo_status mulo_verify(mulo_ctx* ctx, const mulo_params* p, const void* tgt_con
   a.p_tok = p_tok; a.q_tok = q_tok; a.accept_prob = accept_prob;
   a.flags = w.flags;
   a.dev_status = w.status;
-  const size_t dyn = pool_smem_bytes(a.P);
-  if (!raise_smem(k_verify_rows<false>, dyn, ctx)) return MULO_ERR_UNSUPPORTED;
+  const size_t dyn = general_smem(a.P, true);
   cudaStream_t st = (cudaStream_t)stream;
-  k_verify_rows<false><<<(unsigned)((size_t)p->B * p->H * p->W), kThreads, dyn, st>>>(a);
+  if (!MULO_LAUNCH_GENERAL(K_VERIFY, (size_t)p->B * p->H * p->W, dyn, st, a)) return MULO_ERR_UNSUPPORTED;
   MaskArgs m;
   memset(&m, 0, sizeof m);
   m.H = p->H; m.W = p->W; m.r = p->r; m.radius = p->radius; m.clip = a.P.clip; m.resample_mode = p->resample_mode;
@@ -1300,9 +1397,7 @@ mulo_status mulo_resample(mulo_ctx* ctx, const mulo_params* p, const void* tgt_c
   a.expand_bits = expand_bits;
   a.out_tok = out_tok;
   a.dev_status = (uint32_t*)ctx->ws;
-  const size_t dyn = pool_smem_bytes(a.P);
-  if (!raise_smem(k_resample_rows, dyn, ctx)) return MULO_ERR_UNSUPPORTED;
-  k_resample_rows<<<(unsigned)((size_t)p->B * p->H * p->W), kThreads, dyn, (cudaStream_t)stream>>>(a);
+  if (!MULO_LAUNCH_GENERAL(K_RESAMPLE, (size_t)p->B * p->H * p->W, general_smem(a.P, true), (cudaStream_t)stream, a)) return MULO_ERR_UNSUPPORTED;
   return launched(ctx, 1);
 }
 
@@ -1328,9 +1423,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
   a.p_tok = p_tok; a.q_tok = q_tok; a.accept_prob = accept_prob;
   a.flags = w.flags; a.cand_res = w.cand_res; a.cand_tgt = w.cand_tgt;
   a.dev_status = w.status;
-  const size_t dyn = pool_smem_bytes(a.P);
-  if (!raise_smem(k_verify_rows<true>, dyn, ctx)) return MULO_ERR_UNSUPPORTED;
-  if (!raise_smem(k_verify_failed, dyn, ctx)) return MULO_ERR_UNSUPPORTED;
+  const size_t dyn = general_smem(a.P, true);
   cudaStream_t st = (cudaStream_t)stream;
   const bool timed = ctx->ev_used + 2 <= ctx->ev.size();
   if (timed) cudaEventRecord(ctx->ev[ctx->ev_used], st);
@@ -1371,7 +1464,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     ra.n_units = p->B * p->H * p->W;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
     fast = launch_rows(ctx, ra, false, rnw, rdyn, st);
-    if (fast) k_verify_failed<<<2 * ctx->sm_count, kThreads, dyn, st>>>(a, w.fail_list, w.status + kFailCount);
+    if (fast && !MULO_LAUNCH_GENERAL(K_ROUND_FAILED, 2 * ctx->sm_count, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
   }
   StreamArgs sa;
   memset(&sa, 0, sizeof sa);
@@ -1388,9 +1481,9 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
     fast = launch_stream(ctx, sa, sdyn, st);
     // the rows the streaming kernel gave up on (usually a handful, often none)
-    if (fast) k_verify_failed<<<2 * ctx->sm_count, kThreads, dyn, st>>>(a, w.fail_list, w.status + kFailCount);
+    if (fast && !MULO_LAUNCH_GENERAL(K_ROUND_FAILED, 2 * ctx->sm_count, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
   }
-  if (!fast) k_verify_rows<true><<<p->B * a.P.h * a.P.w, kThreads, dyn, st>>>(a);
+  if (!fast && !MULO_LAUNCH_GENERAL(K_ROUND, p->B * a.P.h * a.P.w, dyn, st, a)) return MULO_ERR_UNSUPPORTED;
   if (timed) {
     cudaEventRecord(ctx->ev[ctx->ev_used + 1], st);
     ctx->ev_used += 2;

@@ -2,9 +2,10 @@
 // pre-processing, Philox4x32-10, block reductions/scans, and the "dense" row
 // routines that work on a whole vocabulary row straight from global memory.
 //
-// The dense routines are the general path: any V (multiple of 8), top-k on or
-// off, fp32 or bf16 logits.  They read a row several times (it stays in L1/L2
-// after the first read) and are what the fast top-k path falls back to.
+// The dense routines here are the general path for vocabularies too large for a
+// row to stay in shared memory (mulo_resident.cuh has the others): any V (multiple
+// of 8), top-k on or off, fp32 or bf16 logits.  They read a row several times (it
+// stays in L1/L2 after the first read).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -56,13 +57,21 @@ struct RowSrc {          // one vocabulary row in global memory
   int bf16;
 };
 
+// 16 bytes of a row: through the read-only cache, or (ONCE: a row that is read once, or that another kernel may have
+// written since this one was launched) from L2
+template <bool ONCE>
+__device__ __forceinline__ uint4 load16(const char* p) {
+  return ONCE ? __ldcg(reinterpret_cast<const uint4*>(p)) : __ldg(reinterpret_cast<const uint4*>(p));
+}
+
 // eight consecutive pre-processed logits starting at x (x % 8 == 0)
+template <bool ONCE = false>
 __device__ __forceinline__ void load8(const RowSrc& r, int x, float (&z)[8]) {
   const bool hu = r.uncond != nullptr;
   if (r.bf16) {
-    uint4 c = __ldg(reinterpret_cast<const uint4*>(r.cond + (size_t)x * 2));
+    uint4 c = load16<ONCE>(r.cond + (size_t)x * 2);
     uint4 u = make_uint4(0, 0, 0, 0);
-    if (hu) u = __ldg(reinterpret_cast<const uint4*>(r.uncond + (size_t)x * 2));
+    if (hu) u = load16<ONCE>(r.uncond + (size_t)x * 2);
     z[0] = mix_logit(bf16_lo(c.x), bf16_lo(u.x), hu, r.s, r.invT);
     z[1] = mix_logit(bf16_hi(c.x), bf16_hi(u.x), hu, r.s, r.invT);
     z[2] = mix_logit(bf16_lo(c.y), bf16_lo(u.y), hu, r.s, r.invT);
@@ -72,13 +81,15 @@ __device__ __forceinline__ void load8(const RowSrc& r, int x, float (&z)[8]) {
     z[6] = mix_logit(bf16_lo(c.w), bf16_lo(u.w), hu, r.s, r.invT);
     z[7] = mix_logit(bf16_hi(c.w), bf16_hi(u.w), hu, r.s, r.invT);
   } else {
-    const float4* cp = reinterpret_cast<const float4*>(r.cond + (size_t)x * 4);
-    float4 c0 = __ldg(cp), c1 = __ldg(cp + 1);
+    auto four = [&](const char* p) -> float4 {
+      const uint4 w = load16<ONCE>(p);
+      return make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
+    };
+    const float4 c0 = four(r.cond + (size_t)x * 4), c1 = four(r.cond + (size_t)x * 4 + 16);
     float4 u0 = make_float4(0, 0, 0, 0), u1 = u0;
     if (hu) {
-      const float4* up = reinterpret_cast<const float4*>(r.uncond + (size_t)x * 4);
-      u0 = __ldg(up);
-      u1 = __ldg(up + 1);
+      u0 = four(r.uncond + (size_t)x * 4);
+      u1 = four(r.uncond + (size_t)x * 4 + 16);
     }
     z[0] = mix_logit(c0.x, u0.x, hu, r.s, r.invT);
     z[1] = mix_logit(c0.y, u0.y, hu, r.s, r.invT);
@@ -124,7 +135,6 @@ struct BlockScratch {
   unsigned sel_digit, sel_k;
   int owner;
   int found;
-  int bi[8];
   double bd[8];
 };
 
