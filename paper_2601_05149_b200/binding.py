@@ -78,6 +78,17 @@ def lib() -> C.CDLL:
             fn = getattr(L, name)
             if name not in ("mulo_status_string", "mulo_destroy"):
                 fn.restype = C.c_int
+        # pointers and integers go over as they are: converting them argument by argument costs as much as the call
+        ptr, i32, size = C.c_void_p, C.c_int32, C.c_size_t
+        for name, types in {
+            "mulo_upsample_pool": [ptr] * 9, "mulo_verify": [ptr] * 15, "mulo_local_reject_expand": [ptr] * 7,
+            "mulo_island_schedule": [ptr] * 3 + [i32] + [ptr] * 3, "mulo_sample_draft": [ptr] * 5,
+            "mulo_downsample": [ptr] * 5, "mulo_islands": [ptr] * 5 + [i32] + [ptr] * 3, "mulo_resample": [ptr] * 12,
+            "mulo_redraw_plan": [ptr] * 3 + [i32] + [ptr] * 3, "mulo_redraw_step": [ptr] * 2 + [i32] * 2 + [ptr] * 6,
+            "mulo_round": [ptr] * 17, "mulo_round_static": [ptr] * 18,
+            "mulo_round_host": [ptr] * 3 + [size] + [ptr] * 15,
+        }.items():
+            getattr(L, name).argtypes = types
         _lib = L
     return _lib
 
@@ -112,24 +123,30 @@ def params_from_config(cfg, **over) -> MuloParams:
 
 def _dev(t):
     if t is None:
-        return C.c_void_p(None)
+        return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("tensor arguments must be contiguous CUDA tensors")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _host(t):
     if t is None:
-        return C.c_void_p(None)
+        return None
     if t.is_cuda or not t.is_contiguous():
         raise ValueError("host arguments must be contiguous CPU tensors")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# the handle of the current stream without the Stream object around it (a third of a short call's host time)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _check(status, what):
@@ -167,7 +184,7 @@ class Context:
         return n.value
 
     def set_workspace(self, t: torch.Tensor):
-        _check(lib().mulo_set_workspace(self._ctx, _dev(t), C.c_size_t(t.numel() * t.element_size())),
+        _check(lib().mulo_set_workspace(self._ctx, C.c_void_p(_dev(t)), C.c_size_t(t.numel() * t.element_size())),
                "mulo_set_workspace")
         self._ws = t
 
@@ -180,7 +197,7 @@ class Context:
         """The MULO_DEV_* bits since the last poll; raises MuloError(ERR_TIMEOUT) if a kernel's
         bounded wait gave up (the bits are then in the exception's ``flags``)."""
         f = C.c_uint32()
-        st = lib().mulo_poll_device_status(self._ctx, _stream(stream), C.byref(f))
+        st = lib().mulo_poll_device_status(self._ctx, C.c_void_p(_stream(stream)), C.byref(f))
         if st != OK:
             e = MuloError(st, "mulo_poll_device_status")
             e.flags = f.value
@@ -191,7 +208,7 @@ class Context:
         """[rows redone by the general routines, list full, too few candidates, k-th largest
         above the histogram, crowded bin] since the last poll."""
         c = (C.c_uint32 * 5)()
-        _check(lib().mulo_poll_fallback_counts(self._ctx, _stream(stream), c), "mulo_poll_fallback_counts")
+        _check(lib().mulo_poll_fallback_counts(self._ctx, C.c_void_p(_stream(stream)), c), "mulo_poll_fallback_counts")
         return [int(x) for x in c]
 
     def kernel_launches(self) -> int:
@@ -238,7 +255,7 @@ class Context:
                                               _stream(stream)), "mulo_local_reject_expand")
 
     def mulo_island_schedule(self, p, labels, window, step, n_steps, stream=None):
-        _check(lib().mulo_island_schedule(self._ctx, C.byref(p), _dev(labels), C.c_int32(int(window)), _dev(step),
+        _check(lib().mulo_island_schedule(self._ctx, C.byref(p), _dev(labels), int(window), _dev(step),
                                           _dev(n_steps), _stream(stream)), "mulo_island_schedule")
 
     def mulo_sample_draft(self, p, draft_logits_lo, draft_tok_lo, stream=None):
@@ -258,7 +275,7 @@ class Context:
             elif island_size is not None:
                 max_islands = island_size.shape[1]
         _check(lib().mulo_islands(self._ctx, C.byref(p), _dev(expand_bits), _dev(labels), _dev(n_islands),
-                                  C.c_int32(int(max_islands)), _dev(island_rows), _dev(island_size),
+                                  int(max_islands), _dev(island_rows), _dev(island_size),
                                   _stream(stream)), "mulo_islands")
 
     def mulo_resample(self, p, tgt_cond, tgt_uncond, draft_logits_lo, draft_stats_lo, draft_tok_hi, nn,
@@ -314,7 +331,7 @@ class Context:
         """All tensor arguments except ``arena`` are HOST tensors."""
         self._ws = None     # the arena replaces the workspace
         _check(lib().mulo_round_host(self._ctx, C.byref(p), _dev(arena),
-                                     C.c_size_t(arena.numel() * arena.element_size()),
+                                     arena.numel() * arena.element_size(),
                                      _host(tgt_cond), _host(tgt_uncond), _host(draft_logits_lo),
                                      _host(draft_tok_lo), _host(nn), _host(out_tok),
                                      _host(reject_bits), _host(expand_bits), _host(p_tok),

@@ -122,18 +122,25 @@ __global__ void __launch_bounds__(kThreads, 2) k_upsample_pool(RowKernelArgs a) 
 }
 
 // The inverse-CDF draw of uniform u from softmax(topk(row / T)); one thread writes the token to *out.
-template <bool RES>
-__device__ __forceinline__ void draw_row(const RowSrc& src, int top_k, double u, GeneralScratch<RES>& sc, unsigned char* dyn, int32_t* out) {
+// `before_pick` runs ahead of the last step.
+struct Nothing {
+  __device__ void operator()() const {}
+};
+template <bool RES, bool REG = false, class F = Nothing>
+__device__ __forceinline__ void draw_row(const RowSrc& src, int top_k, double u, GeneralScratch<RES>& sc, unsigned char* dyn,
+                                         int32_t* out, F before_pick = F()) {
   RowStats st;
   if constexpr (RES) {
     const ResRow row(reinterpret_cast<float*>(dyn), src.V);
     int calls = 0;
     float unused;
-    const ResSums sums = res_row_stats(row, src, top_k, sc, calls, -1, unused, st);
+    const ResSums sums = res_row_stats<REG>(row, src, top_k, sc, calls, -1, unused, st);
+    before_pick();
     res_pick(row, sums, u, [&](int x) -> double { return (double)row.at(x); }, out);
   } else {
     dense_row_stats(src, top_k, sc, st.theta, st.m, st.Z);
     __syncthreads();
+    before_pick();
     const float invZ = (float)(1.0 / st.Z);
     // lambda = 0 and no special token: the weights are the probabilities themselves
     const int tok = dense_draw(src, src, st, st, invZ, invZ, 0.0f, -1, 0.0, nullptr, u, sc);
@@ -246,41 +253,67 @@ struct RedrawArgs {
 // Steps follow one another by the thousand, a handful of positions each, so a step is bound by latency: the launch
 // may begin while the kernel before it in the stream still runs (programmatic dependent launch), asks its rows into
 // L2 -- a hint: nothing is read -- and waits for that kernel before it reads anything it uses.
-template <bool RES>
-__global__ void __launch_bounds__(kThreads, 2) k_redraw_step(RedrawArgs a) {
+template <bool RES, bool REG>
+__global__ void __launch_bounds__(kThreads, REG ? 1 : 2) k_redraw_step(RedrawArgs a) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GeneralScratch<RES> sc;
   const DevParams& P = a.P;
   const size_t N = (size_t)P.H * P.W, total = (size_t)P.B * N;
   const size_t bytes = (size_t)P.V * (P.bf16 ? 2 : 4);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (threadIdx.x == 0) {
-    const int beg = ld_fresh(a.offsets + a.s), end = ld_fresh(a.offsets + a.s + 1);
-    const long long i = (long long)beg + (long long)blockIdx.x;
-    if (beg >= 0 && i < end && i < (long long)total) {
-      const size_t g = (size_t)(uint32_t)ld_fresh(a.pos_list + i);
-      if (g < total) {
-        prefetch_l2(a.cond + g * bytes, (uint32_t)bytes);
-        if (a.uncond) prefetch_l2(a.uncond + g * bytes, (uint32_t)bytes);
-      }
+  // what the step will find, if the list stays as it is
+  const int beg0 = ld_fresh(a.offsets + a.s), end0 = ld_fresh(a.offsets + a.s + 1);
+  const long long i0 = (long long)beg0 + (long long)blockIdx.x;
+  size_t g0 = total;
+  if (beg0 >= 0 && i0 < end0 && i0 < (long long)total) {
+    g0 = (size_t)(uint32_t)ld_fresh(a.pos_list + i0);
+    if (g0 < total && threadIdx.x == 0) {
+      prefetch_l2(a.cond + g0 * bytes, (uint32_t)bytes);
+      if (a.uncond) prefetch_l2(a.uncond + g0 * bytes, (uint32_t)bytes);
     }
   }
+  struct Place {
+    RowSrc src;
+    double u;
+  };
+  auto place = [&](size_t g) -> Place {   // (positions fit 32 bits)
+    const uint32_t b = (uint32_t)g / (uint32_t)N, t = (uint32_t)g - b * (uint32_t)N;
+    Place pl;
+    pl.src.cond = a.cond + g * bytes;
+    pl.src.uncond = a.uncond ? a.uncond + g * bytes : nullptr;
+    pl.src.s = P.cfg_scale;
+    pl.src.invT = P.invT;
+    pl.src.V = P.V;
+    pl.src.bf16 = P.bf16;
+    pl.u = uniform24(philox4x32_10(make_uint4(t, b + P.image_offset, P.round, 1u + (uint32_t)a.s),
+                                   make_uint2(P.seed_lo, P.seed_hi)).x);
+    return pl;
+  };
+  const Place first = place(g0 < total ? g0 : 0);
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  int i = -1;
+  if (g0 < total) {   // block-uniform
+    // The position found above is worked on at once, and its token written if the list, read again towards the end,
+    // says so now too: two dependent loads from L2 fewer before the row can be asked for.
+    __shared__ int32_t tok;
+    __shared__ int32_t now[3];
+    draw_row<RES, REG>(first.src, P.top_k, first.u, sc, dyn, &tok, [&]() {
+      if (threadIdx.x < 3) now[threadIdx.x] = ld_fresh(threadIdx.x < 2 ? a.offsets + a.s + threadIdx.x : a.pos_list + i0);
+    });
+    __syncthreads();
+    i = now[0] + (int)blockIdx.x;
+    if (now[0] == beg0 && (size_t)(uint32_t)now[2] == g0 && i < now[1]) {
+      if (threadIdx.x == 0) a.out_tok[g0] = tok;
+      i += (int)gridDim.x;
+    }
+  }
   const int beg = ld_fresh(a.offsets + a.s), end = ld_fresh(a.offsets + a.s + 1);
-  for (int i = beg + (int)blockIdx.x; i < end; i += (int)gridDim.x) {
-    const size_t g = (size_t)ld_fresh(a.pos_list + i);
+  if (i < 0) i = beg + (int)blockIdx.x;
+  for (; i < end; i += (int)gridDim.x) {
+    const size_t g = (size_t)(uint32_t)ld_fresh(a.pos_list + i);
     if (g < total) {   // block-uniform
-      const uint32_t b = (uint32_t)(g / N), t = (uint32_t)(g - (size_t)b * N);
-      RowSrc tr;
-      tr.cond = a.cond + g * bytes;
-      tr.uncond = a.uncond ? a.uncond + g * bytes : nullptr;
-      tr.s = P.cfg_scale;
-      tr.invT = P.invT;
-      tr.V = P.V;
-      tr.bf16 = P.bf16;
-      const uint4 rnd = philox4x32_10(make_uint4(t, b + P.image_offset, P.round, 1u + (uint32_t)a.s),
-                                      make_uint2(P.seed_lo, P.seed_hi));
-      draw_row<RES>(tr, P.top_k, uniform24(rnd.x), sc, dyn, a.out_tok + g);
+      const Place pl = place(g);
+      draw_row<RES, REG>(pl.src, P.top_k, pl.u, sc, dyn, a.out_tok + g);
     }
     __syncthreads();
   }
@@ -1204,8 +1237,9 @@ mulo_status mulo_redraw_step(mulo_ctx* ctx, const mulo_params* p, int32_t s_inde
   cfg.attrs = &at;
   const bool res = resident_fits(a.P.V);
   cfg.numAttrs = res ? 1 : 0;   // (the version for larger vocabularies reads through the read-only cache)
-  if (ctas_per_sm(ctx, res ? k_redraw_step<true> : k_redraw_step<false>, kThreads, cfg.dynamicSmemBytes) < 1) return MULO_ERR_CUDA;
-  if (cudaLaunchKernelEx(&cfg, res ? k_redraw_step<true> : k_redraw_step<false>, a) != cudaSuccess) {
+  auto kern = !res ? k_redraw_step<false, false> : a.P.V <= kResRegs * kThreads ? k_redraw_step<true, true> : k_redraw_step<true, false>;
+  if (ctas_per_sm(ctx, kern, kThreads, cfg.dynamicSmemBytes) < 1) return MULO_ERR_CUDA;
+  if (cudaLaunchKernelEx(&cfg, kern, a) != cudaSuccess) {
     cudaGetLastError();
     return MULO_ERR_CUDA;
   }

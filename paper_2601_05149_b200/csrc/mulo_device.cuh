@@ -64,41 +64,48 @@ __device__ __forceinline__ uint4 load16(const char* p) {
   return ONCE ? __ldcg(reinterpret_cast<const uint4*>(p)) : __ldg(reinterpret_cast<const uint4*>(p));
 }
 
-// eight consecutive pre-processed logits starting at x (x % 8 == 0)
+// eight consecutive logits starting at x (x % 8 == 0): asked for, then mixed
+template <bool BF16>
+struct raw_piece {
+  uint4 w[BF16 ? 1 : 2];
+};
+template <bool ONCE, bool BF16>
+__device__ __forceinline__ void ask8(const RowSrc& r, int x, raw_piece<BF16>& c, raw_piece<BF16>& u) {
+  const size_t o = (size_t)x * (BF16 ? 2 : 4);
+#pragma unroll
+  for (int i = 0; i < (BF16 ? 1 : 2); ++i) {
+    c.w[i] = load16<ONCE>(r.cond + o + 16 * i);
+    if (r.uncond) u.w[i] = load16<ONCE>(r.uncond + o + 16 * i);
+  }
+}
+template <bool BF16>
+__device__ __forceinline__ void mix8(const RowSrc& r, const raw_piece<BF16>& c, const raw_piece<BF16>& u, float (&z)[8]) {
+  const bool hu = r.uncond != nullptr;
+#pragma unroll
+  for (int i = 0; i < (BF16 ? 1 : 2); ++i) {
+    const uint32_t cw[4] = {c.w[i].x, c.w[i].y, c.w[i].z, c.w[i].w}, uw[4] = {u.w[i].x, u.w[i].y, u.w[i].z, u.w[i].w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (BF16) {
+        z[2 * j] = mix_logit(bf16_lo(cw[j]), hu ? bf16_lo(uw[j]) : 0.f, hu, r.s, r.invT);
+        z[2 * j + 1] = mix_logit(bf16_hi(cw[j]), hu ? bf16_hi(uw[j]) : 0.f, hu, r.s, r.invT);
+      } else {
+        z[4 * i + j] = mix_logit(__uint_as_float(cw[j]), hu ? __uint_as_float(uw[j]) : 0.f, hu, r.s, r.invT);
+      }
+    }
+  }
+}
+// eight consecutive pre-processed logits
 template <bool ONCE = false>
 __device__ __forceinline__ void load8(const RowSrc& r, int x, float (&z)[8]) {
-  const bool hu = r.uncond != nullptr;
   if (r.bf16) {
-    uint4 c = load16<ONCE>(r.cond + (size_t)x * 2);
-    uint4 u = make_uint4(0, 0, 0, 0);
-    if (hu) u = load16<ONCE>(r.uncond + (size_t)x * 2);
-    z[0] = mix_logit(bf16_lo(c.x), bf16_lo(u.x), hu, r.s, r.invT);
-    z[1] = mix_logit(bf16_hi(c.x), bf16_hi(u.x), hu, r.s, r.invT);
-    z[2] = mix_logit(bf16_lo(c.y), bf16_lo(u.y), hu, r.s, r.invT);
-    z[3] = mix_logit(bf16_hi(c.y), bf16_hi(u.y), hu, r.s, r.invT);
-    z[4] = mix_logit(bf16_lo(c.z), bf16_lo(u.z), hu, r.s, r.invT);
-    z[5] = mix_logit(bf16_hi(c.z), bf16_hi(u.z), hu, r.s, r.invT);
-    z[6] = mix_logit(bf16_lo(c.w), bf16_lo(u.w), hu, r.s, r.invT);
-    z[7] = mix_logit(bf16_hi(c.w), bf16_hi(u.w), hu, r.s, r.invT);
+    raw_piece<true> c, u = {};
+    ask8<ONCE, true>(r, x, c, u);
+    mix8<true>(r, c, u, z);
   } else {
-    auto four = [&](const char* p) -> float4 {
-      const uint4 w = load16<ONCE>(p);
-      return make_float4(__uint_as_float(w.x), __uint_as_float(w.y), __uint_as_float(w.z), __uint_as_float(w.w));
-    };
-    const float4 c0 = four(r.cond + (size_t)x * 4), c1 = four(r.cond + (size_t)x * 4 + 16);
-    float4 u0 = make_float4(0, 0, 0, 0), u1 = u0;
-    if (hu) {
-      u0 = four(r.uncond + (size_t)x * 4);
-      u1 = four(r.uncond + (size_t)x * 4 + 16);
-    }
-    z[0] = mix_logit(c0.x, u0.x, hu, r.s, r.invT);
-    z[1] = mix_logit(c0.y, u0.y, hu, r.s, r.invT);
-    z[2] = mix_logit(c0.z, u0.z, hu, r.s, r.invT);
-    z[3] = mix_logit(c0.w, u0.w, hu, r.s, r.invT);
-    z[4] = mix_logit(c1.x, u1.x, hu, r.s, r.invT);
-    z[5] = mix_logit(c1.y, u1.y, hu, r.s, r.invT);
-    z[6] = mix_logit(c1.z, u1.z, hu, r.s, r.invT);
-    z[7] = mix_logit(c1.w, u1.w, hu, r.s, r.invT);
+    raw_piece<false> c, u = {};
+    ask8<ONCE, false>(r, x, c, u);
+    mix8<false>(r, c, u, z);
   }
 }
 

@@ -8,7 +8,7 @@
 // place, and one block scan in double gives the partition sum and every thread's slice of the ascending-id CDF.  A
 // draw from the target weights needs nothing more than the walk of the owner's run by its warp.  The routines of
 // mulo_device.cuh / mulo_dense.cuh, which read the row nine times (radix select), took 55 us for a row of 16384
-// bf16 ids with guidance on one CTA; this takes REDRAW_US us.
+// bf16 ids with guidance on one CTA; this takes 7.6 us.
 //
 // A thread owns a contiguous run of E ids; runs are E + 4 floats apart, so that 128-bit accesses of a quarter warp
 // hit different banks.
@@ -20,9 +20,11 @@ namespace mulo {
 
 constexpr int kResBins = 1024;
 constexpr int kResMembers = 128;
+constexpr int kResRegs = 32;     // ids per thread that a kernel with registers for them (REG) keeps until the threshold is known
 
 struct ResScratch {
   unsigned hist[kResBins];
+  unsigned spill[32];           // where the ids outside the bracket are counted
   double scan[2][kWarps];       // block scans; consecutive ones alternate
   float red[2][kWarps][3];      // block maxima, minima, sums
   float sa[kResMembers];
@@ -40,15 +42,16 @@ __host__ inline bool resident_fits(int V) { return V <= 49152; }
 struct ResRow {
   float* w;
   int V, E, beg, end;           // this thread's run
-  __device__ ResRow(float* smem, int V_) : w(smem), V(V_), E(resident_run(V_)) {
+  float inv_E;
+  __device__ ResRow(float* smem, int V_) : w(smem), V(V_), E(resident_run(V_)), inv_E(1.0f / (float)resident_run(V_)) {
     beg = min(V, (int)threadIdx.x * E);
     end = min(V, beg + E);
   }
   __device__ __forceinline__ float* run() const { return w + threadIdx.x * (E + 4); }
-  __device__ __forceinline__ float& at(int x) const {
-    const int o = x / E;
-    return w[o * (E + 4) + x - o * E];
+  __device__ __forceinline__ float* place(int x) const {   // (x + 0.5) / E in fp32 truncates to x / E for x < 2^16)
+    return w + x + 4 * (int)(((float)x + 0.5f) * inv_E);
   }
+  __device__ __forceinline__ float& at(int x) const { return *place(x); }
 };
 
 struct ResSums {      // block scan of one value per thread, in id order
@@ -83,22 +86,86 @@ __device__ __forceinline__ ResSums res_scan(double v, ResScratch& rs, int& calls
   return r;
 }
 
-// The row from global memory into shared memory; every thread gets the row's maximum, minimum and mean.
-__device__ inline void res_load(const ResRow& row, const RowSrc& src, ResScratch& rs, float& mx, float& mn, float& mean) {
+// Eight logits of a piece, two per packed instruction.
+template <bool BF16>
+__device__ __forceinline__ void res_mix(const RowSrc& r, const raw_piece<BF16>& c, const raw_piece<BF16>& u, float (&z)[8]) {
+  const float2 s2 = make_float2(r.s, r.s), t2 = make_float2(r.invT, r.invT);
+  auto all = [&](auto row_u) {
+    constexpr bool U = decltype(row_u)::value;
+#pragma unroll
+    for (int i = 0; i < (BF16 ? 1 : 2); ++i) {
+      float2 q[4];
+      q[0] = row_pair<BF16, U, true, 0>(c.w[i], u.w[i], s2, t2);
+      q[1] = row_pair<BF16, U, true, 1>(c.w[i], u.w[i], s2, t2);
+      if (BF16) {
+        q[2] = row_pair<BF16, U, true, 2>(c.w[i], u.w[i], s2, t2);
+        q[3] = row_pair<BF16, U, true, 3>(c.w[i], u.w[i], s2, t2);
+      }
+#pragma unroll
+      for (int j = 0; j < (BF16 ? 4 : 2); ++j) {
+        z[4 * i + 2 * j] = q[j].x;
+        z[4 * i + 2 * j + 1] = q[j].y;
+      }
+    }
+  };
+  if (r.uncond) all(std::true_type{});
+  else all(std::false_type{});
+}
+
+// The row from global memory into shared memory; every thread gets the row's maximum, minimum and mean.  REG: the ids
+// this thread brought (8 at (c * 512 + tid) * 8 for c = 0 .. 3) also stay in z, -inf past the row's end.
+template <bool REG>
+__device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, ResScratch& rs, float (&z)[kResRegs], float& mx,
+                                         float& mn, float& mean) {
   float hi = -INFINITY, lo = INFINITY, sum = 0.f;
-#pragma unroll 2
-  for (int x = (int)threadIdx.x * 8; x < row.V; x += 8 * kThreads) {
-    float z[8];
-    load8<true>(src, x, z);
-    const int o = x / row.E;
-    float4* const to = reinterpret_cast<float4*>(row.w + o * (row.E + 4) + x - o * row.E);
-    to[0] = make_float4(z[0], z[1], z[2], z[3]);
-    to[1] = make_float4(z[4], z[5], z[6], z[7]);
+  auto take = [&](int x, const float (&v)[8]) {
+    float4* const to = reinterpret_cast<float4*>(row.place(x));
+    to[0] = make_float4(v[0], v[1], v[2], v[3]);
+    to[1] = make_float4(v[4], v[5], v[6], v[7]);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      hi = fmaxf(hi, z[j]);
-      lo = fminf(lo, z[j]);
-      sum += z[j];
+      hi = fmaxf(hi, v[j]);
+      lo = fminf(lo, v[j]);
+      sum += v[j];
+    }
+  };
+  if (REG) {
+    // (four pieces of bf16, two of fp32 asked for before any is used)
+    auto pieces = [&](auto bf16, int first) {
+      constexpr bool BF16 = decltype(bf16)::value;
+      constexpr int F = BF16 ? 4 : 2;
+      raw_piece<BF16> c[F], u[F] = {};
+#pragma unroll
+      for (int k = 0; k < F; ++k) {
+        const int x = ((first + k) * kThreads + (int)threadIdx.x) * 8;
+        if (x < row.V) ask8<true, BF16>(src, x, c[k], u[k]);
+      }
+#pragma unroll
+      for (int k = 0; k < F; ++k) {
+        const int x = ((first + k) * kThreads + (int)threadIdx.x) * 8;
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = -INFINITY;
+        if (x < row.V) {
+          res_mix<BF16>(src, c[k], u[k], v);
+          take(x, v);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) z[8 * (first + k) + j] = v[j];
+      }
+    };
+    if (src.bf16) {
+      pieces(std::true_type{}, 0);
+    } else {
+      pieces(std::false_type{}, 0);
+      pieces(std::false_type{}, 2);
+    }
+  } else {
+#pragma unroll 2
+    for (int x = (int)threadIdx.x * 8; x < row.V; x += 8 * kThreads) {
+      float v[8];
+      load8<true>(src, x, v);
+      take(x, v);
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -133,25 +200,53 @@ __device__ inline void res_load(const ResRow& row, const RowSrc& src, ResScratch
 
 // The top_k-th largest value of the resident row (1 <= top_k < V).  The map z -> bin is monotone, so the crossing
 // bin's entries are consecutive in rank whatever the rounding.
-__device__ inline float res_select(const ResRow& row, int top_k, float mx, float mn, float mean, ResScratch& rs) {
+template <bool REG>
+__device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)[kResRegs], int top_k, float mx, float mn,
+                                            float mean, ResScratch& rs) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n_mine = REG ? kResRegs : row.end - row.beg;
   float zlo = mean > mn && mean < mx ? mean : mn, zhi = mx;
   int above = 0;   // entries above zhi
+#pragma unroll 1
   for (;;) {
     if (!(zlo < zhi)) {   // one value left (uniform)
       __syncthreads();
       return zhi;
     }
     const float sc = (float)(kResBins - 1) / (zhi - zlo);
-    auto bin_of = [&](float v) -> int { return min((int)__fmul_rn(__fsub_rn(v, zlo), sc), kResBins - 1); };
-    const float* const z = row.run();
-#pragma unroll 1
-    for (int i = 0; i < row.end - row.beg; i += 4) {
-      const float4 q = *reinterpret_cast<const float4*>(z + i);
-      const float v[4] = {q.x, q.y, q.z, q.w};
+    // (a range so small that the scale leaves fp32: steps of the order-preserving integer keys instead)
+    const bool by_key = !(sc < 1e30f);
+    const uint32_t key_lo = float_key(zlo);
+    const int shift = max(0, 22 - __clz(float_key(zhi) - key_lo));
+    // the bin of v, or one past the last outside the bracket (v - zlo and the product are monotone; adding 1.5 * 2^23
+    // leaves the rounded integer in the low bits; what rounds up into the first bin from below it does no harm)
+    auto bin_of = [&](float v) -> unsigned {
+      unsigned b = (unsigned)(__float_as_int(fmaf(__fsub_rn(v, zlo), sc, kRMagic)) - __float_as_int(kRMagic));
+      if (by_key) b = v >= zlo ? (float_key(v) - key_lo) >> shift : (unsigned)kResBins;
+      return v <= zhi ? b : (unsigned)kResBins;
+    };
+    // eight of this thread's logits
+    auto eight = [&](int i, float (&v)[8]) {
+      const float4 a = *reinterpret_cast<const float4*>(row.run() + i), b = *reinterpret_cast<const float4*>(row.run() + i + 4);
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+      v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    };
+    const uint32_t hist = smem_u32(rs.hist), spill = smem_u32(rs.spill) + (uint32_t)lane * 4u;
+    auto count = [&](float v) {   // (no branch: what lies outside counts in a word of its lane)
+      const unsigned b = bin_of(v);
+      asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b < (unsigned)kResBins ? hist + 4u * b : spill) : "memory");
+    };
+    if (REG) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (v[j] >= zlo && v[j] <= zhi) atomicAdd(&rs.hist[bin_of(v[j])], 1u);
+      for (int i = 0; i < kResRegs; ++i) count(zr[i]);
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < n_mine; i += 8) {
+        float v[8];
+        eight(i, v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) count(v[j]);
+      }
     }
     __syncthreads();
     // the crossing bin, from the top: every warp finds it (32 bins per lane, lane 0 the highest)
@@ -187,31 +282,45 @@ __device__ inline float res_select(const ResRow& row, int top_k, float mx, float
       if (lane >= o) inc += t;
     }
     const int k = __ffs(__ballot_sync(kFull, over + inc >= want)) - 1;
-    const int bin = (31 - src) * 32 + 31 - k;
+    const unsigned bin = (unsigned)((31 - src) * 32 + 31 - k);
     const int in_bin = (int)__shfl_sync(kFull, h, k);
     over += __shfl_sync(kFull, inc - h, k);
     // its entries: set aside if few, else their range for the next histogram
     float vhi = -INFINITY, vlo = INFINITY;
-#pragma unroll 1
-    for (int i = 0; i < row.end - row.beg; i += 4) {
-      const float4 q = *reinterpret_cast<const float4*>(z + i);
-      const float v[4] = {q.x, q.y, q.z, q.w};
+    auto member = [&](float v) {
+      if (in_bin <= kResMembers) rs.sa[atomicAdd(&rs.n_sa, 1u)] = v;
+      vhi = fmaxf(vhi, v);
+      vlo = fminf(vlo, v);
+    };
+    if (REG) {
+      uint32_t m = 0;
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (v[j] >= zlo && v[j] <= zhi && bin_of(v[j]) == bin) {
-          if (in_bin <= kResMembers) rs.sa[atomicAdd(&rs.n_sa, 1u)] = v[j];
-          vhi = fmaxf(vhi, v[j]);
-          vlo = fminf(vlo, v[j]);
-        }
+      for (int i = 0; i < kResRegs; ++i) m |= bin_of(zr[i]) == bin ? 1u << i : 0u;
+#pragma unroll 1
+      for (; m; m &= m - 1u) {   // (from shared memory: registers cannot be picked by number)
+        const int i = __ffs(m) - 1;
+        member(row.at(((i >> 3) * kThreads + (int)threadIdx.x) * 8 + (i & 7)));
+      }
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < n_mine; i += 8) {
+        float v[8];
+        eight(i, v);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (bin_of(v[j]) == bin) member(v[j]);
+      }
     }
     if (in_bin <= kResMembers) {
       __syncthreads();
       const unsigned r = want - over;   // rank from the top within the bin
       float th = 0.f;
       bool found = false;
+#pragma unroll 1
       for (int i = lane; i < in_bin; i += 32) {
         const float vi = rs.sa[i];
         unsigned more = 0, geq = 0;
+#pragma unroll 4
         for (int j = 0; j < in_bin; ++j) {
           const float vj = rs.sa[j];
           more += vj > vi;
@@ -299,15 +408,18 @@ __device__ inline void res_pick(const ResRow& row, const ResSums& s, double u, W
   if (lane == 0) *out = pick >= 0 ? pick : last >= 0 ? last : x_beg;   // (rounding: the last id with weight)
 }
 
-// Statistics of a row (threshold, maximum, partition sum); the row's weights stay in shared memory.
+// Statistics of a row (threshold, maximum, partition sum); the row's weights stay in shared memory.  REG: in a kernel
+// compiled for 128 registers, for rows of up to 16384 ids.
+template <bool REG = false>
 __device__ inline ResSums res_row_stats(const ResRow& row, const RowSrc& src, int top_k, ResScratch& rs, int& calls,
                                         int tok, float& z_tok, RowStats& st) {
   float mx, mn, mean;
-  res_load(row, src, rs, mx, mn, mean);
+  float z[kResRegs];
+  res_load<REG>(row, src, rs, z, mx, mn, mean);
   z_tok = tok >= 0 ? row.at(tok) : 0.f;   // (before the logits become weights)
   st.m = mx;
   st.theta = -INFINITY;
-  if (top_k > 0 && top_k < row.V) st.theta = res_select(row, top_k, mx, mn, mean, rs);
+  if (top_k > 0 && top_k < row.V) st.theta = res_select<REG>(row, z, top_k, mx, mn, mean, rs);
   else __syncthreads();                   // everybody has z_tok
   const ResSums s = res_weigh(row, st.theta, mx, rs, calls);
   st.Z = s.total;
