@@ -1174,12 +1174,8 @@ mulo_status mulo_island_schedule(mulo_ctx* ctx, const mulo_params* p, const int3
   ScheduleArgs a;
   a.H = p->H; a.W = p->W; a.window = window > p->W ? p->W : window;
   a.labels = labels; a.step = step; a.n_steps = n_steps;
-  const size_t smem = (size_t)4 * p->W * sizeof(int);
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k_island_schedule, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return MULO_ERR_CUDA;
-  }
+  const size_t smem = schedule_smem(p->H, p->W);
+  if (ctas_per_sm(ctx, k_island_schedule, kScheduleThreads, smem) < 1) return MULO_ERR_UNSUPPORTED;
   k_island_schedule<<<p->B, kScheduleThreads, smem, (cudaStream_t)stream>>>(a);
   return launched(ctx, 1);
 }
@@ -1394,12 +1390,7 @@ mulo_status mulo_islands(mulo_ctx* ctx, const mulo_params* p, const uint32_t* ex
   a.rows = max_islands > 0 ? island_rows : nullptr;
   a.size = max_islands > 0 ? island_size : nullptr;
   const size_t smem = ((size_t)2 * p->H * p->W + (size_t)p->H * ((p->W + 31) / 32)) * sizeof(int);
-  if (smem + 1024 > (size_t)ctx->smem_optin) return MULO_ERR_UNSUPPORTED;
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k_islands, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-    cudaGetLastError();
-    return MULO_ERR_CUDA;
-  }
+  if (ctas_per_sm(ctx, k_islands, kIslandThreads, smem) < 1) return MULO_ERR_UNSUPPORTED;
   k_islands<<<p->B, kIslandThreads, smem, (cudaStream_t)stream>>>(a);
   return launched(ctx, 1);
 }

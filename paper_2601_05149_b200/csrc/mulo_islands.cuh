@@ -11,6 +11,7 @@
 // numbering the roots in raster order (a block-wide count) numbers the islands by their
 // first position.
 #pragma once
+#include <climits>
 #include <cstdint>
 
 namespace mulo {
@@ -209,9 +210,14 @@ __global__ void __launch_bounds__(kIslandThreads) k_islands(IslandArgs a) {
 // the sequential step at which each position of R_X is decoded,
 //   step(t) = 1 + max(step of the island's earlier positions in the row,
 //                     step of the island's positions in the row above up to column col(t) + window - 1).
-// Along a row the recurrence s_k = max(s_{k-1} + 1, d_k) has the closed form
-// s_k = max_{l <= k} (d_l + k - l), so the positions of a row are independent of one another: one CTA per
-// image, one thread per column, the rows in sequence.
+// Steps grow along an island's positions in a row, so of the row above only the last position inside the window
+// counts, and along a run of neighbours the recurrence s_k = max(s_{k-1} + 1, d_k) is a prefix maximum of d_k - k.
+// One CTA per image.  All threads first find, for every position, what it depends on -- its run, the position of the
+// row above, for a run the island's previous run in the row -- with bit operations on the rows' masks; nothing of that
+// needs a step.  ONE warp then goes down the rows with shuffles instead of block barriers; the runs of a row share one
+// scan (a term that grows from run to run keeps them apart).  In rows where an island has several runs, a run adds to
+// the next one's steps: lane r takes run r and the chains are followed by doubling.  What bounds the kernel is this
+// chain of H rows (three barriers and two searches per row made them 2.5 us each at 64 columns).
 struct ScheduleArgs {
   int H, W, window;
   const int32_t* labels;   // [B, H, W]
@@ -219,57 +225,194 @@ struct ScheduleArgs {
   int32_t* n_steps;        // [B]
 };
 
-constexpr int kScheduleThreads = 256;
+constexpr int kScheduleThreads = 1024;
+constexpr int kRunTerm = 1 << 15;   // more than two steps, or columns, of one image can differ by
+
+__host__ inline size_t schedule_smem(int H, int W) {
+  const size_t N = (size_t)H * W, nw = (size_t)H * ((W + 31) / 32);
+  return N * 12 + 2 * nw * 4 + (size_t)H * 4;
+}
 
 __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleArgs a) {
-  extern __shared__ int sched_smem[];
-  const int H = a.H, W = a.W, b = blockIdx.x, tid = threadIdx.x;
-  int* const lab_up = sched_smem;           // labels of row i - 1
-  int* const step_up = sched_smem + W;      // steps of row i - 1
-  int* const lab = sched_smem + 2 * W;      // labels of row i
-  int* const dep = sched_smem + 3 * W;      // d_k of row i: 1 + what the row above demands
-  __shared__ int s_max;
-  if (tid == 0) s_max = 0;
-  const int32_t* labels = a.labels + (size_t)b * H * W;
-  int32_t* step = a.step + (size_t)b * H * W;
-  int local_max = 0;
-  for (int i = 0; i < H; ++i) {
-    __syncthreads();   // the previous row's results are in step_up / lab_up
-    for (int j = tid; j < W; j += kScheduleThreads) lab[j] = labels[(size_t)i * W + j];
-    __syncthreads();
-    for (int j = tid; j < W; j += kScheduleThreads) {
-      const int m = lab[j];
-      int d = 1;
-      if (m > 0 && i > 0) {
-        // steps grow along a row of an island: its last position at or before column j + window - 1
-        for (int jj = min(W - 1, j + a.window - 1); jj >= 0; --jj)
-          if (lab_up[jj] == m) {
-            d = step_up[jj] + 1;
-            break;
-          }
-      }
-      dep[j] = d;
-    }
-    __syncthreads();
-    for (int j = tid; j < W; j += kScheduleThreads) {
-      const int m = lab[j];
-      int s = 0;
-      if (m > 0) {
-        int behind = 0;   // k - l: positions of the island between column jj and column j
-        for (int jj = j; jj >= 0; --jj)
-          if (lab[jj] == m) {
-            s = max(s, dep[jj] + behind);
-            ++behind;
-          }
-      }
-      step[(size_t)i * W + j] = s;
-      local_max = max(local_max, s);
-      // becomes the row above (nobody reads step_up / lab_up any more in this row)
-      step_up[j] = s;
-      lab_up[j] = m;
+  extern __shared__ __align__(16) unsigned char sched_smem[];
+  const int H = a.H, W = a.W, N = H * W, Ww = (W + 31) / 32, nw = H * Ww, b = blockIdx.x, tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  int* const lab = reinterpret_cast<int*>(sched_smem);                      // labels, then steps
+  uint32_t* const pos = reinterpret_cast<uint32_t*>(lab + N);               // bit: the position is in R_X
+  uint32_t* const first = pos + nw;                                         // bit: ... and starts a run
+  // by position: number of its run in the row (-1 outside R_X) << 16 | column of the row above (0xffff: none)
+  int* const place = reinterpret_cast<int*>(first + nw);
+  // by run of the row: the island's previous run in the row (-1: none) << 16 | last column
+  int* const table = place + N;
+  int* const linked = table + N;                                            // runs of a row where one has a predecessor, else 0
+  __shared__ int s_max, s_many;
+  if (tid == 0) s_max = s_many = 0;
+  const int32_t* const labels = a.labels + (size_t)b * N;
+  for (int t = tid; t < N; t += kScheduleThreads) lab[t] = labels[t];
+  for (int i = tid; i < H; i += kScheduleThreads) linked[i] = 0;
+  __syncthreads();
+  for (int w = warp; w < nw; w += kScheduleThreads / 32) {   // the rows' masks
+    const int i = w / Ww, j = (w % Ww) * 32 + lane;
+    const int m = j < W ? lab[i * W + j] : 0, left = j > 0 && j < W ? lab[i * W + j - 1] : 0;
+    const unsigned in = __ballot_sync(0xffffffffu, m > 0), fs = __ballot_sync(0xffffffffu, m > 0 && m != left);
+    if (lane == 0) {
+      pos[w] = in;
+      first[w] = fs;
     }
   }
-  atomicMax(&s_max, local_max);
+  __syncthreads();
+  // the last set bit of a row's mask at or before column x, -1: none
+  auto last_at = [&](const uint32_t* row, int x) -> int {
+    if (x < 0) return -1;
+    int w = x >> 5;
+    uint32_t v = row[w] & (0xffffffffu >> (31 - (x & 31)));
+    while (v == 0u && w > 0) v = row[--w];
+    return v ? (w << 5) + 31 - __clz(v) : -1;
+  };
+  // the last position of label m in row i at or before column x: run by run
+  auto last_of = [&](int i, int x, int m) -> int {
+    for (;;) {
+      x = last_at(pos + i * Ww, x);
+      if (x < 0 || lab[i * W + x] == m) return x;
+      x = last_at(first + i * Ww, x) - 1;
+    }
+  };
+  // the number, within the row, of the run that holds column x
+  auto run_of = [&](int i, int x) -> int {
+    int n = -1;
+    for (int w = 0; w < x >> 5; ++w) n += __popc(first[i * Ww + w]);
+    return n + __popc(first[i * Ww + (x >> 5)] & (0xffffffffu >> (31 - (x & 31))));
+  };
+  for (int w = warp; w < nw; w += kScheduleThreads / 32) {
+    const int i = w / Ww, j = (w % Ww) * 32 + lane;
+    if (j >= W) continue;
+    const int t = i * W + j, m = lab[t];
+    int r = -1, u = -1;
+    if (m > 0) {
+      r = run_of(i, j);
+      if (i > 0) u = last_of(i - 1, min(W - 1, j + a.window - 1), m);
+      if (j + 1 == W || lab[t + 1] != m) {   // the run's last position enters it in the row's table
+        const int l = last_of(i, last_at(first + i * Ww, j) - 1, m);
+        table[i * W + r] = (l >= 0 ? run_of(i, l) : -1) << 16 | j;
+        const int nr = run_of(i, W - 1) + 1;
+        if (l >= 0) linked[i] = nr;
+        if (nr > 32) s_many = 1;
+      }
+    }
+    place[t] = r << 16 | (u & 0xffff);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    // the key of a position: what the row above demands, less its column, plus its run's term
+    auto key = [&](int pl, int j, const int* above) -> int {
+      const int u = pl & 0xffff, r = pl >> 16;
+      const int d = u != 0xffff ? above[u] + 1 : 1;
+      return r >= 0 ? d - j + r * kRunTerm : INT_MIN;
+    };
+    // Chains of runs: run r hands on max(c + len, its last step); maps of this kind composed by doubling (lane r: run r).
+    // Returns the step before the run's first one that its predecessor demands (0: none); beg: that first column.
+    auto follow = [&](int i, int nr, const int* row, int& beg) -> int {
+      int top = 0, len = 0, p = -1;
+      beg = 0;
+      if (lane < nr) {
+        const int e = table[i * W + lane];
+        p = e >> 16;
+        top = row[e & 0xffff];
+        beg = last_at(first + i * Ww, e & 0xffff);
+        len = (e & 0xffff) - beg + 1;
+      }
+      const int p0 = p;
+      while (__any_sync(0xffffffffu, p >= 0)) {
+        const int q = max(p, 0);
+        const int t2 = __shfl_sync(0xffffffffu, top, q), l2 = __shfl_sync(0xffffffffu, len, q), p2 = __shfl_sync(0xffffffffu, p, q);
+        if (p >= 0) {
+          top = max(top, t2 + len);
+          len += l2;
+          p = p2;
+        }
+      }
+      const int c = __shfl_sync(0xffffffffu, top, max(p0, 0));
+      return p0 >= 0 ? c : 0;
+    };
+    int* row = lab;
+    if (Ww <= 2 && !s_many) {   // a row is two values per lane, which stay in registers
+      const int j0 = lane, j1 = min(32 + lane, W - 1);
+      const bool in0 = j0 < W, in1 = 32 + lane < W;
+      for (int i = 0; i < H; ++i, row += W) {
+        const int nr = linked[i], p0 = in0 ? place[i * W + j0] : -1, p1 = in1 ? place[i * W + j1] : -1;
+        int v0 = key(p0, j0, row - W), v1 = key(p1, j1, row - W);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          v0 = max(v0, __shfl_up_sync(0xffffffffu, v0, o));   // (the first lanes get their own value)
+          v1 = max(v1, __shfl_up_sync(0xffffffffu, v1, o));
+        }
+        v1 = max(v1, __shfl_sync(0xffffffffu, v0, 31));
+        const int r0 = p0 >> 16, r1 = p1 >> 16;
+        int s0 = r0 >= 0 ? v0 + j0 - r0 * kRunTerm : 0, s1 = r1 >= 0 ? v1 + j1 - r1 * kRunTerm : 0;
+        if (in0) row[j0] = s0;
+        if (in1) row[j1] = s1;
+        __syncwarp();
+        if (nr > 0) {
+          int beg;
+          const int c = follow(i, nr, row, beg);
+          const int c0 = __shfl_sync(0xffffffffu, c, r0 & 31), c1 = __shfl_sync(0xffffffffu, c, r1 & 31);
+          const int b0 = __shfl_sync(0xffffffffu, beg, r0 & 31), b1 = __shfl_sync(0xffffffffu, beg, r1 & 31);
+          if (r0 >= 0 && c0 > 0) row[j0] = max(s0, c0 + 1 + j0 - b0);
+          if (r1 >= 0 && c1 > 0) row[j1] = max(s1, c1 + 1 + j1 - b1);
+          __syncwarp();
+        }
+      }
+    } else {
+      for (int i = 0; i < H; ++i, row += W) {
+        int carry = INT_MIN;
+        for (int w = 0; w < Ww; ++w) {
+          const int j = (w << 5) + lane, pl = j < W ? place[i * W + j] : -1, r = pl >> 16;
+          int v = key(pl, j, row - W);
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) v = max(v, __shfl_up_sync(0xffffffffu, v, o));
+          v = max(v, carry);
+          carry = __shfl_sync(0xffffffffu, v, 31);
+          if (j < W) row[j] = r >= 0 ? v + j - r * kRunTerm : 0;
+        }
+        __syncwarp();
+        const int nr = linked[i];
+        if (nr == 0) continue;
+        int c = 0, beg = 0;
+        if (nr <= 32) {
+          c = follow(i, nr, row, beg);
+        } else {   // run by run
+          if (lane == 0)
+            for (int r = 0; r < nr; ++r) {
+              const int e = table[i * W + r] & 0xffff, p = table[i * W + r] >> 16;
+              if (p >= 0) row[e] = max(row[e], row[table[i * W + p] & 0xffff] + e - last_at(first + i * Ww, e) + 1);
+            }
+          __syncwarp();
+        }
+        for (int w = 0; w < Ww; ++w) {
+          const int j = (w << 5) + lane, r = j < W ? place[i * W + j] >> 16 : -1;
+          int cr = 0, br = 0;
+          if (nr <= 32) {
+            cr = __shfl_sync(0xffffffffu, c, r & 31);
+            br = __shfl_sync(0xffffffffu, beg, r & 31);
+          } else if (r >= 0 && (table[i * W + r] >> 16) >= 0) {
+            cr = row[table[i * W + (table[i * W + r] >> 16)] & 0xffff];
+            br = last_at(first + i * Ww, j);
+          }
+          if (r >= 0 && cr > 0) row[j] = max(row[j], cr + 1 + j - br);
+        }
+        __syncwarp();
+      }
+    }
+  }
+  __syncthreads();
+  int mine = 0;
+  for (int t = tid; t < N; t += kScheduleThreads) {
+    const int s = lab[t];
+    a.step[(size_t)b * N + t] = s;
+    mine = max(mine, s);
+  }
+  mine = __reduce_max_sync(0xffffffffu, mine);
+  if (lane == 0) atomicMax(&s_max, mine);
   __syncthreads();
   if (tid == 0) a.n_steps[b] = s_max;
 }
