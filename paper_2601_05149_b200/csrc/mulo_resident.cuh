@@ -26,7 +26,8 @@ struct ResScratch {
   unsigned hist[kResBins];
   unsigned spill[32];           // where the ids outside the bracket are counted
   double scan[2][kWarps];       // block scans; consecutive ones alternate
-  float red[2][kWarps][3];      // block maxima, minima, sums
+  unsigned top[kWarps], low[kWarps];   // keys of block maxima and minima
+  float sum[kWarps];
   float sa[kResMembers];
   unsigned n_sa;
   int first_bad;
@@ -112,12 +113,12 @@ __device__ __forceinline__ void res_mix(const RowSrc& r, const raw_piece<BF16>& 
   else all(std::false_type{});
 }
 
-// The row from global memory into shared memory; every thread gets the row's maximum, minimum and mean.  REG: the ids
+// The row from global memory into shared memory; every thread gets the row's maximum and mean.  REG: the ids
 // this thread brought (8 at (c * 512 + tid) * 8 for c = 0 .. 3) also stay in z, -inf past the row's end.
 template <bool REG>
 __device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, ResScratch& rs, float (&z)[kResRegs], float& mx,
-                                         float& mn, float& mean) {
-  float hi = -INFINITY, lo = INFINITY, sum = 0.f;
+                                         float& mean) {
+  float hi = -INFINITY, sum = 0.f;
   auto take = [&](int x, const float (&v)[8]) {
     float4* const to = reinterpret_cast<float4*>(row.place(x));
     to[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -125,7 +126,6 @@ __device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, R
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       hi = fmaxf(hi, v[j]);
-      lo = fminf(lo, v[j]);
       sum += v[j];
     }
   };
@@ -164,217 +164,255 @@ __device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, R
 #pragma unroll 2
     for (int x = (int)threadIdx.x * 8; x < row.V; x += 8 * kThreads) {
       float v[8];
-      load8<true>(src, x, v);
+      if (src.bf16) {
+        raw_piece<true> c, u = {};
+        ask8<true, true>(src, x, c, u);
+        res_mix<true>(src, c, u, v);
+      } else {
+        raw_piece<false> c, u = {};
+        ask8<true, false>(src, x, c, u);
+        res_mix<false>(src, c, u, v);
+      }
       take(x, v);
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
-    lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
-    sum += __shfl_xor_sync(kFull, sum, o);
-  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+  const unsigned key = __reduce_max_sync(kFull, float_key(hi));
   if (lane == 0) {
-    rs.red[0][warp][0] = hi;
-    rs.red[0][warp][1] = lo;
-    rs.red[0][warp][2] = sum;
+    rs.top[warp] = key;
+    rs.sum[warp] = sum;
   }
   if (threadIdx.x == 0) rs.n_sa = 0;
 #pragma unroll
   for (int i = 0; i < kResBins / kThreads; ++i) rs.hist[threadIdx.x + i * kThreads] = 0;
   __syncthreads();
-  hi = rs.red[0][lane & (kWarps - 1)][0];
-  lo = rs.red[0][lane & (kWarps - 1)][1];
-  sum = rs.red[0][lane & (kWarps - 1)][2];
+  mx = key_float(__reduce_max_sync(kFull, rs.top[lane & (kWarps - 1)]));
+  sum = rs.sum[lane & (kWarps - 1)];
 #pragma unroll
-  for (int o = kWarps / 2; o > 0; o >>= 1) {
-    hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
-    lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
-    sum += __shfl_xor_sync(kFull, sum, o);
-  }
-  mx = hi;
-  mn = lo;
+  for (int o = kWarps / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
   mean = sum / (float)row.V;
 }
 
-// The top_k-th largest value of the resident row (1 <= top_k < V).  The map z -> bin is monotone, so the crossing
-// bin's entries are consecutive in rank whatever the rounding.
-template <bool REG>
-__device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)[kResRegs], int top_k, float mx, float mn,
-                                            float mean, ResScratch& rs) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int n_mine = REG ? kResRegs : row.end - row.beg;
-  float zlo = mean > mn && mean < mx ? mean : mn, zhi = mx;
-  int above = 0;   // entries above zhi
+// What the histogram of a bracket says about rank `want` from the top: the bin that holds it, the entries above that
+// bin, the entries in it (-1: the bracket holds fewer).  Every warp finds it, 32 bins per lane, lane 0 the highest.
+__device__ __forceinline__ int res_crossing(const ResScratch& rs, unsigned want, unsigned& over, int& in_bin) {
+  const int lane = threadIdx.x & 31;
+  unsigned mine = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint4 h = *reinterpret_cast<const uint4*>(&rs.hist[(31 - lane) * 32 + 4 * ((i + lane) & 7)]);
+    mine += (h.x + h.y) + (h.z + h.w);
+  }
+  unsigned inc = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(kFull, inc, o);
+    if (lane >= o) inc += t;
+  }
+  const unsigned hit = __ballot_sync(kFull, inc >= want);
+  if (hit == 0) return -1;
+  const int src = __ffs(hit) - 1;
+  over = __shfl_sync(kFull, inc - mine, src);
+  const unsigned h = rs.hist[(31 - src) * 32 + 31 - lane];
+  inc = h;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(kFull, inc, o);
+    if (lane >= o) inc += t;
+  }
+  const int k = __ffs(__ballot_sync(kFull, over + inc >= want)) - 1;
+  in_bin = (int)__shfl_sync(kFull, h, k);
+  over += __shfl_sync(kFull, inc - h, k);
+  return (31 - src) * 32 + 31 - k;
+}
+
+// The value of rank r from the top among the entries set aside.
+__device__ __forceinline__ float res_rank(const ResScratch& rs, int n, unsigned r) {
+  float th = 0.f;
+  bool found = false;
 #pragma unroll 1
-  for (;;) {
-    if (!(zlo < zhi)) {   // one value left (uniform)
-      __syncthreads();
-      return zhi;
+  for (int i = threadIdx.x & 31; i < n; i += 32) {
+    const float vi = rs.sa[i];
+    unsigned more = 0, geq = 0;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const float vj = rs.sa[j];
+      more += vj > vi;
+      geq += vj >= vi;
     }
-    const float sc = (float)(kResBins - 1) / (zhi - zlo);
-    // (a range so small that the scale leaves fp32: steps of the order-preserving integer keys instead)
-    const bool by_key = !(sc < 1e30f);
-    const uint32_t key_lo = float_key(zlo);
-    const int shift = max(0, 22 - __clz(float_key(zhi) - key_lo));
-    // the bin of v, or one past the last outside the bracket (v - zlo and the product are monotone; adding 1.5 * 2^23
-    // leaves the rounded integer in the low bits; what rounds up into the first bin from below it does no harm)
-    auto bin_of = [&](float v) -> unsigned {
-      unsigned b = (unsigned)(__float_as_int(fmaf(__fsub_rn(v, zlo), sc, kRMagic)) - __float_as_int(kRMagic));
-      if (by_key) b = v >= zlo ? (float_key(v) - key_lo) >> shift : (unsigned)kResBins;
-      return v <= zhi ? b : (unsigned)kResBins;
-    };
-    // eight of this thread's logits
-    auto eight = [&](int i, float (&v)[8]) {
-      const float4 a = *reinterpret_cast<const float4*>(row.run() + i), b = *reinterpret_cast<const float4*>(row.run() + i + 4);
-      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-      v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-    };
-    const uint32_t hist = smem_u32(rs.hist), spill = smem_u32(rs.spill) + (uint32_t)lane * 4u;
-    auto count = [&](float v) {   // (no branch: what lies outside counts in a word of its lane)
-      const unsigned b = bin_of(v);
-      asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b < (unsigned)kResBins ? hist + 4u * b : spill) : "memory");
-    };
-    if (REG) {
-#pragma unroll
-      for (int i = 0; i < kResRegs; ++i) count(zr[i]);
-    } else {
-#pragma unroll 1
-      for (int i = 0; i < n_mine; i += 8) {
-        float v[8];
-        eight(i, v);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) count(v[j]);
-      }
+    if (more < r && r <= geq) {
+      th = vi;
+      found = true;
+    }
+  }
+  return __shfl_sync(kFull, th, __ffs(__ballot_sync(kFull, found)) - 1);   // (found: the entries hold the rank)
+}
+
+// The top_k-th largest of the row's values in [zlo, zhi], `above` being larger than zhi, by brackets that shrink by a
+// factor of 512 or more per round, in steps of the order-preserving integer keys: for rows whose first histogram did
+// not settle it (many entries in one bin, fewer than top_k above the mean).  The histogram's memory is free (all
+// threads are past a barrier since its last use) and is left so.
+__device__ __noinline__ float res_refine(const ResRow& row, int top_k, int above, float zlo, float zhi, ResScratch& rs) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_mine = row.end - row.beg;
+  const float* const z = row.run();
+  for (;;) {
+    const uint32_t lo = float_key(zlo), hi = float_key(zhi);
+    if (lo == hi) return zhi;
+    const int shift = max(0, 22 - __clz(hi - lo));
+    for (int i = threadIdx.x; i < kResBins; i += kThreads) rs.hist[i] = 0;
+    if (threadIdx.x == 0) rs.n_sa = 0;
+    __syncthreads();
+    for (int i = 0; i < n_mine; ++i) {
+      const uint32_t k = float_key(z[i]);
+      if (k >= lo && k <= hi) atomicAdd(&rs.hist[(k - lo) >> shift], 1u);
     }
     __syncthreads();
-    // the crossing bin, from the top: every warp finds it (32 bins per lane, lane 0 the highest)
-    unsigned mine = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const uint4 h = *reinterpret_cast<const uint4*>(&rs.hist[(31 - lane) * 32 + 4 * ((i + lane) & 7)]);
-      mine += (h.x + h.y) + (h.z + h.w);
-    }
-    unsigned inc = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += t;
-    }
-    const unsigned want = (unsigned)(top_k - above);   // rank from the top within [zlo, zhi]
-    const unsigned hit = __ballot_sync(kFull, inc >= want);
-    if (hit == 0) {   // (fewer than top_k entries reach the mean)
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < kResBins / kThreads; ++i) rs.hist[threadIdx.x + i * kThreads] = 0;
-      __syncthreads();
-      zlo = mn;
-      continue;
-    }
-    const int src = __ffs(hit) - 1;
-    unsigned over = __shfl_sync(kFull, inc - mine, src);
-    const unsigned h = rs.hist[(31 - src) * 32 + 31 - lane];
-    inc = h;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += t;
-    }
-    const int k = __ffs(__ballot_sync(kFull, over + inc >= want)) - 1;
-    const unsigned bin = (unsigned)((31 - src) * 32 + 31 - k);
-    const int in_bin = (int)__shfl_sync(kFull, h, k);
-    over += __shfl_sync(kFull, inc - h, k);
-    // its entries: set aside if few, else their range for the next histogram
-    float vhi = -INFINITY, vlo = INFINITY;
-    auto member = [&](float v) {
-      if (in_bin <= kResMembers) rs.sa[atomicAdd(&rs.n_sa, 1u)] = v;
-      vhi = fmaxf(vhi, v);
-      vlo = fminf(vlo, v);
-    };
-    if (REG) {
-      uint32_t m = 0;
-#pragma unroll
-      for (int i = 0; i < kResRegs; ++i) m |= bin_of(zr[i]) == bin ? 1u << i : 0u;
-#pragma unroll 1
-      for (; m; m &= m - 1u) {   // (from shared memory: registers cannot be picked by number)
-        const int i = __ffs(m) - 1;
-        member(row.at(((i >> 3) * kThreads + (int)threadIdx.x) * 8 + (i & 7)));
-      }
-    } else {
-#pragma unroll 1
-      for (int i = 0; i < n_mine; i += 8) {
-        float v[8];
-        eight(i, v);
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          if (bin_of(v[j]) == bin) member(v[j]);
+    unsigned over = 0;
+    int in_bin = 0;
+    const unsigned want = (unsigned)(top_k - above);
+    const int bin = res_crossing(rs, want, over, in_bin);
+    uint32_t vhi = 0u, vlo = ~0u;
+    for (int i = 0; i < n_mine; ++i) {
+      const uint32_t k = float_key(z[i]);
+      if (k >= lo && k <= hi && (int)((k - lo) >> shift) == bin) {
+        if (in_bin <= kResMembers) rs.sa[atomicAdd(&rs.n_sa, 1u)] = z[i];
+        vhi = max(vhi, k);
+        vlo = min(vlo, k);
       }
     }
-    if (in_bin <= kResMembers) {
-      __syncthreads();
-      const unsigned r = want - over;   // rank from the top within the bin
-      float th = 0.f;
-      bool found = false;
-#pragma unroll 1
-      for (int i = lane; i < in_bin; i += 32) {
-        const float vi = rs.sa[i];
-        unsigned more = 0, geq = 0;
-#pragma unroll 4
-        for (int j = 0; j < in_bin; ++j) {
-          const float vj = rs.sa[j];
-          more += vj > vi;
-          geq += vj >= vi;
-        }
-        if (more < r && r <= geq) {
-          th = vi;
-          found = true;
-        }
-      }
-      return __shfl_sync(kFull, th, __ffs(__ballot_sync(kFull, found)) - 1);   // (found: the bin holds the rank)
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      vhi = fmaxf(vhi, __shfl_xor_sync(kFull, vhi, o));
-      vlo = fminf(vlo, __shfl_xor_sync(kFull, vlo, o));
-    }
+    vhi = __reduce_max_sync(kFull, vhi);
+    vlo = __reduce_min_sync(kFull, vlo);
     if (lane == 0) {
-      rs.red[1][warp][0] = vhi;
-      rs.red[1][warp][1] = vlo;
+      rs.top[warp] = vhi;
+      rs.low[warp] = vlo;
     }
-    __syncthreads();   // (also: everybody is done with the histogram)
-#pragma unroll
-    for (int i = 0; i < kResBins / kThreads; ++i) rs.hist[threadIdx.x + i * kThreads] = 0;
-    vhi = rs.red[1][lane & (kWarps - 1)][0];
-    vlo = rs.red[1][lane & (kWarps - 1)][1];
-#pragma unroll
-    for (int o = kWarps / 2; o > 0; o >>= 1) {
-      vhi = fmaxf(vhi, __shfl_xor_sync(kFull, vhi, o));
-      vlo = fminf(vlo, __shfl_xor_sync(kFull, vlo, o));
-    }
-    zhi = vhi;
-    zlo = vlo;
+    __syncthreads();
+    if (in_bin <= kResMembers) return res_rank(rs, in_bin, want - over);
+    zhi = key_float(__reduce_max_sync(kFull, rs.top[lane & (kWarps - 1)]));
+    zlo = key_float(__reduce_min_sync(kFull, rs.low[lane & (kWarps - 1)]));
     above += (int)over;
     __syncthreads();
   }
 }
 
-// Logits -> weights in place; returns the scan of the threads' sums (total = partition sum).
-__device__ inline ResSums res_weigh(const ResRow& row, float theta, float m, ResScratch& rs, int& calls) {
-  float* const z = row.run();
-  double acc = 0.0;
+// The top_k-th largest value of the resident row (1 <= top_k < V): a histogram between the mean and the maximum, the
+// crossing bin's entries ranked exactly.  The map z -> bin is monotone, so a bin's entries are consecutive in rank
+// whatever the rounding (z - mean and the product round monotonically; adding 1.5 * 2^23 leaves the rounded integer in
+// the low bits; an entry that rounds up into the first bin from below it is simply one of its entries).
+template <bool REG>
+__device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)[kResRegs], int top_k, float mx, float mean,
+                                            ResScratch& rs) {
+  const int lane = threadIdx.x & 31;
+  const float sc = (float)(kResBins - 1) / (mx - mean);
+  if (!(mean < mx) || !(sc < 1e30f)) {   // (uniform)
+    __syncthreads();
+    return res_refine(row, top_k, 0, -3.4028235e38f, mx, rs);
+  }
+  auto bits_of = [&](float v) -> int { return __float_as_int(fmaf(__fsub_rn(v, mean), sc, kRMagic)); };
+  auto eight = [&](int i, float (&v)[8]) {   // eight of this thread's logits
+    const float4 a = *reinterpret_cast<const float4*>(row.run() + i), b = *reinterpret_cast<const float4*>(row.run() + i + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  };
+  const uint32_t hist = smem_u32(rs.hist) - 4u * __float_as_uint(kRMagic), spill = smem_u32(rs.spill) + (uint32_t)lane * 4u;
+  auto count = [&](float v) {   // (no branch: what lies below the first bin counts in a word of its lane)
+    const int b = bits_of(v);
+    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b >= __float_as_int(kRMagic) ? hist + 4u * (uint32_t)b : spill) : "memory");
+  };
+  const int n_mine = row.end - row.beg;
+  if (REG) {
+#pragma unroll
+    for (int i = 0; i < kResRegs; ++i) count(zr[i]);
+  } else {
 #pragma unroll 1
-  for (int i = 0; i < row.end - row.beg; i += 8) {
-    float4 a = *reinterpret_cast<float4*>(z + i), b = *reinterpret_cast<float4*>(z + i + 4);
-    auto weigh = [&](float v) -> float {
-      const float e = expf(__fsub_rn(v, m));
-      return v >= theta ? e : 0.f;
-    };
-    a = make_float4(weigh(a.x), weigh(a.y), weigh(a.z), weigh(a.w));
-    b = make_float4(weigh(b.x), weigh(b.y), weigh(b.z), weigh(b.w));
-    *reinterpret_cast<float4*>(z + i) = a;
-    *reinterpret_cast<float4*>(z + i + 4) = b;
-    acc += (double)(((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w)));
+    for (int i = 0; i < n_mine; i += 8) {
+      float v[8];
+      eight(i, v);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) count(v[j]);
+    }
+  }
+  __syncthreads();
+  unsigned over = 0;
+  int in_bin = 0;
+  const int bin = res_crossing(rs, (unsigned)top_k, over, in_bin);
+  if (bin < 0 || in_bin > kResMembers) {   // (uniform)
+    __syncthreads();
+    return res_refine(row, top_k, 0, -3.4028235e38f, mx, rs);
+  }
+  const int want_bits = bin + __float_as_int(kRMagic);
+  auto aside = [&](float v) { rs.sa[atomicAdd(&rs.n_sa, 1u)] = v; };
+  if (REG) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < kResRegs; ++i) m |= bits_of(zr[i]) == want_bits ? 1u << i : 0u;
+#pragma unroll 1
+    for (; m; m &= m - 1u) {   // (from shared memory: registers cannot be picked by number)
+      const int i = __ffs(m) - 1;
+      aside(row.at(((i >> 3) * kThreads + (int)threadIdx.x) * 8 + (i & 7)));
+    }
+  } else {
+#pragma unroll 1
+    for (int i = 0; i < n_mine; i += 8) {
+      float v[8];
+      eight(i, v);
+      uint32_t m = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) m |= bits_of(v[j]) == want_bits ? 1u << j : 0u;
+#pragma unroll 1
+      for (; m; m &= m - 1u) aside(row.run()[i + __ffs(m) - 1]);
+    }
+  }
+  __syncthreads();
+  return res_rank(rs, in_bin, (unsigned)top_k - over);
+}
+
+// Logits -> weights in place; returns the scan of the threads' sums (total = partition sum).  With a threshold most
+// entries are zero: a thread marks those it keeps and exponentiates only them.
+__device__ __forceinline__ ResSums res_weigh(const ResRow& row, float theta, float m, ResScratch& rs, int& calls) {
+  float* const z = row.run();
+  const int n = row.end - row.beg;
+  double acc = 0.0;
+  if (theta > -INFINITY) {   // uniform
+#pragma unroll 1
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      uint32_t keep = 0;
+#pragma unroll
+      for (int i = 0; i < 32; i += 4)
+        if (i0 + i < n) {
+          float4 a = *reinterpret_cast<float4*>(z + i0 + i);
+          if (a.x >= theta) keep |= 1u << i;
+          else a.x = 0.f;
+          if (a.y >= theta) keep |= 2u << i;
+          else a.y = 0.f;
+          if (a.z >= theta) keep |= 4u << i;
+          else a.z = 0.f;
+          if (a.w >= theta) keep |= 8u << i;
+          else a.w = 0.f;
+          *reinterpret_cast<float4*>(z + i0 + i) = a;
+        }
+      float s = 0.f;
+#pragma unroll 1
+      for (; keep; keep &= keep - 1u) {
+        float* const p = z + i0 + __ffs(keep) - 1;
+        const float e = expf(__fsub_rn(*p, m));
+        *p = e;
+        s += e;
+      }
+      acc += (double)s;
+    }
+  } else {
+#pragma unroll 1
+    for (int i = 0; i < n; i += 8) {
+      float4 a = *reinterpret_cast<float4*>(z + i), b = *reinterpret_cast<float4*>(z + i + 4);
+      a = make_float4(expf(__fsub_rn(a.x, m)), expf(__fsub_rn(a.y, m)), expf(__fsub_rn(a.z, m)), expf(__fsub_rn(a.w, m)));
+      b = make_float4(expf(__fsub_rn(b.x, m)), expf(__fsub_rn(b.y, m)), expf(__fsub_rn(b.z, m)), expf(__fsub_rn(b.w, m)));
+      *reinterpret_cast<float4*>(z + i) = a;
+      *reinterpret_cast<float4*>(z + i + 4) = b;
+      acc += (double)(((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w)));
+    }
   }
   return res_scan(acc, rs, calls);
 }
@@ -413,13 +451,13 @@ __device__ inline void res_pick(const ResRow& row, const ResSums& s, double u, W
 template <bool REG = false>
 __device__ inline ResSums res_row_stats(const ResRow& row, const RowSrc& src, int top_k, ResScratch& rs, int& calls,
                                         int tok, float& z_tok, RowStats& st) {
-  float mx, mn, mean;
+  float mx, mean;
   float z[kResRegs];
-  res_load<REG>(row, src, rs, z, mx, mn, mean);
+  res_load<REG>(row, src, rs, z, mx, mean);
   z_tok = tok >= 0 ? row.at(tok) : 0.f;   // (before the logits become weights)
   st.m = mx;
   st.theta = -INFINITY;
-  if (top_k > 0 && top_k < row.V) st.theta = res_select<REG>(row, z, top_k, mx, mn, mean, rs);
+  if (top_k > 0 && top_k < row.V) st.theta = res_select<REG>(row, z, top_k, mx, mean, rs);
   else __syncthreads();                   // everybody has z_tok
   const ResSums s = res_weigh(row, st.theta, mx, rs, calls);
   st.Z = s.total;
