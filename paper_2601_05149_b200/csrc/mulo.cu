@@ -1008,7 +1008,7 @@ static bool launch_stream(mulo_ctx* ctx, const StreamArgs& s, size_t dyn, cudaSt
 
 // Fills `s` and returns the dynamic shared memory of a CTA of nw warps, or 0 if these parameters are not eligible.
 static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample, int nw, RowsArgs* s) {
-  if (d.top_k <= 0 || (d.pool_k > 1 && !sample)) return 0;
+  if (d.top_k <= 0) return 0;
   const int V = d.V, k = d.top_k;
   if (V < 1024 || d.r > 4) return 0;
   const int esz = d.bf16 ? 2 : 4, ids = 16 / esz;
@@ -1037,7 +1037,7 @@ static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample,
   s->a_boot = (float)inv_norm_cdf(1.0 - (double)(k + margin_boot) / V);
   s->a_max = (float)inv_norm_cdf(1.0 - 0.5 / V);
   const size_t dyn = rows_layout(*s, nw, d.bf16, sample);
-  if (2 * (dyn + sizeof(RowsSmem<8>) + 1024) > (size_t)ctx->smem_optin) return 0;   // too few rows in flight per SM
+  if (2 * (dyn + sizeof(RowsSmem<4, true>) + 1024) > (size_t)ctx->smem_optin) return 0;   // too few rows in flight per SM
   return dyn;
 }
 
@@ -1049,9 +1049,9 @@ static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, Ro
   return 0;
 }
 
-template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
+template <bool BF16, bool HAS_U, bool SAMPLE, bool POOL, bool PLAIN, int NW>
 static bool launch_rows_p(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
-  auto kern = k_round_rows<BF16, HAS_U, SAMPLE, PLAIN, NW>;
+  auto kern = k_round_rows<BF16, HAS_U, SAMPLE, POOL, PLAIN, NW>;
   const int per_sm = ctas_per_sm(ctx, kern, NW * 32, dyn);
   if (per_sm < 1) return false;
   int grid = ctx->sm_count * per_sm;
@@ -1063,8 +1063,12 @@ static bool launch_rows_p(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStre
 template <bool BF16, bool HAS_U, bool SAMPLE, int NW>
 static bool launch_rows_t(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
   const bool plain = s.P.invT == 1.0f && s.row_bytes % (16u * kRPieceBytes * NW) == 0;
-  return plain ? launch_rows_p<BF16, HAS_U, SAMPLE, true, NW>(ctx, s, dyn, st)
-               : launch_rows_p<BF16, HAS_U, SAMPLE, false, NW>(ctx, s, dyn, st);
+  if constexpr (!SAMPLE)
+    if (s.P.pool_k > 1)
+      return plain ? launch_rows_p<BF16, HAS_U, false, true, true, NW>(ctx, s, dyn, st)
+                   : launch_rows_p<BF16, HAS_U, false, true, false, NW>(ctx, s, dyn, st);
+  return plain ? launch_rows_p<BF16, HAS_U, SAMPLE, false, true, NW>(ctx, s, dyn, st)
+               : launch_rows_p<BF16, HAS_U, SAMPLE, false, false, NW>(ctx, s, dyn, st);
 }
 
 template <int NW>
@@ -1482,6 +1486,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
   if (rdyn) {
     ra.P = a.P;
     ra.cond = a.cond; ra.uncond = a.uncond; ra.draft = a.draft; ra.draft_tok_lo = draft_tok_lo;
+    ra.nn = a.nn;
     ra.p_tok = p_tok; ra.q_tok = q_tok; ra.accept_prob = accept_prob;
     ra.flags = w.flags; ra.cand_res = w.cand_res; ra.cand_tgt = w.cand_tgt;
     ra.dev_status = w.status;
@@ -1540,7 +1545,7 @@ mulo_status mulo_round_kernel(const mulo_ctx* ctx, const mulo_params* p, int has
   FullArgs fa;
   memset(&fa, 0, sizeof fa);
   if (plan_full(ctx, d, has_uncond != 0, &fa)) *kernel = MULO_KERNEL_FULL;
-  else if (plan_rows(ctx, d, false, &ra, &nw)) *kernel = MULO_KERNEL_LANE;
+  else if (plan_rows(ctx, d, false, &ra, &nw)) *kernel = d.pool_k > 1 ? MULO_KERNEL_STREAM : MULO_KERNEL_LANE;
   else if (plan_stream(ctx, d, &sa)) *kernel = MULO_KERNEL_STREAM;
   return MULO_OK;
 }

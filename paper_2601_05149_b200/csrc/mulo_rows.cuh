@@ -21,6 +21,10 @@
 //              that both rows kept, found by intersecting the masks) per thread and group.  The group that owns
 //              u * total is searched by the whole CTA, a mask word or so per eight threads; the owner's warp takes
 //              it from there (piece, lane, id) while the others go on with the next row.
+//   pooling    (POOL, Eq. 3-4) between selection and decision: the neighbour list of x~ is walked in tiles, eight
+//              entries per thread, their logits gathered from the row (L2); prefix masses by block scan; the pooled ids'
+//              weights leave the lists (found by popcount on the survivor masks) and their owners' sums (64-bit fixed
+//              point, so the order does not matter).  x~ carries its pooled weight outside the lists.
 //
 // Three block barriers per draft row, four per target row.  Pivot, histogram scale and exp reference are predicted from the CTA's previous
 // rows of the same kind; a row without prediction takes them from the mean and spread of its first pieces.  A
@@ -63,6 +67,7 @@ struct RowsArgs {
   const char* uncond;
   const char* draft;
   const int32_t* draft_tok_lo;
+  const uint16_t* nn;       // POOL
   float* p_tok;
   float* q_tok;
   float* accept_prob;
@@ -82,7 +87,7 @@ struct RowsArgs {
   float a_theta, a_boot, a_max;
 };
 
-template <int NW>
+template <int NW, bool POOL = false>
 struct RowsSmem {
   alignas(16) unsigned hist[kRBins + 4];   // (+ one bin that rounding may reach)
   unsigned spill[32];                      // where the entries outside the window are counted
@@ -102,6 +107,10 @@ struct RowsSmem {
   float red[NW][3];
   unsigned char cnt[NW * 32];
   unsigned char over[NW];
+  // POOL
+  unsigned long long adj[POOL ? NW * 32 : 1];   // weight that left a thread's entries, times 2^40
+  double pool_sum[2][POOL ? NW : 1], pool_cj;
+  int pool_bad[POOL ? NW : 1];
 };
 
 // Dynamic shared memory of a CTA (bytes); the parts' offsets go into `s`.
@@ -250,15 +259,16 @@ __device__ __noinline__ uint4 lane_philox(uint4 c, uint2 k) {
 
 // The optional probability outputs of a position (one thread; out of line: double divisions).
 __device__ __noinline__ void lane_write_probs(float* p_tok, float* q_tok_out, float* accept_prob, size_t g, double e_tok,
-                                              double q_tok, double Z, bool threshold_rule) {
+                                              double mass, double q_tok, double Z, bool threshold_rule) {
   const double p = e_tok / Z;
   if (p_tok) p_tok[g] = (float)p;
   if (q_tok_out) q_tok_out[g] = (float)q_tok;
   if (accept_prob) {
+    const double P = mass / Z;
     double thr;
-    if (threshold_rule) thr = p;
-    else if (q_tok <= 0.0) thr = p > 0.0 ? 1.0 : 0.0;
-    else thr = fmin(1.0, p / q_tok);
+    if (threshold_rule) thr = P;
+    else if (q_tok <= 0.0) thr = P > 0.0 ? 1.0 : 0.0;
+    else thr = fmin(1.0, P / q_tok);
     accept_prob[g] = (float)thr;
   }
 }
@@ -319,13 +329,13 @@ __device__ __noinline__ double rows_div(double a, double b) { return a / b; }
 __host__ __device__ constexpr int rows_warps(bool sample) { return sample ? 24 : 16; }
 
 // PLAIN: T = 1 and every piece a thread's whole 16 bytes (V splits evenly), so no scaling and no bounds checks.
-template <bool BF16, bool HAS_U, bool SAMPLE, bool PLAIN, int NW>
+template <bool BF16, bool HAS_U, bool SAMPLE, bool POOL, bool PLAIN, int NW>
 __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
   constexpr int NT = NW * 32;
   constexpr int IDS = BF16 ? 8 : 4;              // ids per lane per piece
   constexpr int kRDepth = SAMPLE ? 2 : 4;        // pieces in flight per lane
   extern __shared__ __align__(128) unsigned char dyn[];
-  __shared__ RowsSmem<NW> sm;
+  __shared__ RowsSmem<NW, POOL> sm;
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int unit = (int)(((long long)a.n_units * blockIdx.x) / gridDim.x);
@@ -334,6 +344,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
   const int rr = SAMPLE ? 1 : P.r * P.r;
   const uint32_t row_bytes = a.row_bytes;
   const int n_words = a.n_words, R = a.R;
+  const float inv_ppg = 1.0f / (float)a.ppg;
 
   // ---- this thread's places in shared memory.  Lists grow upwards (even warps) or downwards (odd warps).
   const bool up = (warp & 1) == 0;
@@ -968,6 +979,113 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       rot_q = rot;
     } else {
       tries = 0;
+      const double e_tok = !SAMPLE && sm.z_tok >= theta ? sm.e_tok : 0.0;
+      double mass = e_tok;   // x~'s weight with what is pooled onto it
+      // where an id of the row is: the thread, its mask word, the bit in it
+      struct Spot {
+        int thread, word;
+        uint32_t bit;
+      };
+      auto spot_of = [&](int x) -> Spot {
+        const int pc = (x * (BF16 ? 2 : 4)) >> 7, grp = (int)(((float)pc + 0.5f) * inv_ppg), in_grp = pc - grp * a.ppg;
+        return {grp * 8 + ((x / IDS) & 7), in_grp >> 2, 1u << ((in_grp & 3) * IDS + x % IDS)};
+      };
+      const Spot tok_spot = POOL ? spot_of(tok) : Spot{-1, 0, 0u};
+      if constexpr (POOL) {
+        // takes the entry of a kept id out of its owner's list and sum
+        auto remove = [&](int x) {
+          const Spot sp = spot_of(x);
+          const bool o_up = ((sp.thread >> 5) & 1) == 0;
+          const uint32_t o_step = o_up ? 128u : 0u - 128u, o_tm = my + a.o_tmask + (uint32_t)sp.thread * 4u;
+          uint32_t at = my + ((uint32_t)(sp.thread >> 6) * (uint32_t)R + (o_up ? 0u : (uint32_t)(R - 1))) * 128u +
+                        (((uint32_t)sp.thread & 31u) ^ (o_up ? 0u : rot)) * 4u;
+#pragma unroll 1
+          for (int w = 0; w < sp.word; ++w) at += (uint32_t)__popc(lds_u32(o_tm + (uint32_t)(w * NT) * 4u)) * o_step;
+          const uint32_t m = lds_u32(o_tm + (uint32_t)(sp.word * NT) * 4u);
+          if (!(m & sp.bit)) return;   // (cannot be: a kept id is in the list)
+          at += (uint32_t)__popc(m & (sp.bit - 1u)) * o_step;
+          uint32_t old;   // (a list may name an id twice, or x~ itself)
+          asm volatile("atom.shared.exch.b32 %0, [%1], %2;" : "=r"(old) : "r"(at), "r"(0u) : "memory");
+          atomicAdd(&sm.adj[sp.thread], __float2ull_rz(__uint_as_float(old) * 1099511627776.0f));
+        };
+        RowSrc src;
+        src.cond = rc; src.uncond = HAS_U ? ru : nullptr; src.s = P.cfg_scale; src.invT = P.invT; src.V = P.V; src.bf16 = BF16;
+        const uint16_t* const list = a.nn + (size_t)tok * P.pool_k + 1;
+        const int nb = P.pool_k - 1;
+        const double limit = P.pool_delta * Z;
+        double carry = 0.0;
+        sm.adj[tid] = 0ull;
+        if (tid == 0) sm.pool_cj = 0.0;
+        int tile = 0;
+#pragma unroll 1
+        for (int base = 0; base < nb; base += NT * 8, ++tile) {
+          const int j0 = base + tid * 8;
+          float e[8];
+          int id[8];
+          double sum = 0.0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) id[i] = j0 + i < nb ? (int)__ldg(list + j0 + i) : -1;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            e[i] = 0.f;
+            if (id[i] >= P.V) {
+              atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
+              id[i] = P.V - 1;
+            }
+            if (id[i] >= 0) e[i] = load1(src, id[i]);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            e[i] = id[i] >= 0 && e[i] >= theta ? ex2f(fmaf(e[i], kLog2e, c0)) : 0.f;
+            sum += (double)e[i];
+          }
+          double inc = sum;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const double t = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += t;
+          }
+          // (the mass below a thread comes from its neighbour's inclusive sum: inc - sum would cancel small masses)
+          double run = __shfl_up_sync(kFull, inc, 1);
+          if (lane == 0) run = 0.0;
+          if (lane == 31) sm.pool_sum[tile & 1][warp] = inc;
+          __syncthreads();
+          double total = carry;
+#pragma unroll
+          for (int w = 0; w < NW; ++w) {
+            if (w == warp) run += total;
+            total += sm.pool_sum[tile & 1][w];
+          }
+          carry = total;
+          int bad = nb;
+          double c = run;
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (id[i] >= 0) {
+              c += (double)e[i];
+              if (bad == nb && !(c < limit)) bad = j0 + i;
+            }
+          bad = __reduce_min_sync(kFull, bad);
+          if (lane == 0) sm.pool_bad[warp] = bad;
+          __syncthreads();
+          int J = nb;   // the leading run n_1 .. n_J keeps its prefix mass below delta
+#pragma unroll
+          for (int w = 0; w < NW; ++w) J = min(J, sm.pool_bad[w]);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if (id[i] >= 0 && j0 + i < J) {
+              run += (double)e[i];
+              if (j0 + i == J - 1 || (j0 + i == base + NT * 8 - 1)) sm.pool_cj = run;
+              if (e[i] > 0.f) remove(id[i]);
+            }
+          if (J < nb) break;   // (uniform)
+          __syncthreads();     // (the last tile's prefix mass before the next one's)
+        }
+        if (tid == NT - 1 && e_tok > 0.0) remove(tok);   // x~ is drawn with its pooled weight, outside the lists
+        __syncthreads();
+        mass = e_tok + sm.pool_cj;
+        s_t = (float)fmax((double)s_t - (double)sm.adj[tid] * (1.0 / 1099511627776.0), 0.0);
+      }
       // ---- the decision (Eq. 1 / Eq. 5) and what has to be drawn, the same in every warp
       int pending = kDrawTarget;
       double u_res = 0.0, u_tgt;
@@ -977,17 +1095,16 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         u_tgt = uniform24(v.x);
       } else {
         const uint32_t* const rnd = sm.rnd[parent & 1][child];
-        const double e_tok = sm.z_tok >= theta ? sm.e_tok : 0.0;
         int accepted;
-        if (P.accept_mode == MULO_ACCEPT_THRESHOLD) accepted = e_tok >= P.tau * Z;
-        else if (q_tok <= 0.0) accepted = e_tok > 0.0;
-        else accepted = uniform24(rnd[0]) * q_tok * Z < e_tok;
+        if (P.accept_mode == MULO_ACCEPT_THRESHOLD) accepted = mass >= P.tau * Z;
+        else if (q_tok <= 0.0) accepted = mass > 0.0;
+        else accepted = uniform24(rnd[0]) * q_tok * Z < mass;
         u_res = uniform24(rnd[1]);
         u_tgt = uniform24(rnd[2]);
         if (tid == 0) {
           a.flags[g] = accepted ? 0 : 1;
           if (a.p_tok || a.q_tok || a.accept_prob)
-            lane_write_probs(a.p_tok, a.q_tok, a.accept_prob, g, e_tok, q_tok, Z,
+            lane_write_probs(a.p_tok, a.q_tok, a.accept_prob, g, e_tok, mass, q_tok, Z,
                              P.accept_mode == MULO_ACCEPT_THRESHOLD);
         }
         pending = draws_for(P.resample_mode, accepted);
@@ -1034,7 +1151,9 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
           v_t = fmaxf(s_t - mins, 0.f);
         }
         constexpr int NG = NW * 4;   // groups, and sets of eight threads in the search
+        const double w_tok = !POOL ? 0.0 : resid ? fmax(mass - q_tok * Z, 0.0) : mass;   // x~'s weight outside the lists
         double w_grp = (double)v_t;
+        if (POOL && tid == tok_spot.thread) w_grp += w_tok;
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) w_grp += __shfl_xor_sync(kFull, w_grp, o);
         double* const ws = sm.w_draw[dcall & 1];
@@ -1066,6 +1185,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
           // sums over the group's part in fixed point: 2^31 = its weight
           const float to_fx = __fdividef(2147483648.0f, (float)__shfl_sync(kFull, w_grp, og));
           uint32_t y = hit_g ? __double2uint_rz((yt - __shfl_sync(kFull, exc_d, og)) * (double)to_fx) : ~0u;
+          const uint32_t tok_fx = POOL ? __double2uint_rn(fmin(w_tok * (double)to_fx, 4294967294.0)) : 0u;
           // the thread of the group whose entries this thread looks at, and where they are
           const int own = og * 8 + (lane & 7);
           const bool o_up = ((own >> 5) & 1) == 0;
@@ -1125,6 +1245,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
             for (int w = w0; w < w1; ++w) {
               load_word(w);
               v += entries(m, ta);
+              if (POOL && own == tok_spot.thread && w == tok_spot.word) v += tok_fx;
               next_word();
             }
             __syncwarp();
@@ -1153,6 +1274,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
             for (;;) {
               load_word(w);
               v = entries(m & piece_bits, ta + (uint32_t)__popc(m & under) * o_step);
+              if (POOL && own == tok_spot.thread && w == tok_spot.word && (tok_spot.bit & piece_bits)) v += tok_fx;
               __syncwarp();
               const uint32_t t = __reduce_add_sync(kFull, v);
               if (t > 0) last_w = w;
@@ -1182,7 +1304,10 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
             ta = __shfl_sync(kFull, ta, src);
             da = __shfl_sync(kFull, da, src);
             const uint32_t bit = lane < IDS ? m & (1u << ((src >> 3) * IDS + lane)) : 0u;
-            const float wt = weight(bit, ta + (uint32_t)__popc(m & (bit - 1u)) * o_step);
+            float wt = weight(bit, ta + (uint32_t)__popc(m & (bit - 1u)) * o_step);
+            if (POOL && og * 8 + (src & 7) == tok_spot.thread && w == tok_spot.word && lane < IDS &&
+                tok_spot.bit == 1u << ((src >> 3) * IDS + lane))
+              wt += (float)w_tok;
             inc = __float2uint_rn(__fmul_rn(wt, to_fx));
 #pragma unroll
             for (int o = 1; o < IDS; o <<= 1) {
