@@ -13,7 +13,7 @@
 #include "mulo_dense.cuh"
 #include "mulo_islands.cuh"
 #include "mulo_resident.cuh"
-#include "mulo_full.cuh"
+#include "mulo_flat.cuh"
 #include "mulo_rows.cuh"
 #include "mulo_stream.cuh"
 
@@ -1085,41 +1085,57 @@ static bool launch_rows(mulo_ctx* ctx, const RowsArgs& s, bool sample, int nw, s
   return nw == 2 ? launch_rows_nw<2>(ctx, s, sample, dyn, st) : launch_rows_nw<4>(ctx, s, sample, dyn, st);
 }
 
-// ---- rows without a top-k cut: the resident-row kernel ------------------------------------
-// Eligible: top-k off, V = 256 * W with W a multiple of the ids in 16 bytes, and the rows of one
-// position (draft row if q is needed, conditional, unconditional) within a CTA's shared memory.
+// ---- rows without a top-k cut (mulo_flat.cuh) --------------------------------------------
 static bool round_needs_q(const DevParams& d) {
   return !(d.accept_mode == MULO_ACCEPT_THRESHOLD && d.resample_mode == MULO_RESAMPLE_TARGET_ALL);
 }
 
-static size_t plan_full(const mulo_ctx* ctx, const DevParams& d, bool has_u, FullArgs* s) {
+// Fills `s` and returns the dynamic shared memory of a CTA, or 0 if these parameters are not eligible.
+static size_t plan_flat(const mulo_ctx* ctx, const DevParams& d, bool sample, FlatArgs* s, bool* res) {
   if (d.top_k > 0 && d.top_k < d.V) return 0;
-  const int esz = d.bf16 ? 2 : 4, n = 16 / esz;
-  if (d.V % (kFThreads * n) != 0) return 0;
-  const int need_q = round_needs_q(d) ? 1 : 0;
-  const size_t rows = (size_t)need_q + 1 + (has_u ? 1 : 0);
-  const size_t dyn = rows * (size_t)d.V * esz + (size_t)d.V / 8 + (size_t)kFThreads * 8;
-  if (dyn + sizeof(FullSmem) + 1024 > (size_t)ctx->smem_optin) return 0;
-  s->W = d.V / kFThreads;
-  s->need_q = need_q;
+  if (!sample && d.r > kFlatMaxRatio) return 0;
+  *res = !sample && (d.pool_k > 1 || d.resample_mode != MULO_RESAMPLE_TARGET_ALL);   // a row is needed a second time
+  const int nw = *res ? kFlatResWarps : kFlatWarps;
+  s->P = d;
+  s->row_bytes = (uint32_t)(d.V * (d.bf16 ? 2 : 4));
+  const int pieces = (int)((s->row_bytes + kRPieceBytes - 1) / kRPieceBytes);
+  s->ppg = (pieces + 4 * nw - 1) / (4 * nw);
+  s->n_words = (s->ppg + 3) / 4;
+  s->need_q = !sample && round_needs_q(d) ? 1 : 0;
+  const size_t dyn = flat_smem(*s, nw, *res);
+  if (dyn + sizeof(FlatSmem<kFlatResWarps>) + 1024 > (size_t)ctx->smem_optin) return 0;
   return dyn;
 }
 
-template <bool BF16, bool HAS_U>
-static bool launch_full_t(mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
-  auto kern = k_round_full<BF16, HAS_U>;
-  const int per_sm = ctas_per_sm(ctx, kern, kFThreads, dyn);
+template <bool BF16, bool HAS_U, bool SAMPLE, bool POOL, bool RES>
+static bool launch_flat_p(mulo_ctx* ctx, const FlatArgs& s, size_t dyn, cudaStream_t st) {
+  constexpr int nw = RES ? kFlatResWarps : kFlatWarps;
+  const bool plain = s.P.invT == 1.0f && s.row_bytes % (16u * kRPieceBytes * nw) == 0;
+  auto kern = plain ? k_round_flat<BF16, HAS_U, SAMPLE, POOL, RES, true> : k_round_flat<BF16, HAS_U, SAMPLE, POOL, RES, false>;
+  const int per_sm = ctas_per_sm(ctx, kern, nw * 32, dyn);
   if (per_sm < 1) return false;
   int grid = ctx->sm_count * per_sm;
-  if (grid > s.n_parents) grid = s.n_parents;
-  kern<<<grid, kFThreads, dyn, st>>>(s);
+  if (grid > s.n_units) grid = s.n_units;
+  kern<<<grid, nw * 32, dyn, st>>>(s);
   return true;
 }
 
-static bool launch_full(mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
+template <bool BF16, bool HAS_U, bool SAMPLE>
+static bool launch_flat_t(mulo_ctx* ctx, const FlatArgs& s, bool res, size_t dyn, cudaStream_t st) {
+  if constexpr (!SAMPLE) {
+    if (s.P.pool_k > 1) return launch_flat_p<BF16, HAS_U, false, true, true>(ctx, s, dyn, st);
+    if (res) return launch_flat_p<BF16, HAS_U, false, false, true>(ctx, s, dyn, st);
+  }
+  return launch_flat_p<BF16, HAS_U, SAMPLE, false, false>(ctx, s, dyn, st);
+}
+
+static bool launch_flat(mulo_ctx* ctx, const FlatArgs& s, bool sample, bool res, size_t dyn, cudaStream_t st) {
   const bool hu = s.uncond != nullptr;
-  if (s.P.bf16) return hu ? launch_full_t<true, true>(ctx, s, dyn, st) : launch_full_t<true, false>(ctx, s, dyn, st);
-  return hu ? launch_full_t<false, true>(ctx, s, dyn, st) : launch_full_t<false, false>(ctx, s, dyn, st);
+  if (sample)
+    return s.P.bf16 ? launch_flat_t<true, false, true>(ctx, s, res, dyn, st) : launch_flat_t<false, false, true>(ctx, s, res, dyn, st);
+  if (s.P.bf16)
+    return hu ? launch_flat_t<true, true, false>(ctx, s, res, dyn, st) : launch_flat_t<true, false, false>(ctx, s, res, dyn, st);
+  return hu ? launch_flat_t<false, true, false>(ctx, s, res, dyn, st) : launch_flat_t<false, false, false>(ctx, s, res, dyn, st);
 }
 
 static size_t mask_smem(const mulo_params* p) { return (size_t)3 * p->H * ((p->W + 31) / 32) * 4; }
@@ -1262,8 +1278,19 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
   a.draft = (const char*)draft_logits_lo;
   a.out_tok = draft_tok_lo;
   a.dev_status = (uint32_t*)ctx->ws;
-  // fast path: the streaming kernel in its sampling mode (top-k on, and a workspace large
-  // enough for the list of cells it may leave to the general routines)
+  // fast paths: without a top-k cut one kernel does it; with one, a workspace large enough for the list of cells
+  // that the kernel may leave to the general routines
+  FlatArgs fa;
+  memset(&fa, 0, sizeof fa);
+  bool fres = false;
+  const size_t fdyn = ctx->force_dense ? 0 : plan_flat(ctx, a.P, true, &fa, &fres);
+  if (fdyn) {
+    fa.cond = a.draft;
+    fa.sample_out = draft_tok_lo;
+    fa.dev_status = a.dev_status;
+    fa.n_units = p->B * a.P.h * a.P.w;
+    if (launch_flat(ctx, fa, true, fres, fdyn, st)) return launched(ctx, 1);
+  }
   Workspace w;
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
@@ -1465,18 +1492,18 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     a.q_tok = nullptr;
     q_tok = nullptr;
   }
-  FullArgs fa;
+  FlatArgs fa;
   memset(&fa, 0, sizeof fa);
-  const size_t fdyn = ctx->force_dense ? 0 : plan_full(ctx, a.P, tgt_uncond != nullptr, &fa);
+  bool fres = false;
+  const size_t fdyn = ctx->force_dense ? 0 : plan_flat(ctx, a.P, false, &fa, &fres);
   if (fdyn) {
-    fa.P = a.P;
     fa.cond = a.cond; fa.uncond = a.uncond; fa.draft = a.draft; fa.draft_tok_lo = draft_tok_lo;
     fa.nn = a.nn;
     fa.p_tok = p_tok; fa.q_tok = q_tok; fa.accept_prob = accept_prob;
     fa.flags = w.flags; fa.cand_res = w.cand_res; fa.cand_tgt = w.cand_tgt;
     fa.dev_status = w.status;
-    fa.n_parents = p->B * a.P.h * a.P.w;
-    fast = launch_full(ctx, fa, fdyn, st);
+    fa.n_units = p->B * p->H * p->W;
+    fast = launch_flat(ctx, fa, false, fres, fdyn, st);
     if (fast) fast_launches = 1;
   }
   RowsArgs ra;
@@ -1542,9 +1569,10 @@ mulo_status mulo_round_kernel(const mulo_ctx* ctx, const mulo_params* p, int has
   memset(&sa, 0, sizeof sa);
   *kernel = MULO_KERNEL_GENERAL;
   if (ctx->force_dense) return MULO_OK;
-  FullArgs fa;
+  FlatArgs fa;
   memset(&fa, 0, sizeof fa);
-  if (plan_full(ctx, d, has_uncond != 0, &fa)) *kernel = MULO_KERNEL_FULL;
+  bool fres;
+  if (plan_flat(ctx, d, false, &fa, &fres)) *kernel = MULO_KERNEL_FULL;
   else if (plan_rows(ctx, d, false, &ra, &nw)) *kernel = d.pool_k > 1 ? MULO_KERNEL_STREAM : MULO_KERNEL_LANE;
   else if (plan_stream(ctx, d, &sa)) *kernel = MULO_KERNEL_STREAM;
   return MULO_OK;

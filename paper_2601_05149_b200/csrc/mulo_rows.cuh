@@ -36,6 +36,8 @@
 
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "mulo_stream.cuh"
 
 namespace mulo {
@@ -321,8 +323,71 @@ __device__ __noinline__ void lane_learn(LanePredictor* prp, bool ok, int reason,
   *prp = pr;
 }
 
+// One logit as it is in memory, and its value.
+template <bool BF16>
+__device__ __forceinline__ uint32_t raw_logit(const char* row, int x) {
+  if constexpr (BF16) return __ldg(reinterpret_cast<const unsigned short*>(row) + x);
+  else return __ldg(reinterpret_cast<const uint32_t*>(row) + x);
+}
+template <bool BF16>
+__device__ __forceinline__ float wide_logit(uint32_t raw) {
+  return __uint_as_float(BF16 ? raw << 16 : raw);
+}
+
 // Double division, out of line.
 __device__ __noinline__ double rows_div(double a, double b) { return a / b; }
+
+// Eight entries of a neighbour list from `first` (a multiple of eight; entry 0 is x~ itself) on, packed; past the list's
+// end the last ones again.
+__device__ __forceinline__ uint4 pool_ids(const uint16_t* row, int pool_k, int first) {
+  if ((pool_k & 7) == 0 && ((uintptr_t)row & 15) == 0) return __ldg(reinterpret_cast<const uint4*>(row + min(first, pool_k - 8)));
+  uint32_t v[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __ldg(row + min(first + i, pool_k - 1));
+  return make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, v[4] | v[5] << 16, v[6] | v[7] << 16);
+}
+// Puts V - 1 in the place of what is no id; returns whether there was one (entry 0, x~ itself, does not count).
+__device__ __forceinline__ bool pool_clamp(uint4& v, bool from0, int V) {
+  const uint32_t top = (uint32_t)(V - 1) * 0x10001u;
+  const uint4 c = make_uint4(__vminu2(v.x, top), __vminu2(v.y, top), __vminu2(v.z, top), __vminu2(v.w, top));
+  const uint32_t diff = ((c.x ^ v.x) & (from0 ? 0xffff0000u : 0xffffffffu)) | (c.y ^ v.y) | (c.z ^ v.z) | (c.w ^ v.w);
+  v = c;
+  return diff != 0u;
+}
+// One of them.
+__device__ __forceinline__ int pool_id(const uint4& v, int i) {
+  const uint32_t w = i < 2 ? v.x : i < 4 ? v.y : i < 6 ? v.z : v.w;
+  return (int)(w >> (16 * (i & 1)) & 0xffffu);
+}
+// Their logits, in two steps: every load is asked for before one is used.  One entry after the other, that was sixteen
+// round trips to L2 instead of two: 11.5 k of the 25 k cycles that a CTA spent on a pooled row.
+template <bool BF16, bool HAS_U>
+struct PoolRaw {
+  using T = typename std::conditional<BF16, unsigned short, float>::type;
+  T c[8], u[HAS_U ? 8 : 1];
+  __device__ __forceinline__ void ask(const uint4& v, const char* rc, const char* ru) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      c[i] = __ldg(reinterpret_cast<const T*>(rc) + pool_id(v, i));
+      if constexpr (HAS_U) u[i] = __ldg(reinterpret_cast<const T*>(ru) + pool_id(v, i));
+    }
+  }
+  static __device__ __forceinline__ float wide(T v) {
+    if constexpr (BF16) return __uint_as_float((uint32_t)v << 16);
+    else return v;
+  }
+  __device__ __forceinline__ float z(int i, const DevParams& P) const {
+    float uw = 0.f;
+    if constexpr (HAS_U) uw = wide(u[i]);
+    return mix_logit(wide(c[i]), uw, HAS_U, P.cfg_scale, P.invT);
+  }
+};
+
+// Asks a neighbour list into L2 (one thread; the whole 16 bytes in it).
+__device__ __forceinline__ void pool_prefetch(const uint16_t* row, int pool_k) {
+  const uintptr_t from = ((uintptr_t)row + 15) & ~(uintptr_t)15, to = (uintptr_t)(row + pool_k) & ~(uintptr_t)15;
+  if (to > from) prefetch_l2(reinterpret_cast<const char*>(from), (uint32_t)(to - from));
+}
 
 // Warps per SM the kernel is compiled for: 16 (128 registers, four pieces in flight; eight CTAs of two warps are also
 // what the lists of V = 16384, top-k 2000 leave room for), 24 for the sampling kernel, which keeps no draft list.
@@ -696,7 +761,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     const char* const nc = row_c(nq, ng);            // (no row left: this one's first pieces again)
     const char* const nu = more ? row_u(nq, ng) : nullptr;
     // the logit of x~ in this row: asked for now, used after the first pass
-    float raw_c = 0.f, raw_u = 0.f;
+    uint32_t raw_c = 0u, raw_u = 0u;   // (as they are: a conversion here would wait for them)
     if (!SAMPLE) {
       if (is_q) {
         tok = tok_next;
@@ -704,15 +769,11 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
           if (tid == 0) atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
           tok = min(max(tok, 0), P.V - 1);
         }
+        if (POOL && tid == 0) pool_prefetch(a.nn + (size_t)tok * P.pool_k, P.pool_k);
       }
       if (warp == NW - 1) {
-        RowSrc src;
-        src.cond = rc; src.uncond = nullptr; src.s = 0.f; src.invT = 1.f; src.V = P.V; src.bf16 = BF16;
-        raw_c = load1(src, tok);
-        if (HAS_U && !is_q) {
-          src.cond = ru;
-          raw_u = load1(src, tok);
-        }
+        raw_c = raw_logit<BF16>(rc, tok);
+        if (HAS_U && !is_q) raw_u = raw_logit<BF16>(ru, tok);
       }
     }
 
@@ -754,11 +815,11 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     }
     if (!SAMPLE && warp == NW - 1) {
       // the token's own weight, in double from the same exponent as the list entries (its z against theta later)
-      raw_c = mix_logit(raw_c, raw_u, HAS_U && !is_q, P.cfg_scale, P.invT);
-      const double e = lane_exp2((double)raw_c * (double)kLog2e + (double)c0);
+      const float z = mix_logit(wide_logit<BF16>(raw_c), wide_logit<BF16>(raw_u), HAS_U && !is_q, P.cfg_scale, P.invT);
+      const double e = lane_exp2((double)z * (double)kLog2e + (double)c0);
       if (lane == 0) {
         sm.e_tok = e;
-        sm.z_tok = raw_c;
+        sm.z_tok = z;
       }
     }
     if (!SAMPLE && is_q && warp == 0 && lane < rr) {   // the uniforms of the parent's rows
@@ -992,26 +1053,40 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       };
       const Spot tok_spot = POOL ? spot_of(tok) : Spot{-1, 0, 0u};
       if constexpr (POOL) {
-        // takes the entry of a kept id out of its owner's list and sum
-        auto remove = [&](int x) {
-          const Spot sp = spot_of(x);
-          const bool o_up = ((sp.thread >> 5) & 1) == 0;
-          const uint32_t o_step = o_up ? 128u : 0u - 128u, o_tm = my + a.o_tmask + (uint32_t)sp.thread * 4u;
-          uint32_t at = my + ((uint32_t)(sp.thread >> 6) * (uint32_t)R + (o_up ? 0u : (uint32_t)(R - 1))) * 128u +
-                        (((uint32_t)sp.thread & 31u) ^ (o_up ? 0u : rot)) * 4u;
+        // takes the entries of kept ids (those with `in`) out of their owners' lists and sums, N at a time
+        auto remove = [&](auto n_tag, const int* x, const bool* in) {
+          constexpr int N = decltype(n_tag)::value;
+          uint32_t at[N], tm_at[N], last[N];
+          Spot sp[N];
+#pragma unroll
+          for (int i = 0; i < N; ++i) {
+            sp[i] = spot_of(in[i] ? x[i] : 0);
+            const bool o_up = ((sp[i].thread >> 5) & 1) == 0;
+            tm_at[i] = my + a.o_tmask + (uint32_t)sp[i].thread * 4u;
+            at[i] = my + ((uint32_t)(sp[i].thread >> 6) * (uint32_t)R + (o_up ? 0u : (uint32_t)(R - 1))) * 128u +
+                    (((uint32_t)sp[i].thread & 31u) ^ (o_up ? 0u : rot)) * 4u;
+            last[i] = 0u;
+          }
 #pragma unroll 1
-          for (int w = 0; w < sp.word; ++w) at += (uint32_t)__popc(lds_u32(o_tm + (uint32_t)(w * NT) * 4u)) * o_step;
-          const uint32_t m = lds_u32(o_tm + (uint32_t)(sp.word * NT) * 4u);
-          if (!(m & sp.bit)) return;   // (cannot be: a kept id is in the list)
-          at += (uint32_t)__popc(m & (sp.bit - 1u)) * o_step;
-          uint32_t old;   // (a list may name an id twice, or x~ itself)
-          asm volatile("atom.shared.exch.b32 %0, [%1], %2;" : "=r"(old) : "r"(at), "r"(0u) : "memory");
-          atomicAdd(&sm.adj[sp.thread], __float2ull_rz(__uint_as_float(old) * 1099511627776.0f));
+          for (int w = 0; w < n_words; ++w) {
+#pragma unroll
+            for (int i = 0; i < N; ++i) {   // entries of the words before the id's, of its own those below it
+              const uint32_t m = lds_u32(tm_at[i] + (uint32_t)(w * NT) * 4u);
+              const int n = __popc(w < sp[i].word ? m : w == sp[i].word ? m & (sp[i].bit - 1u) : 0u);
+              at[i] += (uint32_t)(sp[i].thread & 32 ? -n : n) * 128u;
+              if (w == sp[i].word) last[i] = m & sp[i].bit;
+            }
+          }
+          uint32_t old[N];   // (a list may name an id twice, or x~ itself)
+#pragma unroll
+          for (int i = 0; i < N; ++i)
+            asm volatile("atom.shared.exch.b32 %0, [%1], %2;" : "=r"(old[i]) : "r"(in[i] && last[i] ? at[i] : spill), "r"(0u) : "memory");
+#pragma unroll
+          for (int i = 0; i < N; ++i)
+            if (in[i] && last[i]) atomicAdd(&sm.adj[sp[i].thread], __float2ull_rz(__uint_as_float(old[i]) * 1099511627776.0f));
         };
-        RowSrc src;
-        src.cond = rc; src.uncond = HAS_U ? ru : nullptr; src.s = P.cfg_scale; src.invT = P.invT; src.V = P.V; src.bf16 = BF16;
-        const uint16_t* const list = a.nn + (size_t)tok * P.pool_k + 1;
-        const int nb = P.pool_k - 1;
+        const uint16_t* const list = a.nn + (size_t)tok * P.pool_k;   // (x~ first)
+        const int nb = P.pool_k;
         const double limit = P.pool_delta * Z;
         double carry = 0.0;
         sm.adj[tid] = 0ull;
@@ -1023,19 +1098,19 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
           float e[8];
           int id[8];
           double sum = 0.0;
+          {
+            uint4 ids = pool_ids(list, nb, j0);
+            if (pool_clamp(ids, j0 == 0, P.V)) atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
+            PoolRaw<BF16, HAS_U> raw;
+            raw.ask(ids, rc, ru);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) id[i] = j0 + i < nb ? (int)__ldg(list + j0 + i) : -1;
+            for (int i = 0; i < 8; ++i) id[i] = pool_id(ids, i);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            e[i] = 0.f;
-            if (id[i] >= P.V) {
-              atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
-              id[i] = P.V - 1;
-            }
-            if (id[i] >= 0) e[i] = load1(src, id[i]);
+            for (int i = 0; i < 8; ++i) e[i] = raw.z(i, P);
           }
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
+            if (j0 + i < 1 || j0 + i >= nb) id[i] = -1;
             e[i] = id[i] >= 0 && e[i] >= theta ? ex2f(fmaf(e[i], kLog2e, c0)) : 0.f;
             sum += (double)e[i];
           }
@@ -1068,20 +1143,29 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
           bad = __reduce_min_sync(kFull, bad);
           if (lane == 0) sm.pool_bad[warp] = bad;
           __syncthreads();
+          bool in[8];
           int J = nb;   // the leading run n_1 .. n_J keeps its prefix mass below delta
 #pragma unroll
           for (int w = 0; w < NW; ++w) J = min(J, sm.pool_bad[w]);
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (id[i] >= 0 && j0 + i < J) {
+          for (int i = 0; i < 8; ++i) {
+            in[i] = id[i] >= 0 && j0 + i < J;
+            if (in[i]) {
               run += (double)e[i];
               if (j0 + i == J - 1 || (j0 + i == base + NT * 8 - 1)) sm.pool_cj = run;
-              if (e[i] > 0.f) remove(id[i]);
             }
+            in[i] = in[i] && e[i] > 0.f;
+          }
+#pragma unroll
+          for (int i = 0; i < 8; i += 4)
+            if (__any_sync(kFull, in[i] || in[i + 1] || in[i + 2] || in[i + 3])) remove(std::integral_constant<int, 4>{}, id + i, in + i);
           if (J < nb) break;   // (uniform)
           __syncthreads();     // (the last tile's prefix mass before the next one's)
         }
-        if (tid == NT - 1 && e_tok > 0.0) remove(tok);   // x~ is drawn with its pooled weight, outside the lists
+        if (warp == NW - 1 && e_tok > 0.0) {
+          const bool one = lane == 0;
+          remove(std::integral_constant<int, 1>{}, &tok, &one);
+        }   // x~ is drawn with its pooled weight, outside the lists
         __syncthreads();
         mass = e_tok + sm.pool_cj;
         s_t = (float)fmax((double)s_t - (double)sm.adj[tid] * (1.0 / 1099511627776.0), 0.0);
