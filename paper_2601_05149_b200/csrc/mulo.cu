@@ -13,7 +13,7 @@
 #include "mulo_dense.cuh"
 #include "mulo_islands.cuh"
 #include "mulo_resident.cuh"
-#include "mulo_flat.cuh"
+#include "mulo_full.cuh"
 #include "mulo_rows.cuh"
 #include "mulo_stream.cuh"
 
@@ -1085,10 +1085,44 @@ static bool launch_rows(mulo_ctx* ctx, const RowsArgs& s, bool sample, int nw, s
   return nw == 2 ? launch_rows_nw<2>(ctx, s, sample, dyn, st) : launch_rows_nw<4>(ctx, s, sample, dyn, st);
 }
 
-// ---- rows without a top-k cut (mulo_flat.cuh) --------------------------------------------
+// ---- rows without a top-k cut (mulo_full.cuh, mulo_flat.cuh) ------------------------------
 static bool round_needs_q(const DevParams& d) {
   return !(d.accept_mode == MULO_ACCEPT_THRESHOLD && d.resample_mode == MULO_RESAMPLE_TARGET_ALL);
 }
+
+// Pooled rows without residual redraws, V = 256 W with W a multiple of the ids in 16 bytes, and the rows of one position
+// (draft row if q is needed, conditional, unconditional) within a CTA's shared memory.
+static size_t plan_full(const mulo_ctx* ctx, const DevParams& d, bool has_u, FullArgs* s) {
+  if (d.top_k > 0 && d.top_k < d.V) return 0;
+  if (d.pool_k <= 1 || d.resample_mode != MULO_RESAMPLE_TARGET_ALL) return 0;
+  const int esz = d.bf16 ? 2 : 4, n = 16 / esz;
+  if (d.V % (kFThreads * n) != 0) return 0;
+  const int need_q = round_needs_q(d) ? 1 : 0;
+  const size_t rows = (size_t)need_q + 1 + (has_u ? 1 : 0);
+  const size_t dyn = rows * (size_t)d.V * esz + (size_t)d.V / 8 + (size_t)kFThreads * 8;
+  if (dyn + sizeof(FullSmem) + 1024 > (size_t)ctx->smem_optin) return 0;
+  s->W = d.V / kFThreads;
+  s->need_q = need_q;
+  return dyn;
+}
+
+template <bool BF16, bool HAS_U>
+static bool launch_full_t(mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
+  auto kern = k_round_full<BF16, HAS_U>;
+  const int per_sm = ctas_per_sm(ctx, kern, kFThreads, dyn);
+  if (per_sm < 1) return false;
+  int grid = ctx->sm_count * per_sm;
+  if (grid > s.n_units) grid = s.n_units;
+  kern<<<grid, kFThreads, dyn, st>>>(s);
+  return true;
+}
+
+static bool launch_full(mulo_ctx* ctx, const FullArgs& s, size_t dyn, cudaStream_t st) {
+  const bool hu = s.uncond != nullptr;
+  if (s.P.bf16) return hu ? launch_full_t<true, true>(ctx, s, dyn, st) : launch_full_t<true, false>(ctx, s, dyn, st);
+  return hu ? launch_full_t<false, true>(ctx, s, dyn, st) : launch_full_t<false, false>(ctx, s, dyn, st);
+}
+
 
 // Fills `s` and returns the dynamic shared memory of a CTA, or 0 if these parameters are not eligible.
 static size_t plan_flat(const mulo_ctx* ctx, const DevParams& d, bool sample, FlatArgs* s, bool* res) {
@@ -1486,16 +1520,30 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
   bool fast = false;
   int fast_launches = 2;   // a fast kernel and the one that redoes the rows it left
   // Eq. 5 with every redraw from the target distribution never looks at q: no kernel reports it
-  // (the resident-row kernel does not even read the draft logits), the output is zero-filled
+  // (the kernels of rows without a cut do not even read the draft logits), the output is zero-filled
   if (!round_needs_q(a.P) && q_tok) {
     if (cudaMemsetAsync(q_tok, 0, sizeof(float) * (size_t)p->B * p->H * p->W, st) != cudaSuccess) return MULO_ERR_CUDA;
     a.q_tok = nullptr;
     q_tok = nullptr;
   }
+  FullArgs ua;
+  memset(&ua, 0, sizeof ua);
+  const size_t udyn = ctx->force_dense ? 0 : plan_full(ctx, a.P, tgt_uncond != nullptr, &ua);
+  if (udyn) {
+    ua.P = a.P;
+    ua.cond = a.cond; ua.uncond = a.uncond; ua.draft = a.draft; ua.draft_tok_lo = draft_tok_lo;
+    ua.nn = a.nn;
+    ua.p_tok = p_tok; ua.q_tok = q_tok; ua.accept_prob = accept_prob;
+    ua.flags = w.flags; ua.cand_tgt = w.cand_tgt;
+    ua.dev_status = w.status;
+    ua.n_units = p->B * p->H * p->W;
+    fast = launch_full(ctx, ua, udyn, st);
+    if (fast) fast_launches = 1;
+  }
   FlatArgs fa;
   memset(&fa, 0, sizeof fa);
   bool fres = false;
-  const size_t fdyn = ctx->force_dense ? 0 : plan_flat(ctx, a.P, false, &fa, &fres);
+  const size_t fdyn = (ctx->force_dense || fast) ? 0 : plan_flat(ctx, a.P, false, &fa, &fres);
   if (fdyn) {
     fa.cond = a.cond; fa.uncond = a.uncond; fa.draft = a.draft; fa.draft_tok_lo = draft_tok_lo;
     fa.nn = a.nn;

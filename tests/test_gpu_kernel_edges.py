@@ -1,0 +1,107 @@
+"""GPU parity at the sizes where the row kernels change: smallest and largest rows, parts of a row that are empty or end
+inside a piece, the lines between the kernels, neighbour lists that do not split evenly, rows that mislead a prediction.
+Everything against the CPU oracle; the bound on probabilities and on excused positions is the one of parity_util."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2601_05149_b200 import binding, synth
+
+import parity_util as pu
+import test_gpu_redraw as redraw
+
+pytestmark = pytest.mark.gpu
+
+EQ5 = dict(accept_mode=binding.ACCEPT_THRESHOLD, tau=1e-3, resample_mode=binding.RESAMPLE_TARGET_ALL)
+ALL = dict(resample_mode=binding.RESAMPLE_RESIDUAL_ALL)
+FLAT = synth.RoundConfig("flat", B=2, H=6, W=4, V=16384, dtype="bf16", sigma=1.0, cfg_scale=3.0, top_k=0, radius=1, seed=501)
+ROWS = synth.RoundConfig("rows", B=1, H=16, W=16, V=16384, dtype="bf16", sigma=1.0, cfg_scale=3.0, top_k=2000, radius=1, seed=601)
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    assert torch.cuda.is_available()
+    binding.lib()
+    c = binding.Context(0)
+    c.set_workspace(torch.empty(1 << 16, dtype=torch.uint8, device="cuda"))
+    yield c
+    c.close()
+
+
+def parity(ctx, cfg, batch=None, kernel=None):
+    p = binding.params_from_config(cfg)
+    ctx.ensure_workspace(p)
+    if kernel:
+        assert ctx.round_kernel(p, cfg.has_uncond) == kernel
+    batch = batch or pu.build_batch(cfg)
+    g = pu.gpu_round(ctx, cfg, batch)
+    pu.check_round(cfg, g, pu.oracle_images(cfg, batch, list(range(cfg.B))))
+    assert ctx.poll_device_status() & ~(binding.DEV_DENSE_FALLBACK | binding.DEV_ZERO_DRAFT_PROB) == 0
+
+
+@pytest.mark.parametrize("over", [
+    dict(V=8, **EQ5), dict(V=8, **ALL),                                      # one lane has ids
+    dict(V=520, dtype="f32", **EQ5), dict(V=520, dtype="f32", **ALL),       # groups without ids
+    dict(V=4096, **EQ5), dict(V=4104, **EQ5),                                # four whole pieces per thread, and one id more
+    dict(V=16384, **ALL), dict(V=16392, **ALL), dict(V=16376, temperature=0.9, **ALL),
+    dict(V=65536, H=2, **EQ5), dict(V=65536, H=2, dtype="f32", cfg_scale=0.0, **EQ5),
+    dict(V=56320, H=2, **ALL), dict(V=65528, H=2, **ALL),                    # the largest weights in shared memory; too large for it
+    dict(V=2048, H=16, W=16, r=8, **ALL),                                    # 64 rows under a draft row
+    dict(V=4096, pool_k=2, pool_delta=0.3), dict(V=4096, pool_k=2048, pool_delta=0.9), dict(V=4096, pool_k=2047, pool_delta=0.9),
+    dict(V=12296, pool_k=257, pool_delta=0.2, **EQ5), dict(V=8192, dtype="f32", pool_k=1000, pool_delta=0.0),
+], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()))
+def test_rows_without_a_cut(ctx, over):
+    cfg = dataclasses.replace(FLAT, **over)
+    parity(ctx, cfg, kernel="general" if cfg.V == 65528 else "full")
+
+
+def test_rows_without_a_cut_that_mislead_the_prediction(ctx):
+    """Consecutive rows whose maxima lie tens apart (every other one is streamed again), constant rows, and one-hot ones."""
+    for over in (EQ5, ALL, dict(pool_k=300, pool_delta=0.2)):
+        cfg = dataclasses.replace(FLAT, V=4104, cfg_scale=0.0, **over)
+        batch = pu.build_batch(cfg)
+        x = batch["cond"].view(-1, cfg.V)
+        x[0::4] += 60.0
+        x[1::4] -= 35.0
+        x[2] = 1.5
+        x[3] = -30.0
+        x[3, 7] = 30.0
+        batch["draft_lo"].view(-1, cfg.V)[1::2] += 50.0
+        pu.redraw_tokens(cfg, batch)
+        parity(ctx, cfg, batch, "full")
+
+
+@pytest.mark.parametrize("over", [
+    dict(V=1024, top_k=16), dict(V=1032, top_k=128), dict(V=2056, top_k=257, dtype="f32", cfg_scale=0.0, temperature=0.9),
+    dict(V=16384, top_k=3276), dict(V=4096, top_k=1024), dict(V=4096, top_k=1200), dict(V=4096, top_k=1900),   # two warps, four, another kernel
+    dict(V=8192, top_k=1000, pool_k=500, pool_delta=0.3), dict(V=8192, top_k=1000, pool_k=513, pool_delta=0.9),
+    dict(V=4104, top_k=500, pool_k=2048, pool_delta=0.05, dtype="f32", radius=2, resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL),
+], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()))
+def test_rows_with_a_cut(ctx, over):
+    parity(ctx, dataclasses.replace(ROWS, **over))
+
+
+@pytest.mark.parametrize("V", [16384, 16392, 49152, 49160])
+@pytest.mark.parametrize("how", ["none", "ties", "const"])
+def test_general_path_around_shared_memory(ctx, V, how):
+    """Rows in registers, in shared memory and beyond it, with masses of ties at the threshold."""
+    cfg = dataclasses.replace(ROWS, H=4, W=4, V=V, top_k=V // 8, cfg_scale=0.0 if how == "const" else 3.0, seed=701, **ALL)
+    batch = pu.build_batch(cfg)
+    for k in ("cond", "uncond", "draft_lo"):
+        if batch[k] is not None and how != "none":
+            x = torch.round(batch[k].float()) if how == "ties" else torch.zeros_like(batch[k].float())
+            batch[k] = x.to(batch[k].dtype).contiguous()
+    pu.redraw_tokens(cfg, batch)
+    ctx.set_general_path_only(True)
+    try:
+        parity(ctx, cfg, batch, "general")
+    finally:
+        ctx.set_general_path_only(False)
+
+
+@pytest.mark.parametrize("V", [16384, 16392, 49152, 65536])
+def test_redraw_around_shared_memory(ctx, V):
+    redraw.test_redraw_steps_against_oracle(ctx, dict(B=1, H=4, W=12, V=V, dtype="bf16", top_k=V // 8, cfg_scale=2.0,
+                                                      temperature=0.9, window=4, density=0.5))
