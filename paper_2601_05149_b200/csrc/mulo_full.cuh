@@ -2,11 +2,11 @@
 // its default sampling setting), when the vocabulary splits evenly over a CTA's 256 threads and the rows of one position
 // fit in shared memory.  The other rows without a cut are mulo_flat.cuh's.
 //
-// A persistent CTA owns a contiguous range of target rows, parent (low-res) cell by parent cell.  Per parent it brings the draft row into shared
-// memory once (plain bulk copies, never multicast) -- unless the decision rule never looks at q (Eq. 5), in which case the
-// draft logits are not read at all -- and then, child by child, the target position's conditional and unconditional rows.
-// Every thread owns a contiguous range of W = V / 256 ids of the resident row, so that per-thread sums are slices of the
-// ascending-id CDF:
+// A persistent CTA owns a contiguous range of target rows, parent (low-res) cell by parent cell.  Per parent it brings the
+// draft row into shared memory once (plain bulk copies, never multicast) -- unless the decision rule never looks at q
+// (Eq. 5), in which case the draft logits are not read at all -- and then, child by child, the target position's
+// conditional and unconditional rows.  Every thread owns a contiguous range of W = V / 256 ids of the resident row, so that
+// per-thread sums are slices of the ascending-id CDF:
 //
 //   softmax      one pass: a running maximum and a sum of exponentials against it per thread
 //                (the sum is rescaled on the rare occasions the maximum moves), then the block
@@ -21,6 +21,11 @@
 // The 128-bit shared loads of a warp are spread over the bank groups by starting every thread
 // at a different 16-byte piece of its range (sums do not depend on the order; the walk of a
 // draw's owner thread is in ascending id).
+//
+// Bound by instruction issue: 13.0 k warp instructions per position of V = 16384 at 0.59 per scheduler cycle, three CTAs
+// per SM.  64 x 64, 16 images, lists of 1000: 1462 us with the list read entry by entry behind the wait for each row, 64-bit
+// atomics (a loop each) and the row kept until the draw was done; 1240 us now, 1280 with these rows on mulo_flat.cuh's
+// kernel.  The next row asked into L2 meanwhile: 5 % slower.
 #pragma once
 
 #include "mulo_flat.cuh"
@@ -57,6 +62,7 @@ struct FullSmem {
   float bf[2][kFWarps];      // block maxima; consecutive reductions alternate
   uint32_t rnd[3];
   double p_tok, q_tok;       // exp(z - max) of x~ at the current position; q(x~) of the parent
+  double p_row;              // p(x~)
   double cJ;                 // pooled prefix mass c_J
   int first_bad;
   int tok;
@@ -136,12 +142,6 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
     fetch(crow, a.cond + g * (size_t)row_bytes, &sm.bar_t);
     if (HAS_U) fetch(urow, a.uncond + g * (size_t)row_bytes, &sm.bar_t);
   };
-  auto position_of = [&](int parent, int child) -> size_t {
-    const int hw = P.h * P.w;
-    const int b = parent / hw, rem = parent - b * hw, ca = rem / P.w, cc = rem - ca * P.w;
-    return (size_t)b * NN + (size_t)(ca * P.r + child / P.r) * P.W + (size_t)(cc * P.r + child % P.r);
-  };
-
   // ---- block helpers (every thread gets the result; fixed order)
   int max_call = 0;
   auto block_max_f = [&](float v) -> float {   // one barrier: consecutive calls alternate buffers
@@ -227,6 +227,9 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
 
   for (int parent = u_begin / rr; parent * rr < u_end; ++parent) {
     const int c_begin = max(0, u_begin - parent * rr), c_end = min(rr, u_end - parent * rr);
+    const int hw = P.h * P.w, b = parent / hw, cell = parent - b * hw, ca = cell / P.w, cc = cell - ca * P.w;
+    int di = c_begin / P.r, dj = c_begin - di * P.r;
+    int t = (ca * P.r + di) * P.W + cc * P.r + dj;   // the row's place in its image
     // ------------------------------------------------------------ the parent's draft row
     if (tid == 0 && !sm.abort) {
       sm.tok = checked_token(__ldg(a.draft_tok_lo + parent), V, a.dev_status);
@@ -235,7 +238,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
         mbar_expect_tx(&sm.bar_q, row_bytes);
         fetch(qrow, a.draft + (size_t)parent * row_bytes, &sm.bar_q);
       }
-      fetch_target(position_of(parent, c_begin));
+      fetch_target((size_t)b * NN + t);
     }
     __syncthreads();
     // A wait of this CTA gave up (block-uniform: raised before the last barrier, and nothing was
@@ -276,8 +279,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
     }
 
     for (int child = c_begin; child < c_end; ++child) {
-      const size_t g = position_of(parent, child);
-      const int b = (int)(g / (size_t)NN), t = (int)(g - (size_t)b * NN);
+      const size_t g = (size_t)b * NN + t;
       if (tid == 32) {
         const uint4 rnd = lane_philox(make_uint4((uint32_t)t, (uint32_t)b + P.image_offset, P.round, 0u),
                                       make_uint2(P.seed_lo, P.seed_hi));
@@ -305,7 +307,10 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
       {
         for (int x = tid; x < V / 32; x += kFThreads) bitmap[x] = 0u;
         adj[tid] = make_uint2(0u, 0u);
-        if (tid == 0) sm.first_bad = nb;
+        if (tid == 0) {
+          sm.first_bad = nb;
+          sm.p_row = sm.p_tok / Z;
+        }
         int id[8];
         bool bad_id = false;
 #pragma unroll
@@ -365,7 +370,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
         __syncthreads();
         if (J > 0) cJ = sm.cJ;
       }
-      const double p_tok = sm.p_tok / Z;
+      const double p_tok = sm.p_row;
       const double mass = p_tok + cJ;   // pooled mass P of Eq. 3
 
       // ---- the decision (Eq. 1 / Eq. 5), the same in every thread
@@ -410,7 +415,12 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
         }
       }
       __syncthreads();   // everybody is done with the resident target row
-      if (tid == 0 && child + 1 < c_end && !sm.abort) fetch_target(position_of(parent, child + 1));
+      if (++dj == P.r) {
+        dj = 0;
+        t += P.W - P.r;
+      }
+      ++t;
+      if (tid == 0 && child + 1 < c_end && !sm.abort) fetch_target((size_t)b * NN + t);
       if (owner_mask) {
         double c = __shfl_sync(kFull, bef, src);
         int pick = -1, last_pos = -1;
