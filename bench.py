@@ -37,7 +37,7 @@ UNIT = "positions/s"
 # (traffic grows in proportion to the positions, every row being read once).  An entry is removed when
 # its kernel changes, and the line then reports null until the counters have been taken again.
 TRAFFIC_BYTES_PER_POSITION = {
-    ("P4", "full"): 66598.0,   # 545.6 MB per launch of 8192 positions (algorithmic: 67,560 B; the lists come from L2)
+    ("C4", "lane"): 79690.0,   # 652.8 MB per launch of 8192 positions (algorithmic: 73,752 B)
 }
 L2_BYTES = 126 << 20
 
@@ -296,7 +296,7 @@ def run_ours(args, cfg):
     row_avg_ms = row_ms / max(1, row_n)
     achieved = alg_bytes / (row_avg_ms * 1e-3) / 1e9
     which = ctx.round_kernel(p, cfg.has_uncond)
-    kernel = {"full": "k_round_full",
+    kernel = {"full": "k_round_full (pooled, target redraws) / k_round_flat",
               "lane": "k_round_rows (+ k_verify_failed for rows that left the fast path)",
               "stream": "k_round_stream (+ k_verify_failed for rows that left the fast path)",
               "general": "k_verify_rows"}[which]

@@ -147,20 +147,19 @@ mulo_status mulo_status_of_device_flags(uint32_t flags);
 mulo_status mulo_poll_fallback_counts(mulo_ctx* ctx, void* stream, uint32_t counts[5]);
 /* Number of kernels this context has launched so far. */
 mulo_status mulo_kernel_launches(const mulo_ctx* ctx, uint64_t* count);
-/* mulo_round picks between four row kernels, mulo_sample_draft between the last two.  All
- * compute the same function; a row a fast kernel cannot handle is redone by the general routines.
- *   MULO_KERNEL_FULL     top-k off (the paper's default sampling), V a multiple of 2048 (bf16) or
- *                        1024 (fp32), the rows of one position within a CTA's shared memory (e.g.
- *                        V <= 16384 in bf16 with classifier-free guidance): rows are made resident
- *                        in shared memory and every entry is exponentiated once; with Eq. 5 and
- *                        redraws from the target distribution the draft logits are not read;
- *   MULO_KERNEL_LANE     top-k on, pooling off, V >= 1024, rows whose candidates fit the kernel's lists (k up
+/* mulo_round picks between these row kernels, mulo_sample_draft too.  All compute the same function; a row a fast kernel
+ * cannot handle is redone by the general routines.
+ *   MULO_KERNEL_FULL     top-k off (the paper's default sampling), r <= 8: every entry is exponentiated once; rows are
+ *                        streamed through registers, with their weights (pooling, residual redraws; V up to about 57000)
+ *                        or the raw rows (pooling with redraws from the target distribution) kept in shared memory; with
+ *                        Eq. 5 and redraws from the target distribution the draft logits are not read;
+ *   MULO_KERNEL_LANE     top-k on, pooling off, V >= 1024, r <= 4, rows whose candidates fit the kernel's lists (k up
  *                        to about a third of V): two or four warps per row, every thread keeps the candidates of
  *                        the ids it reads, rows are streamed once through registers;
- *   MULO_KERNEL_STREAM   top-k on, V >= 1024 (with pooling, V <= 16384), any other shape: rows
- *                        streamed once in chunks, candidates compacted per segment;
- *   MULO_KERNEL_GENERAL  everything else (top-k off, tiny vocabularies): one CTA per row, the
- *                        row read several times (from L2 after the first).
+ *   MULO_KERNEL_STREAM   the same rows with pooling (on the same kernel), and denser cuts (k up to half of V; with pooling
+ *                        V <= 16384): rows streamed once in chunks, candidates compacted per segment;
+ *   MULO_KERNEL_GENERAL  everything else (top-k on with tiny vocabularies, r beyond the limits above, ...): one CTA
+ *                        per row, the row in shared memory (V <= 49152) or read several times.
  * mulo_round_kernel reports the choice for these parameters (and with or without an unconditional
  * tensor) on this context (host arithmetic only; nothing is launched).  mulo_set_general_path_only(on != 0) makes the context always use
  * the general kernel (for testing and comparison). */

@@ -14,7 +14,7 @@
 //              row (L2, one 16-byte load per lane), the id.  The other warps are on their way with the next row.
 //
 // RES: where a row is needed again -- pooling, residual redraws -- its weights (fp32) stay in shared memory, 4 V bytes, and
-// eight warps share a row.
+// eight warps share a row (pooled rows with target redraws only: where mulo_full.cuh's kernel cannot take them).
 //
 //   pooling    (POOL, Eq. 3-4) eight entries of x~'s neighbour list per thread, their weights straight from shared memory;
 //              prefix masses by a block scan; what is pooled is set to zero there, x~'s own weight too (it is drawn apart).
@@ -22,12 +22,13 @@
 //   residual   one pass over the weights and the draft row (L2): sums of max(0, p' - q).
 //   draws      the owning group's weights, 16 ids per lane, then the owning lane's ids, one per lane.
 //
-// Bound: without RES by the loads (V = 16384 bf16 with guidance, 16384 rows, no pooling: 207 us, 5.2 TB/s); with it by
-// instruction issue and by the barriers of a row at two CTAs per SM (pooling, list of 1000: 336 us, 11.0 k warp
-// instructions per row; residual redraws: 416 us).  The kernel before this one copied the raw rows to shared memory, 64 to
-// 96 KB per position, with nothing of the next row in flight: 273, 414 and 724 us, 13.7 k warp instructions.
-// Measured and not kept: logits gathered for the pooling from L2 instead (435 us: the row is out of L2 half of the time),
-// three CTAs per SM at 80 registers (spills, which share what shared memory leaves of L1: 344 to 362 us).
+// Bound: without RES by the loads (16384 rows of V = 16384 bf16 with guidance, no pooling: 207 us, 5.2 TB/s); with it by
+// instruction issue and by the barriers of a row at two CTAs per SM (the same rows with residual redraws: 416 us; with lists
+// of 1000 too: 388 us, 12.7 k warp instructions per row and its quarter of a draft row).  The kernel before this one copied
+// the raw rows to shared memory, 64 to 96 KB per position, with nothing of the next row in flight: 273, 724 and 566 us.
+// Draft draws without a cut went to the general routines: 195 us for 4096 rows, now 35.
+// Measured and not kept: pooled logits gathered from L2 instead of shared memory (470 us: half of the time the row is out of
+// L2), three CTAs per SM at 80 registers (spills, which share what shared memory leaves of L1: 384 to 411 us).
 #pragma once
 
 #include "mulo_rows.cuh"
