@@ -37,6 +37,7 @@ UNIT = "positions/s"
 # (traffic grows in proportion to the positions, every row being read once).  An entry is removed when
 # its kernel changes, and the line then reports null until the counters have been taken again.
 TRAFFIC_BYTES_PER_POSITION = {
+    ("P4", "full"): 66730.0,   # 546.6 MB (algorithmic: 67,560 B; the lists come from L2)
     ("C4", "lane"): 79690.0,   # 652.8 MB per launch of 8192 positions (algorithmic: 73,752 B)
 }
 L2_BYTES = 126 << 20
@@ -617,7 +618,7 @@ def run_draft_io(args, cfg):
         dt = time.time() - t0
         cpu = {"value": n_img * cfg.h * cfg.w / dt, "unit": "cells/s", "cores": 1, "kind": "oracle",
                "sample": f"{n_img} of {cfg.B} images", "seconds": dt}
-    line("mulo_sample_draft", "k_round_stream<sampling mode> (+ k_sample_failed)", "cells_per_sec", cells, ms, cells * (cfg.V * esz + 4), cpu)
+    line("mulo_sample_draft", "k_round_rows<sampling mode> (+ k_sample_failed)", "cells_per_sec", cells, ms, cells * (cfg.V * esz + 4), cpu)
 
     ms = timed(lambda: ctx.mulo_downsample(p, tok_hi, tok_lo))
     cpu = None

@@ -1041,8 +1041,10 @@ static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample,
   return dyn;
 }
 
-// Two warps per row where their lists hold the candidates, else four.  Two is the faster one wherever both do: what
-// every warp of a row repeats (bin search, ranking, decision) is a third of the instructions.
+// Two warps per row where their lists hold the candidates (k / V up to about 0.13 here), else four.  Two is the faster one
+// wherever both do: what every warp of a row repeats (bin search, ranking, decision) is a third of the instructions.
+// 8192 rows of V = 16384, k / V = 0.02, 0.05, 0.1: 248, 255, 269 us with two, 273, 290, 302 with four.  Above, four against the
+// chunked kernel (mulo_stream.cuh): 315 and 585 us at 0.15, 344 and 706 at 0.3.
 static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, RowsArgs* s, int* nw) {
   for (*nw = 2; *nw <= 4; *nw += 2)
     if (const size_t dyn = plan_rows_nw(ctx, d, sample, *nw, s)) return dyn;

@@ -22,7 +22,7 @@
 // at a different 16-byte piece of its range (sums do not depend on the order; the walk of a
 // draw's owner thread is in ascending id).
 //
-// Bound by instruction issue: 13.0 k warp instructions per position of V = 16384 at 0.59 per scheduler cycle, three CTAs
+// Bound by instruction issue: 12.7 k warp instructions per position of V = 16384 at 0.58 per scheduler cycle, three CTAs
 // per SM.  64 x 64, 16 images, lists of 1000: 1462 us with the list read entry by entry behind the wait for each row, 64-bit
 // atomics (a loop each) and the row kept until the draw was done; 1240 us now, 1280 with these rows on mulo_flat.cuh's
 // kernel.  The next row asked into L2 meanwhile: 5 % slower.
