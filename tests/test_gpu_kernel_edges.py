@@ -74,6 +74,7 @@ def test_rows_without_a_cut_that_mislead_the_prediction(ctx):
 
 
 @pytest.mark.parametrize("over", [
+    dict(B=5, H=27, W=34, V=4096, top_k=512, r=1),   # one row under each draft row, several of them per thread block
     dict(V=1024, top_k=16), dict(V=1032, top_k=128), dict(V=2056, top_k=257, dtype="f32", cfg_scale=0.0, temperature=0.9),
     dict(V=16384, top_k=3276), dict(V=4096, top_k=1024), dict(V=4096, top_k=1200), dict(V=4096, top_k=1900),   # two warps, four, another kernel
     dict(V=8192, top_k=1000, pool_k=500, pool_delta=0.3), dict(V=8192, top_k=1000, pool_k=513, pool_delta=0.9),
