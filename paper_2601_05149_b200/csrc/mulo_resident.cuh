@@ -305,8 +305,10 @@ template <bool REG>
 __device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)[kResRegs], int top_k, float mx, float mean,
                                             ResScratch& rs) {
   const int lane = threadIdx.x & 31;
+  // (Finite logits may sum to -inf, or mix to it under guidance: two ids at the lowest value of the type do.  Then there
+  // is no mean, and no first histogram; sc is 0 where mx - mean is infinite.)
   const float sc = (float)(kResBins - 1) / (mx - mean);
-  if (!(mean < mx) || !(sc < 1e30f)) {   // (uniform)
+  if (!(mean < mx) || !(sc > 0.f && sc < 1e30f)) {   // (uniform)
     __syncthreads();
     return res_refine(row, top_k, 0, -3.4028235e38f, mx, rs);
   }
@@ -316,10 +318,12 @@ __device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
   };
-  const uint32_t hist = smem_u32(rs.hist) - 4u * __float_as_uint(kRMagic), spill = smem_u32(rs.spill) + (uint32_t)lane * 4u;
-  auto count = [&](float v) {   // (no branch: what lies below the first bin counts in a word of its lane)
-    const int b = bits_of(v);
-    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b >= __float_as_int(kRMagic) ? hist + 4u * (uint32_t)b : spill) : "memory");
+  const uint32_t hist = smem_u32(rs.hist), spill = smem_u32(rs.spill) + (uint32_t)lane * 4u;
+  // No branch: what lies below the first bin counts in a word of its lane.  Both ends are tested (as unsigned): no value,
+  // whatever its bits, may form an address beyond the bins.
+  auto count = [&](float v) {
+    const uint32_t b = (uint32_t)bits_of(v) - __float_as_uint(kRMagic);
+    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b < (uint32_t)kResBins ? hist + 4u * b : spill) : "memory");
   };
   const int n_mine = row.end - row.beg;
   if (REG) {

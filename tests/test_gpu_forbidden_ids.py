@@ -1,0 +1,94 @@
+"""GPU parity on rows with forbidden ids: logits at the lowest finite value of their type, in the conditional rows alone (guidance
+then takes them to -inf) or in both.  Sums over such a row overflow, so that nothing may be derived from its mean or spread
+without a check.  Everything against the CPU oracle, which sorts and exponentiates such rows like any others."""
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+import oracle as orc
+from paper_2601_05149_b200 import binding, synth
+
+import parity_util as pu
+
+pytestmark = pytest.mark.gpu
+
+ROWS = synth.RoundConfig("forbidden", B=1, H=8, W=8, V=4096, dtype="bf16", sigma=1.0, top_k=500, radius=1, seed=801,
+                         resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL)
+FEW = lambda cfg: 2
+QUARTER = lambda cfg: cfg.V // 4
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    assert torch.cuda.is_available()
+    binding.lib()
+    c = binding.Context(0)
+    c.set_workspace(torch.empty(1 << 16, dtype=torch.uint8, device="cuda"))
+    yield c
+    c.close()
+
+
+def forbid(cfg, n, both=False):
+    """A batch whose rows all forbid the same n ids; the guidance rows only if `both`."""
+    batch = synth.build_batch(cfg, "cuda")
+    ids = torch.from_numpy(np.random.default_rng(cfg.seed).permutation(cfg.V)[:n]).cuda()
+    low = torch.finfo(cfg.torch_dtype).min
+    for k in ("cond", "draft_lo") + (("uncond",) if both and cfg.has_uncond else ()):
+        batch[k][..., ids] = low
+    pu.redraw_tokens(cfg, batch)
+    return batch
+
+
+FORMS = [dict(), dict(temperature=0.7), dict(cfg_scale=3.0), dict(cfg_scale=3.0, both=True), dict(dtype="f32", V=1032, top_k=129),
+         dict(dtype="f32", V=1032, top_k=129, cfg_scale=3.0, temperature=0.9)]
+form_id = lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain"
+
+
+@pytest.mark.parametrize("how", ["stages", "general", "round"])
+@pytest.mark.parametrize("n", [FEW, QUARTER], ids=["few", "quarter"])
+@pytest.mark.parametrize("form", FORMS, ids=form_id)
+def test_rows_with_a_cut(ctx, form, n, how):
+    form = dict(form)
+    both = form.pop("both", False)
+    cfg = dataclasses.replace(ROWS, **form)
+    batch = forbid(cfg, n(cfg), both)
+    ctx.set_general_path_only(how == "general")
+    try:
+        g = pu.gpu_stages(ctx, cfg, batch) if how == "stages" else pu.gpu_round(ctx, cfg, batch)
+    finally:
+        ctx.set_general_path_only(False)
+    pu.check_round(cfg, g, pu.oracle_images(cfg, batch, [0]))
+    assert ctx.poll_device_status() & ~binding.DEV_DENSE_FALLBACK == 0
+
+
+@pytest.mark.parametrize("n", [FEW, QUARTER], ids=["few", "quarter"])
+@pytest.mark.parametrize("V", [4096, 16392])   # the row in registers, in shared memory
+@pytest.mark.parametrize("cfg_scale", [0.0, 3.0])
+def test_redraw_and_draft_draws(ctx, cfg_scale, V, n):
+    cfg = dataclasses.replace(ROWS, V=V, top_k=V // 8, cfg_scale=cfg_scale)
+    batch = forbid(cfg, n(cfg))
+    p = binding.params_from_config(cfg)
+    ctx.ensure_workspace(p)
+    for general in (False, True):
+        tok = torch.full((1, cfg.h, cfg.w), -5, dtype=torch.int32, device="cuda")
+        ctx.set_general_path_only(general)
+        try:
+            ctx.mulo_sample_draft(p, batch["draft_lo"], tok)
+        finally:
+            ctx.set_general_path_only(False)
+        want, edge = orc.sample_draft_tokens(pu.orc_params(cfg, 0), synth.to_numpy_logits(batch["draft_lo"][0]), with_edge=True)
+        assert not ((tok[0].cpu().numpy() != want) & (edge == 0)).any()
+
+    steps = np.arange(1, 65, dtype=np.int32).reshape(8, 8) % 5   # four steps, and positions that stay
+    out = torch.full((1, 8, 8), -7, dtype=torch.int32, device="cuda")
+    pos = torch.empty(64, dtype=torch.int32, device="cuda")
+    offsets = torch.empty(2 * 66, dtype=torch.int32, device="cuda")
+    ctx.mulo_redraw_plan(p, torch.from_numpy(steps).cuda(), 64, pos, offsets)
+    for s in range(1, 5):
+        ctx.mulo_redraw_step(p, s, 64, pos, offsets, batch["cond"], batch["uncond"], out)
+    cond = [synth.to_numpy_logits(batch["cond"][0])] * 4
+    unc = [synth.to_numpy_logits(batch["uncond"][0])] * 4 if cfg.has_uncond else None
+    want, _, edge = orc.redraw_loop(pu.orc_params(cfg, 0), steps, cond, unc, np.full((8, 8), -7, np.int32), with_edge=True)
+    assert not ((out[0].cpu().numpy() != want) & (edge == 0)).any()
