@@ -228,7 +228,7 @@ __device__ __forceinline__ int res_crossing(const ResScratch& rs, unsigned want,
   return (31 - src) * 32 + 31 - k;
 }
 
-// The value of rank r from the top among the entries set aside.
+// The value of rank r from the top among the n >= r entries set aside.
 __device__ __forceinline__ float res_rank(const ResScratch& rs, int n, unsigned r) {
   float th = 0.f;
   bool found = false;
@@ -250,13 +250,15 @@ __device__ __forceinline__ float res_rank(const ResScratch& rs, int n, unsigned 
   return __shfl_sync(kFull, th, __ffs(__ballot_sync(kFull, found)) - 1);   // (found: the entries hold the rank)
 }
 
-// The top_k-th largest of the row's values in [zlo, zhi], `above` being larger than zhi, by brackets that shrink by a
-// factor of 512 or more per round, in steps of the order-preserving integer keys: for rows whose first histogram did
-// not settle it (many entries in one bin, fewer than top_k above the mean).  The histogram's memory is free (all
-// threads are past a barrier since its last use) and is left so.
-__device__ __noinline__ float res_refine(const ResRow& row, int top_k, int above, float zlo, float zhi, ResScratch& rs) {
+// The top_k-th largest of the row's values, zhi being the largest, by brackets that shrink by a factor of 512 or more per
+// round, in steps of the order-preserving integer keys: for rows whose first histogram did not settle it (many entries in
+// one bin, fewer than top_k above the mean).  The first bracket goes down to -inf, which finite logits may mix to.  The
+// histogram's memory is free (all threads are past a barrier since its last use) and is left so.
+__device__ __noinline__ float res_refine(const ResRow& row, int top_k, float zhi, ResScratch& rs) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_mine = row.end - row.beg;
   const float* const z = row.run();
+  float zlo = -INFINITY;
+  int above = 0;   // values larger than zhi
   for (;;) {
     const uint32_t lo = float_key(zlo), hi = float_key(zhi);
     if (lo == hi) return zhi;
@@ -273,6 +275,10 @@ __device__ __noinline__ float res_refine(const ResRow& row, int top_k, int above
     int in_bin = 0;
     const unsigned want = (unsigned)(top_k - above);
     const int bin = res_crossing(rs, want, over, in_bin);
+    if (bin < 0) {   // (uniform; fewer than top_k values are numbers at all: nothing is cut)
+      __syncthreads();
+      return -INFINITY;
+    }
     uint32_t vhi = 0u, vlo = ~0u;
     for (int i = 0; i < n_mine; ++i) {
       const uint32_t k = float_key(z[i]);
@@ -310,7 +316,7 @@ __device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)
   const float sc = (float)(kResBins - 1) / (mx - mean);
   if (!(mean < mx) || !(sc > 0.f && sc < 1e30f)) {   // (uniform)
     __syncthreads();
-    return res_refine(row, top_k, 0, -3.4028235e38f, mx, rs);
+    return res_refine(row, top_k, mx, rs);
   }
   auto bits_of = [&](float v) -> int { return __float_as_int(fmaf(__fsub_rn(v, mean), sc, kRMagic)); };
   auto eight = [&](int i, float (&v)[8]) {   // eight of this thread's logits
@@ -344,7 +350,7 @@ __device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)
   const int bin = res_crossing(rs, (unsigned)top_k, over, in_bin);
   if (bin < 0 || in_bin > kResMembers) {   // (uniform)
     __syncthreads();
-    return res_refine(row, top_k, 0, -3.4028235e38f, mx, rs);
+    return res_refine(row, top_k, mx, rs);
   }
   const int want_bits = bin + __float_as_int(kRMagic);
   auto aside = [&](float v) { rs.sa[atomicAdd(&rs.n_sa, 1u)] = v; };

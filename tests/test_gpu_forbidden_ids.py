@@ -18,6 +18,7 @@ ROWS = synth.RoundConfig("forbidden", B=1, H=8, W=8, V=4096, dtype="bf16", sigma
                          resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL)
 FEW = lambda cfg: 2
 QUARTER = lambda cfg: cfg.V // 4
+MOST = lambda cfg: cfg.V - cfg.top_k + 1   # the top_k-th largest value is a forbidden one
 
 
 @pytest.fixture(scope="module")
@@ -47,7 +48,7 @@ form_id = lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain"
 
 
 @pytest.mark.parametrize("how", ["stages", "general", "round"])
-@pytest.mark.parametrize("n", [FEW, QUARTER], ids=["few", "quarter"])
+@pytest.mark.parametrize("n", [FEW, QUARTER, MOST], ids=["few", "quarter", "most"])
 @pytest.mark.parametrize("form", FORMS, ids=form_id)
 def test_rows_with_a_cut(ctx, form, n, how):
     form = dict(form)
@@ -63,7 +64,7 @@ def test_rows_with_a_cut(ctx, form, n, how):
     assert ctx.poll_device_status() & ~binding.DEV_DENSE_FALLBACK == 0
 
 
-@pytest.mark.parametrize("n", [FEW, QUARTER], ids=["few", "quarter"])
+@pytest.mark.parametrize("n", [FEW, QUARTER, MOST], ids=["few", "quarter", "most"])
 @pytest.mark.parametrize("V", [4096, 16392])   # the row in registers, in shared memory
 @pytest.mark.parametrize("cfg_scale", [0.0, 3.0])
 def test_redraw_and_draft_draws(ctx, cfg_scale, V, n):
