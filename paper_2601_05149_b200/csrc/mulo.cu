@@ -121,7 +121,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_upsample_pool(RowKernelArgs a) 
   }
 }
 
-// The inverse-CDF draw of uniform u from softmax(topk(row / T)); one thread writes the token to *out.
+// The inverse-CDF draw of uniform u from softmax(topk(row / T)); one thread writes the token to *out (-1: no mass, a row
+// whose largest logit mixes to +inf).
 // `before_pick` runs ahead of the last step.
 struct Nothing {
   __device__ void operator()() const {}
@@ -137,6 +138,7 @@ __device__ __forceinline__ void draw_row(const RowSrc& src, int top_k, double u,
     const ResSums sums = res_row_stats<REG>(row, src, top_k, sc, calls, -1, unused, st);
     before_pick();
     res_pick(row, sums, u, [&](int x) -> double { return (double)row.at(x); }, out);
+    if (!(sums.total > 0.0) && threadIdx.x == 0) *out = -1;
   } else {
     dense_row_stats(src, top_k, sc, st.theta, st.m, st.Z);
     __syncthreads();

@@ -415,7 +415,7 @@ __global__ void __launch_bounds__((RES ? kFlatResWarps : kFlatWarps) * 32, (SAMP
       continue;
     }
     again = false;
-    const double Z = gs.total;
+    const double Z = gs.total > 0.0 ? gs.total : (double)NAN;   // (no number, and no probability, where the largest logit is +inf)
     if (is_q) {
       ref_q = mx;
       have_q = true;
@@ -502,7 +502,7 @@ __global__ void __launch_bounds__((RES ? kFlatResWarps : kFlatWarps) * 32, (SAMP
         const uint32_t* const rnd = sm.rnd[parent & 1][di * P.r + dj];
         if (P.accept_mode == MULO_ACCEPT_THRESHOLD) accepted = mass >= P.tau * Z;
         else if (q_tok <= 0.0) accepted = mass > 0.0;
-        else accepted = uniform24(rnd[0]) * q_tok * Z < mass;
+        else accepted = !(uniform24(rnd[0]) * q_tok * Z >= mass);
         u_res = uniform24(rnd[1]);
         u_tgt = uniform24(rnd[2]);
         pending = draws_for(P.resample_mode, accepted);
@@ -575,6 +575,7 @@ __global__ void __launch_bounds__((RES ? kFlatResWarps : kFlatWarps) * 32, (SAMP
             no_mass = true;   // the same draw again, from the target weights
             continue;
           }
+          if (tid == 0) (SAMPLE ? a.sample_out : is_res ? a.cand_res : a.cand_tgt)[g] = -1;
         } else {
           const double yt = (is_res ? u_res : u_tgt) * ds.total;
           const unsigned hit_g = __ballot_sync(kFull, lane < NG && ds.inc > yt), has_g = __ballot_sync(kFull, lane < NG && ds.w > 0.0);

@@ -444,6 +444,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
         if (lane == 0) a.cand_tgt[g] = pick >= 0 ? pick : last_pos >= 0 ? last_pos : o_id0;
       }
       if (tid == 32 * (kFWarps - 1)) {
+        if (!(total > 0.0)) a.cand_tgt[g] = -1;   // (a row whose largest logit mixes to +inf)
         a.flags[g] = accepted ? 0 : 1;
         if (a.p_tok) a.p_tok[g] = (float)p_tok;
         if (a.q_tok) a.q_tok[g] = (float)q_tok;

@@ -93,3 +93,47 @@ def test_redraw_and_draft_draws(ctx, cfg_scale, V, n):
     unc = [synth.to_numpy_logits(batch["uncond"][0])] * 4 if cfg.has_uncond else None
     want, _, edge = orc.redraw_loop(pu.orc_params(cfg, 0), steps, cond, unc, np.full((8, 8), -7, np.int32), with_edge=True)
     assert not ((out[0].cpu().numpy() != want) & (edge == 0)).any()
+
+
+EQ5 = dict(accept_mode=binding.ACCEPT_THRESHOLD, tau=2.0, resample_mode=binding.RESAMPLE_TARGET_ALL)   # nothing is accepted
+
+
+@pytest.mark.parametrize("over", [
+    dict(top_k=0, **EQ5), dict(top_k=0, pool_k=50, **EQ5), dict(top_k=0, V=4104, pool_k=50, **EQ5),
+    dict(top_k=0, **{**EQ5, "resample_mode": binding.RESAMPLE_RESIDUAL_ALL}), dict(top_k=0), dict(**EQ5),
+], ids=["flat", "full", "flat-pooled", "flat-residual", "flat-eq1", "rows"])
+def test_rows_without_a_mass(ctx, over):
+    """An id forbidden in the guidance rows alone mixes to +inf and no probability is a number: every draw says -1, and no
+    token is what the workspace happened to hold."""
+    cfg = dataclasses.replace(ROWS, cfg_scale=3.0, radius=0, **over)
+    batch = pu.build_batch(cfg)
+    batch["uncond"][..., 5] = torch.finfo(cfg.torch_dtype).min
+    p = binding.params_from_config(cfg)
+    ctx.set_workspace(torch.full((ctx.workspace_bytes(p),), 7, dtype=torch.uint8, device="cuda"))
+    g = pu.gpu_round(ctx, cfg, batch)
+    pu.check_round(cfg, g, pu.oracle_images(cfg, batch, [0]))
+    if cfg.accept_mode == binding.ACCEPT_THRESHOLD:
+        assert (g["reject"] == 1).all() and (g["out_tok"] == -1).all()
+
+
+@pytest.mark.parametrize("V", [4096, 16392, 49160])
+def test_draws_without_a_mass(ctx, V):
+    cfg = dataclasses.replace(ROWS, V=V, top_k=V // 8, cfg_scale=3.0, temperature=0.7)
+    batch = synth.build_batch(dataclasses.replace(cfg, H=4, W=4), "cuda")
+    batch["uncond"][..., 5] = torch.finfo(cfg.torch_dtype).min
+    batch["draft_lo"][..., 5] = torch.finfo(cfg.torch_dtype).max
+    for top_k, general in ((0, False), (0, True), (cfg.top_k, False), (cfg.top_k, True)):
+        p = binding.params_from_config(dataclasses.replace(cfg, H=4, W=4, top_k=top_k))
+        ctx.ensure_workspace(p)
+        tok = torch.full((1, 2, 2), 7, dtype=torch.int32, device="cuda")
+        out = torch.full((1, 4, 4), 7, dtype=torch.int32, device="cuda")
+        pos = torch.empty(16, dtype=torch.int32, device="cuda")
+        offsets = torch.empty(2 * 18, dtype=torch.int32, device="cuda")
+        ctx.set_general_path_only(general)
+        try:
+            ctx.mulo_sample_draft(p, batch["draft_lo"], tok)
+        finally:
+            ctx.set_general_path_only(False)
+        ctx.mulo_redraw_plan(p, torch.ones((1, 4, 4), dtype=torch.int32, device="cuda"), 16, pos, offsets)
+        ctx.mulo_redraw_step(p, 1, 16, pos, offsets, batch["cond"], batch["uncond"], out)
+        assert (tok == -1).all() and (out == -1).all(), (top_k, general)
