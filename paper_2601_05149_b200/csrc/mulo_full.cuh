@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
     constexpr bool SCALE = decltype(scale_tag)::value;
     constexpr int NP = N / 2;   // pairs per piece
     const float2 s2 = make_float2(s, s), t2 = make_float2(P.invT, P.invT), l2 = make_float2(kLog2e, kLog2e);
-    m = -INFINITY;
+    m = -1e30f;   // (not -inf: pieces whose ids are all forbidden, at -inf under guidance, would be inf - inf)
     float2 acc = make_float2(0.f, 0.f);
     int ci = start;
 #pragma unroll 1
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
 #pragma unroll
       for (int j = 1; j < NP; ++j) cm = fmaxf(cm, fmaxf(z[j].x, z[j].y));
       if (cm > m) {
-        const float f = ex2f((m - cm) * kLog2e);   // (0 * 2^-inf = 0 on the first piece)
+        const float f = ex2f((m - cm) * kLog2e);   // (0 * 0 on the first piece)
         acc = __fmul2_rn(acc, make_float2(f, f));
         m = cm;
       }

@@ -16,6 +16,8 @@ pytestmark = pytest.mark.gpu
 
 ROWS = synth.RoundConfig("forbidden", B=1, H=8, W=8, V=4096, dtype="bf16", sigma=1.0, top_k=500, radius=1, seed=801,
                          resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL)
+EQ5 = dict(accept_mode=binding.ACCEPT_THRESHOLD, tau=1e-3, resample_mode=binding.RESAMPLE_TARGET_ALL)
+NONE = dict(EQ5, tau=2.0)   # nothing is accepted
 FEW = lambda cfg: 2
 QUARTER = lambda cfg: cfg.V // 4
 MOST = lambda cfg: cfg.V - cfg.top_k + 1   # the top_k-th largest value is a forbidden one
@@ -31,10 +33,11 @@ def ctx():
     c.close()
 
 
-def forbid(cfg, n, both=False):
-    """A batch whose rows all forbid the same n ids; the guidance rows only if `both`."""
+def forbid(cfg, n, both=False, block=False):
+    """A batch whose rows all forbid the same n ids (`block`: consecutive ones); the guidance rows only if `both`."""
     batch = synth.build_batch(cfg, "cuda")
-    ids = torch.from_numpy(np.random.default_rng(cfg.seed).permutation(cfg.V)[:n]).cuda()
+    ids = np.arange(8, 8 + n) if block else np.random.default_rng(cfg.seed).permutation(cfg.V)[:n]
+    ids = torch.from_numpy(ids).cuda()
     low = torch.finfo(cfg.torch_dtype).min
     for k in ("cond", "draft_lo") + (("uncond",) if both and cfg.has_uncond else ()):
         batch[k][..., ids] = low
@@ -62,6 +65,19 @@ def test_rows_with_a_cut(ctx, form, n, how):
         ctx.set_general_path_only(False)
     pu.check_round(cfg, g, pu.oracle_images(cfg, batch, [0]))
     assert ctx.poll_device_status() & ~binding.DEV_DENSE_FALLBACK == 0
+
+
+@pytest.mark.parametrize("block", [False, True], ids=["scattered", "block"])
+@pytest.mark.parametrize("n", [FEW, QUARTER, lambda cfg: cfg.V - 24], ids=["few", "quarter", "all-but-24"])
+@pytest.mark.parametrize("cfg_scale", [0.0, 3.0])
+@pytest.mark.parametrize("over", [
+    dict(**EQ5), dict(pool_k=100, pool_delta=0.3, **EQ5), dict(V=4104, pool_k=100, pool_delta=0.3), dict(),
+], ids=["flat", "full", "flat-pooled", "flat-residual"])
+def test_rows_without_a_cut(ctx, over, cfg_scale, n, block):
+    cfg = dataclasses.replace(ROWS, top_k=0, cfg_scale=cfg_scale, **over)
+    batch = forbid(cfg, n(cfg), block=block)
+    pu.check_round(cfg, pu.gpu_round(ctx, cfg, batch), pu.oracle_images(cfg, batch, [0]))
+    assert ctx.poll_device_status() & ~binding.DEV_ZERO_DRAFT_PROB == 0
 
 
 @pytest.mark.parametrize("n", [FEW, QUARTER, MOST], ids=["few", "quarter", "most"])
@@ -95,12 +111,9 @@ def test_redraw_and_draft_draws(ctx, cfg_scale, V, n):
     assert not ((out[0].cpu().numpy() != want) & (edge == 0)).any()
 
 
-EQ5 = dict(accept_mode=binding.ACCEPT_THRESHOLD, tau=2.0, resample_mode=binding.RESAMPLE_TARGET_ALL)   # nothing is accepted
-
-
 @pytest.mark.parametrize("over", [
-    dict(top_k=0, **EQ5), dict(top_k=0, pool_k=50, **EQ5), dict(top_k=0, V=4104, pool_k=50, **EQ5),
-    dict(top_k=0, **{**EQ5, "resample_mode": binding.RESAMPLE_RESIDUAL_ALL}), dict(top_k=0), dict(**EQ5),
+    dict(top_k=0, **NONE), dict(top_k=0, pool_k=50, **NONE), dict(top_k=0, V=4104, pool_k=50, **NONE),
+    dict(top_k=0, **{**NONE, "resample_mode": binding.RESAMPLE_RESIDUAL_ALL}), dict(top_k=0), dict(**NONE),
 ], ids=["flat", "full", "flat-pooled", "flat-residual", "flat-eq1", "rows"])
 def test_rows_without_a_mass(ctx, over):
     """An id forbidden in the guidance rows alone mixes to +inf and no probability is a number: every draw says -1, and no
