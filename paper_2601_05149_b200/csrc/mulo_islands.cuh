@@ -230,7 +230,7 @@ constexpr int kRunTerm = 1 << 15;   // more than two steps, or columns, of one i
 
 __host__ inline size_t schedule_smem(int H, int W) {
   const size_t N = (size_t)H * W, nw = (size_t)H * ((W + 31) / 32);
-  return N * 12 + 2 * nw * 4 + (size_t)H * 4;
+  return N * 12 + 2 * nw * 4 + (size_t)H * 2;   // (at most 232,000 bytes: 4000 x 4; an SM has 232,448)
 }
 
 __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleArgs a) {
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
   int* const place = reinterpret_cast<int*>(first + nw);
   // by run of the row: the island's previous run in the row (-1: none) << 16 | last column
   int* const table = place + N;
-  int* const linked = table + N;                                            // runs of a row where one has a predecessor, else 0
+  uint16_t* const linked = reinterpret_cast<uint16_t*>(table + N);          // runs of a row where one has a predecessor, else 0
   __shared__ int s_max, s_many;
   if (tid == 0) s_max = s_many = 0;
   const int32_t* const labels = a.labels + (size_t)b * N;
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
         const int l = last_of(i, last_at(first + i * Ww, j) - 1, m);
         table[i * W + r] = (l >= 0 ? run_of(i, l) : -1) << 16 | j;
         const int nr = run_of(i, W - 1) + 1;
-        if (l >= 0) linked[i] = nr;
+        if (l >= 0) linked[i] = (uint16_t)nr;
         if (nr > 32) s_many = 1;
       }
     }

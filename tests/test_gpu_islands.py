@@ -129,6 +129,22 @@ def test_schedule_random_masks(ctx, shape, window):
         schedule_both(ctx, mask, window)
 
 
+@pytest.mark.parametrize("shape", [(1, 4000, 4), (1, 3276, 5), (1, 2730, 6), (1, 4000, 3), (1, 1, 16384), (1, 8, 2048)])
+def test_schedule_of_narrow_and_wide_grids(ctx, shape):
+    """Grids of up to 16384 positions at the ends of the admitted range (4000 x 4 needs most shared memory), and labels that
+    no call of mulo_islands gives: neighbours of different labels, large and negative ones."""
+    rng = np.random.default_rng(shape[1] + shape[2])
+    for window in (1, 16):
+        schedule_both(ctx, (rng.random(shape) < 0.6).astype(np.uint8), window)
+    labels = rng.choice(np.array([0, 1, 2, 3, 1_000_000, -4], np.int32), shape)
+    step = torch.full(shape, -7, dtype=torch.int32, device="cuda")
+    n = torch.full((1,), -7, dtype=torch.int32, device="cuda")
+    ctx.mulo_island_schedule(binding.make_params(*shape, 8, 1, binding.F32), torch.from_numpy(labels).cuda(), 3, step, n)
+    want, nfe = oracle.island_schedule(labels[0], 3)
+    np.testing.assert_array_equal(step[0].cpu().numpy(), want)
+    assert n[0] == nfe
+
+
 def test_schedule_closed_forms(ctx):
     H, W = 32, 48
     mask = np.zeros((3, H, W), np.uint8)
