@@ -380,7 +380,9 @@ __device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)
 }
 
 // Logits -> weights in place; returns the scan of the threads' sums (total = partition sum).  With a threshold most
-// entries are zero: a thread marks those it keeps and exponentiates only them.
+// entries are zero: a thread marks those it keeps and exponentiates only them.  Every weight goes into a double by itself:
+// partial sums in fp32, even of eight, show in Z (relative error of Z_q, 512 draft rows of 264 to 49152 ids: at most 3.3e-8 so,
+// 1.8e-7 with them).
 __device__ __forceinline__ ResSums res_weigh(const ResRow& row, float theta, float m, ResScratch& rs, int& calls) {
   float* const z = row.run();
   const int n = row.end - row.beg;
@@ -403,15 +405,13 @@ __device__ __forceinline__ ResSums res_weigh(const ResRow& row, float theta, flo
           else a.w = 0.f;
           *reinterpret_cast<float4*>(z + i0 + i) = a;
         }
-      float s = 0.f;
 #pragma unroll 1
       for (; keep; keep &= keep - 1u) {
         float* const p = z + i0 + __ffs(keep) - 1;
         const float e = expf(__fsub_rn(*p, m));
         *p = e;
-        s += e;
+        acc += (double)e;
       }
-      acc += (double)s;
     }
   } else {
 #pragma unroll 1
@@ -421,7 +421,7 @@ __device__ __forceinline__ ResSums res_weigh(const ResRow& row, float theta, flo
       b = make_float4(expf(__fsub_rn(b.x, m)), expf(__fsub_rn(b.y, m)), expf(__fsub_rn(b.z, m)), expf(__fsub_rn(b.w, m)));
       *reinterpret_cast<float4*>(z + i) = a;
       *reinterpret_cast<float4*>(z + i + 4) = b;
-      acc += (double)(((a.x + a.y) + (a.z + a.w)) + ((b.x + b.y) + (b.z + b.w)));
+      acc += (((double)a.x + (double)a.y) + ((double)a.z + (double)a.w)) + (((double)b.x + (double)b.y) + ((double)b.z + (double)b.w));
     }
   }
   return res_scan(acc, rs, calls);
@@ -574,7 +574,7 @@ __device__ inline void res_position(const DevParams& P, const ResRow& row, const
       double acc = 0.0;
       for (int i = 0; i < row.end - row.beg; i += 4) {
         const float4 a = *reinterpret_cast<const float4*>(w + i);
-        acc += (double)((a.x + a.y) + (a.z + a.w));
+        acc += ((double)a.x + (double)a.y) + ((double)a.z + (double)a.w);
       }
       if (own_tok) acc += mass * sp.Z - (double)row.at(tok);
       sums = res_scan(fmax(acc, 0.0), rs, calls);
@@ -598,13 +598,11 @@ __device__ inline void res_position(const DevParams& P, const ResRow& row, const
       load8(qr, x, zq);
       const float4 a = *reinterpret_cast<const float4*>(w + x - row.beg), b = *reinterpret_cast<const float4*>(w + x - row.beg + 4);
       const float e[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-      float s = 0.f;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const float q = prob_f(zq[j], sq.theta, sq.m, invZq);
-        s += x + j == tok ? 0.f : fmaxf(__fsub_rn(__fmul_rn(e[j], invZp), q), 0.f);
+        acc += x + j == tok ? 0.0 : (double)fmaxf(__fsub_rn(__fmul_rn(e[j], invZp), q), 0.f);
       }
-      acc += (double)s;
     }
     if (own_tok) acc += fmax(0.0, mass - q_tok);
     const ResSums r = res_scan(acc, rs, calls);
