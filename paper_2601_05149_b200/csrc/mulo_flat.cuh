@@ -377,9 +377,9 @@ __global__ void __launch_bounds__((RES ? kFlatResWarps : kFlatWarps) * 32, (SAMP
       if (lane == 0) sm.wmax[call & 1][warp] = mk;
     }
     if (!SAMPLE && warp == NW - 1) {
-      // the token's own weight, in double from the same exponent as the others
+      // the token's own weight
       const float z = mix_logit(wide_logit<BF16>(raw_c), wide_logit<BF16>(raw_u), HAS_U && !is_q, P.cfg_scale, P.invT);
-      const double e = lane_exp2((double)z * (double)kLog2e + (double)c0);
+      const double e = token_weight(z, ref, c0);
       if (lane == 0) sm.e_tok[call & 1] = e;
     }
     if (warp == 0 && first) {   // the uniforms of the parent's rows (the cell's)
