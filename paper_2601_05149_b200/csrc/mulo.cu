@@ -1622,10 +1622,12 @@ mulo_status mulo_round_kernel(const mulo_ctx* ctx, const mulo_params* p, int has
   memset(&sa, 0, sizeof sa);
   *kernel = MULO_KERNEL_GENERAL;
   if (ctx->force_dense) return MULO_OK;
+  FullArgs ua;
   FlatArgs fa;
+  memset(&ua, 0, sizeof ua);
   memset(&fa, 0, sizeof fa);
   bool fres;
-  if (plan_flat(ctx, d, false, &fa, &fres)) *kernel = MULO_KERNEL_FULL;
+  if (plan_full(ctx, d, has_uncond != 0, &ua) || plan_flat(ctx, d, false, &fa, &fres)) *kernel = MULO_KERNEL_FULL;
   else if (plan_rows(ctx, d, false, &ra, &nw)) *kernel = d.pool_k > 1 ? MULO_KERNEL_STREAM : MULO_KERNEL_LANE;
   else if (plan_stream(ctx, d, &sa)) *kernel = MULO_KERNEL_STREAM;
   return MULO_OK;

@@ -57,6 +57,13 @@ def test_rows_without_a_cut(ctx, over):
     parity(ctx, cfg, kernel="general" if cfg.V == 65528 else "full")
 
 
+@pytest.mark.parametrize("V,cfg_scale,kernel", [(57344, 0.0, "full"), (65536, 0.0, "full"), (65528, 0.0, "general"), (65536, 3.0, "general")])
+def test_pooled_rows_of_large_vocabularies(ctx, V, cfg_scale, kernel):
+    """Weights of so many ids do not fit in shared memory, a raw bf16 row without guidance does."""
+    cfg = dataclasses.replace(FLAT, V=V, H=2, cfg_scale=cfg_scale, pool_k=64, pool_delta=0.2, **EQ5)
+    parity(ctx, cfg, kernel=kernel)
+
+
 def test_rows_without_a_cut_that_mislead_the_prediction(ctx):
     """Consecutive rows whose maxima lie tens apart (every other one is streamed again), constant rows, and one-hot ones."""
     for over in (EQ5, ALL, dict(pool_k=300, pool_delta=0.2)):
