@@ -80,15 +80,22 @@ def test_rows_without_a_cut_that_mislead_the_prediction(ctx):
         parity(ctx, cfg, batch, "full")
 
 
-@pytest.mark.parametrize("over", [
-    dict(B=5, H=27, W=34, V=4096, top_k=512, r=1),   # one row under each draft row, several of them per thread block
-    dict(V=1024, top_k=16), dict(V=1032, top_k=128), dict(V=2056, top_k=257, dtype="f32", cfg_scale=0.0, temperature=0.9),
-    dict(V=16384, top_k=3276), dict(V=4096, top_k=1024), dict(V=4096, top_k=1200), dict(V=4096, top_k=1900),   # two warps, four, another kernel
-    dict(V=8192, top_k=1000, pool_k=500, pool_delta=0.3), dict(V=8192, top_k=1000, pool_k=513, pool_delta=0.9),
-    dict(V=4104, top_k=500, pool_k=2048, pool_delta=0.05, dtype="f32", radius=2, resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL),
-], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()))
-def test_rows_with_a_cut(ctx, over):
-    parity(ctx, dataclasses.replace(ROWS, **over))
+@pytest.mark.parametrize("over,kernel", [
+    (dict(B=5, H=27, W=34, V=4096, top_k=512, r=1), "lane"),   # one row under each draft row, several of them per thread block
+    (dict(V=1024, top_k=16), "lane"), (dict(V=1032, top_k=128), "lane"),
+    (dict(V=2056, top_k=257, dtype="f32", cfg_scale=0.0, temperature=0.9), "lane"),
+    (dict(V=16384, top_k=3276), "lane"), (dict(V=4096, top_k=1024), "lane"), (dict(V=4096, top_k=1200), "lane"),   # two warps, four
+    (dict(V=49152, top_k=6144, H=4, W=8), "stream"), (dict(V=4096, top_k=1900), "general"),   # lists too long for it; half of the row
+    (dict(V=8192, top_k=1000, pool_k=500, pool_delta=0.3), "stream"), (dict(V=8192, top_k=1000, pool_k=513, pool_delta=0.9), "stream"),
+    (dict(V=4104, top_k=500, pool_k=2048, pool_delta=0.05, dtype="f32", radius=2, resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL),
+     "stream"),
+], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) if isinstance(o, dict) else o)
+def test_rows_with_a_cut(ctx, over, kernel):
+    cfg = dataclasses.replace(ROWS, **over)
+    ctx.poll_fallback_counts()
+    parity(ctx, cfg, kernel=kernel)
+    # (the kernel did its rows itself: what it hands to the general routines is the exception)
+    assert ctx.poll_fallback_counts()[0] <= cfg.B * cfg.H * cfg.W // 20
 
 
 @pytest.mark.parametrize("V", [16384, 16392, 49152, 49160])

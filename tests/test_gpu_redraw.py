@@ -108,3 +108,79 @@ def test_redraw_arguments_are_checked(ctx):
         with pytest.raises(binding.MuloError) as e:
             ctx.mulo_redraw_step(p, s, 64, t, off, logits, None, t)
         assert e.value.status == binding.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("V", [512, 16392, 49160])   # the row in registers, in shared memory, beyond it
+@pytest.mark.parametrize("captured", [False, True], ids=["stream", "graph"])
+def test_logits_and_plan_are_rewritten_between_steps(ctx, captured, V):
+    """What a host with a model does: one logits buffer that every step's model call writes anew, one pair of plan buffers that the
+    next round's plan overwrites while the last steps may still run -- on one stream without a wait, and as one graph.  Steps are
+    launched ahead of their predecessors' end, so each must see what was written just before it."""
+    B, H, W = 2, 6, 10
+    rng = np.random.default_rng(V)
+    cfg = synth.RoundConfig("rewritten", B=B, H=H, W=W, V=V, r=1, dtype="bf16", top_k=V // 8, cfg_scale=2.0, seed=77, round=1)
+    plans = [_schedule(rng, B, H, W, 3, density) for density in (0.10, 0.25)]
+    n_steps = [int(s.max()) for s in plans]
+    g = torch.Generator(device="cuda").manual_seed(V)
+    cond = [(2.0 * torch.randn((B, H, W, V), generator=g, device="cuda")).bfloat16() for _ in range(sum(n_steps))]
+    unc = [(c.float() + torch.randn((B, H, W, V), generator=g, device="cuda")).bfloat16() for c in cond]
+    start = torch.from_numpy(rng.integers(0, V, (B, H, W)).astype(np.int32)).cuda()
+    d_plans = [torch.from_numpy(s).cuda() for s in plans]
+    p = binding.params_from_config(cfg)
+    buf_c, buf_u = torch.empty_like(cond[0]), torch.empty_like(cond[0])
+    pos_list = torch.empty(B * H * W, dtype=torch.int32, device="cuda")
+    offsets = torch.empty(2 * (H * W + 2), dtype=torch.int32, device="cuda")
+    out = torch.empty_like(start)
+
+    def rounds():
+        out.copy_(start)
+        at = 0
+        for d_step, n in zip(d_plans, n_steps):
+            ctx.mulo_redraw_plan(p, d_step, H * W, pos_list, offsets)
+            for s in range(1, n + 1):
+                buf_c.copy_(cond[at])
+                buf_u.copy_(unc[at])
+                at += 1
+                ctx.mulo_redraw_step(p, s, H * W, pos_list, offsets, buf_c, buf_u, out)
+
+    if captured:
+        rounds()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            rounds()
+        for t in (buf_c, buf_u, pos_list, offsets, out):
+            t.zero_()
+        graph.replay()
+        graph.replay()
+    else:
+        rounds()
+    torch.cuda.synchronize()
+    got = out.cpu().numpy()
+    for b in range(B):
+        tok, edge, at = start[b].cpu().numpy(), np.zeros((H, W), bool), 0
+        for steps, n in zip(plans, n_steps):
+            tok, _, e = orc.redraw_loop(pu.orc_params(cfg, b), steps[b], [synth.to_numpy_logits(c[b]) for c in cond[at:at + n]],
+                                        [synth.to_numpy_logits(u[b]) for u in unc[at:at + n]], tok, with_edge=True)
+            edge |= e != 0
+            at += n
+        bad = got[b] != tok
+        assert not (bad & ~edge).any(), np.argwhere(bad & ~edge)[:5]
+        assert bad.sum() <= 1
+
+
+def test_a_step_of_more_positions_than_thread_blocks(ctx):
+    B, H, W, V = 3, 16, 24, 264
+    cfg = synth.RoundConfig("many", B=B, H=H, W=W, V=V, r=1, dtype="f32", top_k=40, cfg_scale=0.0, seed=78)
+    cond = synth.build_batch(cfg, "cuda")["cond"]
+    steps = np.ones((B, H, W), np.int32)
+    p = binding.params_from_config(cfg)
+    pos_list = torch.empty(B * H * W, dtype=torch.int32, device="cuda")
+    offsets = torch.empty(2 * 3, dtype=torch.int32, device="cuda")
+    out = torch.full((B, H, W), -7, dtype=torch.int32, device="cuda")
+    ctx.mulo_redraw_plan(p, torch.from_numpy(steps).cuda(), 1, pos_list, offsets)
+    ctx.mulo_redraw_step(p, 1, 1, pos_list, offsets, cond, None, out)
+    for b in range(B):
+        want, _, edge = orc.redraw_loop(pu.orc_params(cfg, b), steps[b], [synth.to_numpy_logits(cond[b])], None,
+                                        np.zeros((H, W), np.int32), with_edge=True)
+        assert not ((out[b].cpu().numpy() != want) & (edge == 0)).any()
