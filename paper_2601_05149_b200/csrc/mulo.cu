@@ -4,6 +4,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 #include <new>
 #include <type_traits>
@@ -656,7 +657,11 @@ struct mulo_ctx {
   size_t ev_used;
   int force_dense;               // diagnostics: never take the fast top-k path
   struct Ready { const void* kernel; size_t dyn; int per_sm; };
-  std::vector<Ready> ready;      // kernels whose shared-memory cap is raised, and the CTAs of them an SM holds
+  // Kernels whose shared-memory cap is raised, and the CTAs of them an SM holds.  A fixed table (nothing on the way to a
+  // launch may throw) whose entries stay as they are once counted: calls from several threads read it without a lock.
+  Ready ready[64];
+  std::atomic<int> n_ready;
+  std::mutex ready_mutex;        // for adding an entry
 };
 
 static const size_t kStatusBytes = 256;
@@ -778,6 +783,7 @@ mulo_status mulo_create(mulo_ctx** out, int device) {
   c->launches = 0;
   c->ev_used = 0;
   c->force_dense = 0;
+  c->n_ready = 0;
   *out = c;
   return MULO_OK;
 }
@@ -896,8 +902,9 @@ static size_t general_smem(const DevParams& d, bool pooling) {
 template <class K>
 static int ctas_per_sm(mulo_ctx* ctx, K kernel, int threads, size_t dyn) {
   const void* const key = (const void*)kernel;
-  for (const mulo_ctx::Ready& r : ctx->ready)
-    if (r.kernel == key && r.dyn == dyn) return r.per_sm;
+  const int n = ctx->n_ready.load(std::memory_order_acquire);
+  for (int i = 0; i < n; ++i)
+    if (ctx->ready[i].kernel == key && ctx->ready[i].dyn == dyn) return ctx->ready[i].per_sm;
   cudaFuncAttributes fa;
   int per_sm = 0;
   if (cudaFuncGetAttributes(&fa, key) != cudaSuccess || dyn + fa.sharedSizeBytes > (size_t)ctx->smem_optin ||
@@ -906,8 +913,12 @@ static int ctas_per_sm(mulo_ctx* ctx, K kernel, int threads, size_t dyn) {
     cudaGetLastError();
     return 0;
   }
-  if (ctx->ready.size() >= 64) ctx->ready.clear();
-  ctx->ready.push_back({key, dyn, per_sm});
+  std::lock_guard<std::mutex> lock(ctx->ready_mutex);
+  const int at = ctx->n_ready.load(std::memory_order_relaxed);
+  if (at < (int)(sizeof ctx->ready / sizeof ctx->ready[0])) {   // (full: asked again on each call)
+    ctx->ready[at] = {key, dyn, per_sm};
+    ctx->n_ready.store(at + 1, std::memory_order_release);
+  }
   return per_sm;
 }
 

@@ -184,3 +184,47 @@ def test_a_step_of_more_positions_than_thread_blocks(ctx):
         want, _, edge = orc.redraw_loop(pu.orc_params(cfg, b), steps[b], [synth.to_numpy_logits(cond[b])], None,
                                         np.zeros((H, W), np.int32), with_edge=True)
         assert not ((out[b].cpu().numpy() != want) & (edge == 0)).any()
+
+
+def test_one_context_from_several_threads():
+    """Calls that need no workspace, from four threads on one new context, each on its own stream and over its own sizes (every one
+    asks for its kernels' limits anew): the tokens and steps are those of one thread."""
+    import concurrent.futures as cf
+    rng = np.random.default_rng(5)
+    jobs = []
+    for k in range(4):
+        per = []
+        for V in (256 + 1024 * k, 4104 + 4096 * k, 20000 + 4000 * k):
+            H, W = 6 + k, 9
+            labels = torch.from_numpy(orc.islands((rng.random((H, W)) < 0.5).astype(np.uint8))[0][None]).cuda()
+            cfg = synth.RoundConfig("threads", B=1, H=H, W=W, V=V, r=1, dtype="bf16", top_k=V // 8, seed=k)
+            per.append((cfg, labels, synth.build_batch(cfg, "cuda")["cond"]))
+        jobs.append(per)
+
+    def work(ctx, per, stream):
+        res = []
+        with torch.cuda.stream(stream):
+            for cfg, labels, cond in per:
+                p = binding.params_from_config(cfg)
+                n = cfg.H * cfg.W
+                step, out = torch.empty_like(labels), torch.zeros_like(labels)
+                n_steps = torch.empty(1, dtype=torch.int32, device="cuda")
+                pos, off = torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(2 * (n + 2), dtype=torch.int32, device="cuda")
+                ctx.mulo_island_schedule(p, labels, 3, step, n_steps)
+                ctx.mulo_redraw_plan(p, step, n, pos, off)
+                for s in range(1, 9):
+                    ctx.mulo_redraw_step(p, s, n, pos, off, cond, None, out)
+                res += [step.cpu().numpy(), out.cpu().numpy()]
+        return res
+
+    torch.cuda.synchronize()
+    alone = binding.Context(0)
+    want = [work(alone, per, torch.cuda.Stream()) for per in jobs]
+    shared = binding.Context(0)
+    with cf.ThreadPoolExecutor(4) as ex:
+        got = list(ex.map(lambda per: work(shared, per, torch.cuda.Stream()), jobs))
+    for a, b in zip(want, got):
+        for x, y in zip(a, b):
+            np.testing.assert_array_equal(x, y)
+    alone.close()
+    shared.close()
