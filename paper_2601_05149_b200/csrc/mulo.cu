@@ -1160,8 +1160,10 @@ static size_t plan_flat(const mulo_ctx* ctx, const DevParams& d, bool sample, Fl
 template <bool BF16, bool HAS_U, bool SAMPLE, bool POOL, bool RES>
 static bool launch_flat_p(mulo_ctx* ctx, const FlatArgs& s, size_t dyn, cudaStream_t st) {
   constexpr int nw = RES ? kFlatResWarps : kFlatWarps;
-  const bool plain = s.P.invT == 1.0f && s.row_bytes % (16u * kRPieceBytes * nw) == 0;
-  auto kern = plain ? k_round_flat<BF16, HAS_U, SAMPLE, POOL, RES, true> : k_round_flat<BF16, HAS_U, SAMPLE, POOL, RES, false>;
+  const bool even = s.row_bytes % (16u * kRPieceBytes * nw) == 0;
+  auto kern = !even ? k_round_flat<BF16, HAS_U, SAMPLE, POOL, RES, false, true>
+              : s.P.invT != 1.0f ? k_round_flat<BF16, HAS_U, SAMPLE, POOL, RES, true, true>
+                                 : k_round_flat<BF16, HAS_U, SAMPLE, POOL, RES, true, false>;
   const int per_sm = ctas_per_sm(ctx, kern, nw * 32, dyn);
   if (per_sm < 1) return false;
   int grid = ctx->sm_count * per_sm;

@@ -46,6 +46,8 @@ def parity(ctx, cfg, batch=None, kernel=None):
     dict(V=520, dtype="f32", **EQ5), dict(V=520, dtype="f32", **ALL),       # groups without ids
     dict(V=4096, **EQ5), dict(V=4104, **EQ5),                                # four whole pieces per thread, and one id more
     dict(V=16384, **ALL), dict(V=16392, **ALL), dict(V=16376, temperature=0.9, **ALL),
+    dict(V=16384, temperature=0.9, **EQ5), dict(V=16384, temperature=0.9, **ALL), dict(V=4096, dtype="f32", temperature=1.3, **ALL),   # even, scaled
+    dict(V=8192, temperature=0.9, pool_k=300, pool_delta=0.2),
     dict(V=65536, H=2, **EQ5), dict(V=65536, H=2, dtype="f32", cfg_scale=0.0, **EQ5),
     dict(V=56320, H=2, **ALL), dict(V=65528, H=2, **ALL),                    # the largest weights in shared memory; too large for it
     dict(V=2048, H=16, W=16, r=8, **ALL),                                    # 64 rows under a draft row
