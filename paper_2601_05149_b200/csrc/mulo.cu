@@ -1046,9 +1046,6 @@ static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample,
   s->R = (int)ceil(fmax(rows_for(k + margin, 2.0, 3.6), rows_for(k + margin_boot, 2.0, 3.0))) + 1 + kRSlack;
   if (s->R < 32) s->R = 32;
   s->margin = margin;
-  s->a_theta = (float)inv_norm_cdf(1.0 - p);
-  s->a_boot = (float)inv_norm_cdf(1.0 - (double)(k + margin_boot) / V);
-  s->a_max = (float)inv_norm_cdf(1.0 - 0.5 / V);
   const size_t dyn = rows_layout(*s, nw, d.bf16, sample);
   if (2 * (dyn + sizeof(RowsSmem<4, true>) + 1024) > (size_t)ctx->smem_optin) return 0;   // too few rows in flight per SM
   return dyn;
@@ -1058,10 +1055,26 @@ static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample,
 // wherever both do: what every warp of a row repeats (bin search, ranking, decision) is a third of the instructions.
 // 8192 rows of V = 16384, k / V = 0.02, 0.05, 0.1: 248, 255, 269 us with two, 273, 290, 302 with four.  Above, four against the
 // chunked kernel (mulo_stream.cuh): 315 and 585 us at 0.15, 344 and 706 at 0.3.
+// ... unless the lists of a two-warp CTA (fp32: those of the draft row are twice as long in bytes) leave room for fewer than
+// seven of them per SM.  4608 rows, guidance, k = V / 8: V = 16384 fp32 (five) 279 us with two, 210 with four; 12288 fp32 (six)
+// 6 to 22 % for four; 16384 bf16 (seven) 5 % for two, 8192 fp32 (eight) 10 % for two.
 static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, RowsArgs* s, int* nw) {
-  for (*nw = 2; *nw <= 4; *nw += 2)
-    if (const size_t dyn = plan_rows_nw(ctx, d, sample, *nw, s)) return dyn;
-  return 0;
+  *nw = 2;
+  size_t dyn = plan_rows_nw(ctx, d, sample, 2, s);
+  if (!dyn || (!sample && 7 * (dyn + sizeof(RowsSmem<2, false>) + 1024) > (size_t)ctx->smem_optin + 1024)) {
+    RowsArgs four = *s;
+    if (const size_t dyn4 = plan_rows_nw(ctx, d, sample, 4, &four)) {
+      *s = four;
+      *nw = 4;
+      dyn = dyn4;
+    }
+  }
+  if (!dyn) return 0;
+  const int k_boot = d.top_k + s->margin + 3 * s->margin / 4;
+  s->a_theta = (float)inv_norm_cdf(1.0 - (double)d.top_k / d.V);
+  s->a_boot = (float)inv_norm_cdf(1.0 - (double)k_boot / d.V);
+  s->a_max = (float)inv_norm_cdf(1.0 - 0.5 / d.V);
+  return dyn;
 }
 
 template <bool BF16, bool HAS_U, bool SAMPLE, bool POOL, bool PLAIN, int NW>

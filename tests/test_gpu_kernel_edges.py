@@ -87,6 +87,8 @@ def test_rows_without_a_cut_that_mislead_the_prediction(ctx):
     (dict(V=1024, top_k=16), "lane"), (dict(V=1032, top_k=128), "lane"),
     (dict(V=2056, top_k=257, dtype="f32", cfg_scale=0.0, temperature=0.9), "lane"),
     (dict(V=16384, top_k=3276), "lane"), (dict(V=4096, top_k=1024), "lane"), (dict(V=4096, top_k=1200), "lane"),   # two warps, four
+    (dict(V=16384, top_k=2048, dtype="f32"), "lane"), (dict(V=16384, top_k=1024, dtype="f32"), "lane"),   # four again, for their lists' bytes; two
+    (dict(V=16384, top_k=2048, dtype="f32", pool_k=300, pool_delta=0.3), "stream"),
     (dict(V=49152, top_k=6144, H=4, W=8), "stream"), (dict(V=4096, top_k=1900), "general"),   # lists too long for it; half of the row
     (dict(V=8192, top_k=1000, pool_k=500, pool_delta=0.3), "stream"), (dict(V=8192, top_k=1000, pool_k=513, pool_delta=0.9), "stream"),
     (dict(V=4104, top_k=500, pool_k=2048, pool_delta=0.05, dtype="f32", radius=2, resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL),
