@@ -1356,11 +1356,21 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
     fa.n_units = p->B * a.P.h * a.P.w;
     if (launch_flat(ctx, fa, true, fres, fdyn, st)) return launched(ctx, 1);
   }
+  // With one, few rows go to the chunked kernel, whose eight warps bring a row through sooner: up to four per SM for 4096 ids
+  // (64, 576, 1024 cells with k = V / 8: 24, 25, 35 us there, 28, 28, 31 us with two warps per row), three for 8192, two for more
+  // (16384 ids, 256, 400, 576 cells: 31, 38, 59 us, 39, 42, 43 us); above 16384 ids only short lists, k up to V / 25 (32768 ids,
+  // 64 cells, k = V / 8: 50 us there, 15 us).
   Workspace w;
+  const bool listed = !ctx->force_dense && check_ws(ctx, p, &w) == MULO_OK;   // (there is room for the list)
+  StreamArgs sa;
+  memset(&sa, 0, sizeof sa);
+  const int V = a.P.V, per_sm = V <= 4096 ? 4 : V <= 8192 ? 3 : 2;
+  const bool few = p->B * a.P.h * a.P.w <= per_sm * ctx->sm_count && (V <= 16384 || a.P.top_k <= V / 25);
+  size_t sdyn = listed && few ? plan_stream(ctx, a.P, &sa) : 0;
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
   int rnw = 0;
-  const size_t rdyn = (ctx->force_dense || check_ws(ctx, p, &w) != MULO_OK) ? 0 : plan_rows(ctx, a.P, true, &ra, &rnw);
+  const size_t rdyn = listed && !sdyn ? plan_rows(ctx, a.P, true, &ra, &rnw) : 0;
   if (rdyn) {
     ra.P = a.P;
     ra.cond = a.draft;
@@ -1374,9 +1384,7 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
       return launched(ctx, 2);
     }
   }
-  StreamArgs sa;
-  memset(&sa, 0, sizeof sa);
-  const size_t sdyn = (ctx->force_dense || check_ws(ctx, p, &w) != MULO_OK) ? 0 : plan_stream(ctx, a.P, &sa);
+  if (listed && !sdyn) sdyn = plan_stream(ctx, a.P, &sa);
   if (sdyn) {
     sa.P = a.P;
     sa.draft = a.draft;

@@ -86,6 +86,19 @@ def test_sample_draft_fast_path(ctx, cfg):
         ctx.set_general_path_only(False)
 
 
+@pytest.mark.parametrize("more", [False, True], ids=["few", "many"])   # four, three, two cells per SM, and one row of cells more
+@pytest.mark.parametrize("over,cells", [
+    (dict(V=1032, top_k=129), 592), (dict(V=4096, dtype="bf16", top_k=500, temperature=0.8), 592), (dict(V=8192, top_k=1000), 444),
+    (dict(V=16384, dtype="bf16", top_k=2000), 296), (dict(V=32768, top_k=600), 296), (dict(V=32768, dtype="bf16", top_k=4000), 16),
+], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) if isinstance(o, dict) else str(o))
+def test_sample_draft_on_either_side_of_the_line(ctx, over, cells, more):
+    cfg = dataclasses.replace(TINY, B=1, H=cells // 4 + more, W=4, r=1, seed=335, **over)
+    ctx.ensure_workspace(binding.params_from_config(cfg))
+    ctx.poll_fallback_counts()
+    sample_both(ctx, cfg)
+    assert ctx.poll_fallback_counts()[0] <= max(1, cells // 20)
+
+
 def test_sample_draft_fast_path_rows_that_are_not_normal(ctx):
     """Heavy-tailed rows defeat the pivot prediction now and then: those cells go through the list."""
     cfg = dataclasses.replace(TINY, B=2, H=32, W=32, V=4096, dtype="f32", top_k=400, seed=334)
