@@ -57,55 +57,53 @@ struct RowSrc {          // one vocabulary row in global memory
   int bf16;
 };
 
-// 16 bytes of a row: through the read-only cache, or (ONCE: a row that is read once, or that another kernel may have
-// written since this one was launched) from L2
-template <bool ONCE>
-__device__ __forceinline__ uint4 load16(const char* p) {
-  return ONCE ? __ldcg(reinterpret_cast<const uint4*>(p)) : __ldg(reinterpret_cast<const uint4*>(p));
-}
-
-// eight consecutive logits starting at x (x % 8 == 0): asked for, then mixed
+// eight consecutive logits starting at x (x % 8 == 0) as they are, asked for from L2 (a row that is read once, or that another
+// kernel may have written since this one was launched)
 template <bool BF16>
 struct raw_piece {
   uint4 w[BF16 ? 1 : 2];
 };
-template <bool ONCE, bool BF16>
+template <bool BF16>
 __device__ __forceinline__ void ask8(const RowSrc& r, int x, raw_piece<BF16>& c, raw_piece<BF16>& u) {
   const size_t o = (size_t)x * (BF16 ? 2 : 4);
 #pragma unroll
   for (int i = 0; i < (BF16 ? 1 : 2); ++i) {
-    c.w[i] = load16<ONCE>(r.cond + o + 16 * i);
-    if (r.uncond) u.w[i] = load16<ONCE>(r.uncond + o + 16 * i);
-  }
-}
-template <bool BF16>
-__device__ __forceinline__ void mix8(const RowSrc& r, const raw_piece<BF16>& c, const raw_piece<BF16>& u, float (&z)[8]) {
-  const bool hu = r.uncond != nullptr;
-#pragma unroll
-  for (int i = 0; i < (BF16 ? 1 : 2); ++i) {
-    const uint32_t cw[4] = {c.w[i].x, c.w[i].y, c.w[i].z, c.w[i].w}, uw[4] = {u.w[i].x, u.w[i].y, u.w[i].z, u.w[i].w};
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (BF16) {
-        z[2 * j] = mix_logit(bf16_lo(cw[j]), hu ? bf16_lo(uw[j]) : 0.f, hu, r.s, r.invT);
-        z[2 * j + 1] = mix_logit(bf16_hi(cw[j]), hu ? bf16_hi(uw[j]) : 0.f, hu, r.s, r.invT);
-      } else {
-        z[4 * i + j] = mix_logit(__uint_as_float(cw[j]), hu ? __uint_as_float(uw[j]) : 0.f, hu, r.s, r.invT);
-      }
-    }
+    c.w[i] = __ldcg(reinterpret_cast<const uint4*>(r.cond + o + 16 * i));
+    if (r.uncond) u.w[i] = __ldcg(reinterpret_cast<const uint4*>(r.uncond + o + 16 * i));
   }
 }
 // eight consecutive pre-processed logits
-template <bool ONCE = false>
 __device__ __forceinline__ void load8(const RowSrc& r, int x, float (&z)[8]) {
+  const bool hu = r.uncond != nullptr;
   if (r.bf16) {
-    raw_piece<true> c, u = {};
-    ask8<ONCE, true>(r, x, c, u);
-    mix8<true>(r, c, u, z);
+    uint4 c = __ldg(reinterpret_cast<const uint4*>(r.cond + (size_t)x * 2));
+    uint4 u = make_uint4(0, 0, 0, 0);
+    if (hu) u = __ldg(reinterpret_cast<const uint4*>(r.uncond + (size_t)x * 2));
+    z[0] = mix_logit(bf16_lo(c.x), bf16_lo(u.x), hu, r.s, r.invT);
+    z[1] = mix_logit(bf16_hi(c.x), bf16_hi(u.x), hu, r.s, r.invT);
+    z[2] = mix_logit(bf16_lo(c.y), bf16_lo(u.y), hu, r.s, r.invT);
+    z[3] = mix_logit(bf16_hi(c.y), bf16_hi(u.y), hu, r.s, r.invT);
+    z[4] = mix_logit(bf16_lo(c.z), bf16_lo(u.z), hu, r.s, r.invT);
+    z[5] = mix_logit(bf16_hi(c.z), bf16_hi(u.z), hu, r.s, r.invT);
+    z[6] = mix_logit(bf16_lo(c.w), bf16_lo(u.w), hu, r.s, r.invT);
+    z[7] = mix_logit(bf16_hi(c.w), bf16_hi(u.w), hu, r.s, r.invT);
   } else {
-    raw_piece<false> c, u = {};
-    ask8<ONCE, false>(r, x, c, u);
-    mix8<false>(r, c, u, z);
+    const float4* cp = reinterpret_cast<const float4*>(r.cond + (size_t)x * 4);
+    float4 c0 = __ldg(cp), c1 = __ldg(cp + 1);
+    float4 u0 = make_float4(0, 0, 0, 0), u1 = u0;
+    if (hu) {
+      const float4* up = reinterpret_cast<const float4*>(r.uncond + (size_t)x * 4);
+      u0 = __ldg(up);
+      u1 = __ldg(up + 1);
+    }
+    z[0] = mix_logit(c0.x, u0.x, hu, r.s, r.invT);
+    z[1] = mix_logit(c0.y, u0.y, hu, r.s, r.invT);
+    z[2] = mix_logit(c0.z, u0.z, hu, r.s, r.invT);
+    z[3] = mix_logit(c0.w, u0.w, hu, r.s, r.invT);
+    z[4] = mix_logit(c1.x, u1.x, hu, r.s, r.invT);
+    z[5] = mix_logit(c1.y, u1.y, hu, r.s, r.invT);
+    z[6] = mix_logit(c1.z, u1.z, hu, r.s, r.invT);
+    z[7] = mix_logit(c1.w, u1.w, hu, r.s, r.invT);
   }
 }
 

@@ -138,7 +138,7 @@ __device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, R
 #pragma unroll
       for (int k = 0; k < F; ++k) {
         const int x = ((first + k) * kThreads + (int)threadIdx.x) * 8;
-        if (x < row.V) ask8<true, BF16>(src, x, c[k], u[k]);
+        if (x < row.V) ask8<BF16>(src, x, c[k], u[k]);
       }
 #pragma unroll
       for (int k = 0; k < F; ++k) {
@@ -166,11 +166,11 @@ __device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, R
       float v[8];
       if (src.bf16) {
         raw_piece<true> c, u = {};
-        ask8<true, true>(src, x, c, u);
+        ask8<true>(src, x, c, u);
         res_mix<true>(src, c, u, v);
       } else {
         raw_piece<false> c, u = {};
-        ask8<true, false>(src, x, c, u);
+        ask8<false>(src, x, c, u);
         res_mix<false>(src, c, u, v);
       }
       take(x, v);
