@@ -1244,7 +1244,15 @@ mulo_status mulo_upsample_pool(mulo_ctx* ctx, const mulo_params* p, const void* 
   a.stats_out = draft_stats_lo;
   a.q_tok_hi_out = q_tok_hi;
   a.dev_status = (uint32_t*)ctx->ws;
+  // Without a cut there is nothing to search: many rows (more than four per SM) are read twice from L1 / L2 by four thread
+  // blocks per SM instead of kept in shared memory by two -- 4096 rows of 1024, 4096, 16392, 49152 bf16 ids: 26, 34, 81, 206 us,
+  // 38, 47, 106, 346 us resident; fp32 up to 8192 ids likewise (56, 71 us), above it the row no longer stays in L1 (16384 ids:
+  // 148, 106 us).  64 rows: 14 to 17 us, 9 to 14 us resident.
   const int cells = p->B * a.P.h * a.P.w;
+  if (a.P.top_k == 0 && cells > 4 * ctx->sm_count && (a.P.bf16 || a.P.V <= 8192)) {
+    if (!launch_general(ctx, K_UPSAMPLE(false), (unsigned)cells, 0, (cudaStream_t)stream, a)) return MULO_ERR_CUDA;
+    return launched(ctx, 1);
+  }
   if (!MULO_LAUNCH_GENERAL(K_UPSAMPLE, cells, general_smem(a.P, false), (cudaStream_t)stream, a)) return MULO_ERR_CUDA;
   return launched(ctx, 1);
 }

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle as orc
 from paper_2601_05149_b200 import binding, synth
 
 import parity_util as pu
@@ -100,6 +101,26 @@ def test_rows_with_a_cut(ctx, over, kernel):
     parity(ctx, cfg, kernel=kernel)
     # (the kernel did its rows itself: what it hands to the general routines is the exception)
     assert ctx.poll_fallback_counts()[0] <= cfg.B * cfg.H * cfg.W // 20
+
+
+@pytest.mark.parametrize("W", [37, 38], ids=["few", "many"])   # 592 and 608 draft rows: four per SM, and more
+@pytest.mark.parametrize("V,dtype", [(264, "bf16"), (8192, "f32"), (16392, "bf16")])
+def test_draft_sums_without_a_cut(ctx, V, dtype, W):
+    """Sums in double of fp32 weights of 2^-22 each, as an fp32 pair; q(x~) is rounded to fp32 besides."""
+    cfg = dataclasses.replace(FLAT, B=1, H=16, W=W, r=1, V=V, dtype=dtype, temperature=0.9)
+    batch = pu.build_batch(cfg)
+    p = binding.params_from_config(cfg)
+    ctx.ensure_workspace(p)
+    hi, q = torch.empty((1, 16, W), dtype=torch.int32, device="cuda"), torch.empty((1, 16, W), device="cuda")
+    stats = torch.empty((1, 16, W, 4), device="cuda")
+    ctx.mulo_upsample_pool(p, batch["draft_lo"], batch["tok_lo"], None, hi, stats, q)
+    tok = batch["tok_lo"][0].cpu().numpy()
+    want = orc.upsample_pool_image(pu.orc_params(cfg, 0), synth.to_numpy_logits(batch["draft_lo"][0]), tok)
+    got = stats[0].double().cpu().numpy()
+    assert np.array_equal(hi[0].cpu().numpy(), tok) and np.array_equal(got[..., 0], want["stats"][..., 0])
+    assert np.array_equal(got[..., 1], want["stats"][..., 1])
+    np.testing.assert_allclose(got[..., 2] + got[..., 3], want["stats"][..., 2], rtol=2.0 ** -22)
+    np.testing.assert_allclose(q[0].cpu().numpy(), want["q_tok"], rtol=2.0 ** -22 + 2.0 ** -24)
 
 
 @pytest.mark.parametrize("V", [16384, 16392, 49152, 49160])
