@@ -1024,7 +1024,7 @@ static bool launch_stream(mulo_ctx* ctx, const StreamArgs& s, size_t dyn, cudaSt
 static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample, int nw, RowsArgs* s) {
   if (d.top_k <= 0) return 0;
   const int V = d.V, k = d.top_k;
-  if (V < 1024 || d.r > 4) return 0;
+  if (V < 1024) return 0;
   const int esz = d.bf16 ? 2 : 4, ids = 16 / esz;
   // Candidates aimed for beyond k: 3.5 standard deviations of the count of entries above a fixed value near the
   // k-th largest (a row that misses, about one in two thousand, is streamed again); more for rows without a

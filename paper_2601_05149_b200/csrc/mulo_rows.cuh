@@ -102,7 +102,7 @@ struct RowsSmem {
   uint32_t fx[2][NW * 4];                  // ... and of the parts of the owning group
   double e_tok;
   float z_tok;
-  uint32_t rnd[2][16][3];                  // uniforms of the parent's children, by parity of the parent
+  uint32_t rnd[2][16][3];                  // uniforms of sixteen of the parent's children, by parity of the parent
   unsigned n_sa;
   int wn[NW];
   unsigned wmax[NW];
@@ -831,8 +831,11 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         sm.z_tok = z;
       }
     }
-    if (!SAMPLE && is_q && warp == 0 && lane < rr) {   // the uniforms of the parent's rows
-      const int ddi = lane / P.r, ddj = lane - ddi * P.r;
+    // the uniforms of the parent's rows, sixteen at a time: those around the first one with the draft row, the next with every
+    // sixteenth row (barrier 3 of the row before lies behind everybody who read the last ones)
+    if (!SAMPLE && warp == 0 && lane < min(rr, 16) && (is_q || (rr > 16 && (child & 15) == 0))) {
+      const int i = rr > 16 ? ((is_q ? di * P.r + dj : child) & ~15) + lane : lane;
+      const int ddi = i / P.r, ddj = i - ddi * P.r;
       const uint32_t t = (uint32_t)(ca * P.r + ddi) * P.W + (uint32_t)(cc * P.r + ddj);
       const uint4 v = lane_philox(make_uint4(t, (uint32_t)b + P.image_offset, P.round, 0u), make_uint2(P.seed_lo, P.seed_hi));
       sm.rnd[parent & 1][lane][0] = v.x;
@@ -1187,7 +1190,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         const uint4 v = lane_philox(make_uint4(cell, (uint32_t)b + P.image_offset, P.round, 1u), make_uint2(P.seed_lo, P.seed_hi));
         u_tgt = uniform24(v.x);
       } else {
-        const uint32_t* const rnd = sm.rnd[parent & 1][child];
+        const uint32_t* const rnd = sm.rnd[parent & 1][child & 15];
         int accepted;
         if (P.accept_mode == MULO_ACCEPT_THRESHOLD) accepted = mass >= P.tau * Z;
         else if (q_tok <= 0.0) accepted = mass > 0.0;

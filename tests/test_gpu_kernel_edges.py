@@ -67,6 +67,13 @@ def test_pooled_rows_of_large_vocabularies(ctx, V, cfg_scale, kernel):
     parity(ctx, cfg, kernel=kernel)
 
 
+@pytest.mark.parametrize("r,H,W", [(5, 20, 35), (8, 16, 32), (9, 18, 27), (16, 32, 16), (12, 12, 12)])
+@pytest.mark.parametrize("over,kernel", [(dict(top_k=300), "lane"), (dict(top_k=300, pool_k=40, pool_delta=0.3), "stream")], ids=["plain", "pooled"])
+def test_many_rows_with_a_cut_under_a_draft_row(ctx, over, kernel, r, H, W):
+    """More children than the sixteen whose uniforms are kept at a time, and parents split over thread blocks."""
+    parity(ctx, dataclasses.replace(ROWS, H=H, W=W, r=r, V=2048, **over), kernel=kernel)
+
+
 def test_rows_without_a_cut_that_mislead_the_prediction(ctx):
     """Consecutive rows whose maxima lie tens apart (every other one is streamed again), constant rows, and one-hot ones."""
     for over in (EQ5, ALL, dict(pool_k=300, pool_delta=0.2)):
