@@ -74,6 +74,14 @@ def test_many_rows_with_a_cut_under_a_draft_row(ctx, over, kernel, r, H, W):
     parity(ctx, dataclasses.replace(ROWS, H=H, W=W, r=r, V=2048, **over), kernel=kernel)
 
 
+@pytest.mark.parametrize("over", [dict(), EQ5, ALL, dict(pool_k=40, pool_delta=0.3, **EQ5)], ids=["mixed", "eq5", "residual", "pooled-eq5"])
+def test_rows_without_a_cut_at_large_ratios(ctx, over):
+    """Beyond k_round_flat's ratio: the general routines."""
+    pooled_target = over.get("pool_k", 1) > 1   # k_round_full's, whatever the ratio
+    cfg = dataclasses.replace(ROWS, H=24, W=12, r=12, V=2048, top_k=0, **over)
+    parity(ctx, cfg, kernel="full" if pooled_target else "general")
+
+
 def test_rows_without_a_cut_that_mislead_the_prediction(ctx):
     """Consecutive rows whose maxima lie tens apart (every other one is streamed again), constant rows, and one-hot ones."""
     for over in (EQ5, ALL, dict(pool_k=300, pool_delta=0.2)):
