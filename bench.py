@@ -297,9 +297,10 @@ def run_ours(args, cfg):
     row_avg_ms = row_ms / max(1, row_n)
     achieved = alg_bytes / (row_avg_ms * 1e-3) / 1e9
     which = ctx.round_kernel(p, cfg.has_uncond)
-    kernel = {"full": "k_round_full (pooled, target redraws) / k_round_flat",
-              "lane": "k_round_rows (+ k_verify_failed for rows that left the fast path)",
-              "stream": "k_round_stream (+ k_verify_failed for rows that left the fast path)",
+    # (of the workloads here: "full" is k_round_full for pooled rows with target redraws, pooled "stream" rows are k_round_rows')
+    pooled, failed = cfg.pool_k > 1, " (+ k_verify_failed for rows that left the fast path)"
+    kernel = {"full": "k_round_full" if pooled and cfg.resample_mode == binding.RESAMPLE_TARGET_ALL else "k_round_flat",
+              "lane": "k_round_rows" + failed, "stream": ("k_round_rows" if pooled else "k_round_stream") + failed,
               "general": "k_verify_rows"}[which]
     roofline = {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak,
                 "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_src,

@@ -111,9 +111,9 @@ typedef struct mulo_params {
 
 /* ---- context, workspace, diagnostics (no counterpart in the paper) ------------------- */
 
-/* Creates a context bound to CUDA device `device` (queries its limits, raises the
- * kernels' dynamic shared-memory caps).  Returns MULO_ERR_CUDA if the device cannot be
- * used.  The context is host memory owned by the library until mulo_destroy. */
+/* Creates a context bound to CUDA device `device` (queries its limits; a kernel's dynamic
+ * shared-memory cap is raised before its first launch).  Returns MULO_ERR_CUDA if the device
+ * cannot be used.  The context is host memory owned by the library until mulo_destroy. */
 mulo_status mulo_create(mulo_ctx** out, int device);
 void mulo_destroy(mulo_ctx* ctx);
 const char* mulo_status_string(mulo_status s);
@@ -153,13 +153,14 @@ mulo_status mulo_kernel_launches(const mulo_ctx* ctx, uint64_t* count);
  *                        streamed through registers, with their weights (pooling, residual redraws; V up to about 57000)
  *                        or the raw rows (pooling with redraws from the target distribution) kept in shared memory; with
  *                        Eq. 5 and redraws from the target distribution the draft logits are not read;
- *   MULO_KERNEL_LANE     top-k on, pooling off, V >= 1024, r <= 4, rows whose candidates fit the kernel's lists (k up
+ *   MULO_KERNEL_LANE     top-k on, pooling off, V >= 1024, rows whose candidates fit the kernel's lists (k up
  *                        to about a third of V): two or four warps per row, every thread keeps the candidates of
  *                        the ids it reads, rows are streamed once through registers;
- *   MULO_KERNEL_STREAM   the same rows with pooling (on the same kernel), and denser cuts (k up to half of V; with pooling
+ *   MULO_KERNEL_STREAM   the same rows with pooling (on the same kernel), and longer lists (k up to half of V; with pooling
  *                        V <= 16384): rows streamed once in chunks, candidates compacted per segment;
- *   MULO_KERNEL_GENERAL  everything else (top-k on with tiny vocabularies, r beyond the limits above, ...): one CTA
+ *   MULO_KERNEL_GENERAL  everything else (top-k on with tiny vocabularies, top-k off with r > 8, ...): one CTA
  *                        per row, the row in shared memory (V <= 49152) or read several times.
+ * mulo_sample_draft takes the chunked kernel of MULO_KERNEL_STREAM while there are few cells, too.
  * mulo_round_kernel reports the choice for these parameters (and with or without an unconditional
  * tensor) on this context (host arithmetic only; nothing is launched).  mulo_set_general_path_only(on != 0) makes the context always use
  * the general kernel (for testing and comparison). */

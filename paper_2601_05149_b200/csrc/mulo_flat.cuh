@@ -388,7 +388,7 @@ __global__ void __launch_bounds__((RES ? kFlatResWarps : kFlatWarps) * 32, (SAMP
       for (int i = lane; i < rr; i += 32) {
         const int ddi = SAMPLE ? 0 : i / P.r, ddj = i - ddi * P.r;
         const uint32_t t = SAMPLE ? (uint32_t)ca * P.w + (uint32_t)cc : (uint32_t)(ca * P.r + ddi) * P.W + (uint32_t)(cc * P.r + ddj);
-        const uint4 v = lane_philox(make_uint4(t, (uint32_t)b + P.image_offset, P.round, SAMPLE ? 1u : 0u),
+        const uint4 v = row_philox(make_uint4(t, (uint32_t)b + P.image_offset, P.round, SAMPLE ? 1u : 0u),
                                     make_uint2(P.seed_lo, P.seed_hi));
         sm.rnd[parent & 1][i][0] = v.x;
         sm.rnd[parent & 1][i][1] = v.y;
@@ -721,7 +721,7 @@ __global__ void __launch_bounds__((RES ? kFlatResWarps : kFlatWarps) * 32, (SAMP
       if (!SAMPLE && tid == ((owner + 1) & (NW - 1)) * 32) {   // (the owner is the last one on its way already)
         a.flags[g] = accepted ? 0 : 1;
         if (a.p_tok || a.q_tok || a.accept_prob)
-          lane_write_probs(a.p_tok, a.q_tok, a.accept_prob, g, e_tok, mass, q_tok, Z, P.accept_mode == MULO_ACCEPT_THRESHOLD);
+          row_write_probs(a.p_tok, a.q_tok, a.accept_prob, g, e_tok, mass, q_tok, Z, P.accept_mode == MULO_ACCEPT_THRESHOLD);
       }
     }
 

@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
       const double Zq = block_scan(mine, before, incl);
       if (tid == 0) {
         const float zq = full_one<BF16, false>(qrow, qrow, tok, 0.f, P.invT);
-        const double q = lane_exp2(((double)zq - (double)m_q) * 1.4426950408889634) / Zq;
+        const double q = row_exp2(((double)zq - (double)m_q) * 1.4426950408889634) / Zq;
         if (q <= 0.0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
         sm.q_tok = q;
       }
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
     for (int child = c_begin; child < c_end; ++child) {
       const size_t g = (size_t)b * NN + t;
       if (tid == 32) {
-        const uint4 rnd = lane_philox(make_uint4((uint32_t)t, (uint32_t)b + P.image_offset, P.round, 0u),
+        const uint4 rnd = row_philox(make_uint4((uint32_t)t, (uint32_t)b + P.image_offset, P.round, 0u),
                                       make_uint2(P.seed_lo, P.seed_hi));
         sm.rnd[0] = rnd.x;
         sm.rnd[1] = rnd.y;
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
       const float z_tok = full_one<BF16, HAS_U>(crow, urow, tok, P.cfg_scale, P.invT);
       const float e_tok = ex2f(fmaf(z_tok, kLog2e, c0));
       // exp(z_tok - M) in double by one thread, published by the scan's barrier
-      if (tid == 0) sm.p_tok = lane_exp2(((double)z_tok - (double)M) * 1.4426950408889634);
+      if (tid == 0) sm.p_tok = row_exp2(((double)z_tok - (double)M) * 1.4426950408889634);
       double before, incl;
       const double Z = block_scan((double)S_t, before, incl);
 

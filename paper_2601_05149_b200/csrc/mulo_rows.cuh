@@ -34,8 +34,6 @@
 // on the prediction.
 #pragma once
 
-#include <cuda.h>
-
 #include <type_traits>
 
 #include "mulo_stream.cuh"
@@ -54,7 +52,7 @@ constexpr float kNearRefGap = 8.0f;      // a row whose maximum lies further fro
                                          // against its own maximum (large exponents cost relative accuracy)
 
 // running prediction for one kind of row (draft / target), per CTA
-struct LanePredictor {
+struct RowPredictor {
   int have;
   int age;                    // rows learnt from since the prediction was last lost
   float theta, rho, mx;       // running k-th largest, density below it, row maximum
@@ -96,7 +94,7 @@ struct RowsSmem {
   alignas(16) float closer[4][32];         // -inf: what a thread past its list's end reads
   alignas(16) float sa_z[kRSetAside];      // (before the set-aside: where such a thread writes)
   unsigned short sa_at[kRSetAside];        // the entry's place (index in its owner's list << 8 | thread)
-  LanePredictor pred[2];                   // draft rows / target rows
+  RowPredictor pred[2];                   // draft rows / target rows
   double w_all[NW];                        // exp sums of each warp without the crossing bin
   double w_draw[2][NW * 4];                // weights of a draw, per group; consecutive draws alternate
   uint32_t fx[2][NW * 4];                  // ... and of the parts of the owning group
@@ -243,7 +241,7 @@ __device__ __forceinline__ void row_piece(const uint4& c, const uint4& u, float2
 }
 
 // 2^x in double, out of line: three call sites, a few hundred instructions each otherwise
-__device__ __noinline__ double lane_exp2(double x) { return exp2(x); }
+__device__ __noinline__ double row_exp2(double x) { return exp2(x); }
 
 // x~'s own weight, in double, beside weights 2^(z * kLog2e + c0), c0 = -ref * kLog2e in fp32.  That constant is off by 1.3e-8
 // (relative), which acts on z - ref: it averages out in sums near the maximum, a single weight far below it shows it whole
@@ -255,7 +253,7 @@ __device__ __noinline__ double token_weight(float z, float ref, float c0) {   //
 }
 
 // Philox4x32-10 as a rolled loop (one thread per row runs it; the unrolled form is ten times the code)
-__device__ __noinline__ uint4 lane_philox(uint4 c, uint2 k) {
+__device__ __noinline__ uint4 row_philox(uint4 c, uint2 k) {
 #pragma unroll 1
   for (int i = 0; i < 10; ++i) {
     const uint32_t a = 0xD2511F53u, b = 0xCD9E8D57u;
@@ -269,7 +267,7 @@ __device__ __noinline__ uint4 lane_philox(uint4 c, uint2 k) {
 }
 
 // The optional probability outputs of a position (one thread; out of line: double divisions).
-__device__ __noinline__ void lane_write_probs(float* p_tok, float* q_tok_out, float* accept_prob, size_t g, double e_tok,
+__device__ __noinline__ void row_write_probs(float* p_tok, float* q_tok_out, float* accept_prob, size_t g, double e_tok,
                                               double mass, double q_tok, double Z, bool threshold_rule) {
   const double p = e_tok / Z;
   if (p_tok) p_tok[g] = (float)p;
@@ -285,9 +283,9 @@ __device__ __noinline__ void lane_write_probs(float* p_tok, float* q_tok_out, fl
 }
 
 // The predictor of one kind of row after a row (ok: theta found exactly).  One thread; out of line.
-__device__ __noinline__ void lane_learn(LanePredictor* prp, bool ok, int reason, float theta, float pivot, int n,
+__device__ __noinline__ void row_learn(RowPredictor* prp, bool ok, int reason, float theta, float pivot, int n,
                                         int n_ge, float mx, int margin, float a_theta, float a_boot) {
-  LanePredictor pr = *prp;
+  RowPredictor pr = *prp;
   if (!ok) {
     pr.have = 0;
     pr.age = 0;
@@ -442,7 +440,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
 #pragma unroll 1
   for (int i = tid; i < 128; i += NT) (&sm.closer[0][0])[i] = -INFINITY;
   if (tid < 2) {
-    LanePredictor& pr = sm.pred[tid];
+    RowPredictor& pr = sm.pred[tid];
     pr.have = 0;
     pr.age = 0;
     pr.theta = 0.f; pr.rho = 1.f; pr.mx = 0.f;
@@ -786,7 +784,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       }
     }
 
-    LanePredictor& pr = sm.pred[is_q ? 0 : 1];
+    RowPredictor& pr = sm.pred[is_q ? 0 : 1];
     if (tries == 0) {   // (a row streamed again keeps its corrected values)
       lo = -INFINITY;
       hi = INFINITY;
@@ -837,7 +835,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       const int i = rr > 16 ? ((is_q ? di * P.r + dj : child) & ~15) + lane : lane;
       const int ddi = i / P.r, ddj = i - ddi * P.r;
       const uint32_t t = (uint32_t)(ca * P.r + ddi) * P.W + (uint32_t)(cc * P.r + ddj);
-      const uint4 v = lane_philox(make_uint4(t, (uint32_t)b + P.image_offset, P.round, 0u), make_uint2(P.seed_lo, P.seed_hi));
+      const uint4 v = row_philox(make_uint4(t, (uint32_t)b + P.image_offset, P.round, 0u), make_uint2(P.seed_lo, P.seed_hi));
       sm.rnd[parent & 1][lane][0] = v.x;
       sm.rnd[parent & 1][lane][1] = v.y;
       sm.rnd[parent & 1][lane][2] = v.z;
@@ -976,7 +974,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     const bool ok = reason == 0 && Z > 0.0 && Z < 1e300;
     const bool again = !ok && reason != 0 && reason != 4 && tries + 1 < kRTries;
     if (tid == 32 && !again)
-      lane_learn(&pr, ok, reason, theta, pivot, n_all, n_ge, mx, a.margin, a.a_theta, a.a_boot);
+      row_learn(&pr, ok, reason, theta, pivot, n_all, n_ge, mx, a.margin, a.a_theta, a.a_boot);
 
     if (!ok) {   // CTA-uniform
       __syncthreads();   // ---- barrier 3
@@ -1187,7 +1185,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       double u_res = 0.0, u_tgt;
       if (SAMPLE) {
         const uint32_t cell = g - (uint32_t)b * (uint32_t)(P.h * P.w);
-        const uint4 v = lane_philox(make_uint4(cell, (uint32_t)b + P.image_offset, P.round, 1u), make_uint2(P.seed_lo, P.seed_hi));
+        const uint4 v = row_philox(make_uint4(cell, (uint32_t)b + P.image_offset, P.round, 1u), make_uint2(P.seed_lo, P.seed_hi));
         u_tgt = uniform24(v.x);
       } else {
         const uint32_t* const rnd = sm.rnd[parent & 1][child & 15];
@@ -1200,7 +1198,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         if (tid == 0) {
           a.flags[g] = accepted ? 0 : 1;
           if (a.p_tok || a.q_tok || a.accept_prob)
-            lane_write_probs(a.p_tok, a.q_tok, a.accept_prob, g, e_tok, mass, q_tok, Z,
+            row_write_probs(a.p_tok, a.q_tok, a.accept_prob, g, e_tok, mass, q_tok, Z,
                              P.accept_mode == MULO_ACCEPT_THRESHOLD);
         }
         pending = draws_for(P.resample_mode, accepted);
