@@ -1269,9 +1269,14 @@ mulo_status mulo_island_schedule(mulo_ctx* ctx, const mulo_params* p, const int3
   ScheduleArgs a;
   a.H = p->H; a.W = p->W; a.window = window > p->W ? p->W : window;
   a.labels = labels; a.step = step; a.n_steps = n_steps;
-  const size_t smem = schedule_smem(p->H, p->W);
-  if (ctas_per_sm(ctx, k_island_schedule, kScheduleThreads, smem) < 1) return MULO_ERR_UNSUPPORTED;
-  k_island_schedule<<<p->B, kScheduleThreads, smem, (cudaStream_t)stream>>>(a);
+  auto launch = [&](auto kernel, size_t smem) -> bool {
+    if (ctas_per_sm(ctx, kernel, kScheduleThreads, smem) < 1) return false;
+    kernel<<<p->B, kScheduleThreads, smem, (cudaStream_t)stream>>>(a);
+    return true;
+  };
+  if (!launch(k_island_schedule<int>, schedule_smem<int>(p->H, p->W)) &&
+      !launch(k_island_schedule<uint16_t>, schedule_smem<uint16_t>(p->H, p->W)))
+    return MULO_ERR_UNSUPPORTED;
   return launched(ctx, 1);
 }
 

@@ -228,11 +228,14 @@ struct ScheduleArgs {
 constexpr int kScheduleThreads = 1024;
 constexpr int kRunTerm = 1 << 15;   // more than two steps, or columns, of one image can differ by
 
+// Linked: the type of a row's number of runs -- int where it fits (16-bit loads in the chain of rows cost 5 %).
+template <class Linked>
 __host__ inline size_t schedule_smem(int H, int W) {
   const size_t N = (size_t)H * W, nw = (size_t)H * ((W + 31) / 32);
-  return N * 12 + 2 * nw * 4 + (size_t)H * 2;   // (at most 232,000 bytes: 4000 x 4; an SM has 232,448)
+  return N * 12 + 2 * nw * 4 + (size_t)H * sizeof(Linked);   // (in 16 bits at most 232,000 bytes: 4000 x 4; an SM has 232,448)
 }
 
+template <class Linked>
 __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleArgs a) {
   extern __shared__ __align__(16) unsigned char sched_smem[];
   const int H = a.H, W = a.W, N = H * W, Ww = (W + 31) / 32, nw = H * Ww, b = blockIdx.x, tid = threadIdx.x;
@@ -244,7 +247,7 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
   int* const place = reinterpret_cast<int*>(first + nw);
   // by run of the row: the island's previous run in the row (-1: none) << 16 | last column
   int* const table = place + N;
-  uint16_t* const linked = reinterpret_cast<uint16_t*>(table + N);          // runs of a row where one has a predecessor, else 0
+  Linked* const linked = reinterpret_cast<Linked*>(table + N);              // runs of a row where one has a predecessor, else 0
   __shared__ int s_max, s_many;
   if (tid == 0) s_max = s_many = 0;
   const int32_t* const labels = a.labels + (size_t)b * N;
@@ -295,7 +298,7 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
         const int l = last_of(i, last_at(first + i * Ww, j) - 1, m);
         table[i * W + r] = (l >= 0 ? run_of(i, l) : -1) << 16 | j;
         const int nr = run_of(i, W - 1) + 1;
-        if (l >= 0) linked[i] = (uint16_t)nr;
+        if (l >= 0) linked[i] = (Linked)nr;
         if (nr > 32) s_many = 1;
       }
     }
