@@ -15,6 +15,7 @@
 #include "mulo_islands.cuh"
 #include "mulo_resident.cuh"
 #include "mulo_full.cuh"
+#include "mulo_redraw.cuh"
 #include "mulo_rows.cuh"
 #include "mulo_stream.cuh"
 
@@ -125,26 +126,20 @@ __global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_pool(RowKern
 
 // The inverse-CDF draw of uniform u from softmax(topk(row / T)); one thread writes the token to *out (-1: no mass, a row
 // whose largest logit mixes to +inf).
-// `before_pick` runs ahead of the last step.
-struct Nothing {
-  __device__ void operator()() const {}
-};
-template <bool RES, bool REG = false, class F = Nothing>
+template <bool RES>
 __device__ __forceinline__ void draw_row(const RowSrc& src, int top_k, double u, GeneralScratch<RES>& sc, unsigned char* dyn,
-                                         int32_t* out, F before_pick = F()) {
+                                         int32_t* out) {
   RowStats st;
   if constexpr (RES) {
     const ResRow row(reinterpret_cast<float*>(dyn), src.V);
     int calls = 0;
     float unused;
-    const ResSums sums = res_row_stats<REG>(row, src, top_k, sc, calls, -1, unused, st);
-    before_pick();
+    const ResSums sums = res_row_stats(row, src, top_k, sc, calls, -1, unused, st);
     res_pick(row, sums, u, [&](int x) -> double { return (double)row.at(x); }, out);
     if (!(sums.total > 0.0) && threadIdx.x == 0) *out = -1;
   } else {
     dense_row_stats(src, top_k, sc, st.theta, st.m, st.Z);
     __syncthreads();
-    before_pick();
     const float invZ = (float)(1.0 / st.Z);
     // lambda = 0 and no special token: the weights are the probabilities themselves
     const int tok = dense_draw(src, src, st, st, invZ, invZ, 0.0f, -1, 0.0, nullptr, u, sc);
@@ -232,94 +227,6 @@ __global__ void __launch_bounds__(256) k_redraw_fill(const int32_t* __restrict__
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int s = step[i];
     if (s >= 1 && s <= max_step) pos_list[atomicAdd(&cursor[s], 1)] = i;
-  }
-}
-
-// a 4-byte load that is neither taken from the read-only cache nor moved
-__device__ __forceinline__ int ld_fresh(const int32_t* p) {
-  int v;
-  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-struct RedrawArgs {
-  DevParams P;
-  const char* cond;
-  const char* uncond;
-  const int32_t* pos_list;
-  const int32_t* offsets;
-  int32_t* out_tok;
-  int s;
-};
-
-// One step: every position of the step's slice of the list draws its token from the target
-// distribution of the given logits; uniform = word 0 of Philox at (t, image, round, 1 + s).
-// Steps follow one another by the thousand, a handful of positions each, so a step is bound by latency: the launch
-// may begin while the kernel before it in the stream still runs (programmatic dependent launch), asks its rows into
-// L2 -- a hint: nothing is read -- and waits for that kernel before it reads anything it uses.
-template <bool RES, bool REG>
-__global__ void __launch_bounds__(kThreads, REG ? 1 : 2) k_redraw_step(RedrawArgs a) {
-  extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ GeneralScratch<RES> sc;
-  const DevParams& P = a.P;
-  const size_t N = (size_t)P.H * P.W, total = (size_t)P.B * N;
-  const size_t bytes = (size_t)P.V * (P.bf16 ? 2 : 4);
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  // what the step will find, if the list stays as it is
-  const int beg0 = ld_fresh(a.offsets + a.s), end0 = ld_fresh(a.offsets + a.s + 1);
-  const long long i0 = (long long)beg0 + (long long)blockIdx.x;
-  size_t g0 = total;
-  if (beg0 >= 0 && i0 < end0 && i0 < (long long)total) {
-    g0 = (size_t)(uint32_t)ld_fresh(a.pos_list + i0);
-    if (RES && g0 < total && threadIdx.x == 0) {
-      prefetch_l2(a.cond + g0 * bytes, (uint32_t)bytes);
-      if (a.uncond) prefetch_l2(a.uncond + g0 * bytes, (uint32_t)bytes);
-    }
-  }
-  struct Place {
-    RowSrc src;
-    double u;
-  };
-  auto place = [&](size_t g) -> Place {   // (positions fit 32 bits)
-    const uint32_t b = (uint32_t)g / (uint32_t)N, t = (uint32_t)g - b * (uint32_t)N;
-    Place pl;
-    pl.src.cond = a.cond + g * bytes;
-    pl.src.uncond = a.uncond ? a.uncond + g * bytes : nullptr;
-    pl.src.s = P.cfg_scale;
-    pl.src.invT = P.invT;
-    pl.src.V = P.V;
-    pl.src.bf16 = P.bf16;
-    pl.u = uniform24(philox4x32_10(make_uint4(t, b + P.image_offset, P.round, 1u + (uint32_t)a.s),
-                                   make_uint2(P.seed_lo, P.seed_hi)).x);
-    return pl;
-  };
-  const Place first = place(g0 < total ? g0 : 0);
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  int i = -1;
-  if (g0 < total) {   // block-uniform
-    // The position found above is worked on at once, and its token written if the list, read again towards the end,
-    // says so now too: two dependent loads from L2 fewer before the row can be asked for.
-    __shared__ int32_t tok;
-    __shared__ int32_t now[3];
-    draw_row<RES, REG>(first.src, P.top_k, first.u, sc, dyn, &tok, [&]() {
-      if (threadIdx.x < 3) now[threadIdx.x] = ld_fresh(threadIdx.x < 2 ? a.offsets + a.s + threadIdx.x : a.pos_list + i0);
-    });
-    __syncthreads();
-    i = now[0] + (int)blockIdx.x;
-    if (now[0] == beg0 && (size_t)(uint32_t)now[2] == g0 && i < now[1]) {
-      if (threadIdx.x == 0) a.out_tok[g0] = tok;
-      i += (int)gridDim.x;
-    }
-  }
-  const int beg = ld_fresh(a.offsets + a.s), end = ld_fresh(a.offsets + a.s + 1);
-  if (i < 0) i = beg + (int)blockIdx.x;
-  for (; i < end; i += (int)gridDim.x) {
-    const size_t g = (size_t)(uint32_t)ld_fresh(a.pos_list + i);
-    if (g < total) {   // block-uniform
-      const Place pl = place(g);
-      draw_row<RES, REG>(pl.src, P.top_k, pl.u, sc, dyn, a.out_tok + g);
-    }
-    __syncthreads();
   }
 }
 
@@ -1320,21 +1227,32 @@ mulo_status mulo_redraw_step(mulo_ctx* ctx, const mulo_params* p, int32_t s_inde
   a.offsets = step_offsets;
   a.out_tok = out_tok;
   a.s = s_index;
-  // the step's positions are counted on the device: a fixed grid strides over them
+  const int np = a.P.V <= kRedrawIds ? 1 : a.P.V <= 2 * kRedrawIds ? 2 : 4, ctas = (a.P.V + np * kRedrawIds - 1) / (np * kRedrawIds);
+  // The step's positions are counted on the device: a fixed number of clusters strides over them.  A schedule of window 8 to 16
+  // has W / 8 to W / 16 of them per image at a time; twice the larger as long as half of the chip holds them -- what is left
+  // over draws the next step's rows meanwhile -- and that many beyond.  64 x 64, 4 images, V = 16384 (15 positions, 64 clusters):
+  // 5.3 us a step, 8.5 before; 16 x 16, 29 images (54 positions): 74 clusters, where 116, which leave no room, took 12.1 us, 11.6
+  // before.  32 x 32, 64 images, V = 2048 (234 positions): 9.2 us, 15.5 before.
+  const int room = ctx->sm_count * (np == 4 ? 1 : 2) / ctas;
+  const long long twice = (long long)p->B * (p->W > 4 ? p->W / 4 : 1), likely = twice <= room / 2 ? twice : twice / 2 > room / 2 ? twice / 2 : room / 2;
+  const int clusters = likely < room ? (int)likely : room;
+  auto kern = a.P.bf16 ? (np == 1 ? k_redraw_step<true, 1> : np == 2 ? k_redraw_step<true, 2> : k_redraw_step<true, 4>)
+                       : (np == 1 ? k_redraw_step<false, 1> : np == 2 ? k_redraw_step<false, 2> : k_redraw_step<false, 4>);
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3((unsigned)(2 * ctx->sm_count));
+  cfg.gridDim = dim3((unsigned)(clusters * ctas));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = general_smem(a.P, false);
+  cfg.dynamicSmemBytes = (size_t)ctas * kRedrawWords * sizeof(uint32_t);
   cfg.stream = (cudaStream_t)stream;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  const bool res = resident_fits(a.P.V);
-  cfg.numAttrs = res ? 1 : 0;   // (the version for larger vocabularies reads through the read-only cache)
-  auto kern = !res ? k_redraw_step<false, false> : a.P.V <= kResRegs * kThreads ? k_redraw_step<true, true> : k_redraw_step<true, false>;
-  if (ctas_per_sm(ctx, kern, kThreads, cfg.dynamicSmemBytes) < 1) return MULO_ERR_CUDA;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)ctas;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  if (clusters < 1 || ctas_per_sm(ctx, kern, kThreads, cfg.dynamicSmemBytes) < 1) return MULO_ERR_CUDA;
   if (cudaLaunchKernelEx(&cfg, kern, a) != cudaSuccess) {
     cudaGetLastError();
     return MULO_ERR_CUDA;

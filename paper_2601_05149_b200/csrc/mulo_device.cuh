@@ -33,6 +33,11 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
   return c;
 }
 
+// Programmatic dependent launch: a kernel launched so may begin once every CTA of the kernel before it has said that it may
+// (or ended), and waits for that kernel's end, and so for what it wrote, before it reads anything of it.
+__device__ __forceinline__ void let_next_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // top 24 bits of a word as a uniform in [0,1): exact in fp32 and fp64
 __device__ __forceinline__ double uniform24(uint32_t w) { return (double)(w >> 8) * (1.0 / 16777216.0); }
 

@@ -20,7 +20,6 @@ namespace mulo {
 
 constexpr int kResBins = 1024;
 constexpr int kResMembers = 128;
-constexpr int kResRegs = 32;     // ids per thread that a kernel with registers for them (REG) keeps until the threshold is known
 
 struct ResScratch {
   unsigned hist[kResBins];
@@ -113,13 +112,21 @@ __device__ __forceinline__ void res_mix(const RowSrc& r, const raw_piece<BF16>& 
   else all(std::false_type{});
 }
 
-// The row from global memory into shared memory; every thread gets the row's maximum and mean.  REG: the ids
-// this thread brought (8 at (c * 512 + tid) * 8 for c = 0 .. 3) also stay in z, -inf past the row's end.
-template <bool REG>
-__device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, ResScratch& rs, float (&z)[kResRegs], float& mx,
-                                         float& mean) {
+// The row from global memory into shared memory; every thread gets the row's maximum and mean.
+__device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, ResScratch& rs, float& mx, float& mean) {
   float hi = -INFINITY, sum = 0.f;
-  auto take = [&](int x, const float (&v)[8]) {
+#pragma unroll 2
+  for (int x = (int)threadIdx.x * 8; x < row.V; x += 8 * kThreads) {
+    float v[8];
+    if (src.bf16) {
+      raw_piece<true> c, u = {};
+      ask8<true>(src, x, c, u);
+      res_mix<true>(src, c, u, v);
+    } else {
+      raw_piece<false> c, u = {};
+      ask8<false>(src, x, c, u);
+      res_mix<false>(src, c, u, v);
+    }
     float4* const to = reinterpret_cast<float4*>(row.place(x));
     to[0] = make_float4(v[0], v[1], v[2], v[3]);
     to[1] = make_float4(v[4], v[5], v[6], v[7]);
@@ -127,53 +134,6 @@ __device__ __forceinline__ void res_load(const ResRow& row, const RowSrc& src, R
     for (int j = 0; j < 8; ++j) {
       hi = fmaxf(hi, v[j]);
       sum += v[j];
-    }
-  };
-  if (REG) {
-    // (four pieces of bf16, two of fp32 asked for before any is used)
-    auto pieces = [&](auto bf16, int first) {
-      constexpr bool BF16 = decltype(bf16)::value;
-      constexpr int F = BF16 ? 4 : 2;
-      raw_piece<BF16> c[F], u[F] = {};
-#pragma unroll
-      for (int k = 0; k < F; ++k) {
-        const int x = ((first + k) * kThreads + (int)threadIdx.x) * 8;
-        if (x < row.V) ask8<BF16>(src, x, c[k], u[k]);
-      }
-#pragma unroll
-      for (int k = 0; k < F; ++k) {
-        const int x = ((first + k) * kThreads + (int)threadIdx.x) * 8;
-        float v[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = -INFINITY;
-        if (x < row.V) {
-          res_mix<BF16>(src, c[k], u[k], v);
-          take(x, v);
-        }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) z[8 * (first + k) + j] = v[j];
-      }
-    };
-    if (src.bf16) {
-      pieces(std::true_type{}, 0);
-    } else {
-      pieces(std::false_type{}, 0);
-      pieces(std::false_type{}, 2);
-    }
-  } else {
-#pragma unroll 2
-    for (int x = (int)threadIdx.x * 8; x < row.V; x += 8 * kThreads) {
-      float v[8];
-      if (src.bf16) {
-        raw_piece<true> c, u = {};
-        ask8<true>(src, x, c, u);
-        res_mix<true>(src, c, u, v);
-      } else {
-        raw_piece<false> c, u = {};
-        ask8<false>(src, x, c, u);
-        res_mix<false>(src, c, u, v);
-      }
-      take(x, v);
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -307,9 +267,7 @@ __device__ __noinline__ float res_refine(const ResRow& row, int top_k, float zhi
 // crossing bin's entries ranked exactly.  The map z -> bin is monotone, so a bin's entries are consecutive in rank
 // whatever the rounding (z - mean and the product round monotonically; adding 1.5 * 2^23 leaves the rounded integer in
 // the low bits; an entry that rounds up into the first bin from below it is simply one of its entries).
-template <bool REG>
-__device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)[kResRegs], int top_k, float mx, float mean,
-                                            ResScratch& rs) {
+__device__ __forceinline__ float res_select(const ResRow& row, int top_k, float mx, float mean, ResScratch& rs) {
   const int lane = threadIdx.x & 31;
   // (Finite logits may sum to -inf, or mix to it under guidance: two ids at the lowest value of the type do.  Then there
   // is no mean, and no first histogram; sc is 0 where mx - mean is infinite.)
@@ -332,17 +290,12 @@ __device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)
     asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(b < (uint32_t)kResBins ? hist + 4u * b : spill) : "memory");
   };
   const int n_mine = row.end - row.beg;
-  if (REG) {
-#pragma unroll
-    for (int i = 0; i < kResRegs; ++i) count(zr[i]);
-  } else {
 #pragma unroll 1
-    for (int i = 0; i < n_mine; i += 8) {
-      float v[8];
-      eight(i, v);
+  for (int i = 0; i < n_mine; i += 8) {
+    float v[8];
+    eight(i, v);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) count(v[j]);
-    }
+    for (int j = 0; j < 8; ++j) count(v[j]);
   }
   __syncthreads();
   unsigned over = 0;
@@ -354,26 +307,15 @@ __device__ __forceinline__ float res_select(const ResRow& row, const float (&zr)
   }
   const int want_bits = bin + __float_as_int(kRMagic);
   auto aside = [&](float v) { rs.sa[atomicAdd(&rs.n_sa, 1u)] = v; };
-  if (REG) {
+#pragma unroll 1
+  for (int i = 0; i < n_mine; i += 8) {
+    float v[8];
+    eight(i, v);
     uint32_t m = 0;
 #pragma unroll
-    for (int i = 0; i < kResRegs; ++i) m |= bits_of(zr[i]) == want_bits ? 1u << i : 0u;
+    for (int j = 0; j < 8; ++j) m |= bits_of(v[j]) == want_bits ? 1u << j : 0u;
 #pragma unroll 1
-    for (; m; m &= m - 1u) {   // (from shared memory: registers cannot be picked by number)
-      const int i = __ffs(m) - 1;
-      aside(row.at(((i >> 3) * kThreads + (int)threadIdx.x) * 8 + (i & 7)));
-    }
-  } else {
-#pragma unroll 1
-    for (int i = 0; i < n_mine; i += 8) {
-      float v[8];
-      eight(i, v);
-      uint32_t m = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) m |= bits_of(v[j]) == want_bits ? 1u << j : 0u;
-#pragma unroll 1
-      for (; m; m &= m - 1u) aside(row.run()[i + __ffs(m) - 1]);
-    }
+    for (; m; m &= m - 1u) aside(row.run()[i + __ffs(m) - 1]);
   }
   __syncthreads();
   return res_rank(rs, in_bin, (unsigned)top_k - over);
@@ -456,18 +398,15 @@ __device__ inline void res_pick(const ResRow& row, const ResSums& s, double u, W
   if (lane == 0) *out = pick >= 0 ? pick : last >= 0 ? last : x_beg;   // (rounding: the last id with weight)
 }
 
-// Statistics of a row (threshold, maximum, partition sum); the row's weights stay in shared memory.  REG: in a kernel
-// compiled for 128 registers, for rows of up to 16384 ids.
-template <bool REG = false>
+// Statistics of a row (threshold, maximum, partition sum); the row's weights stay in shared memory.
 __device__ inline ResSums res_row_stats(const ResRow& row, const RowSrc& src, int top_k, ResScratch& rs, int& calls,
                                         int tok, float& z_tok, RowStats& st) {
   float mx, mean;
-  float z[kResRegs];
-  res_load<REG>(row, src, rs, z, mx, mean);
+  res_load(row, src, rs, mx, mean);
   z_tok = tok >= 0 ? row.at(tok) : 0.f;   // (before the logits become weights)
   st.m = mx;
   st.theta = -INFINITY;
-  if (top_k > 0 && top_k < row.V) st.theta = res_select<REG>(row, z, top_k, mx, mean, rs);
+  if (top_k > 0 && top_k < row.V) st.theta = res_select(row, top_k, mx, mean, rs);
   else __syncthreads();                   // everybody has z_tok
   const ResSums s = res_weigh(row, st.theta, mx, rs, calls);
   st.Z = s.total;

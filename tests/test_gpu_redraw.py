@@ -228,3 +228,84 @@ def test_one_context_from_several_threads():
             np.testing.assert_array_equal(x, y)
     alone.close()
     shared.close()
+
+
+_EARLY_WRITER = r"""
+extern "C" __global__ void early_writer(const uint4* src, uint4* dst, long long n, const int* new_list, int* list, int n_list) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // what comes after may begin now, and is to find the old contents: 60 us and no more
+  const long long t0 = clock64();
+  while (clock64() - t0 < 120000) {}
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) dst[i] = src[i];
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < n_list; i += blockDim.x) list[i] = new_list[i];
+}
+"""
+
+
+@pytest.mark.parametrize("V", [520, 8192, 16384, 20000, 49160])   # one, two, four pieces per thread; two and four CTAs to a row
+@pytest.mark.parametrize("what", ["logits", "one id", "list", "nothing"])
+def test_a_row_drawn_ahead_of_its_inputs(ctx, V, what):
+    """The kernel before the step lets it begin and only then rewrites the row's logits (all of them, or one id of each row's last
+    pieces) or the list: the step's token is that of what stands there when that kernel is done."""
+    B, H, W = 2, 4, 16
+    cfg = synth.RoundConfig("ahead", B=B, H=H, W=W, V=V, r=1, dtype="bf16", top_k=V // 8, cfg_scale=0.0, seed=79)
+    p = binding.params_from_config(cfg)
+    g = torch.Generator(device="cuda").manual_seed(V)
+    old = (2.0 * torch.randn((B, H, W, V), generator=g, device="cuda")).bfloat16()
+    new = old.clone()
+    if what == "logits":
+        new.copy_(2.0 * torch.randn((B, H, W, V), generator=g, device="cuda"))
+    elif what == "one id":
+        new[..., V - 3] = 40.0       # takes the whole mass
+    steps = torch.zeros((B, H, W), dtype=torch.int32, device="cuda")
+    steps.view(-1)[::17] = 1
+    n = B * H * W
+    pos, off = torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(2 * 3, dtype=torch.int32, device="cuda")
+    ctx.mulo_redraw_plan(p, steps, 1, pos, off)
+    listed = pos.clone()
+    if what == "list":
+        listed[:8] = (listed[:8] + 5) % n
+    want = torch.full((B, H, W), -7, dtype=torch.int32, device="cuda")
+    ctx.mulo_redraw_step(p, 1, 1, listed, off, new, None, want)
+    torch.cuda.synchronize()
+    kernel = torch.cuda._compile_kernel(_EARLY_WRITER, "early_writer", compute_capability="100a")
+    for _ in range(3):
+        buf, lst = old.clone(), pos.clone()
+        out = torch.full_like(want, -7)
+        torch.cuda.synchronize()
+        kernel(grid=(16, 1, 1), block=(256, 1, 1), args=[new, buf, buf.numel() // 8, listed, lst, 8])
+        ctx.mulo_redraw_step(p, 1, 1, lst, off, buf, None, out)
+        assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("case", [
+    dict(V=8, top_k=3), dict(V=4096, top_k=4095), dict(V=4104, top_k=1), dict(V=8200, top_k=1000), dict(V=16384, top_k=0), dict(V=16392, top_k=2000),
+    dict(V=65536, top_k=4000), dict(V=65536, top_k=0), dict(V=32776, top_k=30000, dtype="f32"),
+    dict(V=4096, top_k=500, level=-300.0, scale=3.0), dict(V=4096, top_k=500, scale=1e-3), dict(V=8192, top_k=500, quantum=0.5),
+    dict(V=16384, top_k=100, scale=0.0), dict(V=20480, top_k=5000, level=5000.0, scale=100.0, dtype="f32"), dict(V=4096, top_k=2100, quantum=0.25),
+    dict(V=8192, top_k=700, dtype="f32", cfg_scale=2.0, temperature=0.8),
+], ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()))
+def test_rows_of_all_sizes_and_shapes(ctx, case):
+    """Edges of the kernel's pieces and clusters; values outside the first histogram, crowded bins, ties, thresholds below zero."""
+    B, H, W, V = 2, 3, 4, case["V"]
+    dtype, cfg_scale = case.get("dtype", "bf16"), case.get("cfg_scale", 0.0)
+    cfg = synth.RoundConfig("shape", B=B, H=H, W=W, V=V, r=1, dtype=dtype, top_k=case["top_k"], cfg_scale=cfg_scale,
+                            temperature=case.get("temperature", 1.0), seed=80)
+    g = torch.Generator(device="cuda").manual_seed(V + case["top_k"])
+    z = case.get("level", 0.0) + case.get("scale", 2.0) * torch.randn((B, H, W, V), generator=g, device="cuda")
+    if "quantum" in case:
+        z = (z / case["quantum"]).round() * case["quantum"] + 0.0
+        z[..., ::2] = torch.where(z[..., ::2] == 0, -0.0, z[..., ::2])   # both zeros are one value
+    cond = z.to(cfg.torch_dtype).contiguous()
+    unc = (z + 0.3).to(cfg.torch_dtype).contiguous() if cfg_scale else None
+    p = binding.params_from_config(cfg)
+    n = B * H * W
+    pos, off = torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(2 * 3, dtype=torch.int32, device="cuda")
+    out = torch.full((B, H, W), -7, dtype=torch.int32, device="cuda")
+    ctx.mulo_redraw_plan(p, torch.ones((B, H, W), dtype=torch.int32, device="cuda"), 1, pos, off)
+    ctx.mulo_redraw_step(p, 1, 1, pos, off, cond, unc, out)
+    for b in range(B):
+        want, _, edge = orc.redraw_loop(pu.orc_params(cfg, b), np.ones((H, W), np.int32), [synth.to_numpy_logits(cond[b])],
+                                        None if unc is None else [synth.to_numpy_logits(unc[b])], np.zeros((H, W), np.int32), with_edge=True)
+        assert not ((out[b].cpu().numpy() != want) & (edge == 0)).any()
