@@ -1176,14 +1176,10 @@ mulo_status mulo_island_schedule(mulo_ctx* ctx, const mulo_params* p, const int3
   ScheduleArgs a;
   a.H = p->H; a.W = p->W; a.window = window > p->W ? p->W : window;
   a.labels = labels; a.step = step; a.n_steps = n_steps;
-  auto launch = [&](auto kernel, size_t smem) -> bool {
-    if (ctas_per_sm(ctx, kernel, kScheduleThreads, smem) < 1) return false;
-    kernel<<<p->B, kScheduleThreads, smem, (cudaStream_t)stream>>>(a);
-    return true;
-  };
-  if (!launch(k_island_schedule<int>, schedule_smem<int>(p->H, p->W)) &&
-      !launch(k_island_schedule<uint16_t>, schedule_smem<uint16_t>(p->H, p->W)))
-    return MULO_ERR_UNSUPPORTED;
+  const auto kernel = p->W <= 32 ? k_island_schedule<1> : p->W <= 64 ? k_island_schedule<2> : k_island_schedule<4>;
+  const size_t smem = schedule_smem(p->H, p->W);
+  if (ctas_per_sm(ctx, kernel, kScheduleThreads, smem) < 1) return MULO_ERR_UNSUPPORTED;
+  kernel<<<p->B, kScheduleThreads, smem, (cudaStream_t)stream>>>(a);
   return launched(ctx, 1);
 }
 

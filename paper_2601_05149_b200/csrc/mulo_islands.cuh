@@ -211,13 +211,12 @@ __global__ void __launch_bounds__(kIslandThreads) k_islands(IslandArgs a) {
 //   step(t) = 1 + max(step of the island's earlier positions in the row,
 //                     step of the island's positions in the row above up to column col(t) + window - 1).
 // Steps grow along an island's positions in a row, so of the row above only the last position inside the window
-// counts, and along a run of neighbours the recurrence s_k = max(s_{k-1} + 1, d_k) is a prefix maximum of d_k - k.
-// One CTA per image.  All threads first find, for every position, what it depends on -- its run, the position of the
-// row above, for a run the island's previous run in the row -- with bit operations on the rows' masks; nothing of that
-// needs a step.  ONE warp then goes down the rows with shuffles instead of block barriers; the runs of a row share one
-// scan (a term that grows from run to run keeps them apart).  In rows where an island has several runs, a run adds to
-// the next one's steps: lane r takes run r and the chains are followed by doubling.  What bounds the kernel is this
-// chain of H rows (three barriers and two searches per row made them 2.5 us each at 64 columns).
+// counts, and along the island's positions of the row the recurrence s_k = max(s_{k-1} + 1, d_k) is a prefix maximum of
+// d_k - k.  One CTA per image.  All threads first find where every position comes when its row is sorted by island, then by
+// column (its slot), and the slot in the row above that it depends on -- with bit operations on the rows' masks; nothing of
+// that needs a step.  ONE warp then goes down the rows: what the row above demands, one scan over the slots (a term that grows
+// from island to island keeps them apart, however their runs interleave), and the steps are there; a row's slots are asked
+// for one row ahead.  What bounds the kernel is this chain of H rows.
 struct ScheduleArgs {
   int H, W, window;
   const int32_t* labels;   // [B, H, W]
@@ -226,33 +225,35 @@ struct ScheduleArgs {
 };
 
 constexpr int kScheduleThreads = 1024;
-constexpr int kRunTerm = 1 << 15;   // more than two steps, or columns, of one image can differ by
+constexpr int kIslandTerm = 1 << 15;   // more than two steps, or columns, of one image can differ by
 
-// Linked: the type of a row's number of runs -- int where it fits (16-bit loads in the chain of rows cost 5 %).
-template <class Linked>
 __host__ inline size_t schedule_smem(int H, int W) {
   const size_t N = (size_t)H * W, nw = (size_t)H * ((W + 31) / 32);
-  return N * 12 + 2 * nw * 4 + (size_t)H * sizeof(Linked);   // (in 16 bits at most 232,000 bytes: 4000 x 4; an SM has 232,448)
+  return N * 12 + 2 * nw * 4;   // (at most 228,608 bytes: 4000 x 4)
 }
 
-template <class Linked>
+// M: slots per lane in the chain of rows; rows of more than 32 M columns take several turns.
+template <int M>
 __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleArgs a) {
   extern __shared__ __align__(16) unsigned char sched_smem[];
   const int H = a.H, W = a.W, N = H * W, Ww = (W + 31) / 32, nw = H * Ww, b = blockIdx.x, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
-  int* const lab = reinterpret_cast<int*>(sched_smem);                      // labels, then steps
-  uint32_t* const pos = reinterpret_cast<uint32_t*>(lab + N);               // bit: the position is in R_X
+  int* const lab = reinterpret_cast<int*>(sched_smem);
+  uint16_t* const steps = reinterpret_cast<uint16_t*>(sched_smem);          // by slot, once the labels are not needed any more
+  // by slot: the slot of the row above that it depends on (0xffff: none) | its number among its island's in the row << 16
+  uint32_t* const dep = reinterpret_cast<uint32_t*>(lab + N);
+  uint32_t* const pos = dep + N;                                            // bit: the position is in R_X
   uint32_t* const first = pos + nw;                                         // bit: ... and starts a run
-  // by position: number of its run in the row (-1 outside R_X) << 16 | column of the row above (0xffff: none)
-  int* const place = reinterpret_cast<int*>(first + nw);
-  // by run of the row: the island's previous run in the row (-1: none) << 16 | last column
-  int* const table = place + N;
-  Linked* const linked = reinterpret_cast<Linked*>(table + N);              // runs of a row where one has a predecessor, else 0
-  __shared__ int s_max, s_many;
-  if (tid == 0) s_max = s_many = 0;
+  uint16_t* const head = reinterpret_cast<uint16_t*>(first + nw);           // by slot: the first slot of its island
+  uint16_t* const slot = head + N;                                          // by column
+  __shared__ int s_max;
+  if (tid == 0) s_max = 0;
   const int32_t* const labels = a.labels + (size_t)b * N;
-  for (int t = tid; t < N; t += kScheduleThreads) lab[t] = labels[t];
-  for (int i = tid; i < H; i += kScheduleThreads) linked[i] = 0;
+  for (int t = tid; t < N; t += kScheduleThreads) {
+    lab[t] = labels[t];
+    dep[t] = 0xffffu;
+    head[t] = 0;
+  }
   __syncthreads();
   for (int w = warp; w < nw; w += kScheduleThreads / 32) {   // the rows' masks
     const int i = w / Ww, j = (w % Ww) * 32 + lane;
@@ -264,6 +265,28 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
     }
   }
   __syncthreads();
+  // slots: the row's runs, cut at the masks' words, one after the other
+  for (int w = warp; w < nw; w += kScheduleThreads / 32) {
+    if (pos[w] == 0u) continue;
+    const int i = w / Ww, j = (w % Ww) * 32 + lane;
+    const int m = pos[w] >> lane & 1u ? lab[i * W + j] : 0;
+    int below = 0, before = 0;   // positions of islands with a lower label; the island's own to the left
+    for (int v = 0; v < Ww; ++v) {
+      const uint32_t in = pos[i * Ww + v], stops = first[i * Ww + v] | ~in;
+      for (uint32_t starts = (first[i * Ww + v] | 1u) & in; starts; starts &= starts - 1u) {
+        const int at = __ffs(starts) - 1;
+        const uint32_t stop = stops & ~((2u << at) - 1u);
+        const int len = (stop ? __ffs(stop) - 1 : 32) - at, x = v * 32 + at, other = lab[i * W + x];
+        if (other < m) below += len;
+        if (other == m) before += min(max(j - x, 0), len);
+      }
+    }
+    if (m > 0) {
+      slot[i * W + j] = (uint16_t)(below + before);
+      head[i * W + below + before] = (uint16_t)below;
+    }
+  }
+  __syncthreads();
   // the last set bit of a row's mask at or before column x, -1: none
   auto last_at = [&](const uint32_t* row, int x) -> int {
     if (x < 0) return -1;
@@ -272,146 +295,74 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
     while (v == 0u && w > 0) v = row[--w];
     return v ? (w << 5) + 31 - __clz(v) : -1;
   };
-  // the last position of label m in row i at or before column x: run by run
-  auto last_of = [&](int i, int x, int m) -> int {
-    for (;;) {
-      x = last_at(pos + i * Ww, x);
-      if (x < 0 || lab[i * W + x] == m) return x;
-      x = last_at(first + i * Ww, x) - 1;
-    }
-  };
-  // the number, within the row, of the run that holds column x
-  auto run_of = [&](int i, int x) -> int {
-    int n = -1;
-    for (int w = 0; w < x >> 5; ++w) n += __popc(first[i * Ww + w]);
-    return n + __popc(first[i * Ww + (x >> 5)] & (0xffffffffu >> (31 - (x & 31))));
-  };
   for (int w = warp; w < nw; w += kScheduleThreads / 32) {
     const int i = w / Ww, j = (w % Ww) * 32 + lane;
-    if (j >= W) continue;
-    const int t = i * W + j, m = lab[t];
-    int r = -1, u = -1;
-    if (m > 0) {
-      r = run_of(i, j);
-      if (i > 0) u = last_of(i - 1, min(W - 1, j + a.window - 1), m);
-      if (j + 1 == W || lab[t + 1] != m) {   // the run's last position enters it in the row's table
-        const int l = last_of(i, last_at(first + i * Ww, j) - 1, m);
-        table[i * W + r] = (l >= 0 ? run_of(i, l) : -1) << 16 | j;
-        const int nr = run_of(i, W - 1) + 1;
-        if (l >= 0) linked[i] = (Linked)nr;
-        if (nr > 32) s_many = 1;
-      }
+    if (!(pos[w] >> lane & 1u)) continue;
+    const int m = lab[i * W + j], at = slot[i * W + j];
+    int u = 0xffff;
+    if (i > 0) {   // the island's last position of the row above inside the window: run by run
+      int x = last_at(pos + (i - 1) * Ww, min(W - 1, j + a.window - 1));
+      while (x >= 0 && lab[(i - 1) * W + x] != m) x = last_at(pos + (i - 1) * Ww, last_at(first + (i - 1) * Ww, x) - 1);
+      if (x >= 0) u = slot[(i - 1) * W + x];
     }
-    place[t] = r << 16 | (u & 0xffff);
+    dep[i * W + at] = (uint32_t)u | (uint32_t)(at - head[i * W + at]) << 16;
   }
   __syncthreads();
   if (warp == 0) {
-    // the key of a position: what the row above demands, less its column, plus its run's term
-    auto key = [&](int pl, int j, const int* above) -> int {
-      const int u = pl & 0xffff, r = pl >> 16;
-      const int d = u != 0xffff ? above[u] + 1 : 1;
-      return r >= 0 ? d - j + r * kRunTerm : INT_MIN;
-    };
-    // Chains of runs: run r hands on max(c + len, its last step); maps of this kind composed by doubling (lane r: run r).
-    // Returns the step before the run's first one that its predecessor demands (0: none); beg: that first column.
-    auto follow = [&](int i, int nr, const int* row, int& beg) -> int {
-      int top = 0, len = 0, p = -1;
-      beg = 0;
-      if (lane < nr) {
-        const int e = table[i * W + lane];
-        p = e >> 16;
-        top = row[e & 0xffff];
-        beg = last_at(first + i * Ww, e & 0xffff);
-        len = (e & 0xffff) - beg + 1;
-      }
-      const int p0 = p;
-      while (__any_sync(0xffffffffu, p >= 0)) {
-        const int q = max(p, 0);
-        const int t2 = __shfl_sync(0xffffffffu, top, q), l2 = __shfl_sync(0xffffffffu, len, q), p2 = __shfl_sync(0xffffffffu, p, q);
-        if (p >= 0) {
-          top = max(top, t2 + len);
-          len += l2;
-          p = p2;
-        }
-      }
-      const int c = __shfl_sync(0xffffffffu, top, max(p0, 0));
-      return p0 >= 0 ? c : 0;
-    };
-    int* row = lab;
-    if (Ww <= 2 && !s_many) {   // a row is two values per lane, which stay in registers
-      const int j0 = lane, j1 = min(32 + lane, W - 1);
-      const bool in0 = j0 < W, in1 = 32 + lane < W;
-      for (int i = 0; i < H; ++i, row += W) {
-        const int nr = linked[i], p0 = in0 ? place[i * W + j0] : -1, p1 = in1 ? place[i * W + j1] : -1;
-        int v0 = key(p0, j0, row - W), v1 = key(p1, j1, row - W);
+    const int turns = (W + 32 * M - 1) / (32 * M);
+    uint32_t d[M];
+    int h[M];
+    auto ask = [&](int i, int c) {   // (slots that are not used come last in a row: whatever they hold reaches nobody)
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          v0 = max(v0, __shfl_up_sync(0xffffffffu, v0, o));   // (the first lanes get their own value)
-          v1 = max(v1, __shfl_up_sync(0xffffffffu, v1, o));
-        }
-        v1 = max(v1, __shfl_sync(0xffffffffu, v0, 31));
-        const int r0 = p0 >> 16, r1 = p1 >> 16;
-        int s0 = r0 >= 0 ? v0 + j0 - r0 * kRunTerm : 0, s1 = r1 >= 0 ? v1 + j1 - r1 * kRunTerm : 0;
-        if (in0) row[j0] = s0;
-        if (in1) row[j1] = s1;
-        __syncwarp();
-        if (nr > 0) {
-          int beg;
-          const int c = follow(i, nr, row, beg);
-          const int c0 = __shfl_sync(0xffffffffu, c, r0 & 31), c1 = __shfl_sync(0xffffffffu, c, r1 & 31);
-          const int b0 = __shfl_sync(0xffffffffu, beg, r0 & 31), b1 = __shfl_sync(0xffffffffu, beg, r1 & 31);
-          if (r0 >= 0 && c0 > 0) row[j0] = max(s0, c0 + 1 + j0 - b0);
-          if (r1 >= 0 && c1 > 0) row[j1] = max(s1, c1 + 1 + j1 - b1);
-          __syncwarp();
+      for (int k = 0; k < M; ++k) {
+        const int q = (c * 32 + lane) * M + k;
+        d[k] = 0xffffu;
+        h[k] = 0;
+        if (q < W && i < H) {
+          d[k] = dep[i * W + q];
+          h[k] = head[i * W + q];
         }
       }
-    } else {
-      for (int i = 0; i < H; ++i, row += W) {
-        int carry = INT_MIN;
-        for (int w = 0; w < Ww; ++w) {
-          const int j = (w << 5) + lane, pl = j < W ? place[i * W + j] : -1, r = pl >> 16;
-          int v = key(pl, j, row - W);
+    };
+    ask(0, 0);
+    const uint16_t* above = steps;
+    for (int i = 0; i < H; ++i) {
+      int carry = INT_MIN;
+      for (int c = 0; c < turns; ++c) {
+        int v[M], back[M];   // back: what turns a key into the step again
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) v = max(v, __shfl_up_sync(0xffffffffu, v, o));
-          v = max(v, carry);
-          carry = __shfl_sync(0xffffffffu, v, 31);
-          if (j < W) row[j] = r >= 0 ? v + j - r * kRunTerm : 0;
+        for (int k = 0; k < M; ++k) {
+          const uint32_t u = d[k] & 0xffffu;
+          back[k] = (int)(d[k] >> 16) - h[k] * kIslandTerm;
+          v[k] = (u != 0xffffu ? (int)above[u] + 1 : 1) - back[k];
         }
-        __syncwarp();
-        const int nr = linked[i];
-        if (nr == 0) continue;
-        int c = 0, beg = 0;
-        if (nr <= 32) {
-          c = follow(i, nr, row, beg);
-        } else {   // run by run
-          if (lane == 0)
-            for (int r = 0; r < nr; ++r) {
-              const int e = table[i * W + r] & 0xffff, p = table[i * W + r] >> 16;
-              if (p >= 0) row[e] = max(row[e], row[table[i * W + p] & 0xffff] + e - last_at(first + i * Ww, e) + 1);
-            }
-          __syncwarp();
+        if (c + 1 < turns) ask(i, c + 1);
+        else ask(i + 1, 0);
+#pragma unroll
+        for (int k = 1; k < M; ++k) v[k] = max(v[k], v[k - 1]);
+        int inc = v[M - 1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) inc = max(inc, __shfl_up_sync(0xffffffffu, inc, o));   // (the first lanes get their own)
+        int exc = __shfl_up_sync(0xffffffffu, inc, 1);
+        exc = max(lane == 0 ? INT_MIN : exc, carry);
+        if (turns > 1) carry = max(carry, __shfl_sync(0xffffffffu, inc, 31));
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+          const int q = (c * 32 + lane) * M + k;
+          if (q < W) steps[i * W + q] = (uint16_t)(max(v[k], exc) + back[k]);
         }
-        for (int w = 0; w < Ww; ++w) {
-          const int j = (w << 5) + lane, r = j < W ? place[i * W + j] >> 16 : -1;
-          int cr = 0, br = 0;
-          if (nr <= 32) {
-            cr = __shfl_sync(0xffffffffu, c, r & 31);
-            br = __shfl_sync(0xffffffffu, beg, r & 31);
-          } else if (r >= 0 && (table[i * W + r] >> 16) >= 0) {
-            cr = row[table[i * W + (table[i * W + r] >> 16)] & 0xffff];
-            br = last_at(first + i * Ww, j);
-          }
-          if (r >= 0 && cr > 0) row[j] = max(row[j], cr + 1 + j - br);
-        }
-        __syncwarp();
       }
+      __syncwarp();
+      above = steps + i * W;
     }
   }
   __syncthreads();
   int mine = 0;
-  for (int t = tid; t < N; t += kScheduleThreads) {
-    const int s = lab[t];
-    a.step[(size_t)b * N + t] = s;
+  for (int w = warp; w < nw; w += kScheduleThreads / 32) {
+    const int i = w / Ww, j = (w % Ww) * 32 + lane;
+    if (j >= W) continue;
+    const int s = pos[w] >> lane & 1u ? (int)steps[i * W + slot[i * W + j]] : 0;
+    a.step[(size_t)b * N + i * W + j] = s;
     mine = max(mine, s);
   }
   mine = __reduce_max_sync(0xffffffffu, mine);
