@@ -15,8 +15,8 @@
 //              with here (their exp replaces the logit in the list); those in the window go into a 256-bin
 //              histogram and a bit mask.
 //   selection  the bin that holds the k-th largest; the window's entries once more: above the bin -> exp, below
-//              -> 0, in the bin -> set aside, ranked exactly, written back.  From here on the list holds the
-//              row's weights, zeros below the threshold included.
+//              -> 0, in the bin -> set aside and ranked exactly; then each thread turns its own ones into weights (a bit
+//              mask says which).  From here on the list holds the row's weights, zeros below the threshold included.
 //   draws      sums of p (target) or of max(0, p - q) (residual; the sum of p minus that of min(p, q) over the ids
 //              that both rows kept, found by intersecting the masks) per thread and group.  The group that owns
 //              u * total is searched by the whole CTA, a mask word or so per eight threads; the owner's warp takes
@@ -93,7 +93,6 @@ struct RowsSmem {
   unsigned spill[32];                      // where the entries outside the window are counted
   alignas(16) float closer[4][32];         // -inf: what a thread past its list's end reads
   alignas(16) float sa_z[kRSetAside];      // (before the set-aside: where such a thread writes)
-  unsigned short sa_at[kRSetAside];        // the entry's place (index in its owner's list << 8 | thread)
   RowPredictor pred[2];                   // draft rows / target rows
   double w_all[NW];                        // exp sums of each warp without the crossing bin
   double w_draw[2][NW * 4];                // weights of a draw, per group; consecutive draws alternate
@@ -654,15 +653,16 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
   };
 
   // ---- the window's entries once more (after the crossing bin is known): the exp of those above it and 0 for those
-  //      below replace the logit (draft row: those below leave the draft list); returns the exp sum of those above
-  auto window = [&](uint32_t low_a, uint32_t low_b, float inv_w, float hoff, float c0, int bstar) -> float {
+  //      below replace the logit (draft row: those below leave the draft list); returns the exp sum of those above.  Of the
+  //      masks, the entries in the crossing bin are left, which keep their logits.
+  const uint32_t flip = up ? 0u : 3u;      // (a mask's bits run along memory)
+  auto window = [&](uint32_t& low_a, uint32_t& low_b, float inv_w, float hoff, float c0, int bstar) -> float {
     const float hm = hoff + kRMagic;
     const uint32_t bm = __float_as_uint(kRMagic) + (uint32_t)bstar;
-    const uint32_t flip = up ? 0u : 3u;
     float s = 0.f;
     uint32_t first = 0;
-    auto one = [&](uint32_t bit, uint32_t& i, float& z) -> bool {   // does the entry lie in the crossing bin?
-      i = first + ((uint32_t)__popc(bit - 1u) ^ flip);
+    auto one = [&](uint32_t bit, float& z) -> bool {   // does the entry lie in the crossing bin?
+      const uint32_t i = first + ((uint32_t)__popc(bit - 1u) ^ flip);
       const uint32_t at = tl + i * step;
       z = lds_f32(bit ? at : closer);
       const uint32_t bin = __float_as_uint(fmaf(z, inv_w, hm));   // (-inf: as unsigned above every bin; its exp is 0)
@@ -672,35 +672,37 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       if (is_q) {
         if (bin < bm) dlist_put<BF16>(dl + i * dstep, -INFINITY);
       } else {
-        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(at), "f"(e), "r"(bit) : "memory");
+        const uint32_t there = bin == bm ? 0u : bit;
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.shared.f32 [%0], %1;\n\t}" ::"r"(at), "f"(e), "r"(there) : "memory");
       }
       return bin == bm;
     };
-    auto aside = [&](uint32_t i, float z) {
-      const unsigned k = atomicAdd(&sm.n_sa, 1u) & (unsigned)(kRSetAside - 1);
-      sm.sa_z[k] = z;
-      sm.sa_at[k] = (unsigned short)(i << 8 | (uint32_t)tid);
-    };
+    auto aside = [&](float z) { sm.sa_z[atomicAdd(&sm.n_sa, 1u) & (unsigned)(kRSetAside - 1)] = z; };
+    uint32_t left_a = 0;
 #pragma unroll 1
     for (int h = 0; h < 2; ++h) {
       const int trips = __reduce_max_sync(kFull, __popc(low_a));
+      uint32_t left = 0;
 #pragma unroll 1
       for (int t = 0; t < trips; t += 2) {
         const uint32_t b0 = low_a & (0u - low_a);
         low_a ^= b0;
         const uint32_t b1 = low_a & (0u - low_a);
         low_a ^= b1;
-        uint32_t i0, i1;
         float z0, z1;
-        const bool h0 = one(b0, i0, z0), h1 = one(b1, i1, z1);
+        const bool h0 = one(b0, z0), h1 = one(b1, z1);
         if (h0 || h1) {
-          if (h0) aside(i0, z0);
-          if (h1) aside(i1, z1);
+          if (h0) aside(z0);
+          if (h1) aside(z1);
+          left |= (h0 ? b0 : 0u) | (h1 ? b1 : 0u);
         }
       }
+      if (h == 0) left_a = left;
       low_a = low_b;
+      low_b = left;
       first = 32;
     }
+    low_a = left_a;
     return s;
   };
 
@@ -904,7 +906,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
 #pragma unroll 1
     for (int i = tid; i < kRBins + 4; i += NT) sm.hist[i] = 0;
     if (reason == 0) {
-      // ---- the crossing bin's entries: exact rank, and back into the lists
+      // ---- the crossing bin's entries: exact rank, and their weights
       const int want = rank - (int)cum, mcount = (int)in_bin;
       float vmin = INFINITY, vmax = -INFINITY;
 #pragma unroll 1
@@ -954,16 +956,20 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       }
       if (kmin != kmax || !is_q) {   // (a draft row keeps its logits: nothing changes unless some fall below)
         double own = 0.0;
+        uint32_t at = tl;
 #pragma unroll 1
-        for (int i = 0; i < mcount; ++i) {
-          const uint32_t at = sm.sa_at[i];
-          if ((int)(at & 0xffu) == tid) {
-            const float v = sm.sa_z[i];
+        for (int h = 0; h < 2; ++h) {   // this thread's own
+#pragma unroll 1
+          for (; low_a; low_a &= low_a - 1u) {
+            const uint32_t i = (uint32_t)(__ffs(low_a) - 1) ^ flip;
+            const float v = lds_f32(at + i * step);
             const float e = v >= theta ? ex2f(fmaf(v, kLog2e, c0)) : 0.f;
             own += (double)e;
-            if (!is_q) sts_f32(tl + (at >> 8) * step, e);
-            else if (!(v >= theta)) dlist_put<BF16>(dl + (at >> 8) * dstep, -INFINITY);
+            if (!is_q) sts_f32(at + i * step, e);
+            else if (!(v >= theta)) dlist_put<BF16>(dl + (i + 32 * h) * dstep, -INFINITY);
           }
+          low_a = low_b;
+          at += 32 * step;
         }
         s_t = (float)((double)s_t + own);
       }
