@@ -172,6 +172,8 @@ __global__ void __launch_bounds__(kThreads, RES ? 2 : 3) k_sample_failed(RowKern
                                                             const uint32_t* fail_count) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GeneralScratch<RES> sc;
+  let_next_begin();
+  wait_for_previous();
   const size_t total = (size_t)a.P.B * a.P.h * a.P.w;
   const size_t n = min((size_t)*fail_count, total);
   for (size_t idx = blockIdx.x; idx < n; idx += gridDim.x) {
@@ -347,6 +349,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_verify_failed(RowKernelArgs a, 
                                                             const uint32_t* fail_count) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GeneralScratch<RES> sc;
+  let_next_begin();
+  wait_for_previous();
   const DevParams& P = a.P;
   const int N = P.H * P.W;
   const size_t total = (size_t)P.B * N;
@@ -459,6 +463,7 @@ __global__ void __launch_bounds__(kMaskThreads) k_mask(MaskArgs a) {
   uint32_t* ex = words + 2 * nw;
   __shared__ int s_nrej, s_first, s_nexp;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  wait_for_previous();
   if (tid == 0) {
     s_nrej = 0;
     s_first = N;
@@ -830,6 +835,25 @@ static int ctas_per_sm(mulo_ctx* ctx, K kernel, int threads, size_t dyn) {
   return per_sm;
 }
 
+// Launches a kernel that may begin while the one before it in the stream still runs (it waits for it itself: wait_for_previous).
+template <class... P, class... A>
+static bool launch_after(void (*kernel)(P...), unsigned grid, int threads, size_t dyn, cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof cfg);
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = dyn;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kernel, P(args)...) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
+}
+
 // Launches one of the general path's kernels in the version for this vocabulary; false if it cannot run.
 #define MULO_LAUNCH_GENERAL(KERNEL, grid, dyn, st, ...)                                     \
   (resident_fits(a.P.V)                                                                     \
@@ -840,6 +864,13 @@ static bool launch_general(mulo_ctx* ctx, K kernel, unsigned grid, size_t dyn, c
   if (ctas_per_sm(ctx, kernel, kThreads, dyn) < 1) return false;
   kernel<<<grid, kThreads, dyn, st>>>(args...);
   return true;
+}
+// ... for the rows that a fast kernel left, after it.
+#define MULO_LAUNCH_LEFT(KERNEL, dyn, st, ...) \
+  (resident_fits(a.P.V) ? launch_left(ctx, KERNEL(true), dyn, st, __VA_ARGS__) : launch_left(ctx, KERNEL(false), dyn, st, __VA_ARGS__))
+template <class K, class... A>
+static bool launch_left(mulo_ctx* ctx, K kernel, size_t dyn, cudaStream_t st, const A&... args) {
+  return ctas_per_sm(ctx, kernel, kThreads, dyn) >= 1 && launch_after(kernel, 2u * (unsigned)ctx->sm_count, kThreads, dyn, st, args...);
 }
 #define K_UPSAMPLE(RES) k_upsample_pool<RES>
 #define K_SAMPLE(RES) k_sample_draft<RES>
@@ -1309,7 +1340,7 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
     ra.n_units = p->B * a.P.h * a.P.w;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
     if (launch_rows(ctx, ra, true, rnw, rdyn, st)) {
-      if (!MULO_LAUNCH_GENERAL(K_SAMPLE_FAILED, 2 * ctx->sm_count, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+      if (!MULO_LAUNCH_LEFT(K_SAMPLE_FAILED, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
       return launched(ctx, 2);
     }
   }
@@ -1325,7 +1356,7 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
     const bool fast = a.P.bf16 ? launch_stream_t<true, false, true>(ctx, sa, sdyn, st)
                                : launch_stream_t<false, false, true>(ctx, sa, sdyn, st);
     if (fast) {
-      if (!MULO_LAUNCH_GENERAL(K_SAMPLE_FAILED, 2 * ctx->sm_count, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+      if (!MULO_LAUNCH_LEFT(K_SAMPLE_FAILED, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
       return launched(ctx, 2);
     }
   }
@@ -1384,7 +1415,7 @@ mulo_status mulo_verify(mulo_ctx* ctx, const mulo_params* p, const void* tgt_con
   m.H = p->H; m.W = p->W; m.r = p->r; m.radius = p->radius; m.clip = a.P.clip; m.resample_mode = p->resample_mode;
   m.flags = w.flags;
   m.reject_bits = reject_bits; m.n_reject = n_reject; m.first_reject = first_reject;
-  k_mask<0><<<p->B, kMaskThreads, mask_smem(p), st>>>(m);
+  if (!launch_after(k_mask<0>, (unsigned)p->B, kMaskThreads, mask_smem(p), st, m)) return MULO_ERR_CUDA;
   return launched(ctx, 2);
 }
 
@@ -1537,7 +1568,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     ra.n_units = p->B * p->H * p->W;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
     fast = launch_rows(ctx, ra, false, rnw, rdyn, st);
-    if (fast && !MULO_LAUNCH_GENERAL(K_ROUND_FAILED, 2 * ctx->sm_count, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+    if (fast && !MULO_LAUNCH_LEFT(K_ROUND_FAILED, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
   }
   StreamArgs sa;
   memset(&sa, 0, sizeof sa);
@@ -1554,7 +1585,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
     fast = launch_stream(ctx, sa, sdyn, st);
     // the rows the streaming kernel gave up on (usually a handful, often none)
-    if (fast && !MULO_LAUNCH_GENERAL(K_ROUND_FAILED, 2 * ctx->sm_count, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+    if (fast && !MULO_LAUNCH_LEFT(K_ROUND_FAILED, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
   }
   if (!fast && !MULO_LAUNCH_GENERAL(K_ROUND, p->B * a.P.h * a.P.w, dyn, st, a)) return MULO_ERR_UNSUPPORTED;
   if (timed) {
@@ -1569,7 +1600,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
   m.n_reject = n_reject; m.first_reject = first_reject; m.n_expand = n_expand;
   m.cand_res = w.cand_res; m.cand_tgt = w.cand_tgt;
   m.draft_tok_lo = draft_tok_lo; m.out_tok = out_tok;
-  k_mask<2><<<p->B, kMaskThreads, mask_smem(p), st>>>(m);
+  if (!launch_after(k_mask<2>, (unsigned)p->B, kMaskThreads, mask_smem(p), st, m)) return MULO_ERR_CUDA;
   return launched(ctx, fast ? 1 + fast_launches : 2);
 }
 

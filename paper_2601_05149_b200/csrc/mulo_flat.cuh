@@ -135,6 +135,7 @@ __global__ void __launch_bounds__((RES ? kFlatResWarps : kFlatWarps) * 32, (SAMP
   __shared__ FlatSmem<NW> sm;
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  let_next_begin();
   int unit = (int)(((long long)a.n_units * blockIdx.x) / gridDim.x);
   const int u_end = (int)(((long long)a.n_units * (blockIdx.x + 1)) / gridDim.x);
   if (unit >= u_end) return;

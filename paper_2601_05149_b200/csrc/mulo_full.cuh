@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_round_full(const __grid_consta
   __shared__ FullSmem sm;
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  let_next_begin();
   const int u_begin = (int)(((long long)a.n_units * blockIdx.x) / gridDim.x);
   const int u_end = (int)(((long long)a.n_units * (blockIdx.x + 1)) / gridDim.x);
   if (u_end <= u_begin) return;

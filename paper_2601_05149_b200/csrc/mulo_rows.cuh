@@ -409,6 +409,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
   __shared__ RowsSmem<NW, POOL> sm;
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  let_next_begin();
   int unit = (int)(((long long)a.n_units * blockIdx.x) / gridDim.x);
   const int u_end = (int)(((long long)a.n_units * (blockIdx.x + 1)) / gridDim.x);
   if (unit >= u_end) return;

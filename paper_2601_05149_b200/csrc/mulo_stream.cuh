@@ -469,6 +469,7 @@ __global__ void __launch_bounds__(kSThreads, 3) k_round_stream(const __grid_cons
   extern __shared__ __align__(128) unsigned char dyn[];
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  let_next_begin();
   // In the list passes a warp's lanes split into up to four groups, one segment per group
   // at a time (group g takes the warp's segment of chunk g, g + groups, ...).
   const int groups = a.n_chunks >= 3 ? 4 : a.n_chunks;   // 1, 2 or 4
