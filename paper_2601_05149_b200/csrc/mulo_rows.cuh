@@ -22,9 +22,10 @@
 //              u * total is searched by the whole CTA, a mask word or so per eight threads; the owner's warp takes
 //              it from there (piece, lane, id) while the others go on with the next row.
 //   pooling    (POOL, Eq. 3-4) between selection and decision: the neighbour list of x~ is walked in tiles, eight
-//              entries per thread, their logits gathered from the row (L2); prefix masses by block scan; the pooled ids'
-//              weights leave the lists (found by popcount on the survivor masks) and their owners' sums (64-bit fixed
-//              point, so the order does not matter).  x~ carries its pooled weight outside the lists.
+//              entries per thread, their weights found in the lists by popcount on the survivor masks (most neighbours are not
+//              kept at all, which their mask bit says); prefix masses by block scan; the pooled ids' weights change their sign,
+//              which counts as nothing from then on, and leave their owners' sums (64-bit fixed point, so the order does not
+//              matter).  x~ carries its pooled weight outside the lists.
 //
 // Three block barriers per draft row, four per target row.  Pivot, histogram scale and exp reference are predicted from the CTA's previous
 // rows of the same kind; a row without prediction takes them from the mean and spread of its first pieces.  A
@@ -365,30 +366,6 @@ __device__ __forceinline__ int pool_id(const uint4& v, int i) {
   const uint32_t w = i < 2 ? v.x : i < 4 ? v.y : i < 6 ? v.z : v.w;
   return (int)(w >> (16 * (i & 1)) & 0xffffu);
 }
-// Their logits, in two steps: every load is asked for before one is used.  One entry after the other, that was sixteen
-// round trips to L2 instead of two: 11.5 k of the 25 k cycles that a CTA spent on a pooled row.
-template <bool BF16, bool HAS_U>
-struct PoolRaw {
-  using T = typename std::conditional<BF16, unsigned short, float>::type;
-  T c[8], u[HAS_U ? 8 : 1];
-  __device__ __forceinline__ void ask(const uint4& v, const char* rc, const char* ru) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      c[i] = __ldg(reinterpret_cast<const T*>(rc) + pool_id(v, i));
-      if constexpr (HAS_U) u[i] = __ldg(reinterpret_cast<const T*>(ru) + pool_id(v, i));
-    }
-  }
-  static __device__ __forceinline__ float wide(T v) {
-    if constexpr (BF16) return __uint_as_float((uint32_t)v << 16);
-    else return v;
-  }
-  __device__ __forceinline__ float z(int i, const DevParams& P) const {
-    float uw = 0.f;
-    if constexpr (HAS_U) uw = wide(u[i]);
-    return mix_logit(wide(c[i]), uw, HAS_U, P.cfg_scale, P.invT);
-  }
-};
-
 // Asks a neighbour list into L2 (one thread; the whole 16 bytes in it).
 __device__ __forceinline__ void pool_prefetch(const uint16_t* row, int pool_k) {
   const uintptr_t from = ((uintptr_t)row + 15) & ~(uintptr_t)15, to = (uintptr_t)(row + pool_k) & ~(uintptr_t)15;
@@ -1070,37 +1047,42 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       };
       const Spot tok_spot = POOL ? spot_of(tok) : Spot{-1, 0, 0u};
       if constexpr (POOL) {
-        // takes the entries of kept ids (those with `in`) out of their owners' lists and sums, N at a time
-        auto remove = [&](auto n_tag, const int* x, const bool* in) {
+        // where N ids' weights are in the lists, and whose (<< 20); 0: not kept
+        auto find = [&](auto n_tag, const int* x, uint32_t* at) {
           constexpr int N = decltype(n_tag)::value;
-          uint32_t at[N], tm_at[N], last[N];
           Spot sp[N];
+          uint32_t tm_at[N], last[N];
 #pragma unroll
           for (int i = 0; i < N; ++i) {
-            sp[i] = spot_of(in[i] ? x[i] : 0);
+            sp[i] = spot_of(max(x[i], 0));
             const bool o_up = ((sp[i].thread >> 5) & 1) == 0;
             tm_at[i] = my + a.o_tmask + (uint32_t)sp[i].thread * 4u;
             at[i] = my + ((uint32_t)(sp[i].thread >> 6) * (uint32_t)R + (o_up ? 0u : (uint32_t)(R - 1))) * 128u +
                     (((uint32_t)sp[i].thread & 31u) ^ (o_up ? 0u : rot)) * 4u;
-            last[i] = 0u;
+            last[i] = x[i] >= 0 ? lds_u32(tm_at[i] + (uint32_t)(sp[i].word * NT) * 4u) & sp[i].bit : 0u;
           }
-#pragma unroll 1
-          for (int w = 0; w < n_words; ++w) {
+          bool any = false;
 #pragma unroll
-            for (int i = 0; i < N; ++i) {   // entries of the words before the id's, of its own those below it
-              const uint32_t m = lds_u32(tm_at[i] + (uint32_t)(w * NT) * 4u);
-              const int n = __popc(w < sp[i].word ? m : w == sp[i].word ? m & (sp[i].bit - 1u) : 0u);
-              at[i] += (uint32_t)(sp[i].thread & 32 ? -n : n) * 128u;
-              if (w == sp[i].word) last[i] = m & sp[i].bit;
+          for (int i = 0; i < N; ++i) any = any || last[i];
+          if (__any_sync(kFull, any)) {
+#pragma unroll 1
+            for (int w = 0; w < n_words; ++w) {
+#pragma unroll
+              for (int i = 0; i < N; ++i) {   // entries of the words before the id's, of its own those below it
+                const uint32_t m = lds_u32(tm_at[i] + (uint32_t)(w * NT) * 4u);
+                const int n = __popc(w < sp[i].word ? m : w == sp[i].word ? m & (sp[i].bit - 1u) : 0u);
+                at[i] += (uint32_t)(sp[i].thread & 32 ? -n : n) * 128u;
+              }
             }
           }
-          uint32_t old[N];   // (a list may name an id twice, or x~ itself)
 #pragma unroll
-          for (int i = 0; i < N; ++i)
-            asm volatile("atom.shared.exch.b32 %0, [%1], %2;" : "=r"(old[i]) : "r"(in[i] && last[i] ? at[i] : spill), "r"(0u) : "memory");
-#pragma unroll
-          for (int i = 0; i < N; ++i)
-            if (in[i] && last[i]) atomicAdd(&sm.adj[sp[i].thread], __float2ull_rz(__uint_as_float(old[i]) * 1099511627776.0f));
+          for (int i = 0; i < N; ++i) at[i] = last[i] ? at[i] | (uint32_t)sp[i].thread << 20 : 0u;
+        };
+        // takes a weight out of its owner's list and sum (a list may name an id twice, or x~ itself)
+        auto remove = [&](float w, uint32_t at) {
+          uint32_t old;
+          asm volatile("atom.shared.exch.b32 %0, [%1], %2;" : "=r"(old) : "r"(at & 0xfffffu), "r"(__float_as_uint(-w)) : "memory");
+          if (__uint_as_float(old) > 0.f) atomicAdd(&sm.adj[at >> 20], __float2ull_rz(w * 1099511627776.0f));
         };
         const uint16_t* const list = a.nn + (size_t)tok * P.pool_k;   // (x~ first)
         const int nb = P.pool_k;
@@ -1108,27 +1090,26 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         double carry = 0.0;
         sm.adj[tid] = 0ull;
         if (tid == 0) sm.pool_cj = 0.0;
+        __syncthreads();   // (every thread's entries are weights)
         int tile = 0;
 #pragma unroll 1
         for (int base = 0; base < nb; base += NT * 8, ++tile) {
           const int j0 = base + tid * 8;
           float e[8];
           int id[8];
+          uint32_t at[8];
           double sum = 0.0;
           {
             uint4 ids = pool_ids(list, nb, j0);
             if (pool_clamp(ids, j0 == 0, P.V)) atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
-            PoolRaw<BF16, HAS_U> raw;
-            raw.ask(ids, rc, ru);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) id[i] = pool_id(ids, i);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) e[i] = raw.z(i, P);
+            for (int i = 0; i < 8; ++i) id[i] = j0 + i < 1 || j0 + i >= nb ? -1 : pool_id(ids, i);
           }
+          find(std::integral_constant<int, 4>{}, id, at);
+          find(std::integral_constant<int, 4>{}, id + 4, at + 4);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            if (j0 + i < 1 || j0 + i >= nb) id[i] = -1;
-            e[i] = id[i] >= 0 && e[i] >= theta ? ex2f(fmaf(e[i], kLog2e, c0)) : 0.f;
+            e[i] = at[i] ? fabsf(lds_f32(at[i] & 0xfffffu)) : 0.f;
             sum += (double)e[i];
           }
           double inc = sum;
@@ -1171,18 +1152,16 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
               run += (double)e[i];
               if (j0 + i == J - 1 || (j0 + i == base + NT * 8 - 1)) sm.pool_cj = run;
             }
-            in[i] = in[i] && e[i] > 0.f;
+            if (in[i] && e[i] > 0.f) remove(e[i], at[i]);
           }
-#pragma unroll
-          for (int i = 0; i < 8; i += 4)
-            if (__any_sync(kFull, in[i] || in[i + 1] || in[i + 2] || in[i + 3])) remove(std::integral_constant<int, 4>{}, id + i, in + i);
           if (J < nb) break;   // (uniform)
           __syncthreads();     // (the last tile's prefix mass before the next one's)
         }
-        if (warp == NW - 1 && e_tok > 0.0) {
-          const bool one = lane == 0;
-          remove(std::integral_constant<int, 1>{}, &tok, &one);
-        }   // x~ is drawn with its pooled weight, outside the lists
+        if (warp == NW - 1 && e_tok > 0.0) {   // x~ is drawn with its pooled weight, outside the lists
+          uint32_t at;
+          find(std::integral_constant<int, 1>{}, &tok, &at);
+          if (lane == 0 && at) remove(fabsf(lds_f32(at & 0xfffffu)), at);
+        }
         __syncthreads();
         mass = e_tok + sm.pool_cj;
         s_t = (float)fmax((double)s_t - (double)sm.adj[tid] * (1.0 / 1099511627776.0), 0.0);
@@ -1239,7 +1218,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
               im ^= bit;
               const float e = lds_f32(tp + (uint32_t)__popc(m & below) * step);
               const float q = q_weight(dp + (uint32_t)__popc(d & below) * dstep);
-              return bit ? fminf(e, q) : 0.f;
+              return bit ? fminf(POOL ? fmaxf(e, 0.f) : e, q) : 0.f;
             };
 #pragma unroll 1
             for (int i = 0; i < trips; i += 4) {   // four at a time: their chains overlap
