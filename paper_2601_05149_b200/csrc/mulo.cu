@@ -208,6 +208,7 @@ constexpr int kScanThreads = 1024;
 
 __global__ void __launch_bounds__(256) k_redraw_count(const int32_t* __restrict__ step, int n, int max_step,
                                                       int32_t* cursor) {
+  let_next_begin();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int s = step[i];
     if (s >= 1 && s <= max_step) atomicAdd(&cursor[s], 1);
@@ -217,6 +218,8 @@ __global__ void __launch_bounds__(256) k_redraw_count(const int32_t* __restrict_
 __global__ void __launch_bounds__(kScanThreads) k_redraw_scan(int max_step, int32_t* offsets, int32_t* cursor) {
   __shared__ int warp_tot[kScanThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  let_next_begin();
+  wait_for_previous();
   const int n = max_step + 1;                       // entries 0 .. max_step (entry 0 counts nothing)
   const int per = (n + kScanThreads - 1) / kScanThreads;
   const int beg = min(n, tid * per), end = min(n, beg + per);
@@ -244,6 +247,7 @@ __global__ void __launch_bounds__(kScanThreads) k_redraw_scan(int max_step, int3
 
 __global__ void __launch_bounds__(256) k_redraw_fill(const int32_t* __restrict__ step, int n, int max_step,
                                                      int32_t* cursor, int32_t* pos_list) {
+  wait_for_previous();   // (the first step is not let in early: its list is being written)
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int s = step[i];
     if (s >= 1 && s <= max_step) pos_list[atomicAdd(&cursor[s], 1)] = i;
@@ -252,9 +256,11 @@ __global__ void __launch_bounds__(256) k_redraw_fill(const int32_t* __restrict__
 
 // mulo_downsample: one thread per low-res cell; the most frequent token of its r x r block,
 // ties to the one that comes first in raster order of the block (Step 7 stand-in).
-__global__ void __launch_bounds__(256) k_downsample(const int32_t* __restrict__ x, int32_t* __restrict__ y,
+__global__ void __launch_bounds__(256) k_downsample(const int32_t* x, int32_t* y,
                                                     int cells, int h, int w, int W, int r) {
   const int cell = blockIdx.x * blockDim.x + threadIdx.x;
+  let_next_begin();
+  wait_for_previous();
   if (cell >= cells) return;
   const int b = cell / (h * w), rem = cell % (h * w), ca = rem / w, cc = rem % w;
   const int32_t* blk = x + ((size_t)b * h * r + (size_t)ca * r) * W + (size_t)cc * r;
@@ -1354,7 +1360,7 @@ mulo_status mulo_island_schedule(mulo_ctx* ctx, const mulo_params* p, const int3
   const auto kernel = p->W <= 32 ? k_island_schedule<1> : p->W <= 64 ? k_island_schedule<2> : k_island_schedule<4>;
   const size_t smem = schedule_smem(p->H, p->W);
   if (ctas_per_sm(ctx, kernel, kScheduleThreads, smem) < 1) return MULO_ERR_UNSUPPORTED;
-  kernel<<<p->B, kScheduleThreads, smem, (cudaStream_t)stream>>>(a);
+  if (!launch_after(kernel, (unsigned)p->B, kScheduleThreads, smem, (cudaStream_t)stream, a)) return MULO_ERR_CUDA;
   return launched(ctx, 1);
 }
 
@@ -1373,8 +1379,9 @@ mulo_status mulo_redraw_plan(mulo_ctx* ctx, const mulo_params* p, const int32_t*
   if (n == 0) return MULO_OK;
   const int blocks = (n + 255) / 256 < 4 * ctx->sm_count ? (n + 255) / 256 : 4 * ctx->sm_count;
   k_redraw_count<<<blocks, 256, 0, st>>>(step, n, max_step, cursor);
-  k_redraw_scan<<<1, kScanThreads, 0, st>>>(max_step, step_offsets, cursor);
-  k_redraw_fill<<<blocks, 256, 0, st>>>(step, n, max_step, cursor, pos_list);
+  if (!launch_after(k_redraw_scan, 1u, kScanThreads, 0, st, max_step, step_offsets, cursor) ||
+      !launch_after(k_redraw_fill, (unsigned)blocks, 256, 0, st, step, n, max_step, cursor, pos_list))
+    return MULO_ERR_CUDA;
   return launched(ctx, 3);
 }
 
@@ -1518,7 +1525,8 @@ mulo_status mulo_downsample(mulo_ctx* ctx, const mulo_params* p, const int32_t* 
   if (p->B == 0) return MULO_OK;
   if ((s = on_context_device(ctx)) != MULO_OK) return s;
   const int h = p->H / p->r, w = p->W / p->r, cells = p->B * h * w;
-  k_downsample<<<(cells + 255) / 256, 256, 0, (cudaStream_t)stream>>>(tok_hi, tok_lo, cells, h, w, p->W, p->r);
+  if (!launch_after(k_downsample, (unsigned)((cells + 255) / 256), 256, 0, (cudaStream_t)stream, tok_hi, tok_lo, cells, h, w, p->W, p->r))
+    return MULO_ERR_CUDA;
   return launched(ctx, 1);
 }
 
@@ -1620,7 +1628,7 @@ mulo_status mulo_islands(mulo_ctx* ctx, const mulo_params* p, const uint32_t* ex
   a.size = max_islands > 0 ? island_size : nullptr;
   const size_t smem = ((size_t)2 * p->H * p->W + (size_t)p->H * ((p->W + 31) / 32)) * sizeof(int);
   if (ctas_per_sm(ctx, k_islands, kIslandThreads, smem) < 1) return MULO_ERR_UNSUPPORTED;
-  k_islands<<<p->B, kIslandThreads, smem, (cudaStream_t)stream>>>(a);
+  if (!launch_after(k_islands, (unsigned)p->B, kIslandThreads, smem, (cudaStream_t)stream, a)) return MULO_ERR_CUDA;
   return launched(ctx, 1);
 }
 

@@ -14,6 +14,8 @@
 #include <climits>
 #include <cstdint>
 
+#include "mulo_device.cuh"
+
 namespace mulo {
 
 constexpr int kIslandThreads = 1024;
@@ -66,6 +68,8 @@ __global__ void __launch_bounds__(kIslandThreads) k_islands(IslandArgs a) {
   __shared__ int s_carry;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
+  let_next_begin();
+  wait_for_previous();
   for (int w = tid; w < nw; w += kIslandThreads) {
     uint32_t v = a.bits[(size_t)b * nw + w];
     if (w % Ww == Ww - 1 && (W & 31)) v &= (1u << (W & 31)) - 1u;   // bits past the row's end do not count
@@ -248,6 +252,8 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
   uint16_t* const slot = head + N;                                          // by column
   __shared__ int s_max;
   if (tid == 0) s_max = 0;
+  let_next_begin();
+  wait_for_previous();
   const int32_t* const labels = a.labels + (size_t)b * N;
   for (int t = tid; t < N; t += kScheduleThreads) {
     lab[t] = labels[t];
