@@ -18,7 +18,9 @@
  *   - All tensor arguments are DEVICE pointers to caller-owned, contiguous,
  *     row-major memory, 16-byte aligned, unless the name says "host".  The
  *     library never allocates or frees device memory; scratch space is the
- *     workspace the caller hands to mulo_set_workspace.
+ *     workspace the caller hands to mulo_set_workspace.  A context's calls share it, so
+ *     those that read logits must not overlap on the device (one context per stream does it),
+ *     but for mulo_redraw_step, which needs none.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).
  *     Calls validate their arguments on the host, enqueue kernels on the stream
  *     and return; outputs are defined once the stream has been synchronised.  Nothing a

@@ -91,11 +91,8 @@ __device__ __forceinline__ void round_z(double& Z) {   // Z_q as the stages hand
 
 // mulo_upsample_pool: one CTA per low-res cell.
 template <bool RES>
-__global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_pool(RowKernelArgs a) {
-  extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ GeneralScratch<RES> sc;
+__device__ __forceinline__ void upsample_cell(const RowKernelArgs& a, int cell, GeneralScratch<RES>& sc, unsigned char* dyn) {
   const DevParams& P = a.P;
-  const int cell = blockIdx.x;   // b*h*w + ca*w + cc
   const int b = cell / (P.h * P.w), rem = cell % (P.h * P.w), ca = rem / P.w, cc = rem % P.w;
   RowSrc qr = draft_row(a, cell);
   const int tok = checked_token(a.draft_tok_lo[cell], P.V, a.dev_status);
@@ -121,6 +118,27 @@ __global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_pool(RowKern
         a.tok_hi_out[t] = a.draft_tok_lo[cell];
         a.q_tok_hi_out[t] = (float)q;
       }
+  }
+}
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_pool(RowKernelArgs a) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
+  upsample_cell<RES>(a, blockIdx.x, sc, dyn);   // b*h*w + ca*w + cc
+}
+// Second launch of its fast path: the cells the fast kernel put on its list.
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_failed(RowKernelArgs a, const int32_t* fail_list,
+                                                                           const uint32_t* fail_count) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
+  let_next_begin();
+  wait_for_previous();
+  const size_t total = (size_t)a.P.B * a.P.h * a.P.w, n = min((size_t)*fail_count, total);
+  for (size_t idx = blockIdx.x; idx < n; idx += gridDim.x) {
+    const size_t cell = (size_t)fail_list[idx];
+    if (cell < total) upsample_cell<RES>(a, (int)cell, sc, dyn);
+    __syncthreads();
   }
 }
 
@@ -303,6 +321,26 @@ __device__ __forceinline__ RowStats given_stats(const RowKernelArgs& a, size_t c
   return sq;
 }
 
+// One position of mulo_verify: draft statistics given.
+template <bool RES>
+__device__ __forceinline__ void verify_position(const RowKernelArgs& a, size_t g, GeneralScratch<RES>& sc, unsigned char* dyn) {
+  const DevParams& P = a.P;
+  const int N = P.H * P.W;
+  const int b = (int)(g / N), t = (int)(g % N), i = t / P.W, j = t % P.W;
+  const size_t cell = ((size_t)b * P.h + i / P.r) * P.w + j / P.r;
+  const RowStats sq = given_stats(a, cell);
+  const int tok = checked_token(a.draft_tok_hi[g], P.V, a.dev_status);
+  PositionOut o;
+  general_position<RES>(a, target_row(a, g), draft_row(a, cell), sq, tok, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
+                        [](int) { return (int)kDrawNone; }, sc, dyn, o);
+  if (threadIdx.x == 0) {
+    a.flags[g] = o.accepted ? 0 : 1;
+    a.p_tok[g] = o.p_tok;
+    a.q_tok[g] = o.q_tok;
+    a.accept_prob[g] = o.accept_prob;
+  }
+}
+
 // mulo_verify (FUSED = false): one CTA per target position, draft statistics given.
 // mulo_round  (FUSED = true):  one CTA per low-res cell: draft statistics, then its
 // r*r children; accept flags and candidate draws go to the workspace.
@@ -331,20 +369,22 @@ __global__ void __launch_bounds__(kThreads, 2) k_verify_rows(RowKernelArgs a) {
         __syncthreads();
       }
   } else {
-    const size_t g = blockIdx.x;
-    const int b = (int)(g / N), t = (int)(g % N), i = t / P.W, j = t % P.W;
-    const size_t cell = ((size_t)b * P.h + i / P.r) * P.w + j / P.r;
-    const RowStats sq = given_stats(a, cell);
-    const int tok = checked_token(a.draft_tok_hi[g], P.V, a.dev_status);
-    PositionOut o;
-    general_position<RES>(a, target_row(a, g), draft_row(a, cell), sq, tok, (uint32_t)b + P.image_offset, (uint32_t)t, true, 0,
-                          [](int) { return (int)kDrawNone; }, sc, dyn, o);
-    if (threadIdx.x == 0) {
-      a.flags[g] = o.accepted ? 0 : 1;
-      a.p_tok[g] = o.p_tok;
-      a.q_tok[g] = o.q_tok;
-      a.accept_prob[g] = o.accept_prob;
-    }
+    verify_position<RES>(a, blockIdx.x, sc, dyn);
+  }
+}
+
+// Second launch of mulo_verify's fast path: the positions the fast kernel put on its list.
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_verify_left(RowKernelArgs a, const int32_t* fail_list, const uint32_t* fail_count) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
+  let_next_begin();
+  wait_for_previous();
+  const size_t total = (size_t)a.P.B * a.P.H * a.P.W, n = min((size_t)*fail_count, total);
+  for (size_t idx = blockIdx.x; idx < n; idx += gridDim.x) {
+    const size_t g = (size_t)fail_list[idx];
+    if (g < total) verify_position<RES>(a, g, sc, dyn);
+    __syncthreads();
   }
 }
 
@@ -395,14 +435,11 @@ __device__ __forceinline__ bool covered_by_other(const uint32_t* rej, int Ww, in
   return false;
 }
 
-// mulo_resample: one CTA per target position; positions outside R_X copy x~.
+// One position of mulo_resample; positions outside R_X copy x~.
 template <bool RES>
-__global__ void __launch_bounds__(kThreads, 2) k_resample_rows(RowKernelArgs a) {
-  extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ GeneralScratch<RES> sc;
+__device__ __forceinline__ void resample_position(const RowKernelArgs& a, size_t g, GeneralScratch<RES>& sc, unsigned char* dyn) {
   const DevParams& P = a.P;
   const int N = P.H * P.W, Ww = (P.W + 31) / 32;
-  const size_t g = blockIdx.x;
   const int b = (int)(g / N), t = (int)(g % N), i = t / P.W, j = t % P.W;
   const int tok_raw = a.draft_tok_hi[g];
   if (!get_bit(a.expand_bits, Ww, P.H, b, i, j)) {
@@ -433,6 +470,79 @@ __global__ void __launch_bounds__(kThreads, 2) k_resample_rows(RowKernelArgs a) 
   general_position<RES>(a, target_row(a, g), draft_row(a, cell), sq, tok, (uint32_t)b + P.image_offset, (uint32_t)t, false,
                         !rejected, [draw](int) { return draw; }, sc, dyn, o);
   if (threadIdx.x == 0) a.out_tok[g] = use_res ? o.tok_residual : o.tok_target;
+}
+// mulo_resample: one CTA per target position.
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_resample_rows(RowKernelArgs a) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
+  resample_position<RES>(a, blockIdx.x, sc, dyn);
+}
+// Third launch of its fast path: the positions the fast kernel put on its list.
+template <bool RES>
+__global__ void __launch_bounds__(kThreads, 2) k_resample_left(RowKernelArgs a, const int32_t* fail_list, const uint32_t* fail_count) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GeneralScratch<RES> sc;
+  let_next_begin();
+  wait_for_previous();
+  const size_t total = (size_t)a.P.B * a.P.H * a.P.W, n = min((size_t)*fail_count, total);
+  for (size_t idx = blockIdx.x; idx < n; idx += gridDim.x) {
+    const size_t g = (size_t)fail_list[idx];
+    if (g < total) resample_position<RES>(a, g, sc, dyn);
+    __syncthreads();
+  }
+}
+
+// First launch of its fast path, one CTA per image: x~ where nothing is drawn, and the list of what is, parent by parent.
+constexpr int kPickThreads = 1024;
+__global__ void __launch_bounds__(kPickThreads) k_resample_list(RowKernelArgs a, uint32_t* list, int32_t* counts, uint32_t* fail_count) {
+  __shared__ int warp_tot[kPickThreads / 32];
+  const DevParams& P = a.P;
+  const int N = P.H * P.W, Ww = (P.W + 31) / 32, cells = P.h * P.w, b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const size_t n0 = (size_t)b * N;
+  if (b == 0 && tid == 0) *fail_count = 0u;
+  int base = 0;
+  for (int c0 = 0; c0 < cells; c0 += kPickThreads) {
+    const int cell = c0 + tid, ca = cell / P.w, cc = cell - ca * P.w;
+    int n = 0, n_res = 0;
+    auto children = [&](auto take) {
+      if (cell < cells)
+        for (int di = 0; di < P.r; ++di)
+          for (int dj = 0; dj < P.r; ++dj) {
+            const int i = ca * P.r + di, j = cc * P.r + dj;
+            take(i * P.W + j, get_bit(a.expand_bits, Ww, P.H, b, i, j), get_bit(a.reject_bits, Ww, P.H, b, i, j));
+          }
+    };
+    auto residual = [&](int rejected) {
+      return P.resample_mode == MULO_RESAMPLE_RESIDUAL_ALL || (P.resample_mode == MULO_RESAMPLE_MIXED && rejected);
+    };
+    children([&](int t, int in, int rejected) {
+      if (!in) a.out_tok[n0 + t] = a.draft_tok_hi[n0 + t];
+      n += in;
+      n_res += in && residual(rejected);
+    });
+    int inc = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += v;
+    }
+    __syncthreads();
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    const int mine = warp_tot[lane];
+    int at = base + inc - n + __reduce_add_sync(kFull, lane < warp ? mine : 0);
+    base += __reduce_add_sync(kFull, mine);
+    children([&](int t, int in, int rejected) {
+      if (!in) return;
+      list[n0 + at++] = (uint32_t)t | (residual(rejected) ? kPickResidual : 0u) | (n_res > 0 ? kPickDraft : 0u);
+      // what the general routines report of a position
+      const RowStats sq = given_stats(a, (size_t)b * cells + cell);
+      const float zq = load1(draft_row(a, (size_t)b * cells + cell), checked_token(a.draft_tok_hi[n0 + t], P.V, a.dev_status));
+      if (!(zq >= sq.theta) || exp((double)zq - (double)sq.m) / sq.Z <= 0.0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
+    });
+  }
+  if (tid == 0) counts[b] = base;
 }
 
 // ============================================================= mask kernel
@@ -879,6 +989,9 @@ static bool launch_left(mulo_ctx* ctx, K kernel, size_t dyn, cudaStream_t st, co
   return ctas_per_sm(ctx, kernel, kThreads, dyn) >= 1 && launch_after(kernel, 2u * (unsigned)ctx->sm_count, kThreads, dyn, st, args...);
 }
 #define K_UPSAMPLE(RES) k_upsample_pool<RES>
+#define K_UPSAMPLE_FAILED(RES) k_upsample_failed<RES>
+#define K_VERIFY_LEFT(RES) k_verify_left<RES>
+#define K_RESAMPLE_LEFT(RES) k_resample_left<RES>
 #define K_SAMPLE(RES) k_sample_draft<RES>
 #define K_SAMPLE_FAILED(RES) k_sample_failed<RES>
 #define K_VERIFY(RES) k_verify_rows<false, RES>
@@ -965,7 +1078,7 @@ static bool launch_stream(mulo_ctx* ctx, const StreamArgs& s, size_t dyn, cudaSt
 // ---- rows with a top-k cut, NW warps per row (mulo_rows.cuh) ----------------------------
 
 // Fills `s` and returns the dynamic shared memory of a CTA of nw warps, or 0 if these parameters are not eligible.
-static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample, int nw, RowsArgs* s) {
+static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, int kind, int nw, RowsArgs* s) {
   if (d.top_k <= 0) return 0;
   const int V = d.V, k = d.top_k;
   if (V < 1024) return 0;
@@ -991,7 +1104,7 @@ static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample,
   s->R = (int)ceil(fmax(rows_for(k + margin, 2.0, 3.6), rows_for(k + margin_boot, 2.0, 3.0))) + 1 + kRSlack;
   if (s->R < 32) s->R = 32;
   s->margin = margin;
-  const size_t dyn = rows_layout(*s, nw, d.bf16, sample);
+  const size_t dyn = rows_layout(*s, nw, d.bf16, kind);
   if (2 * (dyn + sizeof(RowsSmem<4, true>) + 1024) > (size_t)ctx->smem_optin) return 0;   // too few rows in flight per SM
   return dyn;
 }
@@ -1003,12 +1116,12 @@ static size_t plan_rows_nw(const mulo_ctx* ctx, const DevParams& d, bool sample,
 // ... unless the lists of a two-warp CTA (fp32: those of the draft row are twice as long in bytes) leave room for fewer than
 // seven of them per SM.  4608 rows, guidance, k = V / 8: V = 16384 fp32 (five) 279 us with two, 210 with four; 12288 fp32 (six)
 // 6 to 22 % for four; 16384 bf16 (seven) 5 % for two, 8192 fp32 (eight) 10 % for two.
-static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, RowsArgs* s, int* nw) {
+static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, int kind, RowsArgs* s, int* nw) {
   *nw = 2;
-  size_t dyn = plan_rows_nw(ctx, d, sample, 2, s);
-  if (!dyn || (!sample && 7 * (dyn + sizeof(RowsSmem<2, false>) + 1024) > (size_t)ctx->smem_optin + 1024)) {
+  size_t dyn = plan_rows_nw(ctx, d, kind, 2, s);
+  if (!dyn || ((kind == kRowsRound || kind == kRowsResample) && 7 * (dyn + sizeof(RowsSmem<2, false>) + 1024) > (size_t)ctx->smem_optin + 1024)) {
     RowsArgs four = *s;
-    if (const size_t dyn4 = plan_rows_nw(ctx, d, sample, 4, &four)) {
+    if (const size_t dyn4 = plan_rows_nw(ctx, d, kind, 4, &four)) {
       *s = four;
       *nw = 4;
       dyn = dyn4;
@@ -1022,9 +1135,9 @@ static size_t plan_rows(const mulo_ctx* ctx, const DevParams& d, bool sample, Ro
   return dyn;
 }
 
-template <bool BF16, bool HAS_U, bool SAMPLE, bool POOL, bool PLAIN, int NW>
+template <bool BF16, bool HAS_U, int KIND, bool POOL, bool PLAIN, int NW>
 static bool launch_rows_p(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
-  auto kern = k_round_rows<BF16, HAS_U, SAMPLE, POOL, PLAIN, NW>;
+  auto kern = k_round_rows<BF16, HAS_U, KIND, POOL, PLAIN, NW>;
   const int per_sm = ctas_per_sm(ctx, kern, NW * 32, dyn);
   if (per_sm < 1) return false;
   int grid = ctx->sm_count * per_sm;
@@ -1033,29 +1146,27 @@ static bool launch_rows_p(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStre
   return true;
 }
 
-template <bool BF16, bool HAS_U, bool SAMPLE, int NW>
+template <bool BF16, bool HAS_U, int KIND, int NW>
 static bool launch_rows_t(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
   const bool plain = s.P.invT == 1.0f && s.row_bytes % (16u * kRPieceBytes * NW) == 0;
-  if constexpr (!SAMPLE)
+  if constexpr (KIND == kRowsRound)
     if (s.P.pool_k > 1)
-      return plain ? launch_rows_p<BF16, HAS_U, false, true, true, NW>(ctx, s, dyn, st)
-                   : launch_rows_p<BF16, HAS_U, false, true, false, NW>(ctx, s, dyn, st);
-  return plain ? launch_rows_p<BF16, HAS_U, SAMPLE, false, true, NW>(ctx, s, dyn, st)
-               : launch_rows_p<BF16, HAS_U, SAMPLE, false, false, NW>(ctx, s, dyn, st);
+      return plain ? launch_rows_p<BF16, HAS_U, KIND, true, true, NW>(ctx, s, dyn, st)
+                   : launch_rows_p<BF16, HAS_U, KIND, true, false, NW>(ctx, s, dyn, st);
+  return plain ? launch_rows_p<BF16, HAS_U, KIND, false, true, NW>(ctx, s, dyn, st)
+               : launch_rows_p<BF16, HAS_U, KIND, false, false, NW>(ctx, s, dyn, st);
 }
 
-template <int NW>
-static bool launch_rows_nw(mulo_ctx* ctx, const RowsArgs& s, bool sample, size_t dyn, cudaStream_t st) {
-  const bool hu = s.uncond != nullptr;
-  if (sample)
-    return s.P.bf16 ? launch_rows_t<true, false, true, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, true, NW>(ctx, s, dyn, st);
-  if (s.P.bf16)
-    return hu ? launch_rows_t<true, true, false, NW>(ctx, s, dyn, st) : launch_rows_t<true, false, false, NW>(ctx, s, dyn, st);
-  return hu ? launch_rows_t<false, true, false, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, false, NW>(ctx, s, dyn, st);
+template <int KIND, int NW>
+static bool launch_rows_nw(mulo_ctx* ctx, const RowsArgs& s, size_t dyn, cudaStream_t st) {
+  if constexpr (KIND == kRowsRound || KIND == kRowsVerify || KIND == kRowsResample)
+    if (s.uncond) return s.P.bf16 ? launch_rows_t<true, true, KIND, NW>(ctx, s, dyn, st) : launch_rows_t<false, true, KIND, NW>(ctx, s, dyn, st);
+  return s.P.bf16 ? launch_rows_t<true, false, KIND, NW>(ctx, s, dyn, st) : launch_rows_t<false, false, KIND, NW>(ctx, s, dyn, st);
 }
 
-static bool launch_rows(mulo_ctx* ctx, const RowsArgs& s, bool sample, int nw, size_t dyn, cudaStream_t st) {
-  return nw == 2 ? launch_rows_nw<2>(ctx, s, sample, dyn, st) : launch_rows_nw<4>(ctx, s, sample, dyn, st);
+template <int KIND>
+static bool launch_rows(mulo_ctx* ctx, const RowsArgs& s, int nw, size_t dyn, cudaStream_t st) {
+  return nw == 2 ? launch_rows_nw<KIND, 2>(ctx, s, dyn, st) : launch_rows_nw<KIND, 4>(ctx, s, dyn, st);
 }
 
 // ---- rows without a top-k cut (mulo_full.cuh, mulo_flat.cuh) ------------------------------
@@ -1148,6 +1259,15 @@ static bool launch_flat(mulo_ctx* ctx, const FlatArgs& s, bool sample, bool res,
   return hu ? launch_flat_t<false, true, false>(ctx, s, res, dyn, st) : launch_flat_t<false, false, false>(ctx, s, res, dyn, st);
 }
 
+// Are there enough rows with a cut for the stages to stream them (two warps each) instead of keeping each in one CTA's shared
+// memory?  That CTA is the sooner done with a row.  us streamed / kept: draft rows, 1024 of 16384 ids: 31 / 45, of 4096: 34 / 25, 576 of 16384:
+// 28 / 28; verified, 784 rows of 16384: 38 / 43, of 4096: 37 / 29, of 8192 fp32: 39 / 36, 1296 rows: 44 / 68, 39 / 41, 38 / 54; redrawn,
+// 784 rows: 43 / 56, 36 / 31, 38 / 43, 1296 rows: 77 / 90, 41 / 48, 57 / 68.
+static bool many_rows(const mulo_ctx* ctx, int kind, int V, long long rows) {
+  const int per_sm = kind == kRowsStats ? (V > 4096 ? 4 : 16) : V >= (kind == kRowsVerify ? 12288 : 8192) ? 4 : 8;
+  return !ctx->force_dense && rows > (long long)per_sm * ctx->sm_count;
+}
+
 static size_t mask_smem(const mulo_params* p) { return (size_t)3 * p->H * ((p->W + 31) / 32) * 4; }
 
 // Everything mulo_round can refuse without touching the device.
@@ -1193,11 +1313,35 @@ mulo_status mulo_upsample_pool(mulo_ctx* ctx, const mulo_params* p, const void* 
   // 38, 47, 106, 346 us resident; fp32 up to 8192 ids likewise (56, 71 us), above it the row no longer stays in L1 (16384 ids:
   // 148, 106 us).  64 rows: 14 to 17 us, 9 to 14 us resident.
   const int cells = p->B * a.P.h * a.P.w;
+  const cudaStream_t st = (cudaStream_t)stream;
+  // With one, many rows are streamed, if there is room for the list of rows that this may leave.
+  Workspace w;
+  RowsArgs ra;
+  memset(&ra, 0, sizeof ra);
+  int rnw = 0;
+  const bool many = many_rows(ctx, kRowsStats, a.P.V, cells) && check_ws(ctx, p, &w) == MULO_OK &&
+                    ((uintptr_t)draft_stats_lo & 15u) == 0;
+  if (const size_t rdyn = many ? plan_rows(ctx, a.P, kRowsStats, &ra, &rnw) : 0) {
+    ra.P = a.P;
+    ra.cond = a.draft;
+    ra.tok_of = draft_tok_lo;
+    ra.stats_out = draft_stats_lo;
+    ra.tok_hi_out = draft_tok_hi;
+    ra.q_hi_out = q_tok_hi;
+    ra.dev_status = w.status;
+    ra.fail_list = w.fail_list;
+    ra.n_units = cells;
+    if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
+    if (launch_rows<kRowsStats>(ctx, ra, rnw, rdyn, st)) {
+      if (!MULO_LAUNCH_LEFT(K_UPSAMPLE_FAILED, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+      return launched(ctx, 2);
+    }
+  }
   if (a.P.top_k == 0 && cells > 4 * ctx->sm_count && (a.P.bf16 || a.P.V <= 8192)) {
-    if (!launch_general(ctx, K_UPSAMPLE(false), (unsigned)cells, 0, (cudaStream_t)stream, a)) return MULO_ERR_CUDA;
+    if (!launch_general(ctx, K_UPSAMPLE(false), (unsigned)cells, 0, st, a)) return MULO_ERR_CUDA;
     return launched(ctx, 1);
   }
-  if (!MULO_LAUNCH_GENERAL(K_UPSAMPLE, cells, general_smem(a.P, false), (cudaStream_t)stream, a)) return MULO_ERR_CUDA;
+  if (!MULO_LAUNCH_GENERAL(K_UPSAMPLE, cells, general_smem(a.P, false), st, a)) return MULO_ERR_CUDA;
   return launched(ctx, 1);
 }
 
@@ -1337,7 +1481,7 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
   int rnw = 0;
-  const size_t rdyn = listed && !sdyn ? plan_rows(ctx, a.P, true, &ra, &rnw) : 0;
+  const size_t rdyn = listed && !sdyn ? plan_rows(ctx, a.P, kRowsSample, &ra, &rnw) : 0;
   if (rdyn) {
     ra.P = a.P;
     ra.cond = a.draft;
@@ -1346,7 +1490,7 @@ mulo_status mulo_sample_draft(mulo_ctx* ctx, const mulo_params* p, const void* d
     ra.fail_list = w.fail_list;
     ra.n_units = p->B * a.P.h * a.P.w;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
-    if (launch_rows(ctx, ra, true, rnw, rdyn, st)) {
+    if (launch_rows<kRowsSample>(ctx, ra, rnw, rdyn, st)) {
       if (!MULO_LAUNCH_LEFT(K_SAMPLE_FAILED, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
       return launched(ctx, 2);
     }
@@ -1417,14 +1561,35 @@ mulo_status mulo_verify(mulo_ctx* ctx, const mulo_params* p, const void* tgt_con
   a.dev_status = w.status;
   const size_t dyn = general_smem(a.P, true);
   cudaStream_t st = (cudaStream_t)stream;
-  if (!MULO_LAUNCH_GENERAL(K_VERIFY, (size_t)p->B * p->H * p->W, dyn, st, a)) return MULO_ERR_UNSUPPORTED;
+  // Many rows with a cut and without pooling are streamed.
+  bool fast = false;
+  RowsArgs ra;
+  memset(&ra, 0, sizeof ra);
+  int rnw = 0;
+  const long long rows = (long long)p->B * p->H * p->W;
+  const bool many = a.P.pool_k <= 1 && many_rows(ctx, kRowsVerify, a.P.V, rows);
+  if (const size_t rdyn = many ? plan_rows(ctx, a.P, kRowsVerify, &ra, &rnw) : 0) {
+    ra.P = a.P;
+    ra.cond = a.cond; ra.uncond = a.uncond; ra.draft = a.draft;
+    ra.tok_of = draft_tok_hi;
+    ra.stats_in = draft_stats_lo;
+    ra.p_tok = p_tok; ra.q_tok = q_tok; ra.accept_prob = accept_prob;
+    ra.flags = w.flags;
+    ra.dev_status = w.status;
+    ra.fail_list = w.fail_list;
+    ra.n_units = (int)rows;
+    if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
+    fast = launch_rows<kRowsVerify>(ctx, ra, rnw, rdyn, st);
+    if (fast && !MULO_LAUNCH_LEFT(K_VERIFY_LEFT, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+  }
+  if (!fast && !MULO_LAUNCH_GENERAL(K_VERIFY, rows, dyn, st, a)) return MULO_ERR_UNSUPPORTED;
   MaskArgs m;
   memset(&m, 0, sizeof m);
   m.H = p->H; m.W = p->W; m.r = p->r; m.radius = p->radius; m.clip = a.P.clip; m.resample_mode = p->resample_mode;
   m.flags = w.flags;
   m.reject_bits = reject_bits; m.n_reject = n_reject; m.first_reject = first_reject;
   if (!launch_after(k_mask<0>, (unsigned)p->B, kMaskThreads, mask_smem(p), st, m)) return MULO_ERR_CUDA;
-  return launched(ctx, 2);
+  return launched(ctx, fast ? 3 : 2);
 }
 
 mulo_status mulo_local_reject_expand(mulo_ctx* ctx, const mulo_params* p, const uint32_t* reject_bits,
@@ -1494,7 +1659,34 @@ mulo_status mulo_resample(mulo_ctx* ctx, const mulo_params* p, const void* tgt_c
   a.expand_bits = expand_bits;
   a.out_tok = out_tok;
   a.dev_status = (uint32_t*)ctx->ws;
-  if (!MULO_LAUNCH_GENERAL(K_RESAMPLE, (size_t)p->B * p->H * p->W, general_smem(a.P, true), (cudaStream_t)stream, a)) return MULO_ERR_UNSUPPORTED;
+  const cudaStream_t st = (cudaStream_t)stream;
+  const size_t dyn = general_smem(a.P, true);
+  const long long rows = (long long)p->B * p->H * p->W;
+  // Many rows with a cut and without pooling are streamed, if there is room for the lists.  (Whether a rejection is isolated
+  // depends on its neighbours, which the general kernel looks up.)
+  Workspace w;
+  RowsArgs ra;
+  memset(&ra, 0, sizeof ra);
+  int rnw = 0;
+  const bool many = a.P.pool_k <= 1 && many_rows(ctx, kRowsResample, a.P.V, rows) &&
+                    (size_t)p->H * p->W <= (size_t)kPickIndex && p->resample_mode != MULO_RESAMPLE_ISOLATED_RESIDUAL && check_ws(ctx, p, &w) == MULO_OK;
+  if (const size_t rdyn = many ? plan_rows(ctx, a.P, kRowsResample, &ra, &rnw) : 0) {
+    ra.P = a.P;
+    ra.cond = a.cond; ra.uncond = a.uncond; ra.draft = a.draft;
+    ra.stats_in = draft_stats_lo;
+    ra.sample_out = out_tok;
+    ra.list = (const uint32_t*)w.cand_tgt;
+    ra.counts = w.cand_res;
+    ra.dev_status = w.status;
+    ra.fail_list = w.fail_list;
+    ra.n_units = (int)rows;   // (at most)
+    k_resample_list<<<p->B, kPickThreads, 0, st>>>(a, (uint32_t*)w.cand_tgt, w.cand_res, w.status + kFailCount);
+    if (launch_rows<kRowsResample>(ctx, ra, rnw, rdyn, st)) {
+      if (!MULO_LAUNCH_LEFT(K_RESAMPLE_LEFT, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+      return launched(ctx, 3);
+    }
+  }
+  if (!MULO_LAUNCH_GENERAL(K_RESAMPLE, rows, dyn, st, a)) return MULO_ERR_UNSUPPORTED;
   return launched(ctx, 1);
 }
 
@@ -1564,7 +1756,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
   int rnw = 0;
-  const size_t rdyn = (ctx->force_dense || fast) ? 0 : plan_rows(ctx, a.P, false, &ra, &rnw);
+  const size_t rdyn = (ctx->force_dense || fast) ? 0 : plan_rows(ctx, a.P, kRowsRound, &ra, &rnw);
   if (rdyn) {
     ra.P = a.P;
     ra.cond = a.cond; ra.uncond = a.uncond; ra.draft = a.draft; ra.draft_tok_lo = draft_tok_lo;
@@ -1575,7 +1767,7 @@ mulo_status mulo_round(mulo_ctx* ctx, const mulo_params* p, const void* tgt_cond
     ra.fail_list = w.fail_list;
     ra.n_units = p->B * p->H * p->W;
     if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
-    fast = launch_rows(ctx, ra, false, rnw, rdyn, st);
+    fast = launch_rows<kRowsRound>(ctx, ra, rnw, rdyn, st);
     if (fast && !MULO_LAUNCH_LEFT(K_ROUND_FAILED, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
   }
   StreamArgs sa;
@@ -1630,7 +1822,7 @@ mulo_status mulo_round_kernel(const mulo_ctx* ctx, const mulo_params* p, int has
   memset(&fa, 0, sizeof fa);
   bool fres;
   if (plan_full(ctx, d, has_uncond != 0, &ua) || plan_flat(ctx, d, false, &fa, &fres)) *kernel = MULO_KERNEL_FULL;
-  else if (plan_rows(ctx, d, false, &ra, &nw)) *kernel = d.pool_k > 1 ? MULO_KERNEL_STREAM : MULO_KERNEL_LANE;
+  else if (plan_rows(ctx, d, kRowsRound, &ra, &nw)) *kernel = d.pool_k > 1 ? MULO_KERNEL_STREAM : MULO_KERNEL_LANE;
   else if (plan_stream(ctx, d, &sa)) *kernel = MULO_KERNEL_STREAM;
   return MULO_OK;
 }

@@ -52,6 +52,18 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kNearRefGap = 8.0f;      // a row whose maximum lies further from the predicted exp reference is streamed again
                                          // against its own maximum (large exponents cost relative accuracy)
 
+// What the kernel is run for: a whole round; the drafter's draws; or one stage of a round, which wants sums of a row and
+// nothing drawn: the target rows' probabilities of x~ and its acceptance, the draft rows' statistics.  A stage hands its sums
+// on to whoever calls the next one, so they are no less exact than the general routines': weights within 0.51 units in the last
+// place (sums_exp), added in double, the maximum's own in double.  (The exp reference is a whole number: subtracting it loses no
+// bits of the logits near the maximum.)
+// kRowsResample draws for the listed positions, with the draft rows' statistics given: a draft row is only streamed, its
+// entries above the given threshold are its list.
+constexpr int kRowsRound = 0, kRowsSample = 1, kRowsVerify = 2, kRowsStats = 3, kRowsResample = 4;
+// An entry of kRowsResample's list: the position in its image, whether it is drawn from the residual, whether any position of its
+// parent is (the draft row is not read otherwise).
+constexpr uint32_t kPickIndex = (1u << 30) - 1u, kPickResidual = 1u << 31, kPickDraft = 1u << 30;
+
 // running prediction for one kind of row (draft / target), per CTA
 struct RowPredictor {
   int have;
@@ -75,10 +87,17 @@ struct RowsArgs {
   uint8_t* flags;
   int32_t* cand_res;
   int32_t* cand_tgt;
-  int32_t* sample_out;      // SAMPLE: the drafter's token per cell
+  int32_t* sample_out;      // kRowsSample: the drafter's token per cell
+  const int32_t* tok_of;    // kRowsVerify, kRowsStats: x~ of each row
+  const float* stats_in;    // kRowsVerify, kRowsResample: the draft rows' statistics
+  const uint32_t* list;     // kRowsResample: [B][H * W], an image's positions of R_X (see kPickIndex), parent by parent
+  const int32_t* counts;    // ... and how many they are
+  float* stats_out;         // kRowsStats
+  int32_t* tok_hi_out;
+  float* q_hi_out;
   uint32_t* dev_status;
   int32_t* fail_list;
-  int n_units;              // target rows, parent by parent (SAMPLE: low-res cells)
+  int n_units;              // rows: target rows, parent by parent (kRowsSample, kRowsStats: low-res cells; kRowsVerify: in raster order)
   uint32_t row_bytes;
   int ppg;                  // pieces of a group's part of a row
   int n_words;              // mask words per thread: ceil(ppg / 4)
@@ -114,7 +133,7 @@ struct RowsSmem {
 };
 
 // Dynamic shared memory of a CTA (bytes); the parts' offsets go into `s`.
-inline uint32_t rows_layout(RowsArgs& s, int nw, bool bf16, bool sample) {
+inline uint32_t rows_layout(RowsArgs& s, int nw, bool bf16, int kind) {
   const uint32_t cols = (uint32_t)s.R * (uint32_t)(nw / 2);
   uint32_t off = cols * 128u;   // the target row's lists
   auto take = [&](uint32_t bytes) {
@@ -122,9 +141,10 @@ inline uint32_t rows_layout(RowsArgs& s, int nw, bool bf16, bool sample) {
     off += bytes;
     return o;
   };
-  s.o_dlist = take(sample ? 0u : cols * (bf16 ? 64u : 128u));
-  s.o_tmask = take((uint32_t)s.n_words * nw * 128u);
-  s.o_dmask = sample ? s.o_tmask : take((uint32_t)s.n_words * nw * 128u);
+  const bool draws = kind == kRowsRound || kind == kRowsResample;
+  s.o_dlist = take(draws ? cols * (bf16 ? 64u : 128u) : 0u);
+  s.o_tmask = take(draws || kind == kRowsSample ? (uint32_t)s.n_words * nw * 128u : 0u);
+  s.o_dmask = draws ? take((uint32_t)s.n_words * nw * 128u) : s.o_tmask;
   return off;
 }
 
@@ -186,10 +206,19 @@ __device__ __forceinline__ void prefetch_l2(const char* p, uint32_t bytes) {
 }
 
 // Appends z to the thread's list if z >= pivot (cursor step: one list row of 128 bytes, up or down) and
-// marks its bit.
-template <int BIT>
+// marks its bit (MARK).
+template <bool MARK, int BIT>
 __device__ __forceinline__ void row_put(float z, float pivot, uint32_t& cur, uint32_t step, uint32_t& m) {
-  asm volatile(
+  if constexpr (!MARK)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ge.f32 p, %1, %2;\n\t"
+        "@p st.shared.f32 [%0], %1;\n\t"
+        "@p add.u32 %0, %0, %3;\n\t}"
+        : "+r"(cur)
+        : "f"(z), "f"(pivot), "r"(step)
+        : "memory");
+  else asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ge.f32 p, %2, %3;\n\t"
       "@p st.shared.f32 [%0], %2;\n\t"
@@ -221,27 +250,48 @@ __device__ __forceinline__ float2 row_pair(const uint4& c, const uint4& u, float
   if (SCALE) v = __fmul2_rn(v, t2);
   return v;
 }
-template <bool BF16, bool ROW_U, bool SCALE, int BIT0>
+template <bool BF16, bool ROW_U, bool SCALE, bool MARK, int BIT0>
 __device__ __forceinline__ void row_piece(const uint4& c, const uint4& u, float2 s2, float2 t2, float pivot,
                                           uint32_t& cur, uint32_t step, uint32_t& m) {
   float2 z = row_pair<BF16, ROW_U, SCALE, 0>(c, u, s2, t2);
-  row_put<BIT0>(z.x, pivot, cur, step, m);
-  row_put<BIT0 + 1>(z.y, pivot, cur, step, m);
+  row_put<MARK, BIT0>(z.x, pivot, cur, step, m);
+  row_put<MARK, BIT0 + 1>(z.y, pivot, cur, step, m);
   z = row_pair<BF16, ROW_U, SCALE, 1>(c, u, s2, t2);
-  row_put<BIT0 + 2>(z.x, pivot, cur, step, m);
-  row_put<BIT0 + 3>(z.y, pivot, cur, step, m);
+  row_put<MARK, BIT0 + 2>(z.x, pivot, cur, step, m);
+  row_put<MARK, BIT0 + 3>(z.y, pivot, cur, step, m);
   if (BF16) {
     z = row_pair<BF16, ROW_U, SCALE, 2>(c, u, s2, t2);
-    row_put<(BIT0 + 4) & 31>(z.x, pivot, cur, step, m);
-    row_put<(BIT0 + 5) & 31>(z.y, pivot, cur, step, m);
+    row_put<MARK, (BIT0 + 4) & 31>(z.x, pivot, cur, step, m);
+    row_put<MARK, (BIT0 + 5) & 31>(z.y, pivot, cur, step, m);
     z = row_pair<BF16, ROW_U, SCALE, 3>(c, u, s2, t2);
-    row_put<(BIT0 + 6) & 31>(z.x, pivot, cur, step, m);
-    row_put<(BIT0 + 7) & 31>(z.y, pivot, cur, step, m);
+    row_put<MARK, (BIT0 + 6) & 31>(z.x, pivot, cur, step, m);
+    row_put<MARK, (BIT0 + 7) & 31>(z.y, pivot, cur, step, m);
   }
 }
 
 // 2^x in double, out of line: three call sites, a few hundred instructions each otherwise
 __device__ __noinline__ double row_exp2(double x) { return exp2(x); }
+
+__device__ __noinline__ double row_exp(double x) { return exp(x); }
+
+// e^d for d from -80 (below: that of -80) to 80, within 6.0e-8, 2.6e-8 rms: d = n ln 2 + f, and on |f| <= ln 2 / 2 a polynomial
+// 1 + f + f^2 q(f), q of degree four fitted to (e^f - 1 - f) / f^2 (largest error in e^f 3.1e-9).  expf leaves twice the error
+// in a row's sum.
+__device__ __forceinline__ float sums_exp(float d) {
+  d = fmaxf(d, -80.0f);
+  const float t = fmaf(d, kLog2e, kRMagic), n = t - kRMagic;   // n to nearest
+  float f = fmaf(n, -0.693145751953125f, d);                   // (n times these sixteen bits of ln 2 is exact)
+  f = fmaf(n, -1.4286068203094e-6f, f);
+  float q = fmaf(1.3950488064e-3f, f, 8.3688879386e-3f);
+  q = fmaf(q, f, 4.1666205972e-2f);
+  q = fmaf(q, f, 1.6666518152e-1f);
+  q = fmaf(q, f, 0.5f);
+  q = fmaf(q, f, 1.0f);
+  q = fmaf(q, f, 1.0f);
+  return __fmul_rn(q, __int_as_float((__float_as_int(t) + 127) << 23));
+}
+// What the weight of the row's maximum in a sum of these lacks: with one id far above the rest that is the sum's whole error.
+__device__ __forceinline__ double sums_exp_rest(float d) { return exp((double)d) - (double)sums_exp(d); }
 
 // x~'s own weight, in double, beside weights 2^(z * kLog2e + c0), c0 = -ref * kLog2e in fp32.  That constant is off by 1.3e-8
 // (relative), which acts on z - ref: it averages out in sums near the maximum, a single weight far below it shows it whole
@@ -373,22 +423,72 @@ __device__ __forceinline__ void pool_prefetch(const uint16_t* row, int pool_k) {
 }
 
 // Warps per SM the kernel is compiled for: 16 (128 registers, four pieces in flight; eight CTAs of two warps are also
-// what the lists of V = 16384, top-k 2000 leave room for), 24 for the sampling kernel, which keeps no draft list.
-__host__ __device__ constexpr int rows_warps(bool sample) { return sample ? 24 : 16; }
+// what the lists of V = 16384, top-k 2000 leave room for), 24 for the draft rows' kernels, which keep no draft list, 20 for the
+// target rows' sums.
+__host__ __device__ constexpr int rows_warps(int kind) { return kind == kRowsRound || kind == kRowsResample ? 16 : kind == kRowsVerify ? 20 : 24; }
+
+// The end of a row of the stages (out of line: double divisions and exponentials).  One thread; e_tok: weight of x~ in the row's
+// units, 0 below its threshold.
+__device__ __noinline__ void rows_verified(const RowsArgs* a, uint32_t g, double e_tok, double Z, float m, float ref, float zq,
+                                           float theta_q, float m_q, double Zq) {
+  const DevParams& P = a->P;
+  Z += sums_exp_rest(__fsub_rn(m, ref));
+  const uint32_t N = (uint32_t)P.H * (uint32_t)P.W, b = g / N, t = g - b * N;
+  const double p = e_tok / Z, q = zq >= theta_q ? exp((double)zq - (double)m_q) / Zq : 0.0;
+  if (q <= 0.0) atomicOr(a->dev_status, MULO_DEV_ZERO_DRAFT_PROB);
+  double thr;
+  bool accepted;
+  if (P.accept_mode == MULO_ACCEPT_THRESHOLD) {
+    thr = p;
+    accepted = p >= P.tau;
+  } else {
+    thr = q <= 0.0 ? (p > 0.0 ? 1.0 : 0.0) : fmin(1.0, p / q);
+    accepted = uniform24(row_philox(make_uint4(t, b + P.image_offset, P.round, 0u), make_uint2(P.seed_lo, P.seed_hi)).x) < thr;
+  }
+  a->flags[g] = accepted ? 0 : 1;
+  a->p_tok[g] = (float)p;
+  a->q_tok[g] = (float)q;
+  a->accept_prob[g] = (float)thr;
+}
+__device__ __noinline__ void rows_stats(const RowsArgs* a, uint32_t cell, float z_tok, float theta, float m, float ref, double Z) {
+  const DevParams& P = a->P;
+  Z = (Z + sums_exp_rest(__fsub_rn(m, ref))) * exp((double)ref - (double)m);
+  const float hi = (float)Z, lo = (float)(Z - (double)hi);
+  reinterpret_cast<float4*>(a->stats_out)[cell] = make_float4(theta, m, hi, lo);
+  const float q = z_tok >= theta ? (float)(exp((double)z_tok - (double)m) / ((double)hi + (double)lo)) : 0.f;
+  const uint32_t hw = (uint32_t)P.h * (uint32_t)P.w, b = cell / hw, ca = (cell - b * hw) / P.w, cc = cell - b * hw - ca * P.w;
+  const int32_t tok = a->tok_of[cell];
+  for (int di = 0; di < P.r; ++di)
+    for (int dj = 0; dj < P.r; ++dj) {
+      const size_t t = ((size_t)b * P.H + (size_t)ca * P.r + di) * P.W + (size_t)cc * P.r + dj;
+      a->tok_hi_out[t] = tok;
+      a->q_hi_out[t] = q;
+    }
+}
 
 // PLAIN: T = 1 and every piece a thread's whole 16 bytes (V splits evenly), so no scaling and no bounds checks.
-template <bool BF16, bool HAS_U, bool SAMPLE, bool POOL, bool PLAIN, int NW>
-__global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
+template <bool BF16, bool HAS_U, int KIND, bool POOL, bool PLAIN, int NW>
+__global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
+  constexpr bool LISTED = KIND == kRowsResample;
+  constexpr bool SAMPLE = KIND != kRowsRound && !LISTED;   // one kind of row, and no parents
+  constexpr bool SUMS = KIND == kRowsVerify || KIND == kRowsStats;   // nothing is drawn
   constexpr int NT = NW * 32;
   constexpr int IDS = BF16 ? 8 : 4;              // ids per lane per piece
-  constexpr int kRDepth = SAMPLE ? 2 : 4;        // pieces in flight per lane
+  constexpr int kRDepth = KIND == kRowsSample || KIND == kRowsStats ? 2 : 4;   // pieces in flight per lane
+  using Sum = typename std::conditional<SUMS, double, float>::type;
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ RowsSmem<NW, POOL> sm;
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   let_next_begin();
-  int unit = (int)(((long long)a.n_units * blockIdx.x) / gridDim.x);
-  const int u_end = (int)(((long long)a.n_units * (blockIdx.x + 1)) / gridDim.x);
+  int n_units = a.n_units;
+  if constexpr (LISTED) {
+    n_units = 0;
+    for (int i = lane; i < P.B; i += 32) n_units += a.counts[i];
+    n_units = __reduce_add_sync(kFull, n_units);
+  }
+  int unit = (int)(((long long)n_units * blockIdx.x) / gridDim.x);
+  const int u_end = (int)(((long long)n_units * (blockIdx.x + 1)) / gridDim.x);
   if (unit >= u_end) return;
   const int rr = SAMPLE ? 1 : P.r * P.r;
   const uint32_t row_bytes = a.row_bytes;
@@ -441,7 +541,34 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       dj = child - di * P.r;
     }
   }
+  // LISTED: the entry in work, the one after it, and where that is
+  uint32_t pick = 0, pick_next = 0;
+  int img_at = 0, left = 0;
+  uint32_t N = 0;
+  auto pick_parent = [&](uint32_t p, int image) -> int {
+    const int t = (int)(p & kPickIndex), i = t / P.W, j = t - i * P.W;
+    return (image * P.h + i / P.r) * P.w + j / P.r;
+  };
+  int b_next = 0;      // the image of the entry after this one (b: of that in work)
+  auto next_pick = [&]() {   // (there is one)
+    while (img_at >= a.counts[b_next]) {
+      ++b_next;
+      img_at = 0;
+    }
+    pick_next = a.list[(size_t)b_next * N + (uint32_t)img_at++];
+  };
+  if constexpr (LISTED) {
+    N = (uint32_t)P.H * (uint32_t)P.W;
+    b = 0;
+    img_at = unit;
+    while (img_at >= a.counts[b]) img_at -= a.counts[b++];
+    pick = a.list[(size_t)b * N + (uint32_t)img_at++];
+    parent = pick_parent(pick, b);
+    b_next = b;
+    left = u_end - unit - 1;
+  }
   auto target_index = [&]() -> uint32_t {
+    if constexpr (LISTED) return (uint32_t)b * N + (pick & kPickIndex);
     return ((uint32_t)b * P.H + (uint32_t)(ca * P.r + di)) * P.W + (uint32_t)(cc * P.r + dj);
   };
   auto next_parent = [&]() {
@@ -491,7 +618,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     constexpr int S = J % kRDepth, A = (J + kRDepth) & 3;                                                  \
     constexpr bool SAME = J + kRDepth < 4;                                                                 \
     cur = up ? min(cur, lim) : max(cur, lim);                                                              \
-    row_piece<BF16, ROW_U, !PLAIN, J * IDS>(c[S], u[S], s2, t2, pivot, cur, step, m);                      \
+    row_piece<BF16, ROW_U, !PLAIN, !SUMS, J * IDS>(c[S], u[S], s2, t2, pivot, cur, step, m);                      \
     const char* const pc = SAME ? rc : fc;                                                                 \
     const char* const pu = SAME ? ru : fu;                                                                 \
     const bool want_u = SAME ? ROW_U : do_u;                                                               \
@@ -506,7 +633,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
   }
       MULO_PIECE(0) MULO_PIECE(1) MULO_PIECE(2) MULO_PIECE(3)
 #undef MULO_PIECE
-      sts_u32(mask_at + (uint32_t)(w * NT) * 4u, m);
+      if constexpr (!SUMS) sts_u32(mask_at + (uint32_t)(w * NT) * 4u, m);
       rc += 4 * kRPieceBytes;
       if (HAS_U && ROW_U) ru += 4 * kRPieceBytes;
     }
@@ -565,16 +692,21 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     per = d / (1.75f * (float)a.margin);  // distance per candidate near the pivot
   };
 
-  bool is_q = !SAMPLE;                    // the row in work is a draft row
-  uint32_t g = (uint32_t)parent;          // ... and its index in its tensor
+  bool is_q = LISTED ? (pick & kPickDraft) != 0u : !SAMPLE;   // the row in work is a draft row
+  uint32_t g = !LISTED || is_q ? (uint32_t)parent : target_index();   // ... and its index in its tensor
+  if (LISTED && left > 0) next_pick();
+  int parent_next = 0;
 
   // ---- first pass over the list (see the top of the file); returns the exp sum of the entries above the window.
   //      A draft row (Q) puts its logits into the draft list instead of their exps into its own.  Written with
   //      predicated PTX: left to the compiler, every entry becomes two branches.
-  auto pass_one = [&](auto q_tag, int n, float inv_w, float hoff, float c0, uint32_t& low_a, uint32_t& low_b) -> float {
+  //      (c0: the exp reference as the weights take it, see below)
+  auto weight_of = [&](float z, float c0) -> float { return SUMS ? sums_exp(__fsub_rn(z, c0)) : ex2f(fmaf(z, kLog2e, c0)); };
+  auto pass_one = [&](auto q_tag, int n, float inv_w, float hoff, float c0, uint32_t& low_a, uint32_t& low_b) -> Sum {
     constexpr bool Q = decltype(q_tag)::value;
     const int n_max = __reduce_max_sync(kFull, n);
-    float mx = -INFINITY, s0 = 0.f, s1 = 0.f;
+    float mx = -INFINITY;
+    Sum s0 = 0, s1 = 0;
     low_a = low_b = 0;
     const uint32_t end = tl + (uint32_t)n * step;
 #pragma unroll
@@ -585,7 +717,8 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
 #pragma unroll 1
     for (int i = 0; i < n_max; i += 4, ad += 4 * step, dd += 4 * dstep) {
       const bool in = i < n;
-      const uint32_t from = in ? ad : closer, to = !Q && in ? ad : dump;
+      const uint32_t from = in ? ad : closer;
+      [[maybe_unused]] const uint32_t to = !Q && in ? ad : dump;
       float z[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) z[k] = lds_f32(from + k * 128);
@@ -593,10 +726,23 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
 // (entries outside the window count in a word of their own lane: a predicated reduction becomes a branch)
 #define MULO_ENTRY(K, S)                                                                       \
   {                                                                                            \
-    const float e = ex2f(fmaf(z[K], kLog2e, c0));                                              \
+    float e = weight_of(z[K], c0);                                                             \
     const uint32_t bin = __float_as_uint(fmaf(z[K], inv_w, hm));                               \
     const uint32_t at = hbase + (bin << 2);                                                    \
-    asm volatile(                                                                              \
+    if constexpr (SUMS) {                                                                      \
+      asm volatile(                                                                            \
+          "{\n\t.reg .pred p;\n\t.reg .u32 t, w;\n\t"                                            \
+          "sub.u32 t, %2, %3;\n\t"                                                             \
+          "setp.le.u32 p, t, %4;\n\t"                                                          \
+          "selp.u32 w, %5, %7, p;\n\t"                                                         \
+          "red.shared.add.u32 [w], 1;\n\t"                                                     \
+          "@p or.b32 %0, %0, %6;\n\t"                                                          \
+          "@p mov.f32 %1, 0f00000000;\n\t}"                                                    \
+          : "+r"(l4), "+f"(e)                                                                  \
+          : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(at), "n"(1 << K), "r"(spill)           \
+          : "memory");                                                                         \
+      S += (double)e;                                                                          \
+    } else asm volatile(                                                                       \
         "{\n\t.reg .pred p;\n\t.reg .u32 t, w;\n\t"                                            \
         "sub.u32 t, %2, %3;\n\t"                                                               \
         "setp.le.u32 p, t, %4;\n\t"                                                            \
@@ -605,7 +751,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         "@p or.b32 %0, %0, %6;\n\t"                                                            \
         "@!p add.f32 %1, %1, %7;\n\t"                                                          \
         "@!p st.shared.f32 [%8 + %9], %7;\n\t}"                                                \
-        : "+r"(l4), "+f"(S)                                                                    \
+        : "+r"(l4), "+f"(reinterpret_cast<float&>(S))                                          \
         : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(at), "n"(1 << K), "f"(e), "r"(to), "n"(K * 128), "r"(spill) \
         : "memory");                                                                           \
   }
@@ -634,20 +780,21 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
   //      below replace the logit (draft row: those below leave the draft list); returns the exp sum of those above.  Of the
   //      masks, the entries in the crossing bin are left, which keep their logits.
   const uint32_t flip = up ? 0u : 3u;      // (a mask's bits run along memory)
-  auto window = [&](uint32_t& low_a, uint32_t& low_b, float inv_w, float hoff, float c0, int bstar) -> float {
+  auto window = [&](uint32_t& low_a, uint32_t& low_b, float inv_w, float hoff, float c0, int bstar) -> Sum {
     const float hm = hoff + kRMagic;
     const uint32_t bm = __float_as_uint(kRMagic) + (uint32_t)bstar;
-    float s = 0.f;
+    Sum s = 0;
     uint32_t first = 0;
     auto one = [&](uint32_t bit, float& z) -> bool {   // does the entry lie in the crossing bin?
       const uint32_t i = first + ((uint32_t)__popc(bit - 1u) ^ flip);
       const uint32_t at = tl + i * step;
       z = lds_f32(bit ? at : closer);
       const uint32_t bin = __float_as_uint(fmaf(z, inv_w, hm));   // (-inf: as unsigned above every bin; its exp is 0)
-      float e = ex2f(fmaf(z, kLog2e, c0));
+      float e = weight_of(z, c0);
       e = bin > bm ? e : 0.f;
-      s += e;
-      if (is_q) {
+      s += (Sum)e;
+      if (SUMS) {
+      } else if (is_q) {
         if (bin < bm) dlist_put<BF16>(dl + i * dstep, -INFINITY);
       } else {
         const uint32_t there = bin == bm ? 0u : bit;
@@ -712,10 +859,10 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
   int partner_q = 0;                      // ... and of the draft row's list
   float c0_q = 0.f, Zq = 1.f;             // of the parent's draft row
   double q_tok = 0.0;
-  int tok_next = SAMPLE ? 0 : __ldg(a.draft_tok_lo + parent);
+  int tok_next = KIND == kRowsSample || LISTED ? 0 : __ldg((SUMS ? a.tok_of : a.draft_tok_lo) + parent);
   float pivot = 0.f, inv_w = 0.f, ref = 0.f, per = 0.f, lo = 0.f, hi = 0.f;   // of the row in work
-  prologue(part(row_c(is_q, g)), nullptr);
-  if (tid == 0) prefetch(row_c(is_q, g), nullptr);
+  prologue(part(row_c(is_q, g)), part(row_u(is_q, g)));
+  if (tid == 0) prefetch(row_c(is_q, g), row_u(is_q, g));
 
 #pragma unroll 1
   for (;;) {
@@ -732,6 +879,10 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     } else if (unit + 1 >= u_end) {
       more = false;
       ng = g;
+    } else if (LISTED) {
+      parent_next = pick_parent(pick_next, b_next);
+      nq = parent_next != parent && (pick_next & kPickDraft) != 0u;
+      ng = nq ? (uint32_t)parent_next : (uint32_t)b_next * N + (pick_next & kPickIndex);
     } else {
       if (dj + 1 < P.r || di + 1 < P.r) {
         if (++dj == P.r) {
@@ -749,7 +900,20 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     const char* const nu = more ? row_u(nq, ng) : nullptr;
     // the logit of x~ in this row: asked for now, used after the first pass
     uint32_t raw_c = 0u, raw_u = 0u;   // (as they are: a conversion here would wait for them)
-    if (!SAMPLE) {
+    if constexpr (SUMS) {
+      if (tries == 0) {
+        tok = tok_next;
+        if (tok < 0 || tok >= P.V) {
+          if (tid == 0) atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
+          tok = min(max(tok, 0), P.V - 1);
+        }
+        tok_next = __ldg(a.tok_of + ng);
+      }
+      if (warp == NW - 1) {
+        raw_c = raw_logit<BF16>(rc, tok);
+        if (HAS_U) raw_u = raw_logit<BF16>(ru, tok);
+      }
+    } else if (KIND == kRowsRound) {
       if (is_q) {
         tok = tok_next;
         if (tok < 0 || tok >= P.V) {
@@ -765,7 +929,13 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     }
 
     RowPredictor& pr = sm.pred[is_q ? 0 : 1];
-    if (tries == 0) {   // (a row streamed again keeps its corrected values)
+    float theta_q = 0.f;
+    if (LISTED && is_q) {   // the threshold is given: what lies above it, and no selection
+      const float* const st = a.stats_in + (size_t)g * 4;
+      theta_q = pivot = __ldg(st);
+      ref = __ldg(st + 1);
+      inv_w = 1.0f;
+    } else if (tries == 0) {   // (a row streamed again keeps its corrected values)
       lo = -INFINITY;
       hi = INFINITY;
       if (pr.have) {
@@ -778,6 +948,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       }
     }
 
+    if constexpr (SUMS) ref = rintf(ref);
     col = (uint32_t)lane ^ (up ? 0u : rot);
     tl = my + first_row * 128u + col * 4u;
     if (is_q) dl = my + a.o_dlist + first_row * DROW + col * (DROW / 32u);
@@ -792,18 +963,18 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     // (a list that reached its limit was held there: its entries are incomplete; one of more than R - kRSlack
     // entries would leave its neighbour's next row no room at all)
     const bool over = (up ? end >= lim : end <= lim) || n_raw > 64 || n_raw > R - kRSlack;
-    const float c0 = -ref * kLog2e, hoff = -pivot * inv_w;
+    const float c0 = SUMS ? ref : -ref * kLog2e, hoff = -pivot * inv_w;
     uint32_t low_a, low_b;
-    float s_t = is_q ? pass_one(std::integral_constant<bool, !SAMPLE>{}, n, inv_w, hoff, c0, low_a, low_b)
+    Sum s_t = is_q ? pass_one(std::integral_constant<bool, !SAMPLE>{}, n, inv_w, hoff, c0, low_a, low_b)
                      : pass_one(std::false_type{}, n, inv_w, hoff, c0, low_a, low_b);
     {
       const bool any_over = __any_sync(kFull, over);
       if (lane == 0) sm.over[warp] = any_over;
     }
-    if (!SAMPLE && warp == NW - 1) {
+    if (KIND != kRowsSample && !LISTED && warp == NW - 1) {
       // the token's own weight (its z against theta later)
       const float z = mix_logit(wide_logit<BF16>(raw_c), wide_logit<BF16>(raw_u), HAS_U && !is_q, P.cfg_scale, P.invT);
-      const double e = token_weight(z, ref, c0);
+      const double e = SUMS ? row_exp((double)z - (double)ref) : token_weight(z, ref, c0);
       if (lane == 0) {
         sm.e_tok = e;
         sm.z_tok = z;
@@ -811,7 +982,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     }
     // the uniforms of the parent's rows, sixteen at a time: those around the first one with the draft row, the next with every
     // sixteenth row (barrier 3 of the row before lies behind everybody who read the last ones)
-    if (!SAMPLE && warp == 0 && lane < min(rr, 16) && (is_q || (rr > 16 && (child & 15) == 0))) {
+    if (KIND == kRowsRound && warp == 0 && lane < min(rr, 16) && (is_q || (rr > 16 && (child & 15) == 0))) {
       const int i = rr > 16 ? ((is_q ? di * P.r + dj : child) & ~15) + lane : lane;
       const int ddi = i / P.r, ddj = i - ddi * P.r;
       const uint32_t t = (uint32_t)(ca * P.r + ddi) * P.W + (uint32_t)(cc * P.r + ddj);
@@ -836,12 +1007,14 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     for (int w = 0; w < NW; w += 2)   // (three rows close each of the two lists)
       any_over |= (int)sm.cnt[w * 32 + lane] + (int)sm.cnt[w * 32 + 32 + (lane ^ (int)rot)] + 6 > R;
     if (__any_sync(kFull, any_over)) reason = 1;
+    else if (LISTED && is_q) reason = 0;
     else if (n_all < P.top_k) reason = 2;
     else if (!(fabsf(mx - ref) <= kNearRefGap)) reason = 5;
     unsigned cum = 0, in_bin = 0;
     int bstar = 0;
     const int rank = n_all - P.top_k + 1;   // 1-based rank from the bottom of the k-th largest
-    if (reason == 0) {
+    const bool select = reason == 0 && !(LISTED && is_q);
+    if (select) {
       // ---- the bin that holds the k-th largest: which eight bins, then which of them
       const uint4 h0 = *reinterpret_cast<const uint4*>(sm.hist + lane * 8);
       const uint4 h1 = *reinterpret_cast<const uint4*>(sm.hist + lane * 8 + 4);
@@ -875,7 +1048,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     float theta = 0.f;
     int n_ge = 0;
     double Z = 0.0;
-    if (reason == 0) {
+    if (select && reason == 0) {
       s_t += window(low_a, low_b, inv_w, hoff, c0, bstar);
       const double w = warp_sum((double)s_t);
       if (lane == 0) sm.w_all[warp] = w;
@@ -883,7 +1056,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     __syncthreads();   // ---- barrier 2
 #pragma unroll 1
     for (int i = tid; i < kRBins + 4; i += NT) sm.hist[i] = 0;
-    if (reason == 0) {
+    if (select && reason == 0) {
       // ---- the crossing bin's entries: exact rank, and their weights
       const int want = rank - (int)cum, mcount = (int)in_bin;
       float vmin = INFINITY, vmax = -INFINITY;
@@ -922,17 +1095,17 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
       }
       n_ge = n_all - (int)cum - less_at;
       // (values of one bin share their exponent: sums of them in double are exact, whatever the order)
-      double all = (double)mcount * (double)ex2f(fmaf(theta, kLog2e, c0));
+      double all = (double)mcount * (double)weight_of(theta, c0);
       if (kmin != kmax) {
         all = 0.0;
 #pragma unroll 1
         for (int i = lane; i < mcount; i += 32) {
           const float v = sm.sa_z[i];
-          if (v >= theta) all += (double)ex2f(fmaf(v, kLog2e, c0));
+          if (v >= theta) all += (double)weight_of(v, c0);
         }
         all = warp_sum(all);
       }
-      if (kmin != kmax || !is_q) {   // (a draft row keeps its logits: nothing changes unless some fall below)
+      if (!SUMS && (kmin != kmax || !is_q)) {   // (a draft row keeps its logits: nothing changes unless some fall below)
         double own = 0.0;
         uint32_t at = tl;
 #pragma unroll 1
@@ -949,15 +1122,20 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
           low_a = low_b;
           at += 32 * step;
         }
-        s_t = (float)((double)s_t + own);
+        s_t = (Sum)((double)s_t + own);
       }
       Z = all;
 #pragma unroll
       for (int w = 0; w < NW; ++w) Z += sm.w_all[w];
     }
+    if (LISTED && is_q) {
+      theta = theta_q;
+      const float* const st = a.stats_in + (size_t)g * 4;
+      Z = (double)__ldg(st + 2) + (double)__ldg(st + 3);
+    }
     const bool ok = reason == 0 && Z > 0.0 && Z < 1e300;
     const bool again = !ok && reason != 0 && reason != 4 && tries + 1 < kRTries;
-    if (tid == 32 && !again)
+    if (tid == 32 && !again && !(LISTED && is_q))
       row_learn(&pr, ok, reason, theta, pivot, n_all, n_ge, mx, a.margin, a.a_theta, a.a_boot);
 
     if (!ok) {   // CTA-uniform
@@ -984,7 +1162,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
           pivot = next;
         }
         prologue(part(rc), part(ru));
-        if (!SAMPLE && !is_q && more && !nq) {   // (the position was advanced to the next row above)
+        if (KIND == kRowsRound && !is_q && more && !nq) {   // (the position was advanced to the next row above)
           if (--dj < 0) {
             dj = P.r - 1;
             --di;
@@ -999,6 +1177,23 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         if (tid == 0) defer(g);
       } else {
         // the draft row is lost: its parent's rows go with it (those of this CTA)
+        if constexpr (LISTED) {
+          for (;;) {
+            if (tid == 0) defer(target_index());
+            if (++unit >= u_end) break;
+            const int before = parent;
+            b = b_next;
+            pick = pick_next;
+            parent = pick_parent(pick, b);
+            if (--left > 0) next_pick();
+            if (parent != before) break;
+          }
+          if (unit >= u_end) break;
+          is_q = (pick & kPickDraft) != 0u;
+          g = is_q ? (uint32_t)parent : target_index();
+          prologue(part(row_c(is_q, g)), part(row_u(is_q, g)));
+          continue;
+        } else {
 #pragma unroll 1
         while (true) {
           if (tid == 0) defer(target_index());
@@ -1019,22 +1214,41 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         tok_next = __ldg(a.draft_tok_lo + parent);
         prologue(part(row_c(true, g)), nullptr);
         continue;
+        }
       }
     } else if (!SAMPLE && is_q) {
       tries = 0;
       // ---- a draft row ends here
       c0_q = c0;
       Zq = (float)Z;
-      q_tok = sm.z_tok >= theta ? rows_div(sm.e_tok, Z) : 0.0;
-      if (q_tok <= 0.0 && tid == 0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
+      if (!LISTED) {
+        q_tok = sm.z_tok >= theta ? rows_div(sm.e_tok, Z) : 0.0;
+        if (q_tok <= 0.0 && tid == 0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
+      }
       __syncthreads();   // ---- barrier 3
       if (tid == 0) sm.n_sa = 0;
       partner_n = 0;
       partner_q = pair_n;
       rot_q = rot;
+    } else if constexpr (SUMS) {
+      tries = 0;
+      if (tid == (NW - 1) * 32) {   // (who wrote x~'s weight)
+        if constexpr (KIND == kRowsVerify) {
+          const uint32_t N = (uint32_t)P.H * (uint32_t)P.W, image = g / N, t = g - image * N, i = t / P.W, j = t - i * P.W;
+          const uint32_t cell = (image * P.h + i / P.r) * P.w + j / P.r;
+          const float zq = mix_logit(wide_logit<BF16>(raw_logit<BF16>(a.draft + (size_t)cell * row_bytes, tok)), 0.f, false, 0.f, P.invT);
+          const float* const st = a.stats_in + (size_t)cell * 4;
+          rows_verified(&a, g, sm.z_tok >= theta ? sm.e_tok : 0.0, Z, mx, ref, zq, st[0], st[1], (double)st[2] + (double)st[3]);
+        } else {
+          rows_stats(&a, g, sm.z_tok, theta, mx, ref, Z);
+        }
+      }
+      __syncthreads();   // ---- barrier 3
+      if (tid == 0) sm.n_sa = 0;
+      partner_n = 0;
     } else {
       tries = 0;
-      const double e_tok = !SAMPLE && sm.z_tok >= theta ? sm.e_tok : 0.0;
+      const double e_tok = KIND == kRowsRound && sm.z_tok >= theta ? sm.e_tok : 0.0;
       double mass = e_tok;   // x~'s weight with what is pooled onto it
       // where an id of the row is: the thread, its mask word, the bit in it
       struct Spot {
@@ -1173,6 +1387,11 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
         const uint32_t cell = g - (uint32_t)b * (uint32_t)(P.h * P.w);
         const uint4 v = row_philox(make_uint4(cell, (uint32_t)b + P.image_offset, P.round, 1u), make_uint2(P.seed_lo, P.seed_hi));
         u_tgt = uniform24(v.x);
+      } else if (LISTED) {
+        const uint4 v = row_philox(make_uint4(pick & kPickIndex, (uint32_t)b + P.image_offset, P.round, 0u), make_uint2(P.seed_lo, P.seed_hi));
+        u_res = uniform24(v.y);
+        u_tgt = uniform24(v.z);
+        pending = (pick & kPickResidual) != 0u ? kDrawResidual : kDrawTarget;
       } else {
         const uint32_t* const rnd = sm.rnd[parent & 1][child & 15];
         int accepted;
@@ -1398,7 +1617,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
             has = __ballot_sync(kFull, wt > 0.f);
             // (no id with weight: a sum that was rounding noise of a difference -- to the general routines)
             const int chosen = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : -1;
-            int32_t* const out = SAMPLE ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
+            int32_t* const out = SAMPLE || LISTED ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
             if (lane == chosen) *out = (((og * a.ppg + w * 4 + (src >> 3)) << 3) + (src & 7)) * IDS + chosen;
             if (chosen < 0 && lane == 0) defer(g);
           }
@@ -1417,11 +1636,20 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(SAMPLE) / NW) k_round_rows
     // ---- on to the next row (its first pieces are in registers)
     if (!is_q) ++unit;
     if (!more) break;
-    if (!SAMPLE) {
+    if (KIND == kRowsRound) {
       if (is_q) child = di * P.r + dj;
       else ++child;
     }
-    if (SAMPLE || nq) next_parent();
+    if constexpr (LISTED) {
+      if (!is_q) {
+        b = b_next;
+        pick = pick_next;
+        parent = parent_next;
+        if (--left > 0) next_pick();
+      }
+    } else {
+      if (KIND == kRowsSample || nq) next_parent();
+    }
     is_q = nq;
     g = ng;
   }

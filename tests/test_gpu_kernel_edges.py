@@ -160,3 +160,42 @@ def test_general_path_around_shared_memory(ctx, V, how):
 def test_redraw_around_shared_memory(ctx, V):
     redraw.test_redraw_steps_against_oracle(ctx, dict(B=1, H=4, W=12, V=V, dtype="bf16", top_k=V // 8, cfg_scale=2.0,
                                                       temperature=0.9, window=4, density=0.5))
+
+
+STAGES = synth.RoundConfig("stages", B=2, H=24, W=26, V=4096, dtype="bf16", sigma=1.0, cfg_scale=3.0, top_k=500, radius=1, seed=1201)
+
+
+@pytest.mark.parametrize("over", [
+    dict(), dict(V=1024, top_k=100, dtype="f32"), dict(V=4104, top_k=600, cfg_scale=0.0, temperature=0.8), dict(V=16384, top_k=2000),
+    dict(V=8192, top_k=2600), dict(r=1, H=20, W=31, V=8192, sigma=0.1, cfg_scale=0.0, radius=0), dict(r=3, H=24, W=27, radius=2, sigma=0.3), dict(B=1, H=36, W=36, resample_mode=binding.RESAMPLE_RESIDUAL_ALL),
+    dict(resample_mode=binding.RESAMPLE_TARGET_ALL), dict(accept_mode=binding.ACCEPT_THRESHOLD, tau=1e-3),
+    dict(resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL, radius=3), dict(cubed=True), dict(quantum=0.5, cfg_scale=0.0), dict(B=2, shift=True),
+], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain")
+def test_stages_of_many_rows(ctx, over):
+    """More rows than the stages keep in shared memory: the streaming kernels, rows that mislead their predictions included."""
+    over = dict(over)
+    cubed, quantum, shift = over.pop("cubed", False), over.pop("quantum", 0.0), over.pop("shift", False)
+    cfg = dataclasses.replace(STAGES, **over)
+    batch = pu.build_batch(cfg)
+    for k in ("cond", "uncond", "draft_lo"):
+        if batch[k] is None:
+            continue
+        if cubed:
+            batch[k] = (batch[k].float() ** 3 / 8).to(batch[k].dtype)
+        if quantum:
+            batch[k] = ((batch[k].float() / quantum).round() * quantum).to(batch[k].dtype)
+        if shift:     # every other row lies 20 higher
+            batch[k][:, :, ::2] += 20.0
+    pu.redraw_tokens(cfg, batch)
+    n0 = ctx.kernel_launches()
+    g = pu.gpu_stages(ctx, cfg, batch)
+    isolated = cfg.resample_mode == binding.RESAMPLE_ISOLATED_RESIDUAL
+    assert ctx.kernel_launches() - n0 == (2 if cfg.r == 1 else 1) + 3 + 1 + (1 if isolated else 3)   # the fast paths, but for few draft rows
+    o = pu.oracle_images(cfg, batch, list(range(cfg.B)))
+    pu.check_round(cfg, g, o)
+    for b in range(cfg.B):
+        want = orc.upsample_pool_image(pu.orc_params(cfg, b), synth.to_numpy_logits(batch["draft_lo"][b]), batch["tok_lo"][b].cpu().numpy())
+        np.testing.assert_array_equal(g["tok_hi"][b], want["tok_hi"])
+        np.testing.assert_allclose(g["stats"][b].astype(np.float64)[..., 0:2], want["stats"][..., 0:2], rtol=0, atol=0)
+        np.testing.assert_allclose(g["stats"][b][..., 2].astype(np.float64) + g["stats"][b][..., 3], want["stats"][..., 2], rtol=1e-6)
+    assert ctx.poll_device_status() & ~(binding.DEV_DENSE_FALLBACK | binding.DEV_ZERO_DRAFT_PROB) == 0
