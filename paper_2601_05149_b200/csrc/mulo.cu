@@ -1406,14 +1406,14 @@ mulo_status mulo_redraw_step(mulo_ctx* ctx, const mulo_params* p, int32_t s_inde
   a.out_tok = out_tok;
   a.s = s_index;
   const int np = a.P.V <= kRedrawIds ? 1 : a.P.V <= 2 * kRedrawIds ? 2 : 4, ctas = (a.P.V + np * kRedrawIds - 1) / (np * kRedrawIds);
-  // The step's positions are counted on the device: a fixed number of clusters strides over them.  A schedule of window 8 to 16
-  // has W / 8 to W / 16 of them per image at a time; twice the larger as long as half of the chip holds them -- what is left
-  // over draws the next step's rows meanwhile -- and that many beyond.  64 x 64, 4 images, V = 16384 (15 positions, 64 clusters):
-  // 5.3 us a step, 8.5 before; 16 x 16, 29 images (54 positions): 74 clusters, where 116, which leave no room, took 12.1 us, 11.6
-  // before.  32 x 32, 64 images, V = 2048 (234 positions): 9.2 us, 15.5 before.
+  // The step's positions are counted on the device: a fixed number of clusters strides over them, as many as a schedule of window
+  // 8 has positions at a time (W / 8 per image), and 32 at least.  No more: what is left of the chip draws the next steps' rows
+  // meanwhile.  64 x 64, 4 images, V = 16384 (15 positions): 3.4 us a step with 32 clusters, 5.3 with 64 (as a graph; the host's
+  // calls take 4.9), 8.5 before; 16 x 16, 29 images (54 positions): 9.7 with 58, 12.1 with 116, 11.6 before.  Eight clusters for one image
+  // of sparse islands (10 positions, at most 58) were 1.8 times slower than 16.
   const int room = ctx->sm_count * (np == 4 ? 1 : 2) / ctas;
-  const long long twice = (long long)p->B * (p->W > 4 ? p->W / 4 : 1), likely = twice <= room / 2 ? twice : twice / 2 > room / 2 ? twice / 2 : room / 2;
-  const int clusters = likely < room ? (int)likely : room;
+  const long long likely = (long long)p->B * (p->W > 8 ? p->W / 8 : 1), wanted = likely > 32 ? likely : 32;
+  const int clusters = wanted < room ? (int)wanted : room;
   auto kern = a.P.bf16 ? (np == 1 ? k_redraw_step<true, 1> : np == 2 ? k_redraw_step<true, 2> : k_redraw_step<true, 4>)
                        : (np == 1 ? k_redraw_step<false, 1> : np == 2 ? k_redraw_step<false, 2> : k_redraw_step<false, 4>);
   cudaLaunchConfig_t cfg;
