@@ -221,6 +221,8 @@ __global__ void __launch_bounds__(kIslandThreads) k_islands(IslandArgs a) {
 // that needs a step.  ONE warp then goes down the rows: what the row above demands, one scan over the slots (a term that grows
 // from island to island keeps them apart, however their runs interleave), and the steps are there; a row's slots are asked
 // for one row ahead.  What bounds the kernel is this chain of H rows.
+// (64 x 64, 32 images: 43.1 k of 61 k cycles with the slots' keys formed in the chain, 36 us in all, 44 with a second pass over an
+// island's runs; 25 to 30 us with everything at hand that does not depend on a step.)
 struct ScheduleArgs {
   int H, W, window;
   const int32_t* labels;   // [B, H, W]
@@ -229,11 +231,12 @@ struct ScheduleArgs {
 };
 
 constexpr int kScheduleThreads = 1024;
+constexpr int kScheduleSlack = 128;    // slots past the last row's, which the chain's lanes may touch
 constexpr int kIslandTerm = 1 << 15;   // more than two steps, or columns, of one image can differ by
 
 __host__ inline size_t schedule_smem(int H, int W) {
   const size_t N = (size_t)H * W, nw = (size_t)H * ((W + 31) / 32);
-  return N * 12 + 2 * nw * 4;   // (at most 228,608 bytes: 4000 x 4)
+  return (N + kScheduleSlack) * 12 + 2 * nw * 4;   // (at most 230,144 bytes: 4000 x 4)
 }
 
 // M: slots per lane in the chain of rows; rows of more than 32 M columns take several turns.
@@ -242,14 +245,16 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
   extern __shared__ __align__(16) unsigned char sched_smem[];
   const int H = a.H, W = a.W, N = H * W, Ww = (W + 31) / 32, nw = H * Ww, b = blockIdx.x, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
+  const int S = N + kScheduleSlack;
   int* const lab = reinterpret_cast<int*>(sched_smem);
-  uint16_t* const steps = reinterpret_cast<uint16_t*>(sched_smem);          // by slot, once the labels are not needed any more
-  // by slot: the slot of the row above that it depends on (0xffff: none) | its number among its island's in the row << 16
-  uint32_t* const dep = reinterpret_cast<uint32_t*>(lab + N);
-  uint32_t* const pos = dep + N;                                            // bit: the position is in R_X
+  uint16_t* const steps = reinterpret_cast<uint16_t*>(sched_smem) + 1;      // by slot, once the labels are not needed any more
+  // by slot: what the step loses to become the key of the scan, its number among its island's in the row less a term that grows
+  // with the island's first slot; 1 + the slot of the row above that it depends on, counted through the rows (0: none, steps[-1])
+  int* const less = lab + S;
+  uint32_t* const pos = reinterpret_cast<uint32_t*>(less + S);              // bit: the position is in R_X
   uint32_t* const first = pos + nw;                                         // bit: ... and starts a run
-  uint16_t* const head = reinterpret_cast<uint16_t*>(first + nw);           // by slot: the first slot of its island
-  uint16_t* const slot = head + N;                                          // by column
+  uint16_t* const above = reinterpret_cast<uint16_t*>(first + nw);
+  uint16_t* const slot = above + S;                                         // by column
   __shared__ int s_max;
   if (tid == 0) s_max = 0;
   let_next_begin();
@@ -257,8 +262,12 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
   const int32_t* const labels = a.labels + (size_t)b * N;
   for (int t = tid; t < N; t += kScheduleThreads) {
     lab[t] = labels[t];
-    dep[t] = 0xffffu;
-    head[t] = 0;
+    above[t] = 0;
+    less[t] = 0;
+  }
+  for (int t = N + tid; t < S; t += kScheduleThreads) {
+    above[t] = 0;
+    less[t] = 0;
   }
   __syncthreads();
   for (int w = warp; w < nw; w += kScheduleThreads / 32) {   // the rows' masks
@@ -289,7 +298,7 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
     }
     if (m > 0) {
       slot[i * W + j] = (uint16_t)(below + before);
-      head[i * W + below + before] = (uint16_t)below;
+      less[i * W + below + before] = before - below * kIslandTerm;
     }
   }
   __syncthreads();
@@ -305,61 +314,55 @@ __global__ void __launch_bounds__(kScheduleThreads) k_island_schedule(ScheduleAr
     const int i = w / Ww, j = (w % Ww) * 32 + lane;
     if (!(pos[w] >> lane & 1u)) continue;
     const int m = lab[i * W + j], at = slot[i * W + j];
-    int u = 0xffff;
+    int u = 0;
     if (i > 0) {   // the island's last position of the row above inside the window: run by run
       int x = last_at(pos + (i - 1) * Ww, min(W - 1, j + a.window - 1));
       while (x >= 0 && lab[(i - 1) * W + x] != m) x = last_at(pos + (i - 1) * Ww, last_at(first + (i - 1) * Ww, x) - 1);
-      if (x >= 0) u = slot[(i - 1) * W + x];
+      if (x >= 0) u = 1 + (i - 1) * W + slot[(i - 1) * W + x];
     }
-    dep[i * W + at] = (uint32_t)u | (uint32_t)(at - head[i * W + at]) << 16;
+    above[i * W + at] = (uint16_t)u;
   }
   __syncthreads();
   if (warp == 0) {
+    if (lane == 0) steps[-1] = 0;
+    __syncwarp();
+    // A lane has M slots in a row.  Lanes past the row's end work on the next row's entries, or on slots that are not used: what they
+    // find comes after everything of this row in the scan, and is overwritten when its row's turn comes.
     const int turns = (W + 32 * M - 1) / (32 * M);
-    uint32_t d[M];
-    int h[M];
-    auto ask = [&](int i, int c) {   // (slots that are not used come last in a row: whatever they hold reaches nobody)
+    int u[M], l[M];
+    auto ask = [&](int at) {
 #pragma unroll
       for (int k = 0; k < M; ++k) {
-        const int q = (c * 32 + lane) * M + k;
-        d[k] = 0xffffu;
-        h[k] = 0;
-        if (q < W && i < H) {
-          d[k] = dep[i * W + q];
-          h[k] = head[i * W + q];
-        }
+        u[k] = above[at + k];
+        l[k] = less[at + k];
       }
     };
-    ask(0, 0);
-    const uint16_t* above = steps;
-    for (int i = 0; i < H; ++i) {
+    ask(lane * M);
+    for (int i = 0, row = lane * M; i < H; ++i, row += W) {
       int carry = INT_MIN;
-      for (int c = 0; c < turns; ++c) {
-        int v[M], back[M];   // back: what turns a key into the step again
+      for (int c = 0, at = row; c < turns; ++c, at += 32 * M) {
+        int v[M], back[M];
 #pragma unroll
         for (int k = 0; k < M; ++k) {
-          const uint32_t u = d[k] & 0xffffu;
-          back[k] = (int)(d[k] >> 16) - h[k] * kIslandTerm;
-          v[k] = (u != 0xffffu ? (int)above[u] + 1 : 1) - back[k];
+          back[k] = l[k];
+          v[k] = (int)steps[u[k] - 1] + 1 - l[k];
         }
-        if (c + 1 < turns) ask(i, c + 1);
-        else ask(i + 1, 0);
+        const bool on = c + 1 < turns;
+        if (on ? at + 32 * M < S - M : i + 1 < H) ask(on ? at + 32 * M : row + W);
 #pragma unroll
         for (int k = 1; k < M; ++k) v[k] = max(v[k], v[k - 1]);
         int inc = v[M - 1];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) inc = max(inc, __shfl_up_sync(0xffffffffu, inc, o));   // (the first lanes get their own)
-        int exc = __shfl_up_sync(0xffffffffu, inc, 1);
-        exc = max(lane == 0 ? INT_MIN : exc, carry);
+        const int left = __shfl_up_sync(0xffffffffu, inc, 1);
+        const int exc = max(lane == 0 ? INT_MIN : left, carry);
         if (turns > 1) carry = max(carry, __shfl_sync(0xffffffffu, inc, 31));
+        if (turns == 1 || at < S - M) {
 #pragma unroll
-        for (int k = 0; k < M; ++k) {
-          const int q = (c * 32 + lane) * M + k;
-          if (q < W) steps[i * W + q] = (uint16_t)(max(v[k], exc) + back[k]);
+          for (int k = 0; k < M; ++k) steps[at + k] = (uint16_t)(max(v[k], exc) + back[k]);
         }
       }
       __syncwarp();
-      above = steps + i * W;
     }
   }
   __syncthreads();
