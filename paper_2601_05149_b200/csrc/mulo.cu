@@ -126,18 +126,26 @@ __global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_pool(RowKern
   __shared__ GeneralScratch<RES> sc;
   upsample_cell<RES>(a, blockIdx.x, sc, dyn);   // b*h*w + ca*w + cc
 }
-// Second launch of its fast path: the cells the fast kernel put on its list.
+// Second launch of its fast path: the cells the fast kernel marked.
 template <bool RES>
-__global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_failed(RowKernelArgs a, const int32_t* fail_list,
-                                                                           const uint32_t* fail_count) {
+__global__ void __launch_bounds__(kThreads, RES ? 2 : 4) k_upsample_failed(RowKernelArgs a) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GeneralScratch<RES> sc;
+  __shared__ unsigned found[kWarps];
   let_next_begin();
   wait_for_previous();
-  const size_t total = (size_t)a.P.B * a.P.h * a.P.w, n = min((size_t)*fail_count, total);
-  for (size_t idx = blockIdx.x; idx < n; idx += gridDim.x) {
-    const size_t cell = (size_t)fail_list[idx];
-    if (cell < total) upsample_cell<RES>(a, (int)cell, sc, dyn);
+  const int total = a.P.B * a.P.h * a.P.w;
+  for (int c0 = (int)blockIdx.x * kThreads; c0 < total; c0 += (int)gridDim.x * kThreads) {
+    const int cell = c0 + (int)threadIdx.x;
+    const bool mine = cell < total && __float_as_uint(a.stats_out[(size_t)cell * 4]) == kStatsLeft;
+    const unsigned word = __ballot_sync(kFull, mine);
+    if ((threadIdx.x & 31) == 0) found[threadIdx.x >> 5] = word;
+    if (!__syncthreads_or(mine)) continue;
+    for (int w = 0; w < kWarps; ++w)
+      for (unsigned left = found[w]; left; left &= left - 1u) {   // (block-uniform)
+        upsample_cell<RES>(a, c0 + w * 32 + __ffs(left) - 1, sc, dyn);
+        __syncthreads();
+      }
     __syncthreads();
   }
 }
@@ -1314,13 +1322,11 @@ mulo_status mulo_upsample_pool(mulo_ctx* ctx, const mulo_params* p, const void* 
   // 148, 106 us).  64 rows: 14 to 17 us, 9 to 14 us resident.
   const int cells = p->B * a.P.h * a.P.w;
   const cudaStream_t st = (cudaStream_t)stream;
-  // With one, many rows are streamed, if there is room for the list of rows that this may leave.
-  Workspace w;
+  // With one, many rows are streamed.
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
   int rnw = 0;
-  const bool many = many_rows(ctx, kRowsStats, a.P.V, cells) && check_ws(ctx, p, &w) == MULO_OK &&
-                    ((uintptr_t)draft_stats_lo & 15u) == 0;
+  const bool many = many_rows(ctx, kRowsStats, a.P.V, cells) && ((uintptr_t)draft_stats_lo & 15u) == 0;
   if (const size_t rdyn = many ? plan_rows(ctx, a.P, kRowsStats, &ra, &rnw) : 0) {
     ra.P = a.P;
     ra.cond = a.draft;
@@ -1328,12 +1334,10 @@ mulo_status mulo_upsample_pool(mulo_ctx* ctx, const mulo_params* p, const void* 
     ra.stats_out = draft_stats_lo;
     ra.tok_hi_out = draft_tok_hi;
     ra.q_hi_out = q_tok_hi;
-    ra.dev_status = w.status;
-    ra.fail_list = w.fail_list;
+    ra.dev_status = a.dev_status;
     ra.n_units = cells;
-    if (cudaMemsetAsync(w.status + kFailCount, 0, sizeof(uint32_t), st) != cudaSuccess) return MULO_ERR_CUDA;
     if (launch_rows<kRowsStats>(ctx, ra, rnw, rdyn, st)) {
-      if (!MULO_LAUNCH_LEFT(K_UPSAMPLE_FAILED, general_smem(a.P, false), st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
+      if (!MULO_LAUNCH_LEFT(K_UPSAMPLE_FAILED, general_smem(a.P, false), st, a)) return MULO_ERR_CUDA;
       return launched(ctx, 2);
     }
   }

@@ -62,6 +62,7 @@ constexpr float kNearRefGap = 8.0f;      // a row whose maximum lies further fro
 constexpr int kRowsRound = 0, kRowsSample = 1, kRowsVerify = 2, kRowsStats = 3, kRowsResample = 4;
 // An entry of kRowsResample's list: the position in its image, whether it is drawn from the residual, whether any position of its
 // parent is (the draft row is not read otherwise).
+constexpr uint32_t kStatsLeft = 0xffa5c3e1u;   // in the place of a threshold: a NaN that no logit gives
 constexpr uint32_t kPickIndex = (1u << 30) - 1u, kPickResidual = 1u << 31, kPickDraft = 1u << 30;
 
 // running prediction for one kind of row (draft / target), per CTA
@@ -837,6 +838,12 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     atomicAdd(a.dev_status + slot, 1u);
   };
   auto defer = [&](uint32_t g) {           // one thread: position (cell) g goes to the general routines
+    if constexpr (KIND == kRowsStats) {    // (marked in its own output: no list, and nothing shared with calls on other streams)
+      reinterpret_cast<uint32_t*>(a.stats_out)[(size_t)g * 4] = kStatsLeft;
+      atomicAdd(a.dev_status + kCntRows, 1u);
+      atomicOr(a.dev_status, MULO_DEV_DENSE_FALLBACK);
+      return;
+    }
     const unsigned at = atomicAdd(a.dev_status + kFailCount, 1u);
     a.fail_list[at] = (int32_t)g;
     atomicAdd(a.dev_status + kCntRows, 1u);

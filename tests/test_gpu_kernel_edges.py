@@ -169,7 +169,8 @@ STAGES = synth.RoundConfig("stages", B=2, H=24, W=26, V=4096, dtype="bf16", sigm
     dict(), dict(V=1024, top_k=100, dtype="f32"), dict(V=4104, top_k=600, cfg_scale=0.0, temperature=0.8), dict(V=16384, top_k=2000),
     dict(V=8192, top_k=2600), dict(r=1, H=20, W=31, V=8192, sigma=0.1, cfg_scale=0.0, radius=0), dict(r=3, H=24, W=27, radius=2, sigma=0.3), dict(B=1, H=36, W=36, resample_mode=binding.RESAMPLE_RESIDUAL_ALL),
     dict(resample_mode=binding.RESAMPLE_TARGET_ALL), dict(accept_mode=binding.ACCEPT_THRESHOLD, tau=1e-3),
-    dict(resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL, radius=3), dict(cubed=True), dict(quantum=0.5, cfg_scale=0.0), dict(B=2, shift=True),
+    dict(resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL, radius=3), dict(cubed=True), dict(quantum=0.5, cfg_scale=0.0),
+    dict(r=1, H=20, W=31, V=8192, top_k=1000, quantum=0.5), dict(B=2, shift=True),
 ], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain")
 def test_stages_of_many_rows(ctx, over):
     """More rows than the stages keep in shared memory: the streaming kernels, rows that mislead their predictions included."""
