@@ -14,10 +14,11 @@
 //              its ids.
 //
 // The launch may begin while the kernels before it in the stream still run (programmatic dependent launch).  The first row of
-// a CTA is drawn BEFORE it waits for them, from the list and the logits as they are at that moment; after the wait both are
+// a cluster is drawn BEFORE it waits for them, from the list and the logits as they are at that moment; after the wait both are
 // read again, and the token counts only if every logit mixes to the same value as before and the list names the same
 // position -- otherwise the row is drawn again from what is there now.  So a step costs its successor a re-read instead of
-// the whole chain.
+// the whole chain.  Before the wait anything may be rewritten at any moment: ONE thread of the cluster reads the list and tells
+// the others what it found, and every later verdict is one for the whole cluster, so no barrier is ever met by a part of it.
 #pragma once
 
 #include "mulo_resident.cuh"
@@ -47,6 +48,7 @@ struct RedrawSmem {
   uint32_t w_max[kRedrawMaxCtas * kWarps];
   uint32_t tot[kWarps];
   uint32_t same[kRedrawMaxCtas];
+  uint2 ahead;                                // the list's start and the row to draw before the wait, as one thread found them
   int bin, in_bin;
   unsigned over, n_member;
   float theta;
@@ -125,7 +127,13 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
   };
 
   // what the step will find, if the list stays as it is
-  const int beg0 = ld_fresh(a.offsets + a.s), end0 = ld_fresh(a.offsets + a.s + 1);
+  uint2 found = make_uint2(0u, total);
+  if (rank == 0 && tid == 0) {
+    const int beg = ld_fresh(a.offsets + a.s), end = ld_fresh(a.offsets + a.s + 1);
+    const long long at = (long long)beg + cluster;
+    if (beg >= 0 && at < end && at < (long long)total) found = make_uint2((uint32_t)beg, (uint32_t)ld_fresh(a.pos_list + at));
+    sm.ahead = found;
+  }
   auto clear = [&]() {
     reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < n_warps) sm.m_sum[tid] = 0.0;
@@ -133,9 +141,6 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
   };
   static_assert(kRedrawWords == 4 * kThreads && kRedrawMaxCtas * kWarps <= kThreads, "one 16-byte word per thread");
   clear();
-  const uint32_t i0 = (uint32_t)beg0 + (uint32_t)cluster;
-  uint32_t g = total;
-  if (beg0 >= 0 && (int)i0 < end0 && i0 < total) g = (uint32_t)ld_fresh(a.pos_list + i0);
   RowSrc src;
   src.s = P.cfg_scale;
   src.invT = P.invT;
@@ -171,13 +176,14 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
     return uniform24(philox4x32_10(make_uint4(t, b + P.image_offset, P.round, 1u + (uint32_t)a.s), make_uint2(P.seed_lo, P.seed_hi)).x);
   };
   meet();   // (the peers run, everybody's memory is cleared)
-  bool waited = g >= total;
-  if (ctas > 1) {   // (the CTAs may have read different lists: together or not at all)
-    if (tid < (int)ctas) st_peer(peer_addr(smem_u32(&sm.same[rank]), tid), g < total ? g : 0xffffffffu);
-    meet();
-    for (uint32_t q = 0; q < ctas; ++q) waited = waited || sm.same[q] != g;
+  if (ctas > 1) {
+    if (rank == 0 && tid == 0)
+      for (uint32_t q = 1; q < ctas; ++q) st_peer(peer_addr(smem_u32(&sm.ahead), q), found);
     meet();
   }
+  const uint32_t beg0 = sm.ahead.x;
+  uint32_t g = sm.ahead.y;
+  bool waited = g >= total;
   int i = 0, end = 0;
   if (waited) {
     wait_for_previous();
@@ -478,19 +484,18 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
     waited = true;
     i = ld_fresh(a.offsets + a.s);
     end = ld_fresh(a.offsets + a.s + 1);
-    const int now = ld_fresh(a.pos_list + i0);
-    bool same = true;
+    const int now = ld_fresh(a.pos_list + beg0 + cluster);
+    bool same = i == (int)beg0 && i + cluster < end && (uint32_t)now == g;
     load(g, [&](int j, const float (&v)[8]) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) same = same && __float_as_uint(v[k]) == __float_as_uint(z[j][k]);
     });
-    same = __syncthreads_and(same);
+    bool holds = __syncthreads_and(same);
     if (ctas > 1) {
-      if (tid < (int)ctas) st_peer(peer_addr(smem_u32(&sm.same[rank]), tid), (uint32_t)same);
+      if (tid < (int)ctas) st_peer(peer_addr(smem_u32(&sm.same[rank]), tid), (uint32_t)holds);
       meet();
-      for (uint32_t q = 0; q < ctas; ++q) same = same && sm.same[q] != 0;
+      for (uint32_t q = 0; q < ctas; ++q) holds = holds && sm.same[q] != 0;
     }
-    const bool holds = same && i == beg0 && (int)i0 < end && (uint32_t)now == g;
     i += cluster;
     if (holds) {
       if (mine) a.out_tok[g] = tok;

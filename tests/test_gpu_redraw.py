@@ -279,6 +279,53 @@ def test_a_row_drawn_ahead_of_its_inputs(ctx, V, what):
         assert torch.equal(out, want)
 
 
+_LATE_LISTS = r"""
+extern "C" __global__ void late_lists(const int* new_off, int* off, int n_off, const int* new_list, int* list, int n_list, int cycles) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const long long t0 = clock64();
+  while (clock64() - t0 < cycles) {}
+  for (int i = threadIdx.x; i < n_list; i += blockDim.x) list[i] = new_list[i];
+  for (int i = threadIdx.x; i < n_off; i += blockDim.x) off[i] = new_off[i];
+}
+"""
+
+
+@pytest.mark.parametrize("V", [520, 8192, 16384, 20000, 49160])   # one, two and four CTAs to a row
+def test_a_list_rewritten_while_the_step_begins(ctx, V):
+    """The kernel before the step lets it begin and rewrites offsets and list at any moment of the step's first 10 us: the step before
+    gains a position, so both shift by one and an entry may be seen with either offset.  What counts is what stands there in the end."""
+    B, H, W = 2, 4, 16
+    cfg = synth.RoundConfig("late", B=B, H=H, W=W, V=V, r=1, dtype="bf16", top_k=V // 8, cfg_scale=0.0, seed=81)
+    p = binding.params_from_config(cfg)
+    g = torch.Generator(device="cuda").manual_seed(V)
+    z = (2.0 * torch.randn((B, H, W, V), generator=g, device="cuda")).bfloat16()
+    n = B * H * W
+
+    def plan(steps):
+        pos, off = torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(2 * 4, dtype=torch.int32, device="cuda")
+        ctx.mulo_redraw_plan(p, steps, 2, pos, off)
+        return pos, off
+
+    steps = torch.zeros((B, H, W), dtype=torch.int32, device="cuda")
+    steps.view(-1)[3:24:3] = 2
+    pos0, off0 = plan(steps)
+    pos1 = torch.cat([torch.tensor([1], dtype=torch.int32, device="cuda"), pos0[:-1]]).contiguous()   # position 1 in step 1 now
+    off1 = off0.clone()
+    off1[2:4] += 1
+    want = torch.full((B, H, W), -7, dtype=torch.int32, device="cuda")
+    ctx.mulo_redraw_step(p, 2, 2, pos1, off1, z, None, want)
+    torch.cuda.synchronize()
+    assert int((want >= 0).sum()) == int((steps == 2).sum())
+    kernel = torch.cuda._compile_kernel(_LATE_LISTS, "late_lists", compute_capability="100a")
+    for cycles in range(0, 20000, 500):
+        pos, off = pos0.clone(), off0.clone()
+        out = torch.full_like(want, -7)
+        torch.cuda.synchronize()
+        kernel(grid=(1, 1, 1), block=(64, 1, 1), args=[off1, off, 8, pos1, pos, n, cycles])
+        ctx.mulo_redraw_step(p, 2, 2, pos, off, z, None, out)
+        assert torch.equal(out, want), cycles
+
+
 @pytest.mark.parametrize("case", [
     dict(V=8, top_k=3), dict(V=4096, top_k=4095), dict(V=4104, top_k=1), dict(V=8200, top_k=1000), dict(V=16384, top_k=0), dict(V=16392, top_k=2000),
     dict(V=65536, top_k=4000), dict(V=65536, top_k=0), dict(V=32776, top_k=30000, dtype="f32"),
