@@ -1409,7 +1409,10 @@ mulo_status mulo_redraw_step(mulo_ctx* ctx, const mulo_params* p, int32_t s_inde
   a.offsets = step_offsets;
   a.out_tok = out_tok;
   a.s = s_index;
-  const int np = a.P.V <= kRedrawIds ? 1 : a.P.V <= 2 * kRedrawIds ? 2 : 4, ctas = (a.P.V + np * kRedrawIds - 1) / (np * kRedrawIds);
+  const int np = a.P.V <= 4 * kRedrawIds ? 1 : a.P.V <= 8 * kRedrawIds ? 2 : 4, ctas = (a.P.V + np * kRedrawIds - 1) / (np * kRedrawIds);
+  // Eight ids per thread as long as four CTAs hold the row: a row's chain is the shorter the fewer ids a thread has.  64 x 64, 4 images,
+  // V = 16384, window 16, an ordinary kernel (1.3 us) between any two steps: 12.9 us a step with four CTAs, 15.6 with two, 19.6 with
+  // one; V = 8192: 11.9 with two, 13.6 with one; V = 32768: 17.1 with four, 22.2 with two.
   // The step's positions are counted on the device: a fixed number of clusters strides over them, as many as a schedule of window
   // 8 has positions at a time (W / 8 per image), and 32 at least.  No more: what is left of the chip draws the next steps' rows
   // meanwhile.  64 x 64, 4 images, V = 16384 (15 positions): 3.4 us a step with 32 clusters, 5.3 with 64 (as a graph; the host's

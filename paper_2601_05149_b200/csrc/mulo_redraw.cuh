@@ -2,7 +2,7 @@
 // draws its token from the target distribution of the given logits.
 //
 // Steps follow one another by the thousand with a handful of positions each, so a step is bound by the latency of ONE row.
-// A row's ids stay in the registers of one CTA of 512 threads (a cluster of up to four beyond V = 16384):
+// A row's ids stay in the registers of a cluster of up to four CTAs of 512 threads, eight ids per thread up to V = 16384:
 //
 //   load       128-bit loads, mixed at once
 //   select     a histogram of 4096 bins over the upper bits of the values as they are (the sign, sixteen binary orders of
