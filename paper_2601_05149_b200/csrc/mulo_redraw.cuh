@@ -294,8 +294,12 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
       redraw_range(bin, klo, khi);
       n_in = sm.in_bin;
       above = sm.over;
+      // (Entries of a bin are weighed in any order, so its sums in double have to be exact: 128 weights of 24 bits that lie within
+      // a factor of e^15 of one another.  The bins at the ends of the first histogram have no such bound, nor have ranges of
+      // keys far out.)
+      auto wide = [&]() { return !(key_float(khi) - key_float(klo) <= 15.0f); };
 #pragma unroll 1
-      while (n_in > kRedrawMembers && klo != khi) {   // a crowded bin is split again
+      while ((n_in > kRedrawMembers || wide()) && klo != khi) {   // a crowded or wide bin is split again
         meet();   // (everybody has read the counts)
         reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
         __syncthreads();
@@ -392,7 +396,7 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
       theta = sm.theta;
       if (tid < n_in) {
         const uint2 e = sm.member[tid];
-        // (weights of one bin differ by little: their sums in double are exact, whatever the order)
+        // (exact in double, whatever the order, and so the same in every CTA: see above)
         if (__uint_as_float(e.x) >= theta) atomicAdd(&sm.m_sum[e.y & (kRedrawMaxCtas * kWarps - 1)], (double)weight(__uint_as_float(e.x)));
       }
       __syncthreads();

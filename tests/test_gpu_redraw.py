@@ -332,6 +332,9 @@ def test_a_list_rewritten_while_the_step_begins(ctx, V):
     dict(V=4096, top_k=500, level=-300.0, scale=3.0), dict(V=4096, top_k=500, scale=1e-3), dict(V=8192, top_k=500, quantum=0.5),
     dict(V=16384, top_k=100, scale=0.0), dict(V=20480, top_k=5000, level=5000.0, scale=100.0, dtype="f32"), dict(V=4096, top_k=2100, quantum=0.25),
     dict(V=8192, top_k=700, dtype="f32", cfg_scale=2.0, temperature=0.8),
+    # a few entries in a bin whose values lie far apart: past the first histogram's end, above, below, and up to the type's largest
+    dict(V=20480, top_k=40, level=3000.0, scale=300.0, dtype="f32"), dict(V=49160, top_k=49100, level=-3000.0, scale=300.0, dtype="f32"),
+    dict(V=16384, top_k=20, scale=1e37, dtype="f32"),
 ], ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()))
 def test_rows_of_all_sizes_and_shapes(ctx, case):
     """Edges of the kernel's pieces and clusters; values outside the first histogram, crowded bins, ties, thresholds below zero."""
