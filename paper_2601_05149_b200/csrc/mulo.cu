@@ -1413,21 +1413,29 @@ mulo_status mulo_redraw_step(mulo_ctx* ctx, const mulo_params* p, int32_t s_inde
   // Eight ids per thread as long as four CTAs hold the row: a row's chain is the shorter the fewer ids a thread has.  64 x 64, 4 images,
   // V = 16384, window 16, an ordinary kernel (1.3 us) between any two steps: 12.9 us a step with four CTAs, 15.6 with two, 19.6 with
   // one; V = 8192: 11.9 with two, 13.6 with one; V = 32768: 17.1 with four, 22.2 with two.
-  // The step's positions are counted on the device: a fixed number of clusters strides over them, as many as a schedule of window
-  // 8 has positions at a time (W / 8 per image), and 32 at least.  No more: what is left of the chip draws the next steps' rows
-  // meanwhile.  64 x 64, 4 images, V = 16384 (15 positions): 3.4 us a step with 32 clusters, 5.3 with 64 (as a graph; the host's
-  // calls take 4.9), 8.5 before; 16 x 16, 29 images (54 positions): 9.7 with 58, 12.1 with 116, 11.6 before.  Eight clusters for one image
-  // of sparse islands (10 positions, at most 58) were 1.8 times slower than 16.
+  // The step's positions are counted on the device: a fixed number of clusters strides over them, 128 CTAs' worth, and as many as a
+  // schedule of window 8 has positions at a time (W / 8 per image) if that is more.  No more: what is left of the chip draws the
+  // next steps' rows meanwhile.  64 x 64, 4 images, V = 16384, window 16 (15 positions): 4.7 us a step with 32 clusters of four, 7.5 with 64 (as
+  // a graph; the host's calls take 4.9).
+  // A step of more positions than clusters (small windows; the first steps of sparse islands; any plan of the caller's) is shared out
+  // to single CTAs, each with a whole row in shared memory.  us a step, clusters only / so / the resident kernel with 296 CTAs that
+  // this one replaced: window 4 (64 positions) 14.7 / 12.4 / 9.0, window 1 (up to 256) 39 / 19 / 13, sparse islands at 2 % rejections
+  // (202 positions at first, 40 on average) 13 / 8.5 / 9.9, 4096 positions of one image at once 1050 / 312 / 227; V = 4096, window 1: 24 / 6.3 /
+  // 9.5.  Where two whole rows do not fit an SM (V > 24576) the clusters stride: room for a single row per SM would leave none
+  // for the next steps.
   const int room = ctx->sm_count * (np == 4 ? 1 : 2) / ctas;
-  const long long likely = (long long)p->B * (p->W > 8 ? p->W / 8 : 1), wanted = likely > 32 ? likely : 32;
+  const long long likely = (long long)p->B * (p->W > 8 ? p->W / 8 : 1), base = 128 / ctas, wanted = likely > base ? likely : base;
   const int clusters = wanted < room ? (int)wanted : room;
+  size_t dyn = (size_t)ctas * kRedrawWords * sizeof(uint32_t);
+  a.single = ctas > 1 && np < 4 && 2 * (resident_bytes(a.P.V) + sizeof(RedrawSmem) + sizeof(ResScratch) + 1024) <= (size_t)ctx->smem_optin;
+  if (a.single) dyn = resident_bytes(a.P.V) > dyn ? resident_bytes(a.P.V) : dyn;
   auto kern = a.P.bf16 ? (np == 1 ? k_redraw_step<true, 1> : np == 2 ? k_redraw_step<true, 2> : k_redraw_step<true, 4>)
                        : (np == 1 ? k_redraw_step<false, 1> : np == 2 ? k_redraw_step<false, 2> : k_redraw_step<false, 4>);
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = dim3((unsigned)(clusters * ctas));
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = (size_t)ctas * kRedrawWords * sizeof(uint32_t);
+  cfg.dynamicSmemBytes = dyn;
   cfg.stream = (cudaStream_t)stream;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

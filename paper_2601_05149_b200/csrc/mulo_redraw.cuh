@@ -19,6 +19,9 @@
 // position -- otherwise the row is drawn again from what is there now.  So a step costs its successor a re-read instead of
 // the whole chain.  Before the wait anything may be rewritten at any moment: ONE thread of the cluster reads the list and tells
 // the others what it found, and every later verdict is one for the whole cluster, so no barrier is ever met by a part of it.
+//
+// A step with more positions than clusters is bound by their number instead: after the wait every CTA takes whole rows for itself, by
+// the resident routines, two CTAs to an SM.
 #pragma once
 
 #include "mulo_resident.cuh"
@@ -33,6 +36,7 @@ constexpr int kRedrawIds = 8 * kThreads; // ids of a CTA per piece
 
 struct RedrawArgs {
   DevParams P;
+  int single;              // a step of more positions than clusters: every CTA draws rows of its own
   const char* cond;
   const char* uncond;
   const int32_t* pos_list;
@@ -105,8 +109,9 @@ __device__ __forceinline__ void redraw_range(int bin, uint32_t& lo, uint32_t& hi
 // NP: pieces of eight ids per thread.  A cluster of `ctas` CTAs holds ctas * NP * 4096 >= V ids; a warp's are consecutive.
 template <bool BF16, int NP>
 __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const __grid_constant__ RedrawArgs a) {
-  extern __shared__ __align__(128) unsigned char dyn[];   // [ctas][kRedrawWords]: every CTA's counts, one's own at its rank
+  extern __shared__ __align__(128) unsigned char dyn[];   // [ctas][kRedrawWords]: every CTA's counts, one's own at its rank; or a whole row
   __shared__ RedrawSmem sm;
+  __shared__ typename std::conditional<NP < 4, ResScratch, int>::type rs;   // (rows drawn by one CTA)
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t rank, ctas;
@@ -128,10 +133,19 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
 
   // what the step will find, if the list stays as it is
   uint2 found = make_uint2(0u, total);
-  if (rank == 0 && tid == 0) {
+  if (tid == 0) {
     const int beg = ld_fresh(a.offsets + a.s), end = ld_fresh(a.offsets + a.s + 1);
-    const long long at = (long long)beg + cluster;
-    if (beg >= 0 && at < end && at < (long long)total) found = make_uint2((uint32_t)beg, (uint32_t)ld_fresh(a.pos_list + at));
+    const bool many = a.single && (long long)end - beg > clusters;
+    const long long at = (long long)beg + cluster + (many ? (int)rank * clusters : 0);
+    if (beg >= 0 && at < end && at < (long long)total && (many || rank == 0)) {
+      const uint32_t row = (uint32_t)ld_fresh(a.pos_list + at);
+      if (!many) {
+        found = make_uint2((uint32_t)beg, row);
+      } else if (row < total) {   // (a hint, nothing else: no row is drawn ahead)
+        prefetch_l2(a.cond + (size_t)row * bytes, bytes);
+        if (a.uncond) prefetch_l2(a.uncond + (size_t)row * bytes, bytes);
+      }
+    }
     sm.ahead = found;
   }
   auto clear = [&]() {
@@ -185,16 +199,22 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
   uint32_t g = sm.ahead.y;
   bool waited = g >= total;
   int i = 0, end = 0;
-  if (waited) {
+  bool single = false;
+  auto look = [&]() {   // after the wait: the same in every CTA
     wait_for_previous();
-    i = ld_fresh(a.offsets + a.s) + cluster;
+    i = ld_fresh(a.offsets + a.s);
     end = ld_fresh(a.offsets + a.s + 1);
+    single = a.single && end - i > clusters;
+  };
+  if (waited) {
+    look();
+    i += cluster;
   }
   bool used = false;   // the shared memory, by a row before
 #pragma unroll 1
   for (;;) {   // (what decides here is the same in every CTA of the cluster)
     if (waited) {
-      if (i >= end) break;
+      if (single || i >= end) break;
       g = (uint32_t)ld_fresh(a.pos_list + i);
       if (g >= total) {
         i += clusters;
@@ -484,12 +504,10 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
       continue;
     }
     // ---- drawn ahead: does it hold?
-    wait_for_previous();
+    look();
     waited = true;
-    i = ld_fresh(a.offsets + a.s);
-    end = ld_fresh(a.offsets + a.s + 1);
     const int now = ld_fresh(a.pos_list + beg0 + cluster);
-    bool same = i == (int)beg0 && i + cluster < end && (uint32_t)now == g;
+    bool same = i == (int)beg0 && i + cluster < end && (uint32_t)now == g && !single;
     load(g, [&](int j, const float (&v)[8]) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) same = same && __float_as_uint(v[k]) == __float_as_uint(z[j][k]);
@@ -504,6 +522,27 @@ __global__ void __launch_bounds__(kThreads, NP == 4 ? 1 : 2) k_redraw_step(const
     if (holds) {
       if (mine) a.out_tok[g] = tok;
       i += clusters;
+    }
+  }
+  if constexpr (NP < 4) {
+    if (single) {   // (nothing is under way between the cluster's CTAs any more)
+      const ResRow row(reinterpret_cast<float*>(dyn), P.V);
+#pragma unroll 1
+      for (i += (int)rank * clusters; i < end; i += (int)gridDim.x) {   // (i: the list's start, and this cluster's number)
+        g = (uint32_t)ld_fresh(a.pos_list + i);
+        if (g >= total) continue;
+        src.cond = a.cond + (size_t)g * bytes;
+        src.uncond = a.uncond ? a.uncond + (size_t)g * bytes : nullptr;
+        src.V = P.V;
+        src.bf16 = BF16;
+        int calls = 0;
+        float unused;
+        RowStats st;
+        const ResSums sums = res_row_stats(row, src, P.top_k, rs, calls, -1, unused, st);
+        if (sums.total > 0.0) res_pick(row, sums, uniform_of(g), [&](int x) -> double { return (double)row.at(x); }, a.out_tok + g);
+        else if (tid == 0) a.out_tok[g] = -1;
+        __syncthreads();
+      }
     }
   }
 }

@@ -279,6 +279,13 @@ def test_a_row_drawn_ahead_of_its_inputs(ctx, V, what):
         assert torch.equal(out, want)
 
 
+def _shifted(pos, off):
+    """The plan with position 1 in step 1."""
+    off = off.clone()
+    off[2:4] += 1
+    return torch.cat([torch.tensor([1], dtype=torch.int32, device="cuda"), pos[:-1]]).contiguous(), off
+
+
 _LATE_LISTS = r"""
 extern "C" __global__ void late_lists(const int* new_off, int* off, int n_off, const int* new_list, int* list, int n_list, int cycles) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -291,9 +298,11 @@ extern "C" __global__ void late_lists(const int* new_off, int* off, int n_off, c
 
 
 @pytest.mark.parametrize("V", [520, 8192, 16384, 20000, 49160])   # one, two and four CTAs to a row
-def test_a_list_rewritten_while_the_step_begins(ctx, V):
+@pytest.mark.parametrize("more", [0, 90])
+def test_a_list_rewritten_while_the_step_begins(ctx, V, more):
     """The kernel before the step lets it begin and rewrites offsets and list at any moment of the step's first 10 us: the step before
-    gains a position, so both shift by one and an entry may be seen with either offset.  What counts is what stands there in the end."""
+    gains a position, so both shift by one and an entry may be seen with either offset; or the step itself gains 90, more than it has
+    clusters.  What counts is what stands there in the end."""
     B, H, W = 2, 4, 16
     cfg = synth.RoundConfig("late", B=B, H=H, W=W, V=V, r=1, dtype="bf16", top_k=V // 8, cfg_scale=0.0, seed=81)
     p = binding.params_from_config(cfg)
@@ -309,9 +318,11 @@ def test_a_list_rewritten_while_the_step_begins(ctx, V):
     steps = torch.zeros((B, H, W), dtype=torch.int32, device="cuda")
     steps.view(-1)[3:24:3] = 2
     pos0, off0 = plan(steps)
-    pos1 = torch.cat([torch.tensor([1], dtype=torch.int32, device="cuda"), pos0[:-1]]).contiguous()   # position 1 in step 1 now
-    off1 = off0.clone()
-    off1[2:4] += 1
+    if more:
+        steps.view(-1)[24:24 + more] = 2
+        pos1, off1 = plan(steps)
+    else:
+        pos1, off1 = _shifted(pos0, off0)
     want = torch.full((B, H, W), -7, dtype=torch.int32, device="cuda")
     ctx.mulo_redraw_step(p, 2, 2, pos1, off1, z, None, want)
     torch.cuda.synchronize()
@@ -359,3 +370,40 @@ def test_rows_of_all_sizes_and_shapes(ctx, case):
         want, _, edge = orc.redraw_loop(pu.orc_params(cfg, b), np.ones((H, W), np.int32), [synth.to_numpy_logits(cond[b])],
                                         None if unc is None else [synth.to_numpy_logits(unc[b])], np.zeros((H, W), np.int32), with_edge=True)
         assert not ((out[b].cpu().numpy() != want) & (edge == 0)).any()
+
+
+@pytest.mark.parametrize("case", [
+    dict(V=4096, top_k=500), dict(V=4104, top_k=500), dict(V=8192, top_k=0, dtype="f32"), dict(V=12296, top_k=1500, cfg_scale=3.0, temperature=0.9),
+    dict(V=16384, top_k=2000, cfg_scale=3.0), dict(V=16392, top_k=2000), dict(V=24576, top_k=3000, dtype="f32", cfg_scale=1.5),
+    dict(V=24584, top_k=0), dict(V=40968, top_k=5000),
+], ids=lambda c: "-".join(f"{k}{v}" for k, v in c.items()))
+def test_steps_of_more_positions_than_clusters(ctx, case):
+    """All 300 positions at once, 33 of them, and one more or less than the clusters of each size: every one is drawn, once, and right."""
+    B, H, W, V = 2, 10, 15, case["V"]
+    dtype, cfg_scale = case.get("dtype", "bf16"), case.get("cfg_scale", 0.0)
+    cfg = synth.RoundConfig("many", B=B, H=H, W=W, V=V, r=1, dtype=dtype, top_k=case["top_k"], cfg_scale=cfg_scale,
+                            temperature=case.get("temperature", 1.0), seed=82)
+    g = torch.Generator(device="cuda").manual_seed(V)
+    z = 2.0 * torch.randn((B, H, W, V), generator=g, device="cuda")
+    cond = z.to(cfg.torch_dtype).contiguous()
+    unc = (z + 0.3).to(cfg.torch_dtype).contiguous() if cfg_scale else None
+    p = binding.params_from_config(cfg)
+    n = B * H * W
+    pos, off = torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(2 * 3, dtype=torch.int32, device="cuda")
+    want = None
+    for take in (n, 32, 33, 42, 43, 64, 65, 128, 129):
+        steps = torch.zeros((B, H, W), dtype=torch.int32, device="cuda")
+        steps.view(-1)[:take] = 1
+        out = torch.full((B, H, W), -7, dtype=torch.int32, device="cuda")
+        ctx.mulo_redraw_plan(p, steps, 1, pos, off)
+        ctx.mulo_redraw_step(p, 1, 1, pos, off, cond, unc, out)
+        if want is None:
+            want = out
+            for b in range(B):
+                o, _, edge = orc.redraw_loop(pu.orc_params(cfg, b), np.ones((H, W), np.int32), [synth.to_numpy_logits(cond[b])],
+                                             None if unc is None else [synth.to_numpy_logits(unc[b])], np.zeros((H, W), np.int32),
+                                             with_edge=True)
+                assert not ((out[b].cpu().numpy() != o) & (edge == 0)).any()
+        got = out.view(-1)
+        assert int((got[:take] != want.view(-1)[:take]).sum()) <= 1   # (another order of summation: a draw in 10^4 or fewer)
+        assert bool((got[take:] == -7).all())
