@@ -52,13 +52,12 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kNearRefGap = 8.0f;      // a row whose maximum lies further from the predicted exp reference is streamed again
                                          // against its own maximum (large exponents cost relative accuracy)
 
-// What the kernel is run for: a whole round; the drafter's draws; or one stage of a round, which wants sums of a row and
-// nothing drawn: the target rows' probabilities of x~ and its acceptance, the draft rows' statistics.  A stage hands its sums
-// on to whoever calls the next one, so they are no less exact than the general routines': weights within 0.51 units in the last
-// place (sums_exp), added in double, the maximum's own in double.  (The exp reference is a whole number: subtracting it loses no
-// bits of the logits near the maximum.)
-// kRowsResample draws for the listed positions, with the draft rows' statistics given: a draft row is only streamed, its
-// entries above the given threshold are its list.
+// What the kernel is run for: a whole round; the drafter's draws; or one stage of a round.  Two stages want sums of a row and
+// nothing drawn: the target rows' probabilities of x~ and its acceptance, the draft rows' statistics.  kRowsResample draws for the
+// listed positions, with the draft rows' statistics given: a draft row is only streamed, its entries above the given threshold are
+// its list.  The stages are no less exact than the general routines whose place they take: weights by sums_exp, added in double,
+// the maximum's own in double where the sum is handed on, a draw's sums and its search in double.  (The exp reference is a whole
+// number: subtracting it loses no bits of the logits near the maximum.)
 constexpr int kRowsRound = 0, kRowsSample = 1, kRowsVerify = 2, kRowsStats = 3, kRowsResample = 4;
 // An entry of kRowsResample's list: the position in its image, whether it is drawn from the residual, whether any position of its
 // parent is (the draft row is not read otherwise).
@@ -120,7 +119,7 @@ struct RowsSmem {
   uint32_t fx[2][NW * 4];                  // ... and of the parts of the owning group
   double e_tok;
   float z_tok;
-  uint32_t rnd[2][16][3];                  // uniforms of sixteen of the parent's children, by parity of the parent
+  alignas(8) uint32_t rnd[2][16][3];       // (kRowsResample: `fx` in double) uniforms of sixteen of the parent's children, by parity of the parent
   unsigned n_sa;
   int wn[NW];
   unsigned wmax[NW];
@@ -476,7 +475,8 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   constexpr int NT = NW * 32;
   constexpr int IDS = BF16 ? 8 : 4;              // ids per lane per piece
   constexpr int kRDepth = KIND == kRowsSample || KIND == kRowsStats ? 2 : 4;   // pieces in flight per lane
-  using Sum = typename std::conditional<SUMS, double, float>::type;
+  constexpr bool EXACT = SUMS || LISTED;         // weights by sums_exp, sums in double
+  using Sum = typename std::conditional<EXACT, double, float>::type;
   extern __shared__ __align__(128) unsigned char dyn[];
   __shared__ RowsSmem<NW, POOL> sm;
   const DevParams& P = a.P;
@@ -702,7 +702,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   //      A draft row (Q) puts its logits into the draft list instead of their exps into its own.  Written with
   //      predicated PTX: left to the compiler, every entry becomes two branches.
   //      (c0: the exp reference as the weights take it, see below)
-  auto weight_of = [&](float z, float c0) -> float { return SUMS ? sums_exp(__fsub_rn(z, c0)) : ex2f(fmaf(z, kLog2e, c0)); };
+  auto weight_of = [&](float z, float c0) -> float { return EXACT ? sums_exp(__fsub_rn(z, c0)) : ex2f(fmaf(z, kLog2e, c0)); };
   auto pass_one = [&](auto q_tag, int n, float inv_w, float hoff, float c0, uint32_t& low_a, uint32_t& low_b) -> Sum {
     constexpr bool Q = decltype(q_tag)::value;
     const int n_max = __reduce_max_sync(kFull, n);
@@ -726,11 +726,25 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
       uint32_t l4 = 0;
 // (entries outside the window count in a word of their own lane: a predicated reduction becomes a branch)
 #define MULO_ENTRY(K, S)                                                                       \
-  {                                                                                            \
+  if constexpr (!(LISTED && Q)) {   /* (nothing is selected there, and the sum is given) */    \
     float e = weight_of(z[K], c0);                                                             \
     const uint32_t bin = __float_as_uint(fmaf(z[K], inv_w, hm));                               \
     const uint32_t at = hbase + (bin << 2);                                                    \
-    if constexpr (SUMS) {                                                                      \
+    if constexpr (LISTED) {                                                                    \
+      asm volatile(                                                                            \
+          "{\n\t.reg .pred p;\n\t.reg .u32 t, w;\n\t"                                            \
+          "sub.u32 t, %2, %3;\n\t"                                                             \
+          "setp.le.u32 p, t, %4;\n\t"                                                          \
+          "selp.u32 w, %5, %7, p;\n\t"                                                         \
+          "red.shared.add.u32 [w], 1;\n\t"                                                     \
+          "@p or.b32 %0, %0, %6;\n\t"                                                          \
+          "@!p st.shared.f32 [%8 + %9], %1;\n\t"                                               \
+          "@p mov.f32 %1, 0f00000000;\n\t}"                                                    \
+          : "+r"(l4), "+f"(e)                                                                  \
+          : "r"(bin), "n"(0x4B400000), "n"(kRBins), "r"(at), "n"(1 << K), "r"(spill), "r"(to), "n"(K * 128) \
+          : "memory");                                                                         \
+      S += (double)e;                                                                          \
+    } else if constexpr (SUMS) {                                                               \
       asm volatile(                                                                            \
           "{\n\t.reg .pred p;\n\t.reg .u32 t, w;\n\t"                                            \
           "sub.u32 t, %2, %3;\n\t"                                                             \
@@ -790,7 +804,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
       const uint32_t i = first + ((uint32_t)__popc(bit - 1u) ^ flip);
       const uint32_t at = tl + i * step;
       z = lds_f32(bit ? at : closer);
-      const uint32_t bin = __float_as_uint(fmaf(z, inv_w, hm));   // (-inf: as unsigned above every bin; its exp is 0)
+      const uint32_t bin = __float_as_uint(fmaf(z, inv_w, hm));   // (-inf: as unsigned above every bin; its exp is 0, e^-80 where sums_exp gives it)
       float e = weight_of(z, c0);
       e = bin > bm ? e : 0.f;
       s += (Sum)e;
@@ -864,7 +878,8 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   int tries = 0, tok = 0, child = 0;      // child: which row under the parent
   int partner_n = 0;                      // entries of the previous target row in the list this thread's list grows towards
   int partner_q = 0;                      // ... and of the draft row's list
-  float c0_q = 0.f, Zq = 1.f;             // of the parent's draft row
+  float c0_q = 0.f;                       // of the parent's draft row
+  Sum Zq = 1;
   double q_tok = 0.0;
   int tok_next = KIND == kRowsSample || LISTED ? 0 : __ldg((SUMS ? a.tok_of : a.draft_tok_lo) + parent);
   float pivot = 0.f, inv_w = 0.f, ref = 0.f, per = 0.f, lo = 0.f, hi = 0.f;   // of the row in work
@@ -955,7 +970,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
       }
     }
 
-    if constexpr (SUMS) ref = rintf(ref);
+    if (SUMS || (LISTED && !is_q)) ref = rintf(ref);
     col = (uint32_t)lane ^ (up ? 0u : rot);
     tl = my + first_row * 128u + col * 4u;
     if (is_q) dl = my + a.o_dlist + first_row * DROW + col * (DROW / 32u);
@@ -970,7 +985,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     // (a list that reached its limit was held there: its entries are incomplete; one of more than R - kRSlack
     // entries would leave its neighbour's next row no room at all)
     const bool over = (up ? end >= lim : end <= lim) || n_raw > 64 || n_raw > R - kRSlack;
-    const float c0 = SUMS ? ref : -ref * kLog2e, hoff = -pivot * inv_w;
+    const float c0 = EXACT ? ref : -ref * kLog2e, hoff = -pivot * inv_w;
     uint32_t low_a, low_b;
     Sum s_t = is_q ? pass_one(std::integral_constant<bool, !SAMPLE>{}, n, inv_w, hoff, c0, low_a, low_b)
                      : pass_one(std::false_type{}, n, inv_w, hoff, c0, low_a, low_b);
@@ -1121,7 +1136,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
           for (; low_a; low_a &= low_a - 1u) {
             const uint32_t i = (uint32_t)(__ffs(low_a) - 1) ^ flip;
             const float v = lds_f32(at + i * step);
-            const float e = v >= theta ? ex2f(fmaf(v, kLog2e, c0)) : 0.f;
+            const float e = v >= theta ? weight_of(v, c0) : 0.f;
             own += (double)e;
             if (!is_q) sts_f32(at + i * step, e);
             else if (!(v >= theta)) dlist_put<BF16>(dl + (i + 32 * h) * dstep, -INFINITY);
@@ -1227,7 +1242,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
       tries = 0;
       // ---- a draft row ends here
       c0_q = c0;
-      Zq = (float)Z;
+      Zq = (Sum)Z;
       if (!LISTED) {
         q_tok = sm.z_tok >= theta ? rows_div(sm.e_tok, Z) : 0.0;
         if (q_tok <= 0.0 && tid == 0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
@@ -1416,24 +1431,32 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
         pending = draws_for(P.resample_mode, accepted);
       }
       // weights in units of e = exp(z - ref): p -> e, q -> ratio * e_q
-      const float ratio = __fdividef((float)Z, Zq);
+      const float ratio = LISTED ? (float)(Z / (double)Zq) : __fdividef((float)Z, (float)Zq);
       auto q_weight = [&](uint32_t at) -> float {
         float zq = dlist_get<BF16>(at);
         if (BF16 && !PLAIN) zq = __fmul_rn(zq, P.invT);
-        return __fmul_rn(ex2f(fmaf(zq, kLog2e, c0_q)), ratio);
+        return __fmul_rn(weight_of(zq, c0_q), ratio);
       };
       partner_n = pair_n;   // (this row's entries may still be searched when the next row is streamed)
+      // weights of the owning group's parts: in fixed point, 2^31 = its weight, or (LISTED) as they are
+      using Fx = typename std::conditional<LISTED, double, uint32_t>::type;
+      const Fx past = LISTED ? (Fx)INFINITY : (Fx)~0u;
+      auto fx_of = [&](Sum v, float to_fx) -> Fx {
+        if constexpr (LISTED) return v;
+        else return __float2uint_rn(__fmul_rn(v, to_fx));
+      };
+      static_assert(!LISTED || sizeof sm.rnd[0] >= NW * 4 * sizeof(double), "a double per set of eight threads");
       bool no_mass = false;
       int dcall = 0;
 #pragma unroll 1
       do {
         const bool is_res = (pending & kDrawResidual) != 0;
         const bool resid = !SAMPLE && is_res && !no_mass;
-        float v_t = s_t;
+        Sum v_t = s_t;
         if (resid) {
           // sum of max(0, p - q) = p - min(p, q); min is not zero only where both rows kept the id
           uint32_t tp = tl, dp = dl;
-          float mins = 0.f;
+          Sum mins = 0;
 #pragma unroll 1
           for (int w = 0; w < n_words; ++w) {
             const uint32_t m = lds_u32(tm + (uint32_t)(w * NT) * 4u), d = lds_u32(dm + (uint32_t)(w * NT) * 4u);
@@ -1449,12 +1472,12 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
 #pragma unroll 1
             for (int i = 0; i < trips; i += 4) {   // four at a time: their chains overlap
               const float v0 = both(), v1 = both(), v2 = both(), v3 = both();
-              mins += (v0 + v1) + (v2 + v3);
+              mins += ((Sum)v0 + (Sum)v1) + ((Sum)v2 + (Sum)v3);
             }
             tp += (uint32_t)__popc(m) * step;
             dp += (uint32_t)__popc(d) * dstep;
           }
-          v_t = fmaxf(s_t - mins, 0.f);
+          v_t = s_t > mins ? s_t - mins : (Sum)0;
         }
         constexpr int NG = NW * 4;   // groups, and sets of eight threads in the search
         const double w_tok = !POOL ? 0.0 : resid ? fmax(mass - q_tok * Z, 0.0) : mass;   // x~'s weight outside the lists
@@ -1463,7 +1486,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) w_grp += __shfl_xor_sync(kFull, w_grp, o);
         double* const ws = sm.w_draw[dcall & 1];
-        uint32_t* const fxs = sm.fx[dcall & 1];
+        Fx* const fxs = LISTED ? reinterpret_cast<Fx*>(sm.rnd[dcall & 1]) : reinterpret_cast<Fx*>(sm.fx[dcall & 1]);
         ++dcall;
         if ((lane & 7) == 0) ws[tid >> 3] = w_grp;
         __syncthreads();   // ---- barrier 3
@@ -1488,9 +1511,13 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
           if ((lane & (NG - 1)) == 0) exc_d = 0.0;
           const unsigned hit_g = __ballot_sync(kFull, lane < NG && inc_d > yt), has_g = __ballot_sync(kFull, lane < NG && w_grp > 0.0);
           const int og = hit_g ? __ffs(hit_g) - 1 : 31 - __clz(has_g);
-          // sums over the group's part in fixed point: 2^31 = its weight
           const float to_fx = __fdividef(2147483648.0f, (float)__shfl_sync(kFull, w_grp, og));
-          uint32_t y = hit_g ? __double2uint_rz((yt - __shfl_sync(kFull, exc_d, og)) * (double)to_fx) : ~0u;
+          const double yg = yt - __shfl_sync(kFull, exc_d, og);
+          Fx y = past;
+          if (hit_g) {
+            if constexpr (LISTED) y = yg;
+            else y = __double2uint_rz(yg * (double)to_fx);
+          }
           const uint32_t tok_fx = POOL ? __double2uint_rn(fmin(w_tok * (double)to_fx, 4294967294.0)) : 0u;
           // the thread of the group whose entries this thread looks at, and where they are
           const int own = og * 8 + (lane & 7);
@@ -1509,8 +1536,8 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
             }
             return e;
           };
-          auto entries = [&](uint32_t mm, uint32_t at) -> uint32_t {   // fixed-point sum of the entries at the bits mm
-            float sum = 0.f;
+          auto entries = [&](uint32_t mm, uint32_t at) -> Fx {   // sum of the entries at the bits mm
+            Sum sum = 0;
 #pragma unroll 1
             while (mm) {
               const uint32_t b0 = mm & (0u - mm);
@@ -1520,10 +1547,10 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
               const uint32_t b2 = mm & (0u - mm);
               mm ^= b2;
               const float v0 = weight(b0, at), v1 = weight(b1, at + o_step), v2 = weight(b2, at + 2 * o_step);
-              sum += (v0 + v1) + v2;
+              sum += ((Sum)v0 + (Sum)v1) + (Sum)v2;
               at += 3 * o_step;
             }
-            return __float2uint_rn(__fmul_rn(sum, to_fx));
+            return fx_of(sum, to_fx);
           };
           auto go_to = [&](int w) {   // the state of word w
             ta = o_tl;
@@ -1545,7 +1572,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
           const int wps = (n_words + NG - 1) / NG;   // words per set of eight threads
           {
             const int w0 = min((tid >> 3) * wps, n_words), w1 = min(w0 + wps, n_words);
-            uint32_t v = 0;
+            Fx v = 0;
             go_to(w0);
 #pragma unroll 1
             for (int w = w0; w < w1; ++w) {
@@ -1561,15 +1588,15 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
           }
           __syncthreads();   // ---- barrier 4
           if (warp == (og >> 2)) {
-            uint32_t v = fxs[lane & (NG - 1)], inc = v;
+            Fx v = fxs[lane & (NG - 1)], inc = v;
 #pragma unroll
             for (int o = 1; o < NG; o <<= 1) {
-              const uint32_t t = __shfl_up_sync(kFull, inc, o, NG);
+              const Fx t = __shfl_up_sync(kFull, inc, o, NG);
               if ((lane & (NG - 1)) >= o) inc += t;
             }
             unsigned hit = __ballot_sync(kFull, lane < NG && v > 0 && inc > y), has = __ballot_sync(kFull, lane < NG && v > 0);
             int src = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : 0;
-            y = hit ? y - __shfl_sync(kFull, inc - v, src) : ~0u;
+            y = hit ? y - __shfl_sync(kFull, inc - v, src) : past;
             // the set's words one by one: eight lanes to a piece
             const uint32_t piece_bits = ((1u << IDS) - 1u) << ((lane >> 3) * IDS), under = (1u << ((lane >> 3) * IDS)) - 1u;
             const int w0 = src * wps, w1 = min(w0 + wps, n_words);
@@ -1582,14 +1609,16 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
               v = entries(m & piece_bits, ta + (uint32_t)__popc(m & under) * o_step);
               if (POOL && own == tok_spot.thread && w == tok_spot.word && (tok_spot.bit & piece_bits)) v += tok_fx;
               __syncwarp();
-              const uint32_t t = __reduce_add_sync(kFull, v);
+              Fx t;
+              if constexpr (LISTED) t = warp_sum(v);
+              else t = __reduce_add_sync(kFull, v);
               if (t > 0) last_w = w;
-              if (seek ? w == last_w : y < t) break;
-              if (y != ~0u) y -= t;
+              if (seek ? w == last_w : t > 0 && y < t) break;
+              if (y != past) y -= t;
               next_word();
               if (++w == w1) {
                 seek = true;
-                y = ~0u;
+                y = past;
                 w = last_w;
                 go_to(w);
               }
@@ -1597,13 +1626,13 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
             inc = v;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-              const uint32_t t = __shfl_up_sync(kFull, inc, o);
+              const Fx t = __shfl_up_sync(kFull, inc, o);
               if (lane >= o) inc += t;
             }
             hit = __ballot_sync(kFull, v > 0 && inc > y);
             has = __ballot_sync(kFull, v > 0);
             src = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : 0;
-            y = hit ? y - __shfl_sync(kFull, inc - v, src) : ~0u;
+            y = hit ? y - __shfl_sync(kFull, inc - v, src) : past;
             // ... and the ids of the lane found: lane i takes id i
             m = __shfl_sync(kFull, m, src);
             d = __shfl_sync(kFull, d, src);
@@ -1614,10 +1643,10 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
             if (POOL && og * 8 + (src & 7) == tok_spot.thread && w == tok_spot.word && lane < IDS &&
                 tok_spot.bit == 1u << ((src >> 3) * IDS + lane))
               wt += (float)w_tok;
-            inc = __float2uint_rn(__fmul_rn(wt, to_fx));
+            inc = fx_of((Sum)wt, to_fx);
 #pragma unroll
             for (int o = 1; o < IDS; o <<= 1) {
-              const uint32_t t = __shfl_up_sync(kFull, inc, o);
+              const Fx t = __shfl_up_sync(kFull, inc, o);
               if (lane >= o) inc += t;
             }
             hit = __ballot_sync(kFull, wt > 0.f && inc > y);
