@@ -20,7 +20,8 @@
  *     library never allocates or frees device memory; scratch space is the
  *     workspace the caller hands to mulo_set_workspace.  A context's calls share it, so
  *     those that read logits must not overlap on the device (one context per stream does it),
- *     but for mulo_upsample_pool and mulo_redraw_step, which write nothing there but status bits.
+ *     but for mulo_upsample_pool, mulo_resample and mulo_redraw_step, which write nothing there
+ *     but status bits.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the default stream).
  *     Calls validate their arguments on the host, enqueue kernels on the stream
  *     and return; outputs are defined once the stream has been synchronised.  Nothing a

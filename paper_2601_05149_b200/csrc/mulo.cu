@@ -486,71 +486,28 @@ __global__ void __launch_bounds__(kThreads, 2) k_resample_rows(RowKernelArgs a) 
   __shared__ GeneralScratch<RES> sc;
   resample_position<RES>(a, blockIdx.x, sc, dyn);
 }
-// Third launch of its fast path: the positions the fast kernel put on its list.
+// Second launch of its fast path: the positions the fast kernel marked.
 template <bool RES>
-__global__ void __launch_bounds__(kThreads, 2) k_resample_left(RowKernelArgs a, const int32_t* fail_list, const uint32_t* fail_count) {
+__global__ void __launch_bounds__(kThreads, 2) k_resample_left(RowKernelArgs a) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GeneralScratch<RES> sc;
+  __shared__ unsigned found[kWarps];
   let_next_begin();
   wait_for_previous();
-  const size_t total = (size_t)a.P.B * a.P.H * a.P.W, n = min((size_t)*fail_count, total);
-  for (size_t idx = blockIdx.x; idx < n; idx += gridDim.x) {
-    const size_t g = (size_t)fail_list[idx];
-    if (g < total) resample_position<RES>(a, g, sc, dyn);
+  const size_t total = (size_t)a.P.B * a.P.H * a.P.W;
+  for (size_t g0 = (size_t)blockIdx.x * kThreads; g0 < total; g0 += (size_t)gridDim.x * kThreads) {
+    const size_t g = g0 + threadIdx.x;
+    const bool mine = g < total && a.out_tok[g] == kPickLeft;   // (x~ of such a value: it is copied once more)
+    const unsigned word = __ballot_sync(kFull, mine);
+    if ((threadIdx.x & 31) == 0) found[threadIdx.x >> 5] = word;
+    if (!__syncthreads_or(mine)) continue;
+    for (int w = 0; w < kWarps; ++w)
+      for (unsigned left = found[w]; left; left &= left - 1u) {   // (block-uniform)
+        resample_position<RES>(a, g0 + w * 32 + __ffs(left) - 1, sc, dyn);
+        __syncthreads();
+      }
     __syncthreads();
   }
-}
-
-// First launch of its fast path, one CTA per image: x~ where nothing is drawn, and the list of what is, parent by parent.
-constexpr int kPickThreads = 1024;
-__global__ void __launch_bounds__(kPickThreads) k_resample_list(RowKernelArgs a, uint32_t* list, int32_t* counts, uint32_t* fail_count) {
-  __shared__ int warp_tot[kPickThreads / 32];
-  const DevParams& P = a.P;
-  const int N = P.H * P.W, Ww = (P.W + 31) / 32, cells = P.h * P.w, b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const size_t n0 = (size_t)b * N;
-  if (b == 0 && tid == 0) *fail_count = 0u;
-  int base = 0;
-  for (int c0 = 0; c0 < cells; c0 += kPickThreads) {
-    const int cell = c0 + tid, ca = cell / P.w, cc = cell - ca * P.w;
-    int n = 0, n_res = 0;
-    auto children = [&](auto take) {
-      if (cell < cells)
-        for (int di = 0; di < P.r; ++di)
-          for (int dj = 0; dj < P.r; ++dj) {
-            const int i = ca * P.r + di, j = cc * P.r + dj;
-            take(i * P.W + j, get_bit(a.expand_bits, Ww, P.H, b, i, j), get_bit(a.reject_bits, Ww, P.H, b, i, j));
-          }
-    };
-    auto residual = [&](int rejected) {
-      return P.resample_mode == MULO_RESAMPLE_RESIDUAL_ALL || (P.resample_mode == MULO_RESAMPLE_MIXED && rejected);
-    };
-    children([&](int t, int in, int rejected) {
-      if (!in) a.out_tok[n0 + t] = a.draft_tok_hi[n0 + t];
-      n += in;
-      n_res += in && residual(rejected);
-    });
-    int inc = n;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, inc, o);
-      if (lane >= o) inc += v;
-    }
-    __syncthreads();
-    if (lane == 31) warp_tot[warp] = inc;
-    __syncthreads();
-    const int mine = warp_tot[lane];
-    int at = base + inc - n + __reduce_add_sync(kFull, lane < warp ? mine : 0);
-    base += __reduce_add_sync(kFull, mine);
-    children([&](int t, int in, int rejected) {
-      if (!in) return;
-      list[n0 + at++] = (uint32_t)t | (residual(rejected) ? kPickResidual : 0u) | (n_res > 0 ? kPickDraft : 0u);
-      // what the general routines report of a position
-      const RowStats sq = given_stats(a, (size_t)b * cells + cell);
-      const float zq = load1(draft_row(a, (size_t)b * cells + cell), checked_token(a.draft_tok_hi[n0 + t], P.V, a.dev_status));
-      if (!(zq >= sq.theta) || exp((double)zq - (double)sq.m) / sq.Z <= 0.0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
-    });
-  }
-  if (tid == 0) counts[b] = base;
 }
 
 // ============================================================= mask kernel
@@ -1677,28 +1634,26 @@ mulo_status mulo_resample(mulo_ctx* ctx, const mulo_params* p, const void* tgt_c
   const cudaStream_t st = (cudaStream_t)stream;
   const size_t dyn = general_smem(a.P, true);
   const long long rows = (long long)p->B * p->H * p->W;
-  // Many rows with a cut and without pooling are streamed, if there is room for the lists.  (Whether a rejection is isolated
-  // depends on its neighbours, which the general kernel looks up.)
-  Workspace w;
+  // Many rows with a cut and without pooling are streamed.  (Whether a rejection is isolated depends on its neighbours, which the
+  // general kernel looks up.)
   RowsArgs ra;
   memset(&ra, 0, sizeof ra);
   int rnw = 0;
-  const bool many = a.P.pool_k <= 1 && many_rows(ctx, kRowsResample, a.P.V, rows) &&
-                    (size_t)p->H * p->W <= (size_t)kPickIndex && p->resample_mode != MULO_RESAMPLE_ISOLATED_RESIDUAL && check_ws(ctx, p, &w) == MULO_OK;
+  const bool many = a.P.pool_k <= 1 && many_rows(ctx, kRowsResample, a.P.V, rows) && (size_t)p->H * p->W <= (size_t)kPickIndex &&
+                    p->resample_mode != MULO_RESAMPLE_ISOLATED_RESIDUAL;
   if (const size_t rdyn = many ? plan_rows(ctx, a.P, kRowsResample, &ra, &rnw) : 0) {
     ra.P = a.P;
     ra.cond = a.cond; ra.uncond = a.uncond; ra.draft = a.draft;
+    ra.tok_of = draft_tok_hi;
     ra.stats_in = draft_stats_lo;
+    ra.reject_bits = reject_bits;
+    ra.expand_bits = expand_bits;
     ra.sample_out = out_tok;
-    ra.list = (const uint32_t*)w.cand_tgt;
-    ra.counts = w.cand_res;
-    ra.dev_status = w.status;
-    ra.fail_list = w.fail_list;
+    ra.dev_status = a.dev_status;
     ra.n_units = (int)rows;   // (at most)
-    k_resample_list<<<p->B, kPickThreads, 0, st>>>(a, (uint32_t*)w.cand_tgt, w.cand_res, w.status + kFailCount);
     if (launch_rows<kRowsResample>(ctx, ra, rnw, rdyn, st)) {
-      if (!MULO_LAUNCH_LEFT(K_RESAMPLE_LEFT, dyn, st, a, w.fail_list, w.status + kFailCount)) return MULO_ERR_CUDA;
-      return launched(ctx, 3);
+      if (!MULO_LAUNCH_LEFT(K_RESAMPLE_LEFT, dyn, st, a)) return MULO_ERR_CUDA;
+      return launched(ctx, 2);
     }
   }
   if (!MULO_LAUNCH_GENERAL(K_RESAMPLE, rows, dyn, st, a)) return MULO_ERR_UNSUPPORTED;

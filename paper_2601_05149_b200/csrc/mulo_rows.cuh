@@ -54,14 +54,17 @@ constexpr float kNearRefGap = 8.0f;      // a row whose maximum lies further fro
 
 // What the kernel is run for: a whole round; the drafter's draws; or one stage of a round.  Two stages want sums of a row and
 // nothing drawn: the target rows' probabilities of x~ and its acceptance, the draft rows' statistics.  kRowsResample draws for the
-// listed positions, with the draft rows' statistics given: a draft row is only streamed, its entries above the given threshold are
+// positions of R_X, with the draft rows' statistics given: a draft row is only streamed, its entries above the given threshold are
 // its list.  The stages are no less exact than the general routines whose place they take: weights by sums_exp, added in double,
 // the maximum's own in double where the sum is handed on, a draw's sums and its search in double.  (The exp reference is a whole
 // number: subtracting it loses no bits of the logits near the maximum.)
 constexpr int kRowsRound = 0, kRowsSample = 1, kRowsVerify = 2, kRowsStats = 3, kRowsResample = 4;
-// An entry of kRowsResample's list: the position in its image, whether it is drawn from the residual, whether any position of its
-// parent is (the draft row is not read otherwise).
-constexpr uint32_t kStatsLeft = 0xffa5c3e1u;   // in the place of a threshold: a NaN that no logit gives
+// What is left to the general routines is marked in the stage's own output, so that calls on other streams share nothing but
+// status bits: in the place of a threshold a NaN that no logit gives, in the place of a token what no draw gives.
+constexpr uint32_t kStatsLeft = 0xffa5c3e1u;
+constexpr int32_t kPickLeft = INT32_MIN;
+// A position of R_X: its index in its image, whether it is drawn from the residual, whether any position of its parent is (the
+// draft row is not read otherwise).
 constexpr uint32_t kPickIndex = (1u << 30) - 1u, kPickResidual = 1u << 31, kPickDraft = 1u << 30;
 
 // running prediction for one kind of row (draft / target), per CTA
@@ -88,10 +91,10 @@ struct RowsArgs {
   int32_t* cand_res;
   int32_t* cand_tgt;
   int32_t* sample_out;      // kRowsSample: the drafter's token per cell
-  const int32_t* tok_of;    // kRowsVerify, kRowsStats: x~ of each row
+  const int32_t* tok_of;    // kRowsVerify, kRowsStats, kRowsResample: x~ of each row
   const float* stats_in;    // kRowsVerify, kRowsResample: the draft rows' statistics
-  const uint32_t* list;     // kRowsResample: [B][H * W], an image's positions of R_X (see kPickIndex), parent by parent
-  const int32_t* counts;    // ... and how many they are
+  const uint32_t* reject_bits;   // kRowsResample
+  const uint32_t* expand_bits;
   float* stats_out;         // kRowsStats
   int32_t* tok_hi_out;
   float* q_hi_out;
@@ -482,16 +485,102 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   let_next_begin();
+  const int rr = SAMPLE ? 1 : P.r * P.r;
   int n_units = a.n_units;
+  // LISTED: the unit in work and the one after it are found by going down the positions parent by parent (`found`: how far), 32 at a time.
+  uint32_t found = 0;
+  int left = 0;
+  const uint32_t N = (uint32_t)P.H * (uint32_t)P.W, n_at = (uint32_t)P.B * N;
+  const int Ww = (P.W + 31) >> 5;
+  struct Place {
+    int b, i, j, parent;
+  };
+  auto place_of = [&](uint32_t x) -> Place {
+    Place p;
+    p.parent = (int)(x / (uint32_t)rr);
+    const int c = (int)(x - (uint32_t)p.parent * (uint32_t)rr), hw = P.h * P.w;
+    p.b = p.parent / hw;
+    const int rem = p.parent - p.b * hw, ca = rem / P.w, di = c / P.r;
+    p.i = ca * P.r + di;
+    p.j = (rem - ca * P.w) * P.r + c - di * P.r;
+    return p;
+  };
+  auto bit_of = [&](const uint32_t* bits, const Place& p) -> bool {
+    return bits[((size_t)p.b * P.H + p.i) * Ww + (p.j >> 5)] >> (p.j & 31) & 1u;
+  };
+  // the first position of R_X from x on that has `skip` others before it (every warp for itself; there is one)
+  auto find_pick = [&](uint32_t x, int skip) -> uint32_t {
+#pragma unroll 1
+    for (; x < n_at; x += 32) {
+      const uint32_t mine = x + (uint32_t)lane;
+      uint32_t hit = __ballot_sync(kFull, mine < n_at && bit_of(a.expand_bits, place_of(min(mine, n_at - 1u))));
+      const int n = __popc(hit);
+      if (skip < n) {
+        for (; skip > 0; --skip) hit &= hit - 1u;
+        return x + (uint32_t)__ffs(hit) - 1u;
+      }
+      skip -= n;
+    }
+    return n_at - 1u;
+  };
   if constexpr (LISTED) {
+    // x~ where nothing is drawn; of what is drawn, what the general routines report of a position
+    for (uint32_t x = blockIdx.x * NT + tid; x < n_at; x += gridDim.x * NT) {
+      const int raw = a.tok_of[x], b = (int)(x / N), t = (int)(x - (uint32_t)b * N), i = t / P.W, j = t - i * P.W;
+      if (!bit_of(a.expand_bits, Place{b, i, j, 0})) {
+        a.sample_out[x] = raw;
+      } else {
+        const int tok = min(max(raw, 0), P.V - 1);
+        if (tok != raw) atomicOr(a.dev_status, MULO_DEV_BAD_TOKEN);
+        const size_t cell = ((size_t)b * P.h + i / P.r) * P.w + j / P.r;
+        const float zq = mix_logit(wide_logit<BF16>(raw_logit<BF16>(a.draft + cell * a.row_bytes, tok)), 0.f, false, 0.f, P.invT);
+        const float* const st = a.stats_in + cell * 4;
+        if (!(zq >= st[0]) || row_exp((double)zq - (double)st[1]) / ((double)st[2] + (double)st[3]) <= 0.0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
+      }
+    }
+    // how many positions R_X has, and which is this CTA's first: rows of parents, a run of them per thread
+    const int n_rows = P.B * P.h, per = (n_rows + NT - 1) / NT, r0 = min(n_rows, tid * per), r1 = min(n_rows, r0 + per), words = P.r * Ww;
+    auto count_row = [&](int row) -> int {
+      int n = 0;
+      for (int w = 0; w < words; ++w) {
+        uint32_t v = a.expand_bits[(size_t)row * words + w];
+        if (w % Ww == Ww - 1 && (P.W & 31)) v &= (1u << (P.W & 31)) - 1u;   // (bits past the row's end do not count)
+        n += __popc(v);
+      }
+      return n;
+    };
+    int mine = 0;
+    for (int row = r0; row < r1; ++row) mine += count_row(row);
+    int inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) sm.wn[warp] = inc;
+    __syncthreads();
     n_units = 0;
-    for (int i = lane; i < P.B; i += 32) n_units += a.counts[i];
-    n_units = __reduce_add_sync(kFull, n_units);
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      if (w < warp) inc += sm.wn[w];
+      n_units += sm.wn[w];
+    }
+    const int first = (int)(((long long)n_units * blockIdx.x) / gridDim.x);
+    if (first >= inc - mine && first < inc) {   // (one thread, unless there is nothing to do)
+      int row = r0, skip = first - (inc - mine);
+      for (int n = count_row(row); skip >= n; n = count_row(++row)) skip -= n;
+      sm.n_sa = (unsigned)row;
+      sm.wmax[0] = (unsigned)skip;
+    }
+    __syncthreads();
   }
   int unit = (int)(((long long)n_units * blockIdx.x) / gridDim.x);
   const int u_end = (int)(((long long)n_units * (blockIdx.x + 1)) / gridDim.x);
   if (unit >= u_end) return;
-  const int rr = SAMPLE ? 1 : P.r * P.r;
+  if constexpr (LISTED) {
+    found = find_pick(sm.n_sa * (uint32_t)(P.w * rr), (int)sm.wmax[0]);
+    __syncthreads();
+  }
   const uint32_t row_bytes = a.row_bytes;
   const int n_words = a.n_words, R = a.R;
   const float inv_ppg = 1.0f / (float)a.ppg;
@@ -542,30 +631,31 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
       dj = child - di * P.r;
     }
   }
-  // LISTED: the entry in work, the one after it, and where that is
+  // LISTED: the position in work (b: its image) and the one after it
   uint32_t pick = 0, pick_next = 0;
-  int img_at = 0, left = 0;
-  uint32_t N = 0;
-  auto pick_parent = [&](uint32_t p, int image) -> int {
-    const int t = (int)(p & kPickIndex), i = t / P.W, j = t - i * P.W;
-    return (image * P.h + i / P.r) * P.w + j / P.r;
-  };
-  int b_next = 0;      // the image of the entry after this one (b: of that in work)
-  auto next_pick = [&]() {   // (there is one)
-    while (img_at >= a.counts[b_next]) {
-      ++b_next;
-      img_at = 0;
+  int b_next = 0, parent_next = 0;
+  auto look_at = [&](uint32_t x, uint32_t& p, int& image, int& par) {
+    const Place pl = place_of(x);
+    const int mode = P.resample_mode;
+    bool some = mode == MULO_RESAMPLE_RESIDUAL_ALL;
+    if (mode == MULO_RESAMPLE_MIXED) {
+#pragma unroll 1
+      for (int c0 = 0; c0 < rr; c0 += 32) {
+        const Place c = place_of((uint32_t)pl.parent * (uint32_t)rr + (uint32_t)min(c0 + lane, rr - 1));
+        some = some || __any_sync(kFull, bit_of(a.expand_bits, c) && bit_of(a.reject_bits, c));
+      }
     }
-    pick_next = a.list[(size_t)b_next * N + (uint32_t)img_at++];
+    const bool resid = mode == MULO_RESAMPLE_RESIDUAL_ALL || (mode == MULO_RESAMPLE_MIXED && bit_of(a.reject_bits, pl));
+    p = (uint32_t)(pl.i * P.W + pl.j) | (resid ? kPickResidual : 0u) | (some ? kPickDraft : 0u);
+    image = pl.b;
+    par = pl.parent;
+  };
+  auto next_pick = [&]() {   // (there is one)
+    found = find_pick(found + 1u, 0);
+    look_at(found, pick_next, b_next, parent_next);
   };
   if constexpr (LISTED) {
-    N = (uint32_t)P.H * (uint32_t)P.W;
-    b = 0;
-    img_at = unit;
-    while (img_at >= a.counts[b]) img_at -= a.counts[b++];
-    pick = a.list[(size_t)b * N + (uint32_t)img_at++];
-    parent = pick_parent(pick, b);
-    b_next = b;
+    look_at(found, pick, b, parent);
     left = u_end - unit - 1;
   }
   auto target_index = [&]() -> uint32_t {
@@ -696,7 +786,6 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   bool is_q = LISTED ? (pick & kPickDraft) != 0u : !SAMPLE;   // the row in work is a draft row
   uint32_t g = !LISTED || is_q ? (uint32_t)parent : target_index();   // ... and its index in its tensor
   if (LISTED && left > 0) next_pick();
-  int parent_next = 0;
 
   // ---- first pass over the list (see the top of the file); returns the exp sum of the entries above the window.
   //      A draft row (Q) puts its logits into the draft list instead of their exps into its own.  Written with
@@ -852,8 +941,9 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     atomicAdd(a.dev_status + slot, 1u);
   };
   auto defer = [&](uint32_t g) {           // one thread: position (cell) g goes to the general routines
-    if constexpr (KIND == kRowsStats) {    // (marked in its own output: no list, and nothing shared with calls on other streams)
-      reinterpret_cast<uint32_t*>(a.stats_out)[(size_t)g * 4] = kStatsLeft;
+    if constexpr (KIND == kRowsStats || LISTED) {
+      if (LISTED) a.sample_out[g] = kPickLeft;
+      else reinterpret_cast<uint32_t*>(a.stats_out)[(size_t)g * 4] = kStatsLeft;
       atomicAdd(a.dev_status + kCntRows, 1u);
       atomicOr(a.dev_status, MULO_DEV_DENSE_FALLBACK);
       return;
@@ -902,7 +992,6 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
       more = false;
       ng = g;
     } else if (LISTED) {
-      parent_next = pick_parent(pick_next, b_next);
       nq = parent_next != parent && (pick_next & kPickDraft) != 0u;
       ng = nq ? (uint32_t)parent_next : (uint32_t)b_next * N + (pick_next & kPickIndex);
     } else {
@@ -1206,7 +1295,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
             const int before = parent;
             b = b_next;
             pick = pick_next;
-            parent = pick_parent(pick, b);
+            parent = parent_next;
             if (--left > 0) next_pick();
             if (parent != before) break;
           }

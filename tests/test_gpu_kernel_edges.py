@@ -162,15 +162,15 @@ def test_redraw_around_shared_memory(ctx, V):
                                                       temperature=0.9, window=4, density=0.5))
 
 
-STAGES = synth.RoundConfig("stages", B=2, H=24, W=26, V=4096, dtype="bf16", sigma=1.0, cfg_scale=3.0, top_k=500, radius=1, seed=1201)
+STAGES = synth.RoundConfig("stages", B=4, H=24, W=26, V=4096, dtype="bf16", sigma=1.0, cfg_scale=3.0, top_k=500, radius=1, seed=1201)
 
 
 @pytest.mark.parametrize("over", [
     dict(), dict(V=1024, top_k=100, dtype="f32"), dict(V=4104, top_k=600, cfg_scale=0.0, temperature=0.8), dict(V=16384, top_k=2000),
-    dict(V=8192, top_k=2600), dict(r=1, H=20, W=31, V=8192, sigma=0.1, cfg_scale=0.0, radius=0), dict(r=3, H=24, W=27, radius=2, sigma=0.3), dict(B=1, H=36, W=36, resample_mode=binding.RESAMPLE_RESIDUAL_ALL),
+    dict(V=8192, top_k=2600), dict(r=1, H=20, W=31, V=8192, sigma=0.1, cfg_scale=0.0, radius=0), dict(r=3, H=24, W=27, radius=2, sigma=0.3), dict(B=2, H=36, W=36, resample_mode=binding.RESAMPLE_RESIDUAL_ALL),
     dict(resample_mode=binding.RESAMPLE_TARGET_ALL), dict(accept_mode=binding.ACCEPT_THRESHOLD, tau=1e-3),
     dict(resample_mode=binding.RESAMPLE_ISOLATED_RESIDUAL, radius=3), dict(cubed=True), dict(quantum=0.5, cfg_scale=0.0),
-    dict(r=1, H=20, W=31, V=8192, top_k=1000, quantum=0.5), dict(B=2, shift=True),
+    dict(r=1, H=20, W=31, V=8192, top_k=1000, quantum=0.5), dict(shift=True),
 ], ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain")
 def test_stages_of_many_rows(ctx, over):
     """More rows than the stages keep in shared memory: the streaming kernels, rows that mislead their predictions included."""
@@ -191,7 +191,8 @@ def test_stages_of_many_rows(ctx, over):
     n0 = ctx.kernel_launches()
     g = pu.gpu_stages(ctx, cfg, batch)
     isolated = cfg.resample_mode == binding.RESAMPLE_ISOLATED_RESIDUAL
-    assert ctx.kernel_launches() - n0 == (2 if cfg.r == 1 else 1) + 3 + 1 + (1 if isolated else 3)   # the fast paths, but for few draft rows
+    few = cfg.B * cfg.h * cfg.w <= (4 if cfg.V > 4096 else 16) * torch.cuda.get_device_properties(0).multi_processor_count
+    assert ctx.kernel_launches() - n0 == (1 if few else 2) + 3 + 1 + (1 if isolated else 2)   # the fast paths, but for few draft rows
     o = pu.oracle_images(cfg, batch, list(range(cfg.B)))
     pu.check_round(cfg, g, o)
     for b in range(cfg.B):
@@ -200,3 +201,106 @@ def test_stages_of_many_rows(ctx, over):
         np.testing.assert_allclose(g["stats"][b].astype(np.float64)[..., 0:2], want["stats"][..., 0:2], rtol=0, atol=0)
         np.testing.assert_allclose(g["stats"][b][..., 2].astype(np.float64) + g["stats"][b][..., 3], want["stats"][..., 2], rtol=1e-6)
     assert ctx.poll_device_status() & ~(binding.DEV_DENSE_FALLBACK | binding.DEV_ZERO_DRAFT_PROB) == 0
+
+
+@pytest.mark.parametrize("over", [dict(), dict(r=3, H=24, W=27), dict(V=8192, top_k=1000, dtype="f32", cfg_scale=0.0), dict(V=8192, top_k=900)],
+                         ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain")
+@pytest.mark.parametrize("tied", ["target", "draft"])
+def test_rows_that_the_stages_leave(ctx, tied, over):
+    """Rows with hundreds of equal logits at the threshold crowd a bin (target rows, the draft rows' statistics) or overflow the list
+    of what lies above a given threshold (draft rows of the redraw, with all rows under them): each stage has to leave some to
+    the general routines, and says so."""
+    cfg = dataclasses.replace(STAGES, resample_mode=binding.RESAMPLE_RESIDUAL_ALL, **over)
+    batch = pu.build_batch(cfg)
+    for k in ("cond", "uncond") if tied == "target" else ("draft_lo",):
+        if batch[k] is not None:
+            batch[k] = ((batch[k].float() / 2.0).round() * 2.0).to(batch[k].dtype)
+    pu.redraw_tokens(cfg, batch)
+    p = binding.params_from_config(cfg)
+    ctx.ensure_workspace(p)
+    B, H, W = cfg.B, cfg.H, cfg.W
+    o = binding.alloc_round_outputs(p, "cuda")
+    tok_hi = torch.empty((B, H, W), dtype=torch.int32, device="cuda")
+    stats, q_hi = torch.empty((B, cfg.h, cfg.w, 4), device="cuda"), torch.empty((B, H, W), device="cuda")
+
+    def left():
+        torch.cuda.synchronize()
+        assert ctx.poll_device_status() & ~(binding.DEV_DENSE_FALLBACK | binding.DEV_ZERO_DRAFT_PROB) == 0
+        return ctx.poll_fallback_counts()[0]
+
+    left()
+    n0 = ctx.kernel_launches()
+    ctx.mulo_upsample_pool(p, batch["draft_lo"], batch["tok_lo"], None, tok_hi, stats, q_hi)
+    assert (left() > 0) == (tied == "draft" and ctx.kernel_launches() - n0 == 2)   # (few draft rows are not streamed)
+    ctx.mulo_verify(p, batch["cond"], batch["uncond"], batch["draft_lo"], stats, tok_hi, None, o["p_tok"], o["q_tok"], o["accept_prob"],
+                    o["reject_bits"], o["n_reject"], o["first_reject"])
+    assert (left() > 0) == (tied == "target")
+    ctx.mulo_local_reject_expand(p, o["reject_bits"], o["first_reject"], o["expand_bits"], o["n_expand"])
+    ctx.mulo_resample(p, batch["cond"], batch["uncond"], batch["draft_lo"], stats, tok_hi, None, o["reject_bits"], o["expand_bits"],
+                      o["out_tok"])
+    assert left() > 0
+    pu.check_round(cfg, pu.finish_outputs(o, W), pu.oracle_images(cfg, batch, list(range(B))))
+
+
+@pytest.mark.parametrize("over", [dict(), dict(B=3, H=30, W=37, r=1, V=1024, top_k=100), dict(B=5, H=48, W=45, r=3, radius=2)],
+                         ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain")
+@pytest.mark.parametrize("density", [0.0, 0.0005, 0.02, 0.5, 1.0])
+def test_redraw_of_any_share_of_the_grid(ctx, over, density):
+    """The streamed redraw finds the positions of R_X by itself: none, one or two, some, all; bits past a row's end count as nothing."""
+    cfg = dataclasses.replace(STAGES, resample_mode=binding.RESAMPLE_MIXED, **over)
+    batch = pu.build_batch(cfg)
+    pu.redraw_tokens(cfg, batch)
+    p = binding.params_from_config(cfg)
+    ctx.ensure_workspace(p)
+    B, H, W = cfg.B, cfg.H, cfg.W
+    g = torch.Generator(device="cuda").manual_seed(77)
+    hits = torch.rand((B, H, (W + 31) // 32, 32), generator=g, device="cuda") < density
+    if density == 0.0005:
+        hits.view(-1)[:] = False
+        hits[B - 1, H - 1, (W - 1) // 32, (W - 1) % 32] = True
+        hits[0, 1, 0, 2] = True
+    also = torch.rand(hits.shape, generator=g, device="cuda") < 0.5
+    past = torch.arange(hits.shape[2] * 32, device="cuda").view(1, 1, -1, 32) >= W
+
+    def words(bits):
+        w = (bits.to(torch.int64) << torch.arange(32, device="cuda")).sum(-1)
+        return torch.where(w >= 2 ** 31, w - 2 ** 32, w).to(torch.int32).contiguous()
+
+    expand, reject = words(hits | past), words(hits & also)
+    tok_hi = torch.empty((B, H, W), dtype=torch.int32, device="cuda")
+    stats, q_hi = torch.empty((B, cfg.h, cfg.w, 4), device="cuda"), torch.empty((B, H, W), device="cuda")
+    ctx.mulo_upsample_pool(p, batch["draft_lo"], batch["tok_lo"], None, tok_hi, stats, q_hi)
+    out = {}
+    for how in (False, True):
+        out[how] = torch.full((B, H, W), -9, dtype=torch.int32, device="cuda")
+        ctx.set_general_path_only(how)
+        n0 = ctx.kernel_launches()
+        ctx.mulo_resample(p, batch["cond"], batch["uncond"], batch["draft_lo"], stats, tok_hi, None, reject, expand, out[how])
+        ctx.set_general_path_only(False)
+        assert ctx.kernel_launches() - n0 == (1 if how else 2)
+    inside = (hits & ~past).flatten(2)[..., :W]
+    assert torch.equal(out[False][~inside], tok_hi[~inside])
+    assert int((out[False] != out[True]).sum()) <= 1   # (another order of summation: a draw in 10^4 or fewer)
+
+
+def test_redraws_on_two_streams_of_one_context(ctx):
+    """mulo_resample keeps nothing in the workspace but status bits: two of them at a time on one context."""
+    cfgs = [dataclasses.replace(STAGES, seed=s, resample_mode=m) for s, m in ((1301, binding.RESAMPLE_RESIDUAL_ALL), (1302, binding.RESAMPLE_MIXED))]
+    jobs = []
+    for cfg in cfgs:
+        batch = pu.build_batch(cfg)
+        pu.redraw_tokens(cfg, batch)
+        g = pu.gpu_stages(ctx, cfg, batch)
+        jobs.append((cfg, binding.params_from_config(cfg), batch, {k: torch.from_numpy(g[k]).cuda() for k in ("tok_hi", "stats", "reject_bits", "expand_bits")},
+                     torch.from_numpy(g["out_tok"]).cuda()))
+    streams = [torch.cuda.Stream() for _ in jobs]
+    torch.cuda.synchronize()
+    for _ in range(20):
+        outs = [torch.full_like(j[4], -9) for j in jobs]
+        torch.cuda.synchronize()
+        for (cfg, p, batch, s, _), out, st in zip(jobs, outs, streams):
+            ctx.mulo_resample(p, batch["cond"], batch["uncond"], batch["draft_lo"], s["stats"], s["tok_hi"], None, s["reject_bits"],
+                              s["expand_bits"], out, stream=st)
+        torch.cuda.synchronize()
+        for j, out in zip(jobs, outs):
+            assert torch.equal(out, j[4])
