@@ -236,7 +236,7 @@ constexpr int kIslandTerm = 1 << 15;   // more than two steps, or columns, of on
 
 __host__ inline size_t schedule_smem(int H, int W) {
   const size_t N = (size_t)H * W, nw = (size_t)H * ((W + 31) / 32);
-  return (N + kScheduleSlack) * 12 + 2 * nw * 4;   // (at most 230,144 bytes: 4000 x 4)
+  return (N + kScheduleSlack) * 12 + 2 * nw * 4;   // (at most 225,536 bytes: 4000 x 4)
 }
 
 // M: slots per lane in the chain of rows; rows of more than 32 M columns take several turns.

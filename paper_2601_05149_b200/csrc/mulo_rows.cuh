@@ -277,9 +277,9 @@ __device__ __noinline__ double row_exp2(double x) { return exp2(x); }
 
 __device__ __noinline__ double row_exp(double x) { return exp(x); }
 
-// e^d for d from -80 (below: that of -80) to 80, within 6.0e-8, 2.6e-8 rms: d = n ln 2 + f, and on |f| <= ln 2 / 2 a polynomial
-// 1 + f + f^2 q(f), q of degree four fitted to (e^f - 1 - f) / f^2 (largest error in e^f 3.1e-9).  expf leaves twice the error
-// in a row's sum.
+// e^d for d from -80 (below: that of -80) to 80, within 7.5e-8 (0.91 units in the last place), 2.65e-8 rms, by 4 M values per range:
+// d = n ln 2 + f with ln 2 in two parts (Cody and Waite), and on |f| <= ln 2 / 2 a polynomial 1 + f + f^2 q(f), q of degree four
+// fitted to (e^f - 1 - f) / f^2 (largest error in e^f 5.2e-9; the rest are the roundings of f and of the last two steps).
 __device__ __forceinline__ float sums_exp(float d) {
   d = fmaxf(d, -80.0f);
   const float t = fmaf(d, kLog2e, kRMagic), n = t - kRMagic;   // n to nearest
@@ -473,7 +473,7 @@ __device__ __noinline__ void rows_stats(const RowsArgs* a, uint32_t cell, float 
 template <bool BF16, bool HAS_U, int KIND, bool POOL, bool PLAIN, int NW>
 __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(const __grid_constant__ RowsArgs a) {
   constexpr bool LISTED = KIND == kRowsResample;
-  constexpr bool SAMPLE = KIND != kRowsRound && !LISTED;   // one kind of row, and no parents
+  constexpr bool ONE_KIND = KIND != kRowsRound && !LISTED;       // of row: either target or draft rows, and no parents
   constexpr bool SUMS = KIND == kRowsVerify || KIND == kRowsStats;   // nothing is drawn
   constexpr int NT = NW * 32;
   constexpr int IDS = BF16 ? 8 : 4;              // ids per lane per piece
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   const DevParams& P = a.P;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   let_next_begin();
-  const int rr = SAMPLE ? 1 : P.r * P.r;
+  const int rr = ONE_KIND ? 1 : P.r * P.r;
   int n_units = a.n_units;
   // LISTED: the unit in work and the one after it are found by going down the positions parent by parent (`found`: how far), 32 at a time.
   uint32_t found = 0;
@@ -626,7 +626,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     const int rem = parent - b * hw;
     ca = rem / P.w;
     cc = rem - ca * P.w;
-    if (!SAMPLE) {
+    if (!ONE_KIND) {
       di = child / P.r;
       dj = child - di * P.r;
     }
@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     per = d / (1.75f * (float)a.margin);  // distance per candidate near the pivot
   };
 
-  bool is_q = LISTED ? (pick & kPickDraft) != 0u : !SAMPLE;   // the row in work is a draft row
+  bool is_q = LISTED ? (pick & kPickDraft) != 0u : !ONE_KIND;   // the row in work is a draft row
   uint32_t g = !LISTED || is_q ? (uint32_t)parent : target_index();   // ... and its index in its tensor
   if (LISTED && left > 0) next_pick();
 
@@ -983,7 +983,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     // ---- the row after this one
     bool nq = false, more = true;
     uint32_t ng = 0;
-    if (SAMPLE) {
+    if (ONE_KIND) {
       more = unit + 1 < u_end;
       ng = more ? g + 1 : g;
     } else if (is_q) {
@@ -1076,7 +1076,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     const bool over = (up ? end >= lim : end <= lim) || n_raw > 64 || n_raw > R - kRSlack;
     const float c0 = EXACT ? ref : -ref * kLog2e, hoff = -pivot * inv_w;
     uint32_t low_a, low_b;
-    Sum s_t = is_q ? pass_one(std::integral_constant<bool, !SAMPLE>{}, n, inv_w, hoff, c0, low_a, low_b)
+    Sum s_t = is_q ? pass_one(std::integral_constant<bool, !ONE_KIND>{}, n, inv_w, hoff, c0, low_a, low_b)
                      : pass_one(std::false_type{}, n, inv_w, hoff, c0, low_a, low_b);
     {
       const bool any_over = __any_sync(kFull, over);
@@ -1327,7 +1327,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
         continue;
         }
       }
-    } else if (!SAMPLE && is_q) {
+    } else if (!ONE_KIND && is_q) {
       tries = 0;
       // ---- a draft row ends here
       c0_q = c0;
@@ -1494,7 +1494,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
       // ---- the decision (Eq. 1 / Eq. 5) and what has to be drawn, the same in every warp
       int pending = kDrawTarget;
       double u_res = 0.0, u_tgt;
-      if (SAMPLE) {
+      if (ONE_KIND) {
         const uint32_t cell = g - (uint32_t)b * (uint32_t)(P.h * P.w);
         const uint4 v = row_philox(make_uint4(cell, (uint32_t)b + P.image_offset, P.round, 1u), make_uint2(P.seed_lo, P.seed_hi));
         u_tgt = uniform24(v.x);
@@ -1540,7 +1540,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
 #pragma unroll 1
       do {
         const bool is_res = (pending & kDrawResidual) != 0;
-        const bool resid = !SAMPLE && is_res && !no_mass;
+        const bool resid = !ONE_KIND && is_res && !no_mass;
         Sum v_t = s_t;
         if (resid) {
           // sum of max(0, p - q) = p - min(p, q); min is not zero only where both rows kept the id
@@ -1742,7 +1742,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
             has = __ballot_sync(kFull, wt > 0.f);
             // (no id with weight: a sum that was rounding noise of a difference -- to the general routines)
             const int chosen = hit ? __ffs(hit) - 1 : has ? 31 - __clz(has) : -1;
-            int32_t* const out = SAMPLE || LISTED ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
+            int32_t* const out = ONE_KIND || LISTED ? a.sample_out + g : (is_res ? a.cand_res : a.cand_tgt) + g;
             if (lane == chosen) *out = (((og * a.ppg + w * 4 + (src >> 3)) << 3) + (src & 7)) * IDS + chosen;
             if (chosen < 0 && lane == 0) defer(g);
           }
