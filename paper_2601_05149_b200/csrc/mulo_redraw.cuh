@@ -19,6 +19,9 @@
 // position -- otherwise the row is drawn again from what is there now.  So a step costs its successor a re-read instead of
 // the whole chain.  Before the wait anything may be rewritten at any moment: ONE thread of the cluster reads the list and tells
 // the others what it found, and every later verdict is one for the whole cluster, so no barrier is ever met by a part of it.
+// Where another kernel runs between two steps nothing overlaps, and drawing ahead only costs (the agreement before the row, the
+// re-read after it: 2.5 us).  64 x 64, 4 images, V = 16384, window 16: 4.7 us a step back to back, 13.3 with a copy of 1.3 us between any
+// two; without drawing ahead 9.9 and 10.5.
 //
 // A step with more positions than clusters is bound by their number instead: after the wait every CTA takes whole rows for itself, by
 // the resident routines, two CTAs to an SM.
