@@ -1228,8 +1228,8 @@ static bool launch_flat(mulo_ctx* ctx, const FlatArgs& s, bool sample, bool res,
 // memory?  That CTA is the sooner done with a row.  us streamed / kept: draft rows, 1024 of 16384 ids: 31 / 45, of 4096: 34 / 25, 576 of 16384:
 // 28 / 28; verified, 784 rows of 16384: 38 / 43, of 4096: 37 / 29, of 8192 fp32: 39 / 36, 1296 rows: 44 / 68, 39 / 41, 38 / 54.
 // How many positions are redrawn is not known here, and few of them are sooner done by a CTA each: all of the grid / 30 / 10 / 3 %
-// of it, 2500 positions of 16384 ids: 124 / 172, 56 / 72, 44 / 43, 40 / 35, of 4096: 64 / 96, 34 / 43, 30 / 29, 28 / 25, of 8192 fp32: 101 / 129,
-// 48 / 55, 42 / 35, 34 / 29; 1296 of 16384: 81 / 100, 48 / 47, 46 / 31, 40 / 29.  So the line lies where 10 % are as quick either way.
+// of it, 2500 positions of 16384 ids: 128 / 173, 60 / 72, 48 / 43, 46 / 35, of 4096: 69 / 96, 36 / 43, 34 / 31, 34 / 25, of 8192 fp32: 101 / 129,
+// 50 / 55, 44 / 36, 38 / 29; 1296 of 16384: 81 / 100, 48 / 47, 46 / 31, 40 / 29.  So the line lies where 10 % are nearly as quick either way.
 static bool many_rows(const mulo_ctx* ctx, int kind, int V, long long rows) {
   const int per_sm = kind == kRowsResample ? 16 : kind == kRowsStats ? (V > 4096 ? 4 : 16) : V >= 12288 ? 4 : 8;
   return !ctx->force_dense && rows > (long long)per_sm * ctx->sm_count;

@@ -508,20 +508,57 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   auto bit_of = [&](const uint32_t* bits, const Place& p) -> bool {
     return bits[((size_t)p.b * P.H + p.i) * Ww + (p.j >> 5)] >> (p.j & 31) & 1u;
   };
-  // the first position of R_X from x on that has `skip` others before it (every warp for itself; there is one)
+  // Blocks of 32 parents of a row (r words of r rows of the mask): how many positions of R_X, the first position, the one past the last.
+  const int nb = (P.w + 31) >> 5, n_blocks = P.B * P.h * nb;
+  const uint32_t row_units = (uint32_t)P.w * (uint32_t)rr;
+  auto count_block = [&](int q) -> int {
+    const int row = q / nb, w0 = (q - row * nb) * P.r, w1 = min(w0 + P.r, Ww);
+    int n = 0;
+    for (int i = 0; i < P.r; ++i)
+      for (int w = w0; w < w1; ++w) {
+        uint32_t v = a.expand_bits[((size_t)row * P.r + i) * Ww + w];
+        if (w == Ww - 1 && (P.W & 31)) v &= (1u << (P.W & 31)) - 1u;   // (bits past the row's end do not count)
+        n += __popc(v);
+      }
+    return n;
+  };
+  auto block_start = [&](int q) -> uint32_t {
+    const int row = q / nb;
+    return (uint32_t)row * row_units + (uint32_t)(q - row * nb) * 32u * (uint32_t)rr;
+  };
+  auto block_end = [&](int q) -> uint32_t {
+    const int row = q / nb;
+    return (uint32_t)row * row_units + (uint32_t)min(P.w, (q - row * nb + 1) * 32) * (uint32_t)rr;
+  };
+  // the first position of R_X from x on, which lies in block `q_at` or at its end, that has `skip` others of the block before it (every
+  // warp for itself; there is one)
+  int q_at = 0;
+  uint32_t e_at = 0;
   auto find_pick = [&](uint32_t x, int skip) -> uint32_t {
 #pragma unroll 1
-    for (; x < n_at; x += 32) {
-      const uint32_t mine = x + (uint32_t)lane;
-      uint32_t hit = __ballot_sync(kFull, mine < n_at && bit_of(a.expand_bits, place_of(min(mine, n_at - 1u))));
-      const int n = __popc(hit);
-      if (skip < n) {
-        for (; skip > 0; --skip) hit &= hit - 1u;
-        return x + (uint32_t)__ffs(hit) - 1u;
+    for (;;) {
+#pragma unroll 1
+      for (; x < e_at; x += 32) {
+        const uint32_t mine = x + (uint32_t)lane;
+        uint32_t hit = __ballot_sync(kFull, mine < e_at && bit_of(a.expand_bits, place_of(min(mine, e_at - 1u))));
+        const int n = __popc(hit);
+        if (skip < n) {
+          for (; skip > 0; --skip) hit &= hit - 1u;
+          return x + (uint32_t)__ffs(hit) - 1u;
+        }
+        skip -= n;
       }
-      skip -= n;
+      unsigned some = 0;   // the next block that is not empty, 32 at a time
+#pragma unroll 1
+      for (++q_at; q_at < n_blocks; q_at += 32) {
+        some = __ballot_sync(kFull, q_at + lane < n_blocks && count_block(min(q_at + lane, n_blocks - 1)) > 0);
+        if (some) break;
+      }
+      if (!some) return n_at - 1u;
+      q_at += __ffs(some) - 1;
+      x = block_start(q_at);
+      e_at = block_end(q_at);
     }
-    return n_at - 1u;
   };
   if constexpr (LISTED) {
     // x~ where nothing is drawn; of what is drawn, what the general routines report of a position
@@ -538,19 +575,10 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
         if (!(zq >= st[0]) || row_exp((double)zq - (double)st[1]) / ((double)st[2] + (double)st[3]) <= 0.0) atomicOr(a.dev_status, MULO_DEV_ZERO_DRAFT_PROB);
       }
     }
-    // how many positions R_X has, and which is this CTA's first: rows of parents, a run of them per thread
-    const int n_rows = P.B * P.h, per = (n_rows + NT - 1) / NT, r0 = min(n_rows, tid * per), r1 = min(n_rows, r0 + per), words = P.r * Ww;
-    auto count_row = [&](int row) -> int {
-      int n = 0;
-      for (int w = 0; w < words; ++w) {
-        uint32_t v = a.expand_bits[(size_t)row * words + w];
-        if (w % Ww == Ww - 1 && (P.W & 31)) v &= (1u << (P.W & 31)) - 1u;   // (bits past the row's end do not count)
-        n += __popc(v);
-      }
-      return n;
-    };
+    // how many positions R_X has, and which is this CTA's first: a run of blocks per thread
+    const int per = (n_blocks + NT - 1) / NT, q0 = min(n_blocks, tid * per), q1 = min(n_blocks, q0 + per);
     int mine = 0;
-    for (int row = r0; row < r1; ++row) mine += count_row(row);
+    for (int q = q0; q < q1; ++q) mine += count_block(q);
     int inc = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -567,9 +595,9 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
     }
     const int first = (int)(((long long)n_units * blockIdx.x) / gridDim.x);
     if (first >= inc - mine && first < inc) {   // (one thread, unless there is nothing to do)
-      int row = r0, skip = first - (inc - mine);
-      for (int n = count_row(row); skip >= n; n = count_row(++row)) skip -= n;
-      sm.n_sa = (unsigned)row;
+      int q = q0, skip = first - (inc - mine);
+      for (int n = count_block(q); skip >= n; n = count_block(++q)) skip -= n;
+      sm.n_sa = (unsigned)q;
       sm.wmax[0] = (unsigned)skip;
     }
     __syncthreads();
@@ -578,7 +606,9 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
   const int u_end = (int)(((long long)n_units * (blockIdx.x + 1)) / gridDim.x);
   if (unit >= u_end) return;
   if constexpr (LISTED) {
-    found = find_pick(sm.n_sa * (uint32_t)(P.w * rr), (int)sm.wmax[0]);
+    q_at = (int)sm.n_sa;
+    e_at = block_end(q_at);
+    found = find_pick(block_start(q_at), (int)sm.wmax[0]);
     __syncthreads();
   }
   const uint32_t row_bytes = a.row_bytes;

@@ -242,11 +242,13 @@ def test_rows_that_the_stages_leave(ctx, tied, over):
     pu.check_round(cfg, pu.finish_outputs(o, W), pu.oracle_images(cfg, batch, list(range(B))))
 
 
-@pytest.mark.parametrize("over", [dict(), dict(B=3, H=30, W=37, r=1, V=1024, top_k=100), dict(B=5, H=48, W=45, r=3, radius=2)],
+@pytest.mark.parametrize("over", [dict(), dict(B=3, H=30, W=37, r=1, V=1024, top_k=100), dict(B=5, H=48, W=45, r=3, radius=2),
+                                  dict(B=5, H=3, W=1500, r=3, V=1024, top_k=100)],
                          ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "plain")
-@pytest.mark.parametrize("density", [0.0, 0.0005, 0.02, 0.5, 1.0])
+@pytest.mark.parametrize("density", [0.0, 0.0005, 0.02, 0.5, 1.0, "ends"])
 def test_redraw_of_any_share_of_the_grid(ctx, over, density):
-    """The streamed redraw finds the positions of R_X by itself: none, one or two, some, all; bits past a row's end count as nothing."""
+    """The streamed redraw finds the positions of R_X by itself: none, one or two, some, all; bits past a row's end count as nothing.  "ends": all of the
+    first and of the last image, nothing between."""
     cfg = dataclasses.replace(STAGES, resample_mode=binding.RESAMPLE_MIXED, **over)
     batch = pu.build_batch(cfg)
     pu.redraw_tokens(cfg, batch)
@@ -254,7 +256,9 @@ def test_redraw_of_any_share_of_the_grid(ctx, over, density):
     ctx.ensure_workspace(p)
     B, H, W = cfg.B, cfg.H, cfg.W
     g = torch.Generator(device="cuda").manual_seed(77)
-    hits = torch.rand((B, H, (W + 31) // 32, 32), generator=g, device="cuda") < density
+    hits = torch.rand((B, H, (W + 31) // 32, 32), generator=g, device="cuda") < (1.0 if density == "ends" else density)
+    if density == "ends":
+        hits[1:B - 1] = False
     if density == 0.0005:
         hits.view(-1)[:] = False
         hits[B - 1, H - 1, (W - 1) // 32, (W - 1) % 32] = True
