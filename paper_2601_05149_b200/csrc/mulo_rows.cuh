@@ -1732,7 +1732,7 @@ __global__ void __launch_bounds__(NW * 32, rows_warps(KIND) / NW) k_round_rows(c
               if constexpr (LISTED) t = warp_sum(v);
               else t = __reduce_add_sync(kFull, v);
               if (t > 0) last_w = w;
-              if (seek ? w == last_w : t > 0 && y < t) break;
+              if (seek ? w == last_w : y < t && (!LISTED || t > 0)) break;   // (in double y may be a rounding below 0)
               if (y != past) y -= t;
               next_word();
               if (++w == w1) {
